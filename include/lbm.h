@@ -112,14 +112,18 @@ typedef struct {
                                FP32 phase of a mixed run then hands the instance to the
                                FP64 phase (which ignores it).  0 = never.  Default 200
                                for the mixed precisions, 0 for LBM_FP64 */
-    int32_t pcg_kernel;     /* potential-solve kernel: 0 (default) chooses; 1 the
-                               grid-wide kernel (one CTA for small work, else a
-                               cooperative grid); 2 prefers one thread-block cluster
-                               per group of systems (taken when the batch has a
-                               multiple of 4, at least 16 instances, FP32 work vectors
-                               and z of a cluster's systems fits its shared memory;
-                               otherwise as 1).  0 takes 2 where it qualifies.
-                               Results agree to rounding, not bit for bit */
+    int32_t pcg_kernel;     /* potential-solve kernel: 0 (default) chooses; 1 Jacobi-
+                               preconditioned CG, grid-wide kernel (one CTA for small
+                               work, else a cooperative grid); 2 the same iteration
+                               with one thread-block cluster per group of systems
+                               (taken when the batch has a multiple of 4, at least 16
+                               instances, FP32 work vectors and z of a cluster's
+                               systems fits its shared memory; otherwise as 1).
+                               0 on a Kuhn cube: fast diagonalisation with iterative
+                               refinement to the same residual tests (each iteration
+                               of the counters is one refinement step, at least one a
+                               solve); on a general mesh 2 where it qualifies, else 1.
+                               Results agree to the solves' tolerance */
     int32_t use_graphs;     /* 1 (default): each chunk of check_every iterations is
                                captured once as a CUDA graph (per batch, options and
                                mesh operators) and replayed; the first chunk of a solve

@@ -86,6 +86,8 @@ struct Mesh {
     std::vector<void*> hm_mem;                // its device allocations
     ShellDev* shell = nullptr;                // space-transformation boundary (lbm_mesh_shell), or null
     std::vector<void*> shell_mem;             // its device allocations
+    FastDev* fast = nullptr;                  // fast-diagonalisation tables (Kuhn cubes), or null
+    void* fast_mem = nullptr;                 // their device allocation
     float *tcA = nullptr, *tcAT = nullptr;   // padded FP32 B and B^T for the tensor-core path (lazy)
     // general meshes (lbm_mesh_upload; n == 0)
     bool gen = false;
@@ -105,6 +107,7 @@ struct Mesh {
         v.B64 = B64; v.B32 = B32; v.B32lo = B32lo;
         v.hm = hm;
         v.shell = shell;
+        v.fast = fast;
         v.vsum = gen ? vsum : 24.0 * (double)n * n * n;
         v.cell = cell;
         v.gen = gen ? 1 : 0;
@@ -188,7 +191,12 @@ struct lbm_ctx {
     cudaStream_t cap_stream = nullptr;      // where chunks are captured (lazy)
     ChunkGraph* capturing = nullptr;        // the chunk being captured (profiling events become nodes)
     int64_t graph_stats[3] = {0, 0, 0};     // replays, captures, captures refused
-    Launch launch() { return Launch{stream, num_sms, bar, err, &launches, sweeps, fin, 0}; }
+    bool wait_test = false;                 // lbm_set_wait_limit's hook: solves take kernels with a grid barrier
+    Launch launch() {
+        Launch L{stream, num_sms, bar, err, &launches, sweeps, fin, 0};
+        L.wait_test = wait_test;
+        return L;
+    }
 };
 
 namespace {
@@ -264,7 +272,7 @@ void prof_harvest(lbm_ctx* ctx) {
 // Byte offsets of the per-instance arrays inside one allocation; every array
 // starts on a 256-byte boundary (the PCG reads 8- and 16-byte vectors).
 struct VecLayout {
-    size_t m, g, hout, U1, U2, r, z, p, q, ub_in, ub_out, bem_part, m32, bvec, shx, total;
+    size_t m, g, hout, U1, U2, r, z, p, q, ub_in, ub_out, bem_part, m32, bvec, fs, fs_bytes, shx, total;
 };
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -291,6 +299,14 @@ VecLayout vec_layout(const Mesh& M, int B, int tsize) {
     L.bem_part = take(8 * (32 * nb > df ? 32 * nb : df));
     L.m32 = tsize == 4 ? take(4 * N * 3 * B) : 0;
     L.bvec = take(8 * N * B);
+    // transformed planes of the fast solves of large cubes (FP64 batches: plain and
+    // mixed iterations share the room)
+    L.fs_bytes = 0;
+    if (M.fast) {
+        L.fs_bytes = C * 4 * fast_scratch_words(M.n, 4);
+        if (tsize == 8) L.fs_bytes = std::max(L.fs_bytes, C * 8 * fast_scratch_words(M.n, 8));
+    }
+    L.fs = take(L.fs_bytes);
     // space-transformation boundary: grid potential and CG vectors, FP64 in every mode
     L.shx = M.shell ? take(8 * 6 * (size_t)M.shell->Ng * B) : 0;
     L.total = o;
@@ -318,6 +334,7 @@ BatchView<T> batch_view(const lbm_ctx* ctx, const Mesh& M, const Inst& I, bool w
     v.bem_part = (T*)(base + L.bem_part);
     v.m32 = sizeof(T) == 4 ? (float*)(base + L.m32) : nullptr;
     v.bvec = (double*)(base + L.bvec);
+    v.fs = L.fs_bytes ? (void*)(base + L.fs) : nullptr;
     v.shx = M.shell ? (double*)(base + L.shx) : nullptr;
     v.part = I.part;
     v.st = I.st;
@@ -385,12 +402,65 @@ void free_shell(Mesh* m) {
 void free_mesh(Mesh* m) {
     free_hm(m);
     free_shell(m);
+    if (m->fast_mem) cudaFree(m->fast_mem);
+    delete m->fast;
     void* ptrs[] = {m->rowptr, m->col, m->pkA, m->pkB, m->node, m->bidx, m->tris, m->inc_ptr, m->inc_slot,
                     m->kptr, m->kent, m->B64, m->B32, m->B32lo, m->tcA, m->tcAT, m->tets, m->xyz, m->gA64, m->gB64,
                     m->gA32, m->gB32, m->gk64, m->gV, m->gd64, m->gk32, m->gd32};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete m;
+}
+
+// The fast-diagonalisation tables of a Kuhn cube (fast_solve.cu).
+int fast_upload(lbm_ctx* ctx, Mesh* M) {
+    FastTables t;
+    fast_tables(M->n, t);
+    const size_t nm = t.mat.size(), ni = 2 * t.inv, nr = t.lam_row.size(), nc = t.lam_col.size();
+    const size_t ne = 12 * (size_t)M->n - 4, ne2 = ne * ne;
+    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const size_t o_i64 = up(8 * nm), o_m32 = o_i64 + up(8 * ni), o_i32 = o_m32 + up(4 * nm), o_r = o_i32 + up(4 * ni),
+                 o_c = o_r + up(8 * nr), o_e64 = o_c + up(8 * nc), o_e32 = o_e64 + up(8 * ne2),
+                 total = o_e32 + up(4 * ne2);
+    CK(cudaMalloc(&M->fast_mem, total));
+    char* base = (char*)M->fast_mem;
+    const std::vector<float> m32(t.mat.begin(), t.mat.end());
+    cudaStream_t st = ctx->stream;
+    CK(cudaMemcpyAsync(base, t.mat.data(), 8 * nm, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(base + o_m32, m32.data(), 4 * nm, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(base + o_r, t.lam_row.data(), 8 * nr, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(base + o_c, t.lam_col.data(), 8 * nc, cudaMemcpyHostToDevice, st));
+    launch_fast_inv(M->n, (const double*)(base + o_r), (const double*)(base + o_c), (double*)(base + o_i64),
+                    (float*)(base + o_i32), st);
+    ctx->launches += 2;
+    {   // the correction of the cube's edges
+        std::vector<double> A, X(ne2), H;
+        fast_edge_system(M->n, A);
+        double* w = nullptr;   // A, T1, T2; X in H's place
+        CK(cudaMalloc(&w, 3 * 8 * ne2));
+        cudaError_t e = cudaMemcpyAsync(w, A.data(), 8 * ne2, cudaMemcpyHostToDevice, st);
+        launch_inverse_newton((int)ne, w, (double*)(base + o_e64), w + ne2, w + 2 * ne2, st);
+        ctx->launches += 9;
+        if (e == cudaSuccess) e = cudaMemcpyAsync(X.data(), base + o_e64, 8 * ne2, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        cudaFree(w);
+        CK(e);
+        fast_edge_matrix(M->n, X, H);
+        const std::vector<float> h32(H.begin(), H.end());
+        CK(cudaMemcpyAsync(base + o_e64, H.data(), 8 * ne2, cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(base + o_e32, h32.data(), 4 * ne2, cudaMemcpyHostToDevice, st));
+        CK(cudaStreamSynchronize(st));
+    }
+    CK(cudaGetLastError());
+    M->fast = new FastDev();
+    M->fast->mat64 = (const double*)base;
+    M->fast->inv64 = (const double*)(base + o_i64);
+    M->fast->mat32 = (const float*)(base + o_m32);
+    M->fast->inv32 = (const float*)(base + o_i32);
+    M->fast->edge64 = (const double*)(base + o_e64);
+    M->fast->edge32 = (const float*)(base + o_e32);
+    M->bytes += total;
+    return LBM_OK;
 }
 
 void free_inst(Inst* I) {
@@ -532,7 +602,8 @@ int run_chunk(lbm_ctx* ctx, const Launch& L, const Mesh& M, Inst* I, const Batch
     {
         // the launch shape of the cluster potential solves (it follows the active
         // instances; querying it here also caches its occupancy before a capture)
-        const int64_t shape = pcg_cluster_shape(L, M.view(), I->B, sizeof(T) == 8, o.cg_mixed_iter != 0);
+        int64_t shape = fast_shape(L, M.view(), I->B, sizeof(T) == 8, o.cg_mixed_iter != 0);
+        if (!shape) shape = pcg_cluster_shape(L, M.view(), I->B, sizeof(T) == 8, o.cg_mixed_iter != 0);
         const int64_t k[10] = {chunk, (int64_t)sizeof(T), I->B, (int64_t)(intptr_t)M.hm, (int64_t)(intptr_t)M.B32lo,
                                (int64_t)(intptr_t)M.tcA, ctx->prof ? 1 : 0, (int64_t)(intptr_t)V.m,
                                (int64_t)(intptr_t)M.shell, shape};
@@ -981,7 +1052,11 @@ int lbm_mesh_cube(lbm_ctx* ctx, double cell_m, int32_t n, lbm_mesh* out) {
     cleanup();
     cnt = bflag = bpos = nullptr;
 #undef CKM
-    M->bytes = sizeof(int) * ((size_t)3 * N + 2 + 3 * (size_t)M->nnz + M->nnzK + M->nb + tris.size() +
+    if (int rc = fast_upload(ctx, M)) {
+        free_mesh(M);
+        return rc;
+    }
+    M->bytes += sizeof(int) * ((size_t)3 * N + 2 + 3 * (size_t)M->nnz + M->nnzK + M->nb + tris.size() +
                               incp.size() + incs.size()) + 12 * nb2;
     const int64_t id = ctx->next_id++;
     ctx->meshes[id] = M;
@@ -2047,7 +2122,7 @@ extern "C" int lbm_evaluate_noalloc(lbm_ctx* ctx, lbm_mesh mesh, const lbm_mater
     // what must start at zero: the potentials (cold start), barrier, error word, counters
     CK(cudaMemsetAsync(U1, 0, sizeof(double) * 2 * N, s));
     CK(cudaMemsetAsync(U2, 0, sizeof(double) * 2 * N, s));
-    CK(cudaMemsetAsync(bar, 0, sizeof(unsigned), s));
+    CK(cudaMemsetAsync(bar, 0, 4 * sizeof(unsigned), s));
     CK(cudaMemsetAsync(err, 0, 4 * sizeof(int), s));
     CK(cudaMemcpyAsync(err + 1, ctx->err + 1, 2 * sizeof(int), cudaMemcpyDeviceToDevice, s));
     CK(cudaMemsetAsync(sweeps, 0, 4 * sizeof(unsigned long long), s));
@@ -2086,6 +2161,7 @@ extern "C" int lbm_evaluate_noalloc(lbm_ctx* ctx, lbm_mesh mesh, const lbm_mater
     V.m32 = nullptr;   // FP64 evaluation: no FP32 copy of the trial point
     V.bvec = bv;
     Launch L{s, ctx->num_sms, bar, err, &ctx->launches, sweeps, fin, 0};
+    L.wait_test = ctx->wait_test;
     L.tune = false;   // no waiting inside this call (and it may be captured)
     const MeshView mv = M->view();
     lbm_solve_opts oo = o;
@@ -2119,6 +2195,7 @@ extern "C" int lbm_set_wait_limit(lbm_ctx* ctx, double seconds, int32_t unreacha
     const int cfg[2] = {(int)llround(seconds * 1e3), unreachable ? 1 : 0};
     CK(cudaStreamSynchronize(ctx->stream));
     CK(cudaMemcpy(ctx->err + 1, cfg, sizeof cfg, cudaMemcpyHostToDevice));
+    ctx->wait_test = unreachable != 0;
     return LBM_OK;
     LBM_CATCH
 }

@@ -172,6 +172,28 @@ struct ShellDev {
     const int* magnet = nullptr;       // N: grid node of every magnet node
 };
 
+// Tables of the fast-diagonalisation solves on a Kuhn cube (fast_solve.cu): per
+// kind (0 Neumann, 1 Dirichlet) the 1-D transform matrices and 1 / eigenvalues.
+struct FastDev {
+    const double *mat64 = nullptr, *inv64 = nullptr, *edge64 = nullptr;
+    const float *mat32 = nullptr, *inv32 = nullptr, *edge32 = nullptr;   // edge: H of the edge nodes
+};
+struct FastTables {
+    int words = 0, ldx = 0;            // words of one kind's matrices; row length of a sheet
+    size_t inv = 0;                    // words of one kind's 1 / eigenvalues
+    std::vector<double> mat, lam_row, lam_col;   // [2 kinds]
+};
+void fast_tables(int n, FastTables& t);
+// Correction of the edge nodes: A = 1 + R E, and H = E - E X with X = A^-1 (host,
+// ne x ne row-major, ne = 12 n - 4); launch_inverse_newton: X = A^-1 on the device for
+// an A near 1 (spectral radius of 1 - A at most 1/3), T1 and T2 scratch of the same size
+void fast_edge_system(int n, std::vector<double>& A);
+void fast_edge_matrix(int n, const std::vector<double>& X, std::vector<double>& H);
+void launch_inverse_newton(int n, const double* A, double* X, double* T1, double* T2, cudaStream_t st);
+void launch_fast_inv(int n, const double* lam_row, const double* lam_col, double* inv64, float* inv32, cudaStream_t st);
+// words of global scratch per system (0: none needed) with CG vectors of `word` bytes
+size_t fast_scratch_words(int n, size_t word);
+
 // ---- device view of one mesh --------------------------------------------------------
 struct MeshView {
     int n, N, nb, nnz, F;
@@ -188,6 +210,7 @@ struct MeshView {
     const float* B32lo;  // nb x nb: fp32(B64 - B32), for the FP64-accurate batched product (null: not built)
     const HMDevice* hm = nullptr;   // host pointer: the hierarchical form, when built (lbm_mesh_hmatrix)
     const ShellDev* shell = nullptr;   // host pointer: the space-transformation boundary, when attached
+    const FastDev* fast = nullptr;     // host pointer: fast-diagonalisation tables (Kuhn cubes)
     double vsum;         // sum_i Vint_i = 24 n^3 (general meshes: sum of gV)
     double cell;         // cell edge h (m); general meshes: the length unit L
     // General meshes (gen != 0): the same tables as FP64/FP32 values in the same
@@ -222,6 +245,7 @@ struct BatchView {
     double* hout;              // optional [N][3][B] effective field (nullable)
     float* m32 = nullptr;      // FP32 batches: [N][3][B] FP32 copy of the trial point (else null)
     double* bvec = nullptr;    // [N][B] divergence right-hand side b = G m at the trial point (rhs_eval)
+    void* fs = nullptr;        // transformed planes of the fast solves of large cubes (fast_scratch_words)
     double* shx = nullptr;     // [6][Ng][B] FP64 grid potential and five CG work vectors (space-transformation boundary)
 };
 
@@ -235,6 +259,7 @@ struct Launch {
     double* fin;                 // device scratch for grid reductions (>= 4 * 512 doubles)
     int max_blocks;              // cap on the cooperative PCG grid (0: one block per SM)
     bool tune = true;            // launch-shape autotuning allowed (it waits on events)
+    bool wait_test = false;      // solves must take a kernel with a grid barrier (lbm_set_wait_limit's test hook)
     int pcg_kernel = 0;          // 0 choose, 1 grid-wide kernel, 2 prefer clusters (lbm_solve_opts)
     // host flags [B]: the instances iterating at the start of the chunk (null: all);
     // the cluster potential solves size their launch to the groups still active
@@ -243,6 +268,13 @@ struct Launch {
 // The shape the cluster potential solves take for this launch (CPC * 100 + CL;
 // 0: the grid-wide kernel), from the active flags of L.
 int pcg_cluster_shape(const Launch& L, const MeshView& M, int B, bool fp64, bool mixed_iter);
+// The same for the fast-diagonalisation solves (0: they do not take this launch).
+int64_t fast_shape(const Launch& L, const MeshView& M, int B, bool fp64, bool mixed_iter);
+// CG preconditioned by fast diagonalisation on Kuhn cubes (fast_solve.cu): 1 when
+// launched (*err its status), 0 when it does not qualify.
+template <typename T>
+int fast_solve(const Launch& L, const MeshView& M, const BatchView<T>& V, int mode, double tol, int max_iter,
+               bool mixed_iter, cudaError_t* err);
 
 // u2_S = B_H u1_S and c_S = B_H^T t_S on the [nb][2B] surface arrays (forward
 // columns [0, B), adjoint columns [B, 2B)) with the hierarchical form of B

@@ -599,6 +599,9 @@ static cudaError_t dispatch_pcg(const Launch& L, const MeshView& M, PcgArgs<T>& 
 template <typename T>
 int pcg_solve(const Launch& L, const MeshView& M, const BatchView<T>& V, int mode, double tol, int max_iter,
               bool mixed_iter) {
+    // Kuhn cubes, unless the caller asks for one of the diagonally preconditioned kernels
+    cudaError_t fe;
+    if (fast_solve<T>(L, M, V, mode, tol, max_iter, mixed_iter, &fe)) return fe == cudaSuccess ? 0 : (int)fe;
     if (L.pcg_kernel != 1) {
         cudaError_t ce;
         if (pcg_solve_cluster<T>(L, M, V, mode, tol, max_iter, mixed_iter, &ce)) return ce == cudaSuccess ? 0 : (int)ce;
