@@ -307,8 +307,9 @@ VecLayout vec_layout(const Mesh& M, int B, int tsize) {
         if (tsize == 8) L.fs_bytes = std::max(L.fs_bytes, C * 8 * fast_scratch_words(M.n, 8));
     }
     L.fs = take(L.fs_bytes);
-    // space-transformation boundary: grid potential and CG vectors, FP64 in every mode
-    L.shx = M.shell ? take(8 * 6 * (size_t)M.shell->Ng * B) : 0;
+    // space-transformation boundary: the FP64 grid potential and seven CG vectors, FP32
+    // ones in the room of five FP64 ones in FP32 batches
+    L.shx = M.shell ? take(8 * (tsize == 8 ? 8 : 6) * (size_t)M.shell->Ng * B) : 0;
     L.total = o;
     return L;
 }
@@ -1513,6 +1514,7 @@ int lbm_mesh_shell(lbm_ctx* ctx, lbm_mesh mesh, int32_t a, int32_t s, int64_t in
     std::vector<unsigned char> kind(Ng, 1);
     std::vector<int> gnode(Ng, -1);
     for (int v : G.outer) kind[v] = 0;
+    double bound = 0.0;   // of the eigenvalues of D^-1 K (Gershgorin; 4 for linear tetrahedra)
     for (size_t i = 0; i < G.magnet.size(); ++i) gnode[G.magnet[i]] = (int)i;
     for (int r = 0; r < Ng; ++r) {
         if (kind[r] == 0) continue;
@@ -1529,6 +1531,9 @@ int lbm_mesh_shell(lbm_ctx* ctx, lbm_mesh mesh, int32_t a, int32_t s, int64_t in
         }
         if (!(c[0] > 0.0)) return fail(LBM_E_INVALID, "lbm_mesh_shell: stiffness without a positive diagonal");
         c[15] = 1.0 / c[0];
+        double sum = 0.0;
+        for (int k = 0; k < 15; ++k) sum += fabs(c[k]);
+        bound = std::max(bound, sum * c[15]);
         for (int k = 7; k < 15; ++k)
             if (c[k] != 0.0) kind[r] = 2;
     }
@@ -1545,6 +1550,7 @@ int lbm_mesh_shell(lbm_ctx* ctx, lbm_mesh mesh, int32_t a, int32_t s, int64_t in
     };
     S->Ng = Ng;
     S->n1 = n1;
+    S->jac_bound = (float)std::min(4.0, bound * (1.0 + 1e-6));
     S->coef64 = (const double*)up(c64.data(), sizeof(double) * c64.size());
     S->coef32 = (const float*)up(c32.data(), sizeof(float) * c32.size());
     S->kind = (const unsigned char*)up(kind.data(), kind.size());
@@ -2373,10 +2379,10 @@ size_t group_estimate(int n, int slots, int shell_a, int shell_s) {
     const size_t nb = N - (size_t)(n > 1 ? (n - 1) * (n - 1) * (n - 1) : 0);
     size_t mesh = 12 * nb * nb + 100 * N;
     size_t per_slot = 8 * (2 * N * 3 * 2 + 3 * N) * 2 + (4 + 8) * (12 * N + 4 * nb) + 40 * N;
-    if (shell_a > 0) {   // the grid's stencil records and, per slot, its six FP64 vectors in both batches
+    if (shell_a > 0) {   // the grid's stencil records and, per slot, its FP64 vectors in both batches
         const size_t g1 = (size_t)n + 2 * ((size_t)shell_a + shell_s) + 1, Ng = g1 * g1 * g1;
         mesh += (16 * 12 + 9) * Ng;
-        per_slot += 2 * 6 * 8 * Ng;
+        per_slot += (6 + 8) * 8 * Ng;
     }
     return mesh + per_slot * slots + ((size_t)64 << 20);
 }

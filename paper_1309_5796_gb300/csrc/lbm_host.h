@@ -165,6 +165,7 @@ std::string host_shell_setup(int n, int a, int s, double cell, ShellGrid& G);
 // -(x+y+z), 1/K_ii} (zeros on the outer face).
 struct ShellDev {
     int Ng = 0, n1 = 0;                // grid nodes, grid nodes a side
+    float jac_bound = 4.f;             // bound of the eigenvalues of D^-1 K
     const float* coef32 = nullptr;     // [Ng][16], rounded to FP32
     const double* coef64 = nullptr;    // [Ng][16]
     const unsigned char* kind = nullptr;   // Ng: 0 outer face, 1 seven-point row (M = I), 2 fifteen-point row
@@ -246,7 +247,7 @@ struct BatchView {
     float* m32 = nullptr;      // FP32 batches: [N][3][B] FP32 copy of the trial point (else null)
     double* bvec = nullptr;    // [N][B] divergence right-hand side b = G m at the trial point (rhs_eval)
     void* fs = nullptr;        // transformed planes of the fast solves of large cubes (fast_scratch_words)
-    double* shx = nullptr;     // [6][Ng][B] FP64 grid potential and five CG work vectors (space-transformation boundary)
+    double* shx = nullptr;     // [Ng][B] FP64 grid potential, then seven CG work vectors (space-transformation boundary)
 };
 
 struct Launch {

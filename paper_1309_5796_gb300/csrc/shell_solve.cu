@@ -8,9 +8,10 @@
 // exactly the gradient field of the stray-field energy (no boundary matrix, no
 // adjoint chain).  The host set-up (csrc/shell.cu) builds the grid and its
 // stiffness; here the solve runs on the device for all instances of a batch
-// at once: Jacobi-preconditioned CG, one persistent cooperative kernel per
-// solve (grid barriers with the context's time limit), the grid potential
-// warm-started from the instance's previous solve.
+// at once: CG with a Chebyshev polynomial of the Jacobi-scaled matrix as
+// preconditioner, one persistent cooperative kernel per solve (grid barriers with
+// the context's time limit), the grid potential warm-started from the instance's
+// previous solve.
 //
 // Every row that is not on the outer face is an interior node of the grid, and
 // the Kuhn split couples a node only to the 14 neighbours along +-x, +-y, +-z,
@@ -33,7 +34,7 @@ struct ShellArgs {
     const InstState* st;
     const double* bvec;           // [N][B] divergence right-hand side of the magnet
     double* x;                    // [Ng][B] FP64 grid potential
-    W *r, *z, *p, *q, *d;         // [Ng][B] work vectors (d: this solve's correction of x)
+    W *r, *z, *z2, *dd, *p, *q, *d;   // [Ng][B] work vectors (d: this solve's correction of x)
     double tol2;
     int max_iter;
     unsigned* bar;
@@ -63,8 +64,9 @@ template <> struct CoefLoad<double> {
     }
 };
 
-// VEC consecutive values (instances c0 .. c0+VEC-1 of one row), L2-only loads
-// (CG) for values other blocks write during the kernel.
+// VEC consecutive values (instances c0 .. c0+VEC-1 of one row).  Values that other
+// blocks wrote are read after a grid barrier, whose acquire makes plain loads (and so
+// the L1, which serves a product's neighbours) see them; CG: past the L1.
 template <int VEC, bool CG, typename W>
 __device__ __forceinline__ void ldv(W (&d)[VEC], const W* p) {
     if constexpr (VEC == 1) {
@@ -109,7 +111,7 @@ __device__ __forceinline__ void kuhn_apply(const C (&c)[16], const V* v, ptrdiff
 #pragma unroll
     for (int j = 0; j < 7; ++j) {
         V t[VEC];
-        ldv<VEC, true>(t, v + off[j]);
+        ldv<VEC, false>(t, v + off[j]);
 #pragma unroll
         for (int k = 0; k < VEC; ++k) w[k] += R(c[j]) * R(t[k]);
     }
@@ -117,12 +119,15 @@ __device__ __forceinline__ void kuhn_apply(const C (&c)[16], const V* v, ptrdiff
 #pragma unroll
         for (int j = 7; j < 15; ++j) {
             V t[VEC];
-            ldv<VEC, true>(t, v + off[j]);
+            ldv<VEC, false>(t, v + off[j]);
 #pragma unroll
             for (int k = 0; k < VEC; ++k) w[k] += R(c[j]) * R(t[k]);
         }
     }
 }
+
+constexpr int SH_DEG = 8;             // products of a CG iteration
+constexpr double SH_RATIO = 60.0;     // of the polynomial's interval
 
 // Threads hold VEC consecutive instances of one row: thread tid works on
 // instances c0 = (tid % G) VEC .. c0 + VEC - 1 (G = B / VEC) of row lane tid / G.
@@ -135,9 +140,19 @@ __device__ __forceinline__ void kuhn_apply(const C (&c)[16], const V* v, ptrdiff
 //     FP64 residual f - K x, FP32 CG until it has reduced that residual by
 //     MP_INNER (or met the tolerance), x += d; the solve ends on the FP64
 //     residual test (restarted CG, as the magnet's mixed-iteration solves).
-// Per CG iteration (the same fused form as the magnet's solves):
-//   A: w = K z, p = z + beta p, q = w + beta q (= K p), partial p.q
-//   B: alpha = rho / p.q, d += alpha p, r -= alpha q, z = r / K_ii, partials r.z, r.r
+// Per CG iteration:
+//   B: alpha = rho / p.q, d += alpha p, r -= alpha q, z = dd = D^-1 r / theta, r.r
+//   C: SH_DEG - 1 steps dd = c1 dd + c2 D^-1 (r - K z), z' = z + dd; r.z with the last
+//   A: w = K z, p = z + beta p, q = w + beta q (= K p), p.q
+// The polynomial is Chebyshev's on [b / 60, b], b a bound of the eigenvalues of
+// D^-1 K: on the 54^3-cell grid 51 iterations of eight products where Jacobi-CG
+// takes 358 of one, and a product with its step moves 5 vector words and one
+// barrier where a CG iteration moves 12 and four.  (Multigrid and fast
+// diagonalisation stall on the shell's growing tangential stiffness.)
+// Measured on that grid: 32 instances 14.9 ms a solve, before 24.1; one 3.0, before 5.7.
+// Every block has one run of consecutive rows, so that the L1 serves a product's
+// neighbours along x and y and about three of its fifteen reads go to L2 (with
+// rows dealt round all blocks and loads past the L1, all fifteen did).
 // Outer-face rows keep zero in every vector (and 1/K_ii = 0 there), so they
 // drop out of every product.
 template <typename W, bool RES64, int THREADS, int VEC>
@@ -149,9 +164,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
     const bool lane = tid < RB * G;
     const int g = tid % G, c0 = g * VEC, rl = tid / G;
     const int nrow = (G <= 32 && (32 % G) == 0) ? (bd >> 5) : RB;
-    double* scratch = sm;                          // [4][nrow][B] doubles (or floats in the same room)
-    double* out = scratch + 4 * (size_t)nrow * B;  // [4][B]
-    double* s_rho = out + 4 * B;
+    double* scratch = sm;                          // [2][nrow][B] doubles (or floats in the same room)
+    double* out = scratch + 2 * (size_t)nrow * B;  // [2][B]
+    double* s_rho = out + 2 * B;
     double* s_rhop = s_rho + B;
     double* s_ab = s_rhop + B;
     double* s_tol = s_ab + B;
@@ -177,190 +192,217 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
     const W* coefW;
     if constexpr (std::is_same<W, double>::value) coefW = A.S.coef64;
     else coefW = A.S.coef32;
-    const int row0 = blockIdx.x * RB + rl, rstride = gridDim.x * RB;
+    const int rpb = (Ng + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int rlo = (int)blockIdx.x * rpb, rhi = lane ? min(Ng, rlo + rpb) : 0;   // idle lanes have no rows
+    const int row0 = rlo + rl;
+    const W bnd = W(A.S.jac_bound), th = W(0.5 * (1.0 + 1.0 / SH_RATIO)) * bnd, de = W(0.5 * (1.0 - 1.0 / SH_RATIO)) * bnd;
     unsigned epoch = 0;
-    auto publish = [&]() -> bool {
+    // totals of v over the grid into out (NQ quantities of B instances)
+    auto publish = [&](auto& v) -> bool {
+        constexpr int NQ = sizeof(v) / sizeof(v[0]);
+        using R = typename std::remove_reference<decltype(v[0][0])>::type;
+        block_reduce_cols<NQ, VEC, R>(v, reinterpret_cast<R*>(scratch), out, B, G, RB);
         if (tid < B)
-            for (int k = 0; k < 4; ++k) A.part[((size_t)blockIdx.x * B + tid) * 4 + k] = out[k * B + tid];
-        return grid_reduce<4>(A.part, 0, B, A.fin, out, A.bar, epoch, A.err);
+            for (int k = 0; k < NQ; ++k) A.part[((size_t)blockIdx.x * B + tid) * 4 + k] = out[k * B + tid];
+        return grid_reduce<NQ>(A.part, 0, B, A.fin, out, A.bar, epoch, A.err);
     };
-    const W zero[VEC] = {};
+    W* z = A.z;
+    W* zo = A.z2;   // the steps alternate between the two
     for (int cycle = 0;; ++cycle) {
-        // residual of the current x: r = f - K x, z = r / K_ii, d = p = q = 0
+        // residual of the current x: r = f - K x, z = dd = D^-1 r / theta, zero outer faces
         {
-            R0 v[4][VEC];   // r.z, r.r, f.f
+            R0 v[2][VEC];   // r.r, f.f
 #pragma unroll
-            for (int k = 0; k < VEC; ++k) v[0][k] = v[1][k] = v[2][k] = v[3][k] = R0(0);
-            if (lane)
-                for (int row = row0; row < Ng; row += rstride) {
-                    const size_t i = (size_t)row * B + c0;
-                    const int kind = __ldg(&A.S.kind[row]);
+            for (int k = 0; k < VEC; ++k) v[0][k] = v[1][k] = R0(0);
+            const W zero[VEC] = {};
+            for (int row = row0; row < rhi; row += RB) {
+                const size_t i = (size_t)row * B + c0;
+                const int kind = __ldg(&A.S.kind[row]);
+                if (kind == 0) {   // outer face: u = 0
+                    stv<VEC>(A.r + i, zero);
+                    stv<VEC>(z + i, zero);
+                    stv<VEC>(zo + i, zero);
+                    stv<VEC>(A.dd + i, zero);
                     stv<VEC>(A.p + i, zero);
                     stv<VEC>(A.q + i, zero);
                     stv<VEC>(A.d + i, zero);
-                    if (kind == 0) {   // outer face: u = 0
-                        stv<VEC>(A.r + i, zero);
-                        stv<VEC>(A.z + i, zero);
-                        continue;
-                    }
-                    const int gn = __ldg(&A.S.gnode[row]);
-                    double f[VEC];
-#pragma unroll
-                    for (int k = 0; k < VEC; ++k) f[k] = 0.0;
-                    if (gn >= 0) ldv<VEC, false>(f, A.bvec + (size_t)gn * B + c0);
-                    R0 kx[VEC];
-                    W dinv;
-                    if constexpr (std::is_same<R0, double>::value) {
-                        double c[16];
-                        CoefLoad<double>::row(A.S.coef64 + (size_t)row * 16, c);
-                        kuhn_apply<VEC>(c, A.x + i, sx, sy, sz, kind == 2, kx);
-                        dinv = W(c[15]);
-                    } else {
-                        float c[16];
-                        CoefLoad<float>::row(A.S.coef32 + (size_t)row * 16, c);
-                        kuhn_apply<VEC>(c, A.x + i, sx, sy, sz, kind == 2, kx);
-                        dinv = c[15];
-                    }
-                    W rw[VEC], zw[VEC];
-#pragma unroll
-                    for (int k = 0; k < VEC; ++k) {
-                        if (!act[k]) f[k] = 0.0;
-                        const R0 rv = R0(f[k]) - kx[k];
-                        rw[k] = W(rv);
-                        zw[k] = rw[k] * dinv;
-                        if (act[k]) {
-                            v[0][k] += R0(rw[k]) * R0(zw[k]);
-                            v[1][k] += rv * rv;
-                            v[2][k] += R0(f[k]) * R0(f[k]);
-                        }
-                    }
-                    stv<VEC>(A.r + i, rw);
-                    stv<VEC>(A.z + i, zw);
+                    continue;
                 }
-            block_reduce_cols<4, VEC, R0>(v, reinterpret_cast<R0*>(scratch), out, B, G, RB);
-            if (!publish()) return;
+                const int gn = __ldg(&A.S.gnode[row]);
+                double f[VEC];
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) f[k] = 0.0;
+                if (gn >= 0) ldv<VEC, false>(f, A.bvec + (size_t)gn * B + c0);
+                R0 kx[VEC];
+                W dinv;
+                if constexpr (std::is_same<R0, double>::value) {
+                    double c[16];
+                    CoefLoad<double>::row(A.S.coef64 + (size_t)row * 16, c);
+                    kuhn_apply<VEC>(c, A.x + i, sx, sy, sz, kind == 2, kx);
+                    dinv = W(c[15]);
+                } else {
+                    float c[16];
+                    CoefLoad<float>::row(A.S.coef32 + (size_t)row * 16, c);
+                    kuhn_apply<VEC>(c, A.x + i, sx, sy, sz, kind == 2, kx);
+                    dinv = c[15];
+                }
+                W rw[VEC], zw[VEC];
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) {
+                    if (!act[k]) f[k] = 0.0;
+                    const R0 rv = R0(f[k]) - kx[k];
+                    rw[k] = W(rv);
+                    zw[k] = rw[k] * (dinv / th);
+                    if (act[k]) {
+                        v[0][k] += rv * rv;
+                        v[1][k] += R0(f[k]) * R0(f[k]);
+                    }
+                }
+                stv<VEC>(A.r + i, rw);
+                stv<VEC>(z + i, zw);
+                stv<VEC>(A.dd + i, zw);
+            }
+            if (!publish(v)) return;
         }
         if (tid < B) {
-            const double rr = out[B + tid];
-            if (cycle == 0) s_tol[tid] = A.tol2 * out[2 * B + tid];
+            const double rr = out[tid];
+            if (cycle == 0) s_tol[tid] = A.tol2 * out[B + tid];
             s_done[tid] = !s_act[tid] || rr <= s_tol[tid] || s_it[tid] >= A.max_iter;
             s_tin[tid] = RES64 ? fmax(s_tol[tid], MP_INNER * MP_INNER * rr) : s_tol[tid];
             s_rhop[tid] = 1.0;
         }
         if (__syncthreads_and(tid < B ? s_done[tid] : 1)) break;
-        for (int it = 0;; ++it) {
-            if (tid < B) {
-                const double rho = out[tid], rr = out[B + tid];
-                const int conv = s_done[tid] || rr <= s_tin[tid] || s_it[tid] >= A.max_iter;
-                s_ab[tid] = (it == 0 || conv) ? 0.0 : rho / s_rhop[tid];
-                s_abw[tid] = W(s_ab[tid]);
-                s_rho[tid] = rho;
-                s_flag[tid] = conv;
+        int it = 0;
+        for (;; ++it) {
+            if (tid < B) {   // out: r.r
+                if (it > 0) {
+                    s_rhop[tid] = s_rho[tid];
+                    if (!s_flag[tid]) s_it[tid] += 1;
+                }
+                s_flag[tid] = s_done[tid] || out[tid] <= s_tin[tid] || s_it[tid] >= A.max_iter;
             }
             if (__syncthreads_and(tid < B ? s_flag[tid] : 1)) break;
             bool run[VEC];
-            W beta[VEC];
 #pragma unroll
-            for (int k = 0; k < VEC; ++k) {
-                run[k] = act[k] && !s_flag[c0 + k];
-                beta[k] = s_abw[c0 + k];
-            }
-            W v[4][VEC];
+            for (int k = 0; k < VEC; ++k) run[k] = act[k] && !s_flag[c0 + k];
+            // ---- C: outer-face rows (kind 0) keep zero ----
+            W v1[1][VEC], rho_c = de / th;
+            for (int st = 1; st < SH_DEG; ++st) {
+                const W rn = W(1) / (W(2) * th / de - rho_c), c1 = rn * rho_c, c2 = W(2) * rn / de;
+                rho_c = rn;
 #pragma unroll
-            for (int k = 0; k < VEC; ++k) v[0][k] = v[1][k] = v[2][k] = v[3][k] = W(0);
-            // outer-face rows (kind 0) skip the stencil and keep zero
-            if (lane)
-                for (int row = row0; row < Ng; row += rstride) {
+                for (int k = 0; k < VEC; ++k) v1[0][k] = W(0);
+                for (int row = row0; row < rhi; row += RB) {
                     const int kind = __ldg(&A.S.kind[row]);
                     if (kind == 0) continue;
                     const size_t i = (size_t)row * B + c0;
                     W c[16];
                     CoefLoad<W>::row(coefW + (size_t)row * 16, c);
-                    W w[VEC], zi[VEC], pv[VEC], qv[VEC];
-                    ldv<VEC, false>(zi, A.z + i);
-                    ldv<VEC, false>(pv, A.p + i);
-                    ldv<VEC, false>(qv, A.q + i);
-                    kuhn_apply<VEC>(c, A.z + i, sx, sy, sz, kind == 2, w);
+                    W w[VEC], rv[VEC], tv[VEC], zv[VEC];
+                    ldv<VEC, false>(rv, A.r + i);
+                    ldv<VEC, false>(tv, A.dd + i);
+                    ldv<VEC, false>(zv, z + i);
+                    kuhn_apply<VEC>(c, z + i, sx, sy, sz, kind == 2, w);
+                    const W di = c2 * c[15];
 #pragma unroll
                     for (int k = 0; k < VEC; ++k) {
-                        pv[k] = zi[k] + beta[k] * pv[k];
-                        qv[k] = w[k] + beta[k] * qv[k];
-                        if (run[k]) v[0][k] += pv[k] * qv[k];
+                        tv[k] = c1 * tv[k] + di * (rv[k] - w[k]);
+                        zv[k] += tv[k];
+                        if (run[k]) v1[0][k] += rv[k] * zv[k];
                     }
-                    stv<VEC>(A.p + i, pv);
-                    stv<VEC>(A.q + i, qv);
+                    stv<VEC>(A.dd + i, tv);
+                    stv<VEC>(zo + i, zv);
                 }
-            block_reduce_cols<4, VEC, W>(v, reinterpret_cast<W*>(scratch), out, B, G, RB);
-            if (!publish()) return;
+                W* t = z;
+                z = zo;
+                zo = t;
+                if (st + 1 < SH_DEG && !grid_sync(A.bar, gridDim.x, epoch, A.err)) return;
+            }
+            if (!publish(v1)) return;   // r.z
+            if (tid < B) {
+                const double rho = out[tid];
+                s_ab[tid] = (it == 0 || s_flag[tid]) ? 0.0 : rho / s_rhop[tid];
+                s_abw[tid] = W(s_ab[tid]);
+                s_rho[tid] = rho;
+            }
+            __syncthreads();
+            // ---- A ----
+            W ab[VEC];
+#pragma unroll
+            for (int k = 0; k < VEC; ++k) {
+                ab[k] = s_abw[c0 < B ? c0 + k : 0];
+                v1[0][k] = W(0);
+            }
+            for (int row = row0; row < rhi; row += RB) {
+                const int kind = __ldg(&A.S.kind[row]);
+                if (kind == 0) continue;
+                const size_t i = (size_t)row * B + c0;
+                W c[16];
+                CoefLoad<W>::row(coefW + (size_t)row * 16, c);
+                W w[VEC], zi[VEC], pv[VEC], qv[VEC];
+                ldv<VEC, false>(zi, z + i);
+                if (it) {
+                    ldv<VEC, false>(pv, A.p + i);
+                    ldv<VEC, false>(qv, A.q + i);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k) pv[k] = qv[k] = W(0);
+                }
+                kuhn_apply<VEC>(c, z + i, sx, sy, sz, kind == 2, w);
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) {
+                    pv[k] = zi[k] + ab[k] * pv[k];
+                    qv[k] = w[k] + ab[k] * qv[k];
+                    if (run[k]) v1[0][k] += pv[k] * qv[k];
+                }
+                stv<VEC>(A.p + i, pv);
+                stv<VEC>(A.q + i, qv);
+            }
+            if (!publish(v1)) return;   // p.q
             if (tid < B) {
                 s_ab[tid] = s_flag[tid] ? 0.0 : s_rho[tid] / out[tid];
                 s_abw[tid] = W(s_ab[tid]);
             }
             __syncthreads();
-            W alpha[VEC];
+            // ---- B, and the first step of the next polynomial, into the copy of z that no
+            // block's products still read; outer-face rows need no test: their vectors
+            // and 1/K_ii are zero, and stay so ----
 #pragma unroll
             for (int k = 0; k < VEC; ++k) {
-                alpha[k] = s_abw[c0 + k];
-                v[0][k] = v[1][k] = v[2][k] = v[3][k] = W(0);
+                ab[k] = s_abw[c0 < B ? c0 + k : 0];
+                v1[0][k] = W(0);
             }
-            // two rows per pass (a stream: every load first); outer-face rows
-            // need no test: their vectors and 1/K_ii are zero, and stay so
-            if (lane)
-                for (int row = row0; row < Ng; row += 2 * rstride) {
-                    const int rowb = row + rstride;
-                    const bool two = rowb < Ng;
-                    const size_t ia = (size_t)row * B + c0, ib = (size_t)(two ? rowb : row) * B + c0;
-                    const W da = __ldg(coefW + (size_t)row * 16 + 15);
-                    const W db = __ldg(coefW + (size_t)(two ? rowb : row) * 16 + 15);
-                    W xa[VEC], pa[VEC], ra[VEC], qa[VEC], xb[VEC], pb[VEC], rb[VEC], qb[VEC];
-                    ldv<VEC, false>(xa, A.d + ia);
-                    ldv<VEC, false>(pa, A.p + ia);
-                    ldv<VEC, false>(ra, A.r + ia);
-                    ldv<VEC, false>(qa, A.q + ia);
-                    ldv<VEC, false>(xb, A.d + ib);
-                    ldv<VEC, false>(pb, A.p + ib);
-                    ldv<VEC, false>(rb, A.r + ib);
-                    ldv<VEC, false>(qb, A.q + ib);
+            for (int row = row0; row < rhi; row += RB) {
+                const size_t i = (size_t)row * B + c0;
+                const W dt = __ldg(coefW + (size_t)row * 16 + 15) / th;
+                W xa[VEC], pa[VEC], ra[VEC], qa[VEC];
+                if (it) ldv<VEC, false>(xa, A.d + i);
+                else
 #pragma unroll
-                    for (int k = 0; k < VEC; ++k) {
-                        xa[k] += alpha[k] * pa[k];
-                        ra[k] -= alpha[k] * qa[k];
-                        pa[k] = ra[k] * da;   // z
-                        if (run[k]) {
-                            v[0][k] += ra[k] * pa[k];
-                            v[1][k] += ra[k] * ra[k];
-                        }
-                    }
-                    stv<VEC>(A.d + ia, xa);
-                    stv<VEC>(A.r + ia, ra);
-                    stv<VEC>(A.z + ia, pa);
-                    if (two) {
+                    for (int k = 0; k < VEC; ++k) xa[k] = W(0);
+                ldv<VEC, false>(pa, A.p + i);
+                ldv<VEC, false>(ra, A.r + i);
+                ldv<VEC, false>(qa, A.q + i);
 #pragma unroll
-                        for (int k = 0; k < VEC; ++k) {
-                            xb[k] += alpha[k] * pb[k];
-                            rb[k] -= alpha[k] * qb[k];
-                            pb[k] = rb[k] * db;
-                            if (run[k]) {
-                                v[0][k] += rb[k] * pb[k];
-                                v[1][k] += rb[k] * rb[k];
-                            }
-                        }
-                        stv<VEC>(A.d + ib, xb);
-                        stv<VEC>(A.r + ib, rb);
-                        stv<VEC>(A.z + ib, pb);
-                    }
+                for (int k = 0; k < VEC; ++k) {
+                    xa[k] += ab[k] * pa[k];
+                    ra[k] -= ab[k] * qa[k];
+                    pa[k] = ra[k] * dt;   // z
+                    if (run[k]) v1[0][k] += ra[k] * ra[k];
                 }
-            block_reduce_cols<4, VEC, W>(v, reinterpret_cast<W*>(scratch), out, B, G, RB);
-            if (!publish()) return;
-            if (tid < B) {
-                s_rhop[tid] = s_rho[tid];
-                if (!s_flag[tid]) s_it[tid] += 1;
+                stv<VEC>(A.d + i, xa);
+                stv<VEC>(A.r + i, ra);
+                stv<VEC>(zo + i, pa);
+                stv<VEC>(A.dd + i, pa);
             }
-            __syncthreads();
+            W* t = z;
+            z = zo;
+            zo = t;
+            if (!publish(v1)) return;   // r.r
         }
         // fold the cycle's correction into x before anything reads x
-        if (lane)
-            for (int row = row0; row < Ng; row += rstride) {
+        if (it > 0)
+            for (int row = row0; row < rhi; row += RB) {
                 const size_t i = (size_t)row * B + c0;
                 double xv[VEC];
                 W dv[VEC];
@@ -404,7 +446,7 @@ int launch_shell(const Launch& L, const ShellDev& S, const double* bvec, double*
                  const InstState* st, double tol, int max_iter) {
     const int G = B / VEC, RB = THREADS / G;
     const int nrow = (G <= 32 && (32 % G) == 0) ? (THREADS >> 5) : RB;
-    const size_t smem = sizeof(double) * (4 * (size_t)nrow * B + 9 * (size_t)B) + sizeof(int) * 4 * B + sizeof(W) * B;
+    const size_t smem = sizeof(double) * (2 * (size_t)nrow * B + 7 * (size_t)B) + sizeof(int) * 4 * B + sizeof(W) * B;
     const void* fn = (const void*)k_shell_pcg<W, RES64, THREADS, VEC>;
     int occ = 1;
     cudaError_t e = kernel_smem_attr(fn, 160 * 1024, THREADS, smem, &occ);
@@ -419,12 +461,14 @@ int launch_shell(const Launch& L, const ShellDev& S, const double* bvec, double*
     a.st = st;
     a.bvec = bvec;
     a.x = shx;
-    W* w = reinterpret_cast<W*>(shx + Gv);   // five work vectors after x
+    W* w = reinterpret_cast<W*>(shx + Gv);   // seven work vectors after x
     a.r = w;
     a.z = w + Gv;
     a.p = w + 2 * Gv;
     a.q = w + 3 * Gv;
     a.d = w + 4 * Gv;
+    a.z2 = w + 5 * Gv;
+    a.dd = w + 6 * Gv;
     a.tol2 = tol * tol;
     a.max_iter = max_iter;
     a.bar = L.bar;
@@ -457,8 +501,8 @@ int shell_solve(const Launch& L, const MeshView& M, const BatchView<T>& V, doubl
     if (B < 1 || B > 512) return (int)cudaErrorInvalidValue;
     int e;
     // FP32 iterations for FP32 batches and for FP64 solves with mixed iterations
-    if (sizeof(T) == 4) e = launch_shell_vec<float, false, 512>(L, S, V.bvec, V.shx, V.part, B, V.st, tol, max_iter);
-    else if (mixed_iter) e = launch_shell_vec<float, true, 512>(L, S, V.bvec, V.shx, V.part, B, V.st, tol, max_iter);
+    if (sizeof(T) == 4) e = launch_shell_vec<float, false, 1024>(L, S, V.bvec, V.shx, V.part, B, V.st, tol, max_iter);
+    else if (mixed_iter) e = launch_shell_vec<float, true, 1024>(L, S, V.bvec, V.shx, V.part, B, V.st, tol, max_iter);
     else e = launch_shell_vec<double, false, 512>(L, S, V.bvec, V.shx, V.part, B, V.st, tol, max_iter);
     if (e) return e;
     size_t blocks = ((size_t)M.N * B + 255) / 256;
