@@ -98,6 +98,8 @@ struct Mesh {
     float4 *gA32 = nullptr, *gB32 = nullptr;
     double *gk64 = nullptr, *gV = nullptr, *gd64 = nullptr;
     float *gk32 = nullptr, *gd32 = nullptr;
+    int emax[17] = {0};                      // [c]: most kent entries of one of c equal row blocks
+    float jac_bound = 4.f;                   // bound of the eigenvalues of D^-1 K
     size_t bytes = 0;
     MeshView view() const {
         MeshView v;
@@ -113,6 +115,8 @@ struct Mesh {
         v.gen = gen ? 1 : 0;
         v.gA64 = gA64; v.gA32 = gA32; v.gB64 = gB64; v.gB32 = gB32;
         v.gk64 = gk64; v.gk32 = gk32; v.gV = gV; v.gd64 = gd64; v.gd32 = gd32;
+        memcpy(v.emax, emax, sizeof emax);
+        v.jac_bound = jac_bound;
         return v;
     }
 };
@@ -603,8 +607,12 @@ int run_chunk(lbm_ctx* ctx, const Launch& L, const Mesh& M, Inst* I, const Batch
     {
         // the launch shape of the cluster potential solves (it follows the active
         // instances; querying it here also caches its occupancy before a capture)
-        int64_t shape = fast_shape(L, M.view(), I->B, sizeof(T) == 8, o.cg_mixed_iter != 0);
-        if (!shape) shape = pcg_cluster_shape(L, M.view(), I->B, sizeof(T) == 8, o.cg_mixed_iter != 0);
+        int64_t shape = 0;   // the other solves' shapes do not follow the active instances
+        if (!(M.shell && o.demag)) {
+            shape = fast_shape(L, M.view(), I->B, sizeof(T) == 8, o.cg_mixed_iter != 0);
+            if (!shape && (!M.gen || o.pcg_kernel != 0))
+                shape = pcg_cluster_shape(L, M.view(), I->B, sizeof(T) == 8, o.cg_mixed_iter != 0);
+        }
         const int64_t k[10] = {chunk, (int64_t)sizeof(T), I->B, (int64_t)(intptr_t)M.hm, (int64_t)(intptr_t)M.B32lo,
                                (int64_t)(intptr_t)M.tcA, ctx->prof ? 1 : 0, (int64_t)(intptr_t)V.m,
                                (int64_t)(intptr_t)M.shell, shape};
@@ -1164,10 +1172,28 @@ int lbm_mesh_upload(lbm_ctx* ctx, const double* xyz, int64_t n_nodes, const int3
     CKM(cudaMemcpyAsync(&tot, M->kptr + N, sizeof(int), cudaMemcpyDeviceToHost, st));
     CKM(cudaStreamSynchronize(st));
     M->nnzK = tot;
+    {
+        std::vector<int> kp(N + 1);
+        CKM(cudaMemcpyAsync(kp.data(), M->kptr, sizeof(int) * ((size_t)N + 1), cudaMemcpyDeviceToHost, st));
+        CKM(cudaStreamSynchronize(st));
+        for (int c = 1; c <= 16; ++c) {
+            const int rpc = (N + c - 1) / c;
+            for (int r = 0; r < N; r += rpc) M->emax[c] = std::max(M->emax[c], kp[std::min(N, r + rpc)] - kp[r]);
+        }
+    }
     CKM(cudaMalloc(&M->kent, sizeof(int) * (size_t)M->nnzK));
     CKM(cudaMalloc(&M->gk64, sizeof(double) * (size_t)M->nnzK));
     CKM(cudaMalloc(&M->gk32, sizeof(float) * (size_t)M->nnzK));
     launch_kcsr_fill_gen(N, M->rowptr, M->col, M->gA64, M->kptr, M->kent, M->gk64, M->gk32, st);
+    {   // cnt has served: its first word takes the bound
+        CKM(cudaMemsetAsync(cnt, 0, sizeof(float), st));
+        launch_jac_bound(N, M->kptr, M->gk64, M->gd64, (float*)cnt, st);
+        ctx->launches += 1;
+        CKM(cudaMemcpyAsync(&M->jac_bound, cnt, sizeof(float), cudaMemcpyDeviceToHost, st));
+        CKM(cudaStreamSynchronize(st));
+        // 4 bounds every mesh of linear tetrahedra: D_e^-1 K_e of an element has trace 4
+        M->jac_bound = fminf(4.f, M->jac_bound);
+    }
     ctx->launches += 1;
     const size_t nb2 = (size_t)nb * nb;
     CKM(cudaMalloc(&M->B64, sizeof(double) * nb2));

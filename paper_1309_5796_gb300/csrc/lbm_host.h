@@ -44,6 +44,8 @@ void launch_assemble_gen(int N, const double* xyz, const int* tets, const int* n
 void launch_kcsr_count_gen(int N, const int* rowptr, const Dbl4* A64, int* cnt, cudaStream_t st);
 void launch_kcsr_fill_gen(int N, const int* rowptr, const int* col, const Dbl4* A64, const int* kptr, int* kent,
                           double* k64, float* k32, cudaStream_t st);
+// *bound = max over the rows of sum |K_ij| / K_ii (must be zero before)
+void launch_jac_bound(int N, const int* kptr, const double* k64, const double* d64, float* bound, cudaStream_t st);
 
 // ---- hierarchical form of the boundary matrix: host set-up (csrc/hpartition.cu) --------
 struct HCluster {
@@ -223,6 +225,8 @@ struct MeshView {
     const double* gk64; const float* gk32;     // nnzK values of the stiffness-only CSR
     const double* gV;                          // N    lumped volumes
     const double* gd64; const float* gd32;     // N    K_ii (Jacobi preconditioner)
+    int emax[17] = {0};                        // [c]: most kent entries of one of c equal row blocks
+    float jac_bound = 4.f;                     // bound of the eigenvalues of D^-1 K (general meshes)
 };
 
 // ---- device view of one instance batch (node-major, instance-minor) ------------------
@@ -294,6 +298,12 @@ int shell_solve(const Launch& L, const MeshView& M, const BatchView<T>& V, doubl
 template <typename T>
 int pcg_solve_cluster(const Launch& L, const MeshView& M, const BatchView<T>& V, int mode, double tol, int max_iter,
                       bool mixed_iter, cudaError_t* err);
+// Polynomially preconditioned CG with a cluster per group of systems and its vectors in shared memory
+// (cluster_cg.cu), general meshes: 1 when launched (*err its status), 0 when it does
+// not qualify.
+template <typename T>
+int cluster_cg_fem(const Launch& L, const MeshView& M, const BatchView<T>& V, int mode, double tol, int max_iter,
+                   bool mixed_iter, cudaError_t* err);
 template <typename T>
 int pcg_solve(const Launch& L, const MeshView& M, const BatchView<T>& V, int mode, double tol, int max_iter,
               bool mixed_iter);

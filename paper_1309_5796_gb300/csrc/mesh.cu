@@ -523,6 +523,22 @@ void launch_assemble_gen(int N, const double* xyz, const int* tets, const int* n
 void launch_kcsr_count_gen(int N, const int* rowptr, const Dbl4* A64, int* cnt, cudaStream_t st) {
     k_kcsr_count_gen<<<(N + 255) / 256, 256, 0, st>>>(N, rowptr, A64, cnt);
 }
+// Gershgorin's bound of the eigenvalues of D^-1 K, rounded up (positive floats order as integers)
+__global__ void k_jac_bound(int N, const int* __restrict__ kptr, const double* __restrict__ k64,
+                            const double* __restrict__ d64, float* __restrict__ bound) {
+    float m = 0.f;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+        double s = 0.0;
+        for (int e = kptr[i]; e < kptr[i + 1]; ++e) s += fabs(k64[e]);
+        m = fmaxf(m, __double2float_ru(s / d64[i]));
+    }
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<int*>(bound), __float_as_int(m));
+}
+void launch_jac_bound(int N, const int* kptr, const double* k64, const double* d64, float* bound, cudaStream_t st) {
+    k_jac_bound<<<std::min((N + 255) / 256, 512), 256, 0, st>>>(N, kptr, k64, d64, bound);
+}
+
 void launch_kcsr_fill_gen(int N, const int* rowptr, const int* col, const Dbl4* A64, const int* kptr, int* kent,
                           double* k64, float* k32, cudaStream_t st) {
     k_kcsr_fill_gen<<<(N + 255) / 256, 256, 0, st>>>(N, rowptr, col, A64, kptr, kent, k64, k32);

@@ -602,6 +602,7 @@ int pcg_solve(const Launch& L, const MeshView& M, const BatchView<T>& V, int mod
     // Kuhn cubes, unless the caller asks for one of the diagonally preconditioned kernels
     cudaError_t fe;
     if (fast_solve<T>(L, M, V, mode, tol, max_iter, mixed_iter, &fe)) return fe == cudaSuccess ? 0 : (int)fe;
+    if (cluster_cg_fem<T>(L, M, V, mode, tol, max_iter, mixed_iter, &fe)) return fe == cudaSuccess ? 0 : (int)fe;
     if (L.pcg_kernel != 1) {
         cudaError_t ce;
         if (pcg_solve_cluster<T>(L, M, V, mode, tol, max_iter, mixed_iter, &ce)) return ce == cudaSuccess ? 0 : (int)ce;

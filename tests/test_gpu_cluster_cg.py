@@ -1,0 +1,81 @@
+"""Jacobi-CG with a cluster per group of systems (csrc/cluster_cg.cu) against the
+grid-wide kernels (lbm_solve_opts.pcg_kernel = 1): uploaded meshes and the
+space-transformation boundary.
+
+Both run the same iteration to the same relative residual: 1e-13 (FP64), 1e-10
+(FP64 iterated in FP32) or 1e-6 (FP32).  In FP64 the condition numbers (a few
+hundred for cells of one size, a few thousand for the grids) leave fields and
+potentials within 1e-9 and 1e-6.  An FP32 solve is taken against the FP64 one: no
+further off than 2e-5 (as the FP32 parity tests) or, where the mesh is worse
+conditioned (a ball's flat corner cells), than twice the grid-wide kernel over the
+same batch.
+"""
+import numpy as np
+import pytest
+
+import paper_1309_5796_gb300 as lbm
+from synth.inputs import A_JM, JS_T, K1_JM3, m_perturbed, tilted_axis
+from synth.meshes import ball_mesh, jittered_cube, l_shape
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_1309_5796_gb300 import build
+    build.build()
+    c = lbm.Context(0)
+    yield c
+    c.close()
+
+
+def _run(ctx, mesh, N, B, prec, **opts):
+    inst = ctx.instance_create(mesh, B, prec)
+    inst.set_material(JS_T, A_JM, K1_JM3, tilted_axis(3.0, 0.4))
+    inst.set_field(np.array([0.1, 0.0, -2.0]))
+    inst.set_m(np.stack([m_perturbed(N, 50 + b, 0.3, (0.2 * b, 0.3, 1.0)) for b in range(B)]))
+    res, h, u = inst.evaluate(lbm.default_opts(prec, **opts))
+    inst.destroy()
+    return res, h, u
+
+
+def _off(x, y):
+    return [np.linalg.norm(x[b] - y[b]) / np.linalg.norm(y[b]) for b in range(len(x))]
+
+
+def _compare(ctx, mesh, N, B, prec):
+    ref = _run(ctx, mesh, N, B, 0, pcg_kernel=1)
+    if prec:
+        grid = _run(ctx, mesh, N, B, prec, pcg_kernel=1)
+        new = _run(ctx, mesh, N, B, prec)
+        for k in (1, 2):
+            assert max(_off(new[k], ref[k])) <= max(2e-5, 2.0 * max(_off(grid[k], ref[k])))
+        assert all(r["status"] == lbm.LBM_OK for r in new[0])
+        return
+    for tol, v in ((1e-9, dict()), (1e-6, dict(cg_mixed_iter=1, cg_tol=1e-10))):
+        new = _run(ctx, mesh, N, B, prec, **v)
+        assert all(r["status"] == lbm.LBM_OK for r in new[0])
+        assert max(_off(new[2], ref[2])) <= tol and max(_off(new[1], ref[1])) <= tol, v
+
+
+# one CTA to sixteen, rows that do and do not divide by them, widths 1, 2 and 4, matrix
+# entries in shared memory and (26, FP64 and width 4) not
+@pytest.mark.parametrize("shape,n,B,prec", [
+    ("cube", 1, 1, 0), ("cube", 2, 3, 1), ("cube", 3, 4, 0), ("l", 4, 1, 0), ("l", 6, 2, 1), ("ball", 6, 5, 1),
+    ("ball", 8, 16, 0), ("ball", 10, 1, 0), ("cube", 9, 24, 1), ("ball", 26, 1, 0), ("ball", 26, 1, 1), ("ball", 26, 16, 1)])
+def test_uploaded_meshes(ctx, shape, n, B, prec):
+    xyz, tets = {"cube": jittered_cube, "l": l_shape, "ball": ball_mesh}[shape](n)
+    mesh = ctx.mesh_upload(xyz, tets)
+    _compare(ctx, mesh, xyz.shape[0], B, prec)
+    ctx.mesh_destroy(mesh)
+
+
+# grids of 8^3 to 55^3 nodes: all vectors in shared memory, some, and z alone (FP64)
+@pytest.mark.parametrize("n,a,s,B,prec", [
+    (1, 1, 2, 1, 0), (2, 1, 2, 3, 1), (3, 2, 3, 4, 0), (5, 2, 4, 2, 1), (6, 2, 4, 16, 1), (10, 3, 5, 1, 0),
+    (20, 4, 8, 6, 1), (30, 4, 8, 1, 0), (30, 4, 8, 2, 1)])
+def test_transformed_grid(ctx, n, a, s, B, prec):
+    mesh = ctx.mesh_cube(2e-9, n)
+    ctx.mesh_shell(mesh, a, s)
+    _compare(ctx, mesh, (n + 1) ** 3, B, prec)
+    ctx.mesh_destroy(mesh)
