@@ -26,7 +26,7 @@
 //
 // Measured on GB300 (two stages of both chains, FP64 n = 10 / FP32 n = 20, 80, one
 // instance / FP32 n = 30, 64 instances, before: diagonally preconditioned CG):
-// 0.14 / 0.14 / 1.56 / 1.34 ms, before 6.1 / 5.6 / 36 / 12 ms.
+// 0.13 / 0.12 / 1.5 / 0.96 ms, before 6.1 / 5.6 / 36 / 12 ms.
 //
 // One thread-block cluster solves VEC systems (columns of the [N][2B] layout)
 // of one kind; CTA r owns the z-planes [r ppc, (r+1) ppc).  Per step:
@@ -59,7 +59,7 @@ namespace {
 
 constexpr size_t FS_SMEM_MAX = 226 * 1024;   // dynamic; the rest of the 227 KB is static
 constexpr int FS_MAX_N1 = 97;       // largest cube: 96 cells
-constexpr int FS_NQ = 4;            // most quantities of one reduction
+constexpr int FS_NQ = 5;            // most quantities of one reduction
 constexpr int FS_MAX_CL = 16;
 constexpr int FS_SPLIT = 8;         // parts of a row of H
 
@@ -86,28 +86,12 @@ __device__ __forceinline__ uint32_t peer_addr(uint32_t a, unsigned rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void ld_peer(uint32_t a, float (&v)[4]) {
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
-                 : "r"(a)
-                 : "memory");
-}
-__device__ __forceinline__ void ld_peer(uint32_t a, double (&v)[4]) {
-    asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "r"(a) : "memory");
-    asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v[2]), "=d"(v[3]) : "r"(a + 16) : "memory");
-}
-__device__ __forceinline__ void st_peer(uint32_t a, const float (&v)[4]) {
-    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3])
-                 : "memory");
-}
-__device__ __forceinline__ void st_peer(uint32_t a, const double (&v)[4]) {
-    asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(v[0]), "d"(v[1]) : "memory");
-    asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(a + 16), "d"(v[2]), "d"(v[3]) : "memory");
-}
-__device__ __forceinline__ float ld_peer1(uint32_t a, float) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-    return v;
+// generic address of p in the CTA `rank` of the cluster
+template <typename X>
+__device__ __forceinline__ X* peer_ptr(X* p, unsigned rank) {
+    X* r;
+    asm volatile("mapa.u64 %0, %1, %2;" : "=l"(r) : "l"(p), "r"(rank));
+    return r;
 }
 __device__ __forceinline__ double ld_peer1(uint32_t a, double) {
     double v;
@@ -354,11 +338,13 @@ __device__ __forceinline__ void edge_node(int e, int n, int& i, int& j, int& k) 
 }
 
 // T: type of the potential x and of the residual f - K x; W: type of the
-// refinement (transforms, r, the sum d of the steps) and of the dot products
-// inside a chunk (sums over chunks, planes and CTAs in FP64).  T = W: refinement to the tolerance on the recurrence
-// r -= K z.  T = double, W = float (solves iterated in FP32): cycles of the FP64
-// residual and FP32 refinement until it has reduced that residual by MP_INNER;
-// the solve ends on the FP64 residual test.  Neumann systems (forward in mode 0,
+// refinement (transforms, r, the sum of the steps) and of the dot products inside
+// a chunk (sums over chunks, planes and CTAs in FP64).  T = W: d starts as x and
+// collects the steps; the first residual's stencil runs on a copy of x in the
+// planes' place, so x is read once and written once (a system's values lie 2B words
+// apart in it).  T = double, W = float (solves iterated in FP32): cycles of the FP64
+// residual and FP32 refinement until it has reduced that residual by MP_INNER; the
+// solve ends on the FP64 residual test.  Neumann systems (forward in mode 0,
 // adjoint in mode 1): residual taken without its mean (consistent right-hand
 // side), solution gauged to zero V-weighted mean.  Dirichlet systems: surface
 // values frozen.
@@ -377,18 +363,18 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
     double* s_tol = out + FS_NQ * VEC;
     double* s_tin = s_tol + VEC;
     double* s_mean = s_tin + VEC;
-    int* s_flag = reinterpret_cast<int*>(s_mean + VEC);
+    W** s_plane = reinterpret_cast<W**>(s_mean + VEC);            // [s2] every plane's sheets (peers' shared memory, or gt)
+    uint32_t* s_slot = reinterpret_cast<uint32_t*>(s_plane + FS_MAX_N1);   // [s2] its partial sums (slot 0)
+    int* s_flag = reinterpret_cast<int*>(s_slot + FS_MAX_N1);
     int* s_it = s_flag + VEC;
     int* s_done = s_it + VEC;
-    uint32_t* s_plane = reinterpret_cast<uint32_t*>(s_done + VEC);   // [s2] cluster address of every plane's sheets
-    uint32_t* s_slot = s_plane + FS_MAX_N1;                     // [s2] and of its partial sums (slot 0)
     __shared__ int s_grp;
 
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
     const unsigned rank = cl_rank();
     const int B = A.P.V.B, C = 2 * B, n = g.n, s2 = g.s2, N = A.P.M.N, mode = A.P.mode;
     const int ss = g.ss, ldx = g.ldx, h = g.h, ho = g.ho, hp = g.hp, hop = g.hop;
-    const int gap = hp - h;
+    const int gap = hp - h, pn = s2 * s2;
 
     // the cluster's group of VEC systems: the k-th one with an active instance
     if (warp == 0) {
@@ -416,25 +402,27 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
     const int c0 = (grp < 0 ? 0 : grp) * VEC, b0 = c0 % B;
     const bool neu = (mode == c0 / B);   // B % VEC == 0: one kind per cluster
     const int k0 = (int)rank * g.ppc, k1 = min(s2, k0 + g.ppc), np = max(0, k1 - k0);
-    const int lo = k0 * s2 * s2, hi = max(lo, k1 * s2 * s2);
+    const int lo = k0 * pn, hi = max(lo, k1 * pn);
     int itmax = 0;
     if (grp >= 0) {
         const PcgArgs<T>& P = A.P;
         bool act[VEC];
 #pragma unroll
         for (int k = 0; k < VEC; ++k) act[k] = P.V.st[b0 + k].phase != PH_DONE;
-        // grouped vectors [rows][VEC]; d: the sum of the steps of this solve or cycle
+        // r and d of the own planes, [rows][VEC], and x at the first own row and column
         W *r, *d;
         if (g.vs) {
-            r = reinterpret_cast<W*>(fs_sm + g.o_vec) - (ptrdiff_t)lo * VEC;
-            d = r + (ptrdiff_t)g.ppc * s2 * s2 * VEC;
+            r = reinterpret_cast<W*>(fs_sm + g.o_vec);
+            d = r + (ptrdiff_t)g.ppc * pn * VEC;
         } else {
-            const size_t gb = (size_t)grp * N * VEC;
+            const size_t gb = ((size_t)grp * N + lo) * VEC;
             r = reinterpret_cast<W*>(P.V.r) + gb;
             d = reinterpret_cast<W*>(P.V.z) + gb;
         }
         W* gt = TS ? nullptr : A.gt + (size_t)grp * s2 * VEC * ss;
-        T* __restrict__ x = mode ? P.V.U2 : P.V.U1;
+        T* const x = (mode ? P.V.U2 : P.V.U1) + (size_t)lo * C + c0;
+        const double* const bv = P.V.bvec + (size_t)lo * B + b0;
+        const int* const nodes = P.M.node + lo;
         const int kind = neu ? 0 : 1;
         // transforms: forward F, back G
         const unsigned oFe = g.o_mat, oGe = oFe + (unsigned)(hp * hp * sizeof(W)), oFo = oGe + (unsigned)(hp * hp * sizeof(W)),
@@ -446,7 +434,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
         }
         for (int k = tid; k < s2; k += nt) {
             const int o = k / g.ppc, lp = k - o * g.ppc;
-            s_plane[k] = peer_addr(sm_addr(buf), (unsigned)o) + (uint32_t)((size_t)lp * VEC * ss * sizeof(W));
+            s_plane[k] = TS ? peer_ptr(buf, (unsigned)o) + (size_t)lp * VEC * ss : gt + (size_t)k * VEC * ss;
             s_slot[k] = peer_addr(sm_addr(slots), (unsigned)o) + (uint32_t)(lp * FS_NQ * VEC * sizeof(double));
         }
         if constexpr (TS)   // the gap columns stay zero
@@ -456,6 +444,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
             s_done[tid] = 0;
             s_tin[tid] = 0.0;
         }
+        __syncthreads();
         int par = 0;
         // Totals over the cluster of the nq quantities whose chunk sums the CTA has
         // written to part: chunks of a plane, then planes (lanes stride, then a fixed
@@ -484,8 +473,8 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
             par ^= 1;
             __syncthreads();
         };
-        // chunk sums of the quantities v into part (whole warp)
-        auto put = [&](auto& v, int pl, int ch) {
+        // chunk sums of the quantities a0, a0 + 1, ... in v into part (whole warp)
+        auto put = [&](auto& v, int a0, int pl, int ch) {
             constexpr int NQ = sizeof(v) / sizeof(v[0]);
 #pragma unroll
             for (int a = 0; a < NQ; ++a)
@@ -493,92 +482,253 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                 for (int k = 0; k < VEC; ++k) {
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) v[a][k] += __shfl_xor_sync(0xffffffffu, v[a][k], o);
-                    if (lane == 0) part[((pl * g.nch + ch) * FS_NQ + a) * VEC + k] = (double)v[a][k];
+                    if (lane == 0) part[((pl * g.nch + ch) * FS_NQ + a0 + a) * VEC + k] = (double)v[a][k];
                 }
         };
-        // f(plane, chunk, y, x, mirrored in y, mirrored in x, valid) for every chunk of
-        // the CTA's planes [pa, pb), a warp per chunk, a lane per quadruple (y, x),
-        // (y, n-x), (n-y, x), (n-y, n-x), y, x < h
-        auto chunks = [&](int pa, int pb, auto&& f) {
-            for (int w = pa * g.nch + warp; w < pb * g.nch; w += nw) {
-                const int pl = w / g.nch, ch = w - pl * g.nch, e = ch * 32 + lane;
-                const int y = e / h, xx = e - y * h;
-                f(pl, ch, y, xx, y < ho, xx < ho, y < h);
+        // f(pl, ch, q) for every chunk ch of the CTA's planes [pa, pb), a warp per chunk, a
+        // lane per quadruple of mirrored nodes: u = 0 (y, x), 1 (y, n-x), 2 (n-y, x),
+        // 3 (n-y, n-x), x, y < h.  A warp keeps its chunk from plane to plane where the
+        // CTA has as many warps as a plane has chunks, so q is computed once.
+        struct Quad {
+            int y, x;
+            bool on, has[4];
+            int row[4];    // in a plane of rows
+            int at[4];     // in a sheet
+        };
+        auto quads = [&](int pa, int pb, auto&& f) {
+            const bool wide = nw >= g.nch;
+            const int ps = wide ? nw / g.nch : 1, pf = wide ? warp / g.nch : 0, cf = wide ? warp - pf * g.nch : warp;
+            if (pf >= ps) return;
+            for (int ch = cf; ch < g.nch; ch += wide ? g.nch : nw) {
+                Quad q;
+                const int e = ch * 32 + lane;
+                q.y = e / h;
+                q.x = e - q.y * h;
+                q.on = q.y < h;
+                if (!q.on) q.y = 0;
+                const bool mx = q.x < ho, my = q.y < ho;
+                q.has[0] = q.on;
+                q.has[1] = q.on && mx;
+                q.has[2] = q.on && my;
+                q.has[3] = q.on && mx && my;
+                const int xm = mx ? n - q.x : q.x, ym = my ? n - q.y : q.y, cm = mx ? xm + gap : q.x;
+                q.row[0] = q.y * s2 + q.x;
+                q.row[1] = q.y * s2 + xm;
+                q.row[2] = ym * s2 + q.x;
+                q.row[3] = ym * s2 + xm;
+                q.at[0] = q.y * ldx + q.x;
+                q.at[1] = q.y * ldx + cm;
+                q.at[2] = ym * ldx + q.x;
+                q.at[3] = ym * ldx + cm;
+                for (int pl = pa + pf; pl < pb; pl += ps) f(pl, ch, q);
             }
         };
-        // f(u, exists, row, i, j) for the points of a quadruple (u = 0..3)
-        auto points = [&](int pl, int y, int xx, bool my, bool mx, bool on, auto&& f) {
-            const int row0 = (k0 + pl) * s2 * s2;
+        // The stencil: f(u, value) of (K v) at the quadruple's nodes for column k of the
+        // plane kk's sheets s (own plane), with the planes below and above.  Weights in
+        // units h/6: an axis edge counts 6 times 1/2 per other coordinate on the boundary,
+        // +-1/2 on the cube's edges (same end of both other axes: +).
+        auto stencil = [&](const Quad& q, int kk, const W* s, const W* sm, const W* sp, auto&& f) {
+            const bool ex = q.x == 0, ey = q.y == 0, ek = kk == 0 || kk == n;
+            const W ax = ex ? W(0.5) : W(1), ay = ey ? W(0.5) : W(1), ak = ek ? W(0.5) : W(1);
+            const W wx = W(6) * ay * ak, wy = W(6) * ax * ak, wz = W(6) * ax * ay;
+            const W cx = ey && ek ? (kk == 0 ? W(0.5) : W(-0.5)) : W(0), cy = ex && ek ? (kk == 0 ? W(0.5) : W(-0.5)) : W(0),
+                    cz = ex && ey ? W(0.5) : W(0);
+            const int xo = ex ? 0 : -1, xi = q.x + 1 < h ? 1 : 1 + gap, xim = n - q.x - 1 >= h ? -1 : -1 - gap;
+            const int yo = ey ? 0 : -ldx;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const bool has = on && ((u & 1) == 0 || mx) && ((u & 2) == 0 || my);
-                const int j = (u & 2) ? n - y : y, i = (u & 1) ? n - xx : xx;
-                f(u, has, row0 + j * s2 + i, i, j);
+                if (!q.has[u]) continue;
+                const W* z = s + q.at[u];
+                const W z0 = z[0];
+                const W vx = wx + ((u & 2) ? -cx : cx), vy = wy + ((u & 1) ? -cy : cy), vz = wz + (u == 0 || u == 3 ? cz : -cz);
+                // towards the boundary (none there: the difference vanishes) and away from it
+                W a = vx * (z0 - z[(u & 1) ? -xo : xo]);
+                a = fma_(vx, z0 - z[(u & 1) ? xim : xi], a);
+                a = fma_(vy, z0 - z[(u & 2) ? -yo : yo], a);
+                a = fma_(vy, z0 - z[(u & 2) ? -ldx : ldx], a);
+                a = fma_(vz, z0 - sm[q.at[u]], a);
+                a = fma_(vz, z0 - sp[q.at[u]], a);
+                f(u, z0, a);
             }
         };
+        // the sheets of the planes below and above plane kk (its own where there is none)
+        auto below = [&](int kk, int pl) -> const W* { return kk == 0 ? s_plane[0] : (TS && pl > 0 ? buf + (pl - 1) * VEC * ss : s_plane[kk - 1]); };
+        auto above = [&](int kk, int pl) -> const W* { return kk == n ? s_plane[n] : (TS && pl + 1 < np ? buf + (pl + 1) * VEC * ss : s_plane[kk + 1]); };
+        auto own = [&](int kk, int pl) -> const W* { return TS ? buf + pl * VEC * ss : s_plane[kk]; };
 
-        // Dirichlet systems: surface values (stage 1 adjoint: zero; stage 2 forward: B u1_S)
-        if (!neu)
-            for (int row = lo + tid; row < hi; row += nt) {
-                const int bp = (int)((unsigned)P.M.node[row] >> 16);
+        // Surface values of the Dirichlet systems (stage 1 adjoint: zero; stage 2 forward:
+        // B u1_S).  T = W: x with them into d and into the planes' place.
+        if constexpr (!MP) {
+            quads(0, np, [&](int pl, int, const Quad& q) {
+                const int kk = k0 + pl;
+                const bool surf = q.x == 0 || q.y == 0 || kk == 0 || kk == n;
+                T xv[4][VEC];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (q.has[u]) ldc<VEC, false>(xv[u], x + (ptrdiff_t)(pl * pn + q.row[u]) * C);
+                W* s = const_cast<W*>(own(kk, pl));
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (!q.has[u]) continue;
+                    if (!neu && surf) {
+                        const int bp = (int)((unsigned)nodes[pl * pn + q.row[u]] >> 16);
+#pragma unroll
+                        for (int k = 0; k < VEC; ++k)
+                            if (act[k]) xv[u][k] = mode ? P.V.ub_out[(size_t)(bp - 1) * C + b0 + k] : T(0);
+                    }
+                    W wv[VEC];
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k) {
+                        wv[k] = W(xv[u][k]);
+                        s[k * ss + q.at[u]] = wv[k];
+                    }
+                    stc<VEC>(d + (ptrdiff_t)(pl * pn + q.row[u]) * VEC, wv);
+                }
+            });
+        } else if (!neu) {
+            for (int l = tid; l < hi - lo; l += nt) {
+                const int bp = (int)((unsigned)nodes[l] >> 16);
                 if (!bp) continue;
 #pragma unroll
                 for (int k = 0; k < VEC; ++k)
-                    if (act[k]) x[(size_t)row * C + c0 + k] = mode ? P.V.ub_out[(size_t)(bp - 1) * C + b0 + k] : T(0);
+                    if (act[k]) x[(ptrdiff_t)l * C + k] = mode ? P.V.ub_out[(size_t)(bp - 1) * C + b0 + k] : T(0);
             }
+        }
         cl_sync();
         const int step = TS ? max(np, 1) : g.spl;
+        bool ended = false;
         for (int cycle = 0;; ++cycle) {
-            // residual of the current x into r; sums r.r, r, f.f, f (f: the norm reference)
-            chunks(0, np, [&](int pl, int ch, int y, int xx, bool my, bool mx, bool on) {
-                W v[4][VEC];
-#pragma unroll
-                for (int a = 0; a < 4; ++a)
-#pragma unroll
-                    for (int k = 0; k < VEC; ++k) v[a][k] = W(0);
+            // residual of the current x into r; sums r.r, r, f.f, f (f: the norm
+            // reference, Dirichlet: f - K_IS x_S) and (MP, Neumann) V x for the gauge
+            quads(0, np, [&](int pl, int ch, const Quad& q) {
                 const int kk = k0 + pl;
-                points(pl, y, xx, my, mx, on, [&](int, bool has, int row, int i, int j) {
-                    if (!has) return;
-                    const int bp = (int)((unsigned)P.M.node[row] >> 16);
+                const bool surf = q.x == 0 || q.y == 0 || kk == 0 || kk == n;
+                W v[4][VEC];
+                double vx[1][VEC];
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) {
+                    v[0][k] = v[1][k] = v[2][k] = v[3][k] = W(0);
+                    vx[0][k] = 0.0;
+                }
+                const bool froz = !neu && surf;
+                // the right-hand side at node u (none in the stage-2 forward system)
+                auto rhs = [&](int u, T (&f)[VEC]) {
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k) f[k] = T(0);
+                    if (froz || (mode && !neu)) return;
+                    double fb[VEC];
+                    ldc<VEC, false>(fb, bv + (ptrdiff_t)(pl * pn + q.row[u]) * B);
+                    if (mode && surf) {   // the BEM term of the adjoint Neumann system
+                        const int bp = (int)((unsigned)nodes[pl * pn + q.row[u]] >> 16);
+#pragma unroll
+                        for (int k = 0; k < VEC; ++k) fb[k] += (double)P.V.ub_out[(size_t)(bp - 1) * C + c0 + k];
+                    }
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k) f[k] = act[k] ? T(fb[k]) : T(0);
+                };
+                auto done = [&](int u, const T (&f)[VEC], const T (&kx)[VEC], const T (&ks)[VEC]) {
                     W rv[VEC];
-                    if (!neu && bp) {
 #pragma unroll
-                        for (int k = 0; k < VEC; ++k) rv[k] = W(0);
-                    } else {
-                        const T* xp = x + (size_t)row * C + c0;
-                        T xi[VEC], kx[VEC], f[VEC];
-                        ldc<VEC, true>(xi, xp);
+                    for (int k = 0; k < VEC; ++k) {
+                        rv[k] = W(f[k] - kx[k]);
+                        const W ref = W(f[k] - ks[k]);
+                        v[0][k] = fma_(rv[k], rv[k], v[0][k]);
+                        v[1][k] += rv[k];
+                        v[2][k] = fma_(ref, ref, v[2][k]);
+                        v[3][k] += ref;
+                    }
+                    stc<VEC>(r + (ptrdiff_t)(pl * pn + q.row[u]) * VEC, rv);
+                };
+                if constexpr (!MP) {
+                    T kx[4][VEC], ks[4][VEC];
 #pragma unroll
-                        for (int k = 0; k < VEC; ++k) kx[k] = f[k] = T(0);
-                        if (!(mode == 1 && !neu)) {
-                            double fb[VEC];
-                            ldc<VEC, false>(fb, P.V.bvec + (size_t)row * B + b0);
+                    for (int u = 0; u < 4; ++u)
 #pragma unroll
-                            for (int k = 0; k < VEC; ++k) {
-                                if (!act[k]) fb[k] = 0.0;
-                                if (mode == 1 && bp) fb[k] += (double)P.V.ub_out[(size_t)(bp - 1) * C + c0 + k];
-                                f[k] = T(fb[k]);
+                        for (int k = 0; k < VEC; ++k) kx[u][k] = ks[u][k] = T(0);
+                    if (!froz) {
+                        const W *s = own(kk, pl), *sm = below(kk, pl), *sp = above(kk, pl);
+#pragma unroll
+                        for (int k = 0; k < VEC; ++k) {
+                            stencil(q, kk, s + k * ss, sm + k * ss, sp + k * ss, [&](int u, W, W a) { kx[u][k] = a; });
+                            if (!neu && mode) {   // neighbours on the surface
+                                const bool nx = q.x == 1, nx2 = q.x + 1 == n, ny = q.y == 1, ny2 = q.y + 1 == n;
+                                if (!(nx || nx2 || ny || ny2 || kk == 1 || kk + 1 == n)) continue;
+                                const int xi = q.x + 1 < h ? 1 : 1 + gap, xim = n - q.x - 1 >= h ? -1 : -1 - gap;
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) {
+                                    if (!q.has[u]) continue;
+                                    const W* z = s + k * ss + q.at[u];
+                                    W t = W(0);
+                                    if (nx) t += z[(u & 1) ? 1 : -1];
+                                    if (nx2) t += z[(u & 1) ? xim : xi];
+                                    if (ny) t += z[(u & 2) ? ldx : -ldx];
+                                    if (ny2) t += z[(u & 2) ? -ldx : ldx];
+                                    if (kk == 1) t += sm[k * ss + q.at[u]];
+                                    if (kk + 1 == n) t += sp[k * ss + q.at[u]];
+                                    ks[u][k] = W(-6) * t;
+                                }
                             }
                         }
-                        T ks[VEC] = {};   // Dirichlet: K_IS x_S (norm reference f - K_IS x_S)
-                        const ptrdiff_t st[3] = {(ptrdiff_t)C, (ptrdiff_t)s2 * C, (ptrdiff_t)s2 * s2 * C};
-                        const int co[3] = {i, j, kk};
-                        const int wt[3] = {bp ? edge_weight(j, kk, n) : 6, bp ? edge_weight(i, kk, n) : 6,
-                                           bp ? edge_weight(i, j, n) : 6};
+                    }
 #pragma unroll
-                        for (int a = 0; a < 3; ++a)
+                    for (int u = 0; u < 4; ++u) {
+                        if (!q.has[u]) continue;
+                        T f[VEC];
+                        rhs(u, f);
+                        done(u, f, kx[u], ks[u]);
+                    }
+                } else {
+                    const int co[3] = {q.x, q.y, kk};
+                    const ptrdiff_t st[3] = {(ptrdiff_t)C, (ptrdiff_t)s2 * C, (ptrdiff_t)pn * C};
+#pragma unroll 1
+                    for (int u = 0; u < 4; ++u) {
+                        const bool mx = u & 1, my = u & 2;
+                        if (!(mx ? (my ? q.has[3] : q.has[1]) : (my ? q.has[2] : q.has[0]))) continue;
+                        const int j = my ? n - q.y : q.y, i = mx ? n - q.x : q.x, l = pl * pn + j * s2 + i;
+                        T kx[VEC], ks[VEC], f[VEC];
 #pragma unroll
-                            for (int sgn = -1; sgn <= 1; sgn += 2) {
-                                if (sgn < 0 ? co[a] == 0 : co[a] == n) continue;
-                                T xj[VEC];
-                                ldc<VEC, true>(xj, xp + sgn * st[a]);
-                                const T w = T(wt[a]);
+                        for (int k = 0; k < VEC; ++k) kx[k] = ks[k] = f[k] = T(0);
+                        if (!froz) {
+                            const T* xp = x + (ptrdiff_t)l * C;
+                            T xi[VEC];
+                            ldc<VEC, false>(xi, xp);
+                            const int wt[3] = {surf ? edge_weight(j, kk, n) : 6, surf ? edge_weight(i, kk, n) : 6,
+                                               surf ? edge_weight(i, j, n) : 6};
 #pragma unroll
-                                for (int k = 0; k < VEC; ++k) kx[k] = fma_(w, xi[k] - xj[k], kx[k]);
-                                if (!neu && mode && co[a] == (sgn < 0 ? 1 : n - 1))   // the neighbour lies on the surface
+                            for (int a = 0; a < 3; ++a)
 #pragma unroll
-                                    for (int k = 0; k < VEC; ++k) ks[k] -= T(6) * xj[k];
+                                for (int sg = -1; sg <= 1; sg += 2) {
+                                    // x and y: sg < 0 towards the boundary; z: down
+                                    const int ca = co[a] + sg;
+                                    if (ca < 0 || ca > n) continue;
+                                    const bool flip = (a == 0 && mx) || (a == 1 && my);
+                                    T xj[VEC];
+                                    ldc<VEC, false>(xj, xp + ((sg < 0) != flip ? -st[a] : st[a]));
+                                    const T w = T(wt[a]);
+#pragma unroll
+                                    for (int k = 0; k < VEC; ++k) kx[k] = fma_(w, xi[k] - xj[k], kx[k]);
+                                    if (!neu && mode && (ca == 0 || ca == n))   // the neighbour lies on the surface
+#pragma unroll
+                                        for (int k = 0; k < VEC; ++k) ks[k] -= T(6) * xj[k];
+                                }
+                            if (neu) {
+                                const double vi = (double)(nodes[l] & 0xff);
+#pragma unroll
+                                for (int k = 0; k < VEC; ++k) vx[0][k] = fma_(vi, (double)xi[k], vx[0][k]);
                             }
+                            if (neu || !mode) {
+                                double fb[VEC];
+                                ldc<VEC, false>(fb, bv + (ptrdiff_t)l * B);
+                                if (mode && surf) {   // the BEM term of the adjoint Neumann system
+                                    const int bp = (int)((unsigned)nodes[l] >> 16);
+#pragma unroll
+                                    for (int k = 0; k < VEC; ++k) fb[k] += (double)P.V.ub_out[(size_t)(bp - 1) * C + c0 + k];
+                                }
+#pragma unroll
+                                for (int k = 0; k < VEC; ++k) f[k] = act[k] ? T(fb[k]) : T(0);
+                            }
+                        }
+                        W rv[VEC];
 #pragma unroll
                         for (int k = 0; k < VEC; ++k) {
                             rv[k] = W(f[k] - kx[k]);
@@ -588,12 +738,14 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                             v[2][k] = fma_(ref, ref, v[2][k]);
                             v[3][k] += ref;
                         }
+                        stc<VEC>(r + (ptrdiff_t)l * VEC, rv);
                     }
-                    stc<VEC>(r + (ptrdiff_t)row * VEC, rv);
-                });
-                put(v, pl, ch);
+                }
+                put(v, 0, pl, ch);
+                if constexpr (MP)
+                    if (neu) put(vx, 4, pl, ch);
             });
-            reduce(4);
+            reduce(MP && neu ? 5 : 4);
             int it = 0;
             for (;; ++it) {
                 const bool first = it == 0;
@@ -633,41 +785,45 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                 // ---- P1 ------------------------------------------------------------
                 for (int pa = 0; pa < np; pa += step) {
                     const int pb = min(np, pa + step), nsh = (pb - pa) * VEC;
-                    chunks(pa, pb, [&](int pl, int, int y, int xx, bool my, bool mx, bool on) {
+                    quads(pa, pb, [&](int pl, int, const Quad& q) {
                         W f[4][VEC];
-                        points(pl, y, xx, my, mx, on, [&](int u, bool has, int row, int, int) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
 #pragma unroll
                             for (int k = 0; k < VEC; ++k) f[u][k] = mean[k];
-                            if (has) ldc<VEC, false>(f[u], r + (ptrdiff_t)row * VEC);
-                        });
+                            if (q.has[u]) ldc<VEC, false>(f[u], r + (ptrdiff_t)(pl * pn + q.row[u]) * VEC);
+                        }
 #pragma unroll
                         for (int u = 0; u < 4; ++u)
 #pragma unroll
                             for (int k = 0; k < VEC; ++k) f[u][k] -= mean[k];
-                        if (second)
-                            points(pl, y, xx, my, mx, on, [&](int u, bool has, int, int i, int j) {
-                                const int e = has ? edge_index(i, j, k0 + pl, n) : -1;
-                                if (e >= 0)
+                        if (second) {
+                            const int kk = k0 + pl, bnd = (q.x == 0) + (q.y == 0) + (kk == 0 || kk == n);
+                            if (bnd >= 2)
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) {
+                                    if (!q.has[u]) continue;
+                                    const int e = edge_index((u & 1) ? n - q.x : q.x, (u & 2) ? n - q.y : q.y, kk, n);
 #pragma unroll
                                     for (int k = 0; k < VEC; ++k) f[u][k] += ec[e * VEC + k];
-                            });
-                        if (!on) return;
+                                }
+                        }
+                        if (!q.on) return;
                         // fold about the centre in x, then in y
-                        W* s0 = buf + (pl - pa) * VEC * ss;
-                        const int ya = y * ldx, yb = (n - y) * ldx, xb = n - xx + gap;
+                        W* s = buf + (pl - pa) * VEC * ss;
 #pragma unroll
-                        for (int k = 0; k < VEC; ++k, s0 += ss) {
+                        for (int k = 0; k < VEC; ++k, s += ss) {
                             const W e0 = f[0][k] + f[1][k], e1 = f[2][k] + f[3][k];
                             const W o0 = f[0][k] - f[1][k], o1 = f[2][k] - f[3][k];
-                            s0[ya + xx] = e0 + e1;
-                            if (mx) s0[ya + xb] = o0 + o1;
-                            if (my) s0[yb + xx] = e0 - e1;
-                            if (mx && my) s0[yb + xb] = o0 - o1;
-                            if (!TS && xx == h - 1)   // the gap columns (TS: zero from the start)
+                            s[q.at[0]] = e0 + e1;
+                            if (q.has[1]) s[q.at[1]] = o0 + o1;
+                            if (q.has[2]) s[q.at[2]] = e0 - e1;
+                            if (q.has[3]) s[q.at[3]] = o0 - o1;
+                            if (!TS && q.x == h - 1)   // the gap columns (TS: zero from the start)
                                 for (int c = 0; c < gap + (hop - ho); ++c) {
                                     const int cc = c < gap ? h + c : hp + ho + c - gap;
-                                    s0[ya + cc] = W(0);
-                                    if (my) s0[yb + cc] = W(0);
+                                    s[q.y * ldx + cc] = W(0);
+                                    if (q.has[2]) s[(n - q.y) * ldx + cc] = W(0);
                                 }
                         }
                     });
@@ -687,19 +843,14 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                 // ---- P2 ------------------------------------------------------------
                 const int z0 = (int)rank * g.zc, z1 = min(ss, z0 + g.zc);
                 for (int za = z0; za < z1; za += g.pr) {
-                    const int pc = min(g.pr, z1 - za), ld = VEC * pc, q4 = pc >> 2;
-                    for (int e = tid; e < h * VEC * q4; e += nt) {
-                        const int k = e / (VEC * q4), rem = e - k * VEC * q4, c = rem / q4, pos = za + 4 * (rem - c * q4);
+                    const int pc = min(g.pr, z1 - za), ld = VEC * pc, q4 = pc >> 2, per = VEC * q4;
+                    for (int e = tid; e < h * per; e += nt) {
+                        const int k = e / per, rem = e - k * per, c = VEC == 1 ? 0 : rem / q4, p4 = 4 * (rem - c * q4);
+                        const int off = c * ss + za + p4;
                         W a[4], b[4] = {W(0), W(0), W(0), W(0)}, s[4];
-                        if constexpr (TS) {
-                            const uint32_t off = (uint32_t)((c * ss + pos) * (int)sizeof(W));
-                            ld_peer(s_plane[k] + off, a);
-                            if (k < ho) ld_peer(s_plane[n - k] + off, b);
-                        } else {
-                            ldc<4, true>(a, gt + ((size_t)k * VEC + c) * ss + pos);
-                            if (k < ho) ldc<4, true>(b, gt + ((size_t)(n - k) * VEC + c) * ss + pos);
-                        }
-                        W* zp = zb + k * ld + c * pc + (pos - za);
+                        ld4(s_plane[k] + off, a);
+                        if (k < ho) ld4(s_plane[n - k] + off, b);
+                        W* zp = zb + k * ld + c * pc + p4;
 #pragma unroll
                         for (int j = 0; j < 4; ++j) s[j] = a[j] + b[j];
                         st4(zp, s);
@@ -712,9 +863,10 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                     __syncthreads();
                     pass_left<W>(g.o_z, 1, ld, oFe, oFo, s2, hp, hop, inv + za, pc);
                     pass_left<W>(g.o_z, 1, ld, oGe, oGo, s2, hp, hop, nullptr, 1);
-                    for (int e = tid; e < h * VEC * q4; e += nt) {
-                        const int k = e / (VEC * q4), rem = e - k * VEC * q4, c = rem / q4, pos = za + 4 * (rem - c * q4);
-                        const W* zp = zb + k * ld + c * pc + (pos - za);
+                    for (int e = tid; e < h * per; e += nt) {
+                        const int k = e / per, rem = e - k * per, c = VEC == 1 ? 0 : rem / q4, p4 = 4 * (rem - c * q4);
+                        const int off = c * ss + za + p4;
+                        const W* zp = zb + k * ld + c * pc + p4;
                         W a[4], b[4] = {W(0), W(0), W(0), W(0)}, s[4], t[4];
                         ld4(zp, a);
                         if (k < ho) ld4(zp + (n - 2 * k) * ld, b);
@@ -723,14 +875,8 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                             s[j] = a[j] + b[j];
                             t[j] = a[j] - b[j];
                         }
-                        if constexpr (TS) {
-                            const uint32_t off = (uint32_t)((c * ss + pos) * (int)sizeof(W));
-                            st_peer(s_plane[k] + off, s);
-                            if (k < ho) st_peer(s_plane[n - k] + off, t);
-                        } else {
-                            st4(gt + ((size_t)k * VEC + c) * ss + pos, s);
-                            if (k < ho) st4(gt + ((size_t)(n - k) * VEC + c) * ss + pos, t);
-                        }
+                        st4(s_plane[k] + off, s);
+                        if (k < ho) st4(s_plane[n - k] + off, t);
                     }
                     __syncthreads();
                 }
@@ -748,21 +894,19 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                     }
                     pass_left<W>(0, nsh, ldx, oGe, oGo, s2, hp, hop, nullptr, 1);
                     pass_right<W>(0, nsh, oGe, oGo, s2, hp, hop);
-                    chunks(pa, pb, [&](int pl, int, int y, int xx, bool my, bool mx, bool on) {
-                        if (!on) return;   // unfold, in place
-                        W* s0 = buf + (pl - pa) * VEC * ss;
-                        const int ya = y * ldx, yb = (n - y) * ldx, xb = n - xx + gap;
+                    quads(pa, pb, [&](int pl, int, const Quad& q) {
+                        if (!q.on) return;   // unfold, in place
+                        W* s = buf + (pl - pa) * VEC * ss;
 #pragma unroll
-                        for (int k = 0; k < VEC; ++k, s0 += ss) {
-                            const W ee = s0[ya + xx], eo = mx ? s0[ya + xb] : W(0), oe = my ? s0[yb + xx] : W(0);
-                            const W oo = mx && my ? s0[yb + xb] : W(0);
-                            s0[ya + xx] = (ee + eo) + (oe + oo);
-                            if (mx) s0[ya + xb] = (ee - eo) + (oe - oo);
-                            if (my) s0[yb + xx] = (ee + eo) - (oe + oo);
-                            if (mx && my) s0[yb + xb] = (ee - eo) - (oe - oo);
+                        for (int k = 0; k < VEC; ++k, s += ss) {
+                            const W ee = s[q.at[0]], eo = q.has[1] ? s[q.at[1]] : W(0), oe = q.has[2] ? s[q.at[2]] : W(0);
+                            const W oo = q.has[3] ? s[q.at[3]] : W(0);
+                            s[q.at[0]] = (ee + eo) + (oe + oo);
+                            if (q.has[1]) s[q.at[1]] = (ee - eo) + (oe - oo);
+                            if (q.has[2]) s[q.at[2]] = (ee + eo) - (oe + oo);
+                            if (q.has[3]) s[q.at[3]] = (ee - eo) - (oe - oo);
                         }
                     });
-                    __syncwarp();
                     if constexpr (!TS) {
                         __syncthreads();
                         for (int i = tid * 4; i < nsh * ss; i += nt * 4) {
@@ -778,85 +922,63 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                 W keep[VEC];   // 0: the system has converged and stays as it is
 #pragma unroll
                 for (int k = 0; k < VEC; ++k) keep[k] = s_flag[k] ? W(0) : W(1);
-                chunks(0, np, [&](int pl, int ch, int y, int xx, bool my, bool mx, bool on) {
+                quads(0, np, [&](int pl, int ch, const Quad& q) {
                     W v[2][VEC];   // r.r, sum r
 #pragma unroll
                     for (int k = 0; k < VEC; ++k) v[0][k] = v[1][k] = W(0);
                     const int kk = k0 + pl;
+                    const bool froz = !neu && (q.x == 0 || q.y == 0 || kk == 0 || kk == n);
                     W rv[4][VEC], dv[4][VEC];
-                    points(pl, y, xx, my, mx, on, [&](int u, bool has, int row, int, int) {
-                        if (!has) return;
-                        ldc<VEC, false>(rv[u], r + (ptrdiff_t)row * VEC);
-                        if (!first) ldc<VEC, false>(dv[u], d + (ptrdiff_t)row * VEC);
-                    });
-                    points(pl, y, xx, my, mx, on, [&](int u, bool has, int row, int i, int j) {
-                        if (!has) return;
-                        const bool surf = i == 0 || i == n || j == 0 || j == n || kk == 0 || kk == n;
-                        const W wx = W(surf ? edge_weight(j, kk, n) : 6), wy = W(surf ? edge_weight(i, kk, n) : 6),
-                                wz = W(surf ? edge_weight(i, j, n) : 6);
-                        const int ci = i + (i < h ? 0 : gap), cm = i - 1 + (i - 1 < h ? 0 : gap),
-                                  cp = i + 1 + (i + 1 < h ? 0 : gap);
-                        const W* zr = TS ? buf + pl * VEC * ss + j * ldx : gt + (size_t)kk * VEC * ss + j * ldx;
 #pragma unroll
-                        for (int k = 0; k < VEC; ++k) {
-                            const W* zk = zr + k * ss;
-                            const W zc = TS ? zk[ci] : __ldcg(zk + ci);
-                            W a = W(0);
-                            auto add = [&](W wt, W zj) { a = fma_(wt, zc - zj, a); };
-                            if (kk > 0) {
-                                if constexpr (TS) {
-                                    add(wz, pl > 0 ? zk[ci - VEC * ss]
-                                                   : ld_peer1(s_plane[kk - 1] + (uint32_t)((k * ss + j * ldx + ci) * (int)sizeof(W)), W(0)));
-                                } else {
-                                    add(wz, __ldcg(zk + ci - VEC * ss));
-                                }
-                            }
-                            if (j > 0) add(wy, TS ? zk[ci - ldx] : __ldcg(zk + ci - ldx));
-                            if (i > 0) add(wx, TS ? zk[cm] : __ldcg(zk + cm));
-                            if (i < n) add(wx, TS ? zk[cp] : __ldcg(zk + cp));
-                            if (j < n) add(wy, TS ? zk[ci + ldx] : __ldcg(zk + ci + ldx));
-                            if (kk < n) {
-                                if constexpr (TS) {
-                                    add(wz, pl + 1 < np ? zk[ci + VEC * ss]
-                                                        : ld_peer1(s_plane[kk + 1] + (uint32_t)((k * ss + j * ldx + ci) * (int)sizeof(W)), W(0)));
-                                } else {
-                                    add(wz, __ldcg(zk + ci + VEC * ss));
-                                }
-                            }
-                            if (!neu && surf) a = W(0);
+                    for (int u = 0; u < 4; ++u) {
+                        if (!q.has[u]) continue;
+                        const ptrdiff_t o = (ptrdiff_t)(pl * pn + q.row[u]) * VEC;
+                        ldc<VEC, false>(rv[u], r + o);
+                        if (!MP || !first) ldc<VEC, false>(dv[u], d + o);
+                        else
+#pragma unroll
+                            for (int k = 0; k < VEC; ++k) dv[u][k] = W(0);
+                    }
+                    const W *s = own(kk, pl), *sm = below(kk, pl), *sp = above(kk, pl);
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k)
+                        stencil(q, kk, s + k * ss, sm + k * ss, sp + k * ss, [&](int u, W zc, W a) {
+                            if (froz) a = W(0);
                             rv[u][k] = fma_(-keep[k], a, rv[u][k] - mean[k]);
-                            dv[u][k] = first ? keep[k] * zc : fma_(keep[k], zc, dv[u][k]);
+                            dv[u][k] = fma_(keep[k], zc, dv[u][k]);
                             v[0][k] = fma_(rv[u][k], rv[u][k], v[0][k]);
                             v[1][k] += rv[u][k];
-                        }
-                        stc<VEC>(r + (ptrdiff_t)row * VEC, rv[u]);
-                        stc<VEC>(d + (ptrdiff_t)row * VEC, dv[u]);
-                    });
-                    put(v, pl, ch);
+                        });
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        if (!q.has[u]) continue;
+                        const ptrdiff_t o = (ptrdiff_t)(pl * pn + q.row[u]) * VEC;
+                        stc<VEC>(r + o, rv[u]);
+                        stc<VEC>(d + o, dv[u]);
+                    }
+                    put(v, 0, pl, ch);
                 });
                 if (neu && !second) {
                     // H z on the edge nodes for the second step of the pair: this CTA's
                     // rows, each in FS_SPLIT parts, to the CTAs that own the nodes
                     for (int t = tid; t < g.ne * VEC; t += nt) {
-                        const int k = t / g.ne, e = t - k * g.ne;
+                        const int k = VEC == 1 ? 0 : t / g.ne, e = t - k * g.ne;
                         int i, j, l;
                         edge_node(e, n, i, j, l);
-                        const int at = k * ss + j * ldx + i + (i < h ? 0 : gap);
-                        ev[e * VEC + k] = TS ? ld_peer1(s_plane[l] + (uint32_t)(at * (int)sizeof(W)), W(0))
-                                             : __ldcg(gt + (size_t)l * VEC * ss + at);
+                        ev[e * VEC + k] = s_plane[l][k * ss + j * ldx + i + (i < h ? 0 : gap)];
                     }
                     __syncthreads();
                     const int e0 = (int)rank * g.er, er = max(0, min(g.er, g.ne - e0)), sl = (g.ne + FS_SPLIT - 1) / FS_SPLIT;
                     for (int t = tid; t < er * FS_SPLIT; t += nt) {
-                        const int s = t / er, e = t - s * er;
+                        const int sq = t / er, e = t - sq * er;
                         W acc[VEC];
 #pragma unroll
                         for (int k = 0; k < VEC; ++k) acc[k] = W(0);
                         const W* Hp = A.edge + e0 + e;   // column e0 + e of the symmetric matrix
-                        const int fb = min(g.ne, (s + 1) * sl);
+                        const int fb = min(g.ne, (sq + 1) * sl);
 #pragma unroll 8
-                        for (int f = s * sl; f < fb; ++f) {
-                            const W hv = __ldg(Hp + (size_t)f * g.ne);
+                        for (int f = sq * sl; f < fb; ++f) {
+                            const W hv = __ldg(Hp + f * g.ne);
 #pragma unroll
                             for (int k = 0; k < VEC; ++k) acc[k] = fma_(hv, ev[f * VEC + k], acc[k]);
                         }
@@ -868,7 +990,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                         const int e = t / VEC, k = t - e * VEC;
                         W acc = W(0);
 #pragma unroll
-                        for (int s = 0; s < FS_SPLIT; ++s) acc += ep[(s * er + e) * VEC + k];
+                        for (int sq = 0; sq < FS_SPLIT; ++sq) acc += ep[(sq * er + e) * VEC + k];
                         int i, j, l;
                         edge_node(e0 + e, n, i, j, l);
                         st_peer1(peer_addr(sm_addr(ec + (e0 + e) * VEC + k), (unsigned)(l / g.ppc)), acc);
@@ -876,68 +998,91 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                 }
                 reduce(2);
             }
-            if (it > 0) {   // the sum of the steps into x before anything reads x
-                for (int row = lo + tid; row < hi; row += nt) {
-                    T xv[VEC];
-                    W dv[VEC];
-                    ldc<VEC, false>(xv, x + (size_t)row * C + c0);
-                    ldc<VEC, false>(dv, d + (ptrdiff_t)row * VEC);
-#pragma unroll
-                    for (int k = 0; k < VEC; ++k) xv[k] += T(dv[k]);
-                    stc<VEC>(x + (size_t)row * C + c0, xv);
-                }
-            }
-            cl_sync();
             if constexpr (!MP) {
                 break;
             } else {
                 // done when every system met the tolerance on its true residual at the
-                // start of this cycle (or ran out of iterations or cycles)
-                if (__syncthreads_and(tid < VEC ? s_done[tid] : 1) || cycle + 1 >= MP_MAX_CYCLES) break;
+                // start of this cycle (or ran out of iterations)
+                if (__syncthreads_and(tid < VEC ? s_done[tid] : 1)) {
+                    ended = true;
+                    break;
+                }
+                if (it > 0)   // the cycle's steps into x before anything reads x
+                    for (int l = tid; l < hi - lo; l += nt) {
+                        T xv[VEC];
+                        W dv[VEC];
+                        ldc<VEC, false>(xv, x + (ptrdiff_t)l * C);
+                        ldc<VEC, false>(dv, d + (ptrdiff_t)l * VEC);
+#pragma unroll
+                        for (int k = 0; k < VEC; ++k) xv[k] += T(dv[k]);
+                        stc<VEC>(x + (ptrdiff_t)l * C, xv);
+                    }
+                cl_sync();
+                if (cycle + 1 >= MP_MAX_CYCLES) break;
             }
         }
-        // epilogue: Neumann systems are gauged to zero V-weighted mean and (stage 1)
-        // hand u1_S to the BEM product; stage-1 Dirichlet (adjoint) systems hand
-        // t = b_S - K_SI w (w vanishes on the surface, so K_SI w = (K w)_S)
+        // Neumann systems are gauged to zero V-weighted mean and (stage 1) hand u1_S to
+        // the BEM product; stage-1 Dirichlet (adjoint) systems hand t = b_S - K_SI w (w
+        // vanishes on the surface, so K_SI w = (K w)_S)
+        double mean[VEC];
+#pragma unroll
+        for (int k = 0; k < VEC; ++k) mean[k] = 0.0;
         if (neu) {
-            chunks(0, np, [&](int pl, int ch, int y, int xx, bool my, bool mx, bool on) {
-                double v[1][VEC];
+            if (!ended) {   // MP: the residual pass that ended the solve has summed V x
+                quads(0, np, [&](int pl, int ch, const Quad& q) {
+                    T v[1][VEC];
 #pragma unroll
-                for (int k = 0; k < VEC; ++k) v[0][k] = 0.0;
-                points(pl, y, xx, my, mx, on, [&](int, bool has, int row, int, int) {
-                    if (!has) return;
-                    const double vi = (double)(P.M.node[row] & 0xff);
-                    T xv[VEC];
-                    ldc<VEC, true>(xv, x + (size_t)row * C + c0);
+                    for (int k = 0; k < VEC; ++k) v[0][k] = T(0);
 #pragma unroll
-                    for (int k = 0; k < VEC; ++k) v[0][k] = fma_(vi, (double)xv[k], v[0][k]);
+                    for (int u = 0; u < 4; ++u) {
+                        if (!q.has[u]) continue;
+                        const int l = pl * pn + q.row[u];
+                        const T vi = T(nodes[l] & 0xff);
+                        T xv[VEC];
+                        if constexpr (MP) {
+                            ldc<VEC, false>(xv, x + (ptrdiff_t)l * C);
+                        } else {
+                            ldc<VEC, false>(xv, d + (ptrdiff_t)l * VEC);
+                        }
+#pragma unroll
+                        for (int k = 0; k < VEC; ++k) v[0][k] = fma_(vi, xv[k], v[0][k]);
+                    }
+                    put(v, 4, pl, ch);
                 });
-                put(v, pl, ch);
-            });
-            reduce(1);
-            T mean[VEC];
+                reduce(5);
+            }
 #pragma unroll
-            for (int k = 0; k < VEC; ++k) mean[k] = T(out[k] / P.M.vsum);
-            for (int row = lo + tid; row < hi; row += nt) {
-                const int bp = (int)((unsigned)P.M.node[row] >> 16);
+            for (int k = 0; k < VEC; ++k) mean[k] = out[4 * VEC + k] / P.M.vsum;
+        }
+        if (!MP || neu)
+            for (int l = tid; l < hi - lo; l += nt) {
                 T xv[VEC];
-                ldc<VEC, true>(xv, x + (size_t)row * C + c0);
+                if constexpr (MP) {
+                    ldc<VEC, false>(xv, x + (ptrdiff_t)l * C);
+                } else {
+                    W dv[VEC];
+                    ldc<VEC, false>(dv, d + (ptrdiff_t)l * VEC);
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k) xv[k] = T(dv[k]);
+                }
+                const int bp = neu && mode == 0 ? (int)((unsigned)nodes[l] >> 16) : 0;
 #pragma unroll
                 for (int k = 0; k < VEC; ++k) {
                     if (!act[k]) continue;
-                    xv[k] -= mean[k];
-                    if (mode == 0 && bp) P.V.ub_in[(size_t)(bp - 1) * C + c0 + k] = xv[k];
+                    xv[k] -= T(mean[k]);
+                    if (bp) P.V.ub_in[(size_t)(bp - 1) * C + c0 + k] = xv[k];
                 }
-                stc<VEC>(x + (size_t)row * C + c0, xv);
+                stc<VEC>(x + (ptrdiff_t)l * C, xv);
             }
-        } else if (mode == 0) {
-            for (int row = lo + tid; row < hi; row += nt) {
-                const int bp = (int)((unsigned)P.M.node[row] >> 16);
+        if (!neu && mode == 0) {
+            cl_sync();   // x of the neighbouring planes
+            for (int l = tid; l < hi - lo; l += nt) {
+                const int bp = (int)((unsigned)nodes[l] >> 16);
                 if (!bp) continue;
                 // at most one of the six neighbours of a surface node lies inside
-                const int i = row % s2, j = (row / s2) % s2, k3 = row / (s2 * s2);
-                const T* xp = x + (size_t)row * C + c0;
-                const ptrdiff_t st[3] = {(ptrdiff_t)C, (ptrdiff_t)s2 * C, (ptrdiff_t)s2 * s2 * C};
+                const int row = lo + l, i = row % s2, j = (row / s2) % s2, k3 = row / pn;
+                const T* xp = x + (ptrdiff_t)l * C;
+                const ptrdiff_t st[3] = {(ptrdiff_t)C, (ptrdiff_t)s2 * C, (ptrdiff_t)pn * C};
                 const int co[3] = {i, j, k3};
                 T kw[VEC];
                 double f[VEC];
@@ -953,7 +1098,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
 #pragma unroll
                     for (int k = 0; k < VEC; ++k) kw[k] = T(-6) * xj[k];
                 }
-                ldc<VEC, false>(f, P.V.bvec + (size_t)row * B + b0);
+                ldc<VEC, false>(f, bv + (ptrdiff_t)l * B);
 #pragma unroll
                 for (int k = 0; k < VEC; ++k)
                     if (act[k]) P.V.ub_in[(size_t)(bp - 1) * C + c0 + k] = T(f[k]) - kw[k];
@@ -1020,7 +1165,7 @@ bool fit_geo(FsGeo& g, int vec, int ppc, size_t word, int threads, bool ts) {
     const size_t mat = up(g.matw * word), part = up(sizeof(double) * (size_t)ppc * g.nch * FS_NQ * vec);
     const size_t slot = up(sizeof(double) * 2 * (size_t)ppc * FS_NQ * vec);
     const size_t edge = up(word * vec * (2 * (size_t)g.ne + (size_t)g.er * FS_SPLIT));
-    const size_t col = up(sizeof(double) * (FS_NQ + 3) * vec + sizeof(int) * 3 * vec + 4 * 2 * FS_MAX_N1);
+    const size_t col = up(sizeof(double) * (FS_NQ + 3) * vec + sizeof(int) * 3 * vec + (8 + 4) * FS_MAX_N1);
     const size_t vecs = up(word * vec * 2 * (size_t)ppc * g.s2 * g.s2);
     const size_t fixed = mat + part + slot + edge + col;
     const size_t sheet = (size_t)g.ss * word * vec;
@@ -1098,53 +1243,84 @@ struct FsChoice {
 };
 
 template <typename T, typename W, int VEC, bool TS>
-void try_shapes(const Launch& L, int n, int B, FsChoice& best, double& best_cost) {
+void try_shapes(const Launch& L, int n, int B, int groups, FsChoice& best, double& best_cost) {
     if (B % VEC) return;
-    int groups = 0;   // with an active instance
-    for (int gi = 0; gi < 2 * B / VEC; ++gi) {
-        bool a = L.active == nullptr;
-        for (int i = 0; i < VEC && !a; ++i) a = L.active[(gi * VEC + i) % B] != 0;
-        groups += a;
-    }
-    if (groups == 0) groups = 1;
+    const int most = sizeof(W) == 8 ? 512 : 1024;
     for (int ppc = 1, last = 0; ppc <= n + 1; ++ppc) {
-        FsGeo g = base_geo(n);
-        const int cl = (g.s2 + ppc - 1) / ppc;
+        const int cl = (n + ppc) / ppc;
         if (cl > FS_MAX_CL || cl == last) continue;   // more planes, no fewer CTAs
         last = cl;
-        // threads: about eight nodes each, 256 to the kernel's most
-        const int most = sizeof(W) == 8 ? 512 : 1024;
-        int threads = 256;
-        while (threads < most && (long long)ppc * VEC * g.s2 * g.s2 > 8LL * threads) threads *= 2;
-        if (!fit_geo(g, VEC, ppc, sizeof(W), threads, TS)) continue;
-        int r = resident<T, W, VEC, TS>(g, threads);
-        if (L.max_blocks > 0) r = std::min(r, std::max(1, L.max_blocks / cl));
-        if (r < 1) continue;
-        const int waves = (groups + r - 1) / r;
-        const double cost = waves * ((double)ppc * VEC * g.s2 * g.s2 + 1500.0) * (TS ? 1.0 : 1.5);
-        if (best.vec == 0 || cost < best_cost) {
-            best_cost = cost;
-            best.g = g;
-            best.vec = VEC;
-            best.threads = threads;
-            best.ts = TS;
-            best.clusters = waves > 1 ? 2 * B / VEC : std::min(r, 2 * B / VEC);
+        for (int threads = 256; threads <= most; threads *= 2) {
+            FsGeo g = base_geo(n);
+            if (!fit_geo(g, VEC, ppc, sizeof(W), threads, TS)) continue;
+            int r = resident<T, W, VEC, TS>(g, threads);
+            if (L.max_blocks > 0) r = std::min(r, std::max(1, L.max_blocks / cl));
+            if (r < 1) continue;
+            const int waves = (groups + r - 1) / r;
+            // CTAs that share an SM share its issue slots; a CTA's own rows take their
+            // latencies whatever the others do (us of two stages)
+            const double rows = (double)ppc * VEC * g.s2 * g.s2 * (sizeof(W) == 8 ? 3.9 : 1.0);
+            const double load = std::max(1.0, std::min(groups, r) * (double)cl / L.num_sms);
+            double cost = waves * (5.8 + rows * std::max(1.9e-3 * load, 0.42e-3 * 256 / threads)) * (TS ? 1.0 : 1.5);
+            if (sizeof(T) != sizeof(W))   // FP64 residuals: latencies weigh more, waves overlap
+                cost = std::max(1.0, (double)groups / r) * (TS ? 1.0 : 1.5) * (1.0 + 0.04 * ppc) *
+                       (3.0 + 0.3 * threads / 256 + rows * std::max(1.9e-3 * load, 2.5e-3 * 256 / threads));
+            if (best.vec == 0 || cost < best_cost) {
+                best_cost = cost;
+                best.g = g;
+                best.vec = VEC;
+                best.threads = threads;
+                best.ts = TS;
+                best.clusters = waves > 1 ? 2 * B / VEC : std::min(r, 2 * B / VEC);
+            }
         }
     }
 }
 
-// The launch for a batch: VEC systems per cluster and planes per CTA.  Clusters
-// are independent, so more of them than can be resident at once run in waves; the
-// cost of a wave is the nodes of a CTA's planes plus a constant for the barriers
-// and latencies of an iteration (about 1500 nodes' worth).
+// The launch for a batch: VEC systems per cluster, planes per CTA, threads.  Clusters
+// are independent, so more of them than can be resident at once run in waves.  The
+// constants are fitted to 287 measured shapes of fifteen sizes and batches (n = 10 to
+// 80, 1 to 64 instances), on which the rule picks the fastest to 1 %: 64 instances at
+// n = 30 run one system on two CTAs of 16 planes and 512 threads (0.37 ms a stage; 0.46
+// on sixteen CTAs of two planes, 0.80 on one CTA), one instance at n = 20 on eleven CTAs
+// of two planes (62 us; 120 on two CTAs).
 template <typename T, typename W>
 FsChoice choose(const Launch& L, const MeshView& M, int B) {
+    // groups of 1, 2 and 4 systems with an active instance
+    int groups[3];
+    for (int v = 0; v < 3; ++v) {
+        const int vec = 1 << v;
+        groups[v] = 0;
+        for (int gi = 0; B % vec == 0 && gi < B / vec; ++gi) {
+            bool a = L.active == nullptr;
+            for (int i = 0; i < vec && !a; ++i) a = L.active[gi * vec + i] != 0;
+            groups[v] += 2 * a;   // forward and adjoint systems
+        }
+        groups[v] = std::max(1, groups[v]);
+    }
+    // the search takes some 10 us: its results are kept (a bounded number of them)
+    static std::mutex mu;
+    static std::map<std::tuple<int, int, int, int, int, int, int>, FsChoice> known;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const auto key = std::make_tuple(dev, M.n, B, groups[0], groups[1], groups[2], L.max_blocks);
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        auto it = known.find(key);
+        if (it != known.end()) return it->second;
+    }
     FsChoice c;
     double cost = 0.0;
-    if constexpr (sizeof(W) == 4) try_shapes<T, W, 4, true>(L, M.n, B, c, cost);
-    try_shapes<T, W, 2, true>(L, M.n, B, c, cost);
-    try_shapes<T, W, 1, true>(L, M.n, B, c, cost);
-    if (!c.vec) try_shapes<T, W, 1, false>(L, M.n, B, c, cost);
+    // mixed iterations run one system per cluster: their FP64 residual gathers gain
+    // nothing from vectors of instances (32 at n = 30: 1.9 ms for two stages, 2.2 with
+    // two systems, 3.9 with four; the best shape of all eleven measured sizes has one)
+    if constexpr (sizeof(T) == 4) try_shapes<T, W, 4, true>(L, M.n, B, groups[2], c, cost);
+    if constexpr (sizeof(T) == sizeof(W)) try_shapes<T, W, 2, true>(L, M.n, B, groups[1], c, cost);
+    try_shapes<T, W, 1, true>(L, M.n, B, groups[0], c, cost);
+    if (!c.vec) try_shapes<T, W, 1, false>(L, M.n, B, groups[0], c, cost);
+    std::lock_guard<std::mutex> lk(mu);
+    if (known.size() >= 4096) known.clear();
+    known.emplace(key, c);
     return c;
 }
 
@@ -1189,9 +1365,11 @@ cudaError_t solve_as(const Launch& L, const MeshView& M, const BatchView<T>& V, 
     }
     switch (c.vec * 2 + (c.ts ? 1 : 0)) {
         case 9:
-            if constexpr (sizeof(W) == 4) return launch_fast<T, W, 4, true>(L, a, c);
+            if constexpr (sizeof(T) == 4) return launch_fast<T, W, 4, true>(L, a, c);
             return cudaErrorInvalidValue;
-        case 5: return launch_fast<T, W, 2, true>(L, a, c);
+        case 5:
+            if constexpr (sizeof(T) == sizeof(W)) return launch_fast<T, W, 2, true>(L, a, c);
+            return cudaErrorInvalidValue;
         case 3: return launch_fast<T, W, 1, true>(L, a, c);
         default: return launch_fast<T, W, 1, false>(L, a, c);
     }
