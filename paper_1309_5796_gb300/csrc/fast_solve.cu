@@ -26,7 +26,7 @@
 //
 // Measured on GB300 (two stages of both chains, FP64 n = 10 / FP32 n = 20, 80, one
 // instance / FP32 n = 30, 64 instances, before: diagonally preconditioned CG):
-// 0.13 / 0.12 / 1.5 / 0.96 ms, before 6.1 / 5.6 / 36 / 12 ms.
+// 0.13 / 0.13 / 1.5 / 0.72 ms, before 6.1 / 5.6 / 36 / 12 ms.
 //
 // One thread-block cluster solves VEC systems (columns of the [N][2B] layout)
 // of one kind; CTA r owns the z-planes [r ppc, (r+1) ppc).  Per step:
@@ -1261,7 +1261,9 @@ void try_shapes(const Launch& L, int n, int B, int groups, FsChoice& best, doubl
             // latencies whatever the others do (us of two stages)
             const double rows = (double)ppc * VEC * g.s2 * g.s2 * (sizeof(W) == 8 ? 3.9 : 1.0);
             const double load = std::max(1.0, std::min(groups, r) * (double)cl / L.num_sms);
-            double cost = waves * (5.8 + rows * std::max(1.9e-3 * load, 0.42e-3 * 256 / threads)) * (TS ? 1.0 : 1.5);
+            double cost = waves * (TS ? 1.0 : 1.5) *
+                          (5.8 + 1.1 * threads / 256 +
+                           rows * std::max(0.83e-3 * load, 3.1e-3 * 256 / threads) * (1.0 + 0.14 * (VEC - 1)));
             if (sizeof(T) != sizeof(W))   // FP64 residuals: latencies weigh more, waves overlap
                 cost = std::max(1.0, (double)groups / r) * (TS ? 1.0 : 1.5) * (1.0 + 0.04 * ppc) *
                        (3.0 + 0.3 * threads / 256 + rows * std::max(1.9e-3 * load, 2.5e-3 * 256 / threads));
@@ -1279,11 +1281,11 @@ void try_shapes(const Launch& L, int n, int B, int groups, FsChoice& best, doubl
 
 // The launch for a batch: VEC systems per cluster, planes per CTA, threads.  Clusters
 // are independent, so more of them than can be resident at once run in waves.  The
-// constants are fitted to 287 measured shapes of fifteen sizes and batches (n = 10 to
-// 80, 1 to 64 instances), on which the rule picks the fastest to 1 %: 64 instances at
-// n = 30 run one system on two CTAs of 16 planes and 512 threads (0.37 ms a stage; 0.46
-// on sixteen CTAs of two planes, 0.80 on one CTA), one instance at n = 20 on eleven CTAs
-// of two planes (62 us; 120 on two CTAs).
+// constants are fitted to some 400 measured shapes of 25 sizes and batches (n = 10 to
+// 80, 1 to 64 instances), on which the rule's shape is within 5 % of the fastest (1 % on
+// average): 64 instances at n = 30 run one system on two CTAs of 16 planes and 512
+// threads (0.36 ms a stage; 0.46 on sixteen CTAs of two planes, 0.80 on one CTA), one
+// instance at n = 20 on eleven CTAs of two planes (62 us; 120 on two CTAs).
 template <typename T, typename W>
 FsChoice choose(const Launch& L, const MeshView& M, int B) {
     // groups of 1, 2 and 4 systems with an active instance
