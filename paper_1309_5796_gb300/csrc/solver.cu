@@ -535,32 +535,78 @@ __global__ void __launch_bounds__(SINGLE ? PCG_SINGLE_THREADS : PCG_THREADS, 1) 
         }
 }
 
+// The groups of VEC instances (VEC = 1: instances) that still run, as first instance * 2
+// + its current buffer, ascending, in list[0 .. returned); B <= 256.  The node kernels
+// hand their lanes to these only: with lanes for every instance, the ones that had
+// finished took issue slots to the end (on average over half of a batch of 32 that
+// minimises to 1e-6 of torque).
+template <int VEC>
+__device__ __forceinline__ int active_list(const InstState* st, int B, int* list) {
+    __shared__ int s_n;
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        int n = 0;
+        for (int g0 = 0; g0 < B / VEC; g0 += 32) {
+            const int b = (g0 + lane) * VEC;
+            bool a = false;
+            int cur = 0;
+            if (b < B) {
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) a |= st[b + k].phase != PH_DONE;
+                cur = st[b].cur;
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, a);
+            if (a) list[n + __popc(m & ((1u << lane) - 1))] = b * 2 + cur;
+            n += __popc(m);
+        }
+        if (lane == 0) s_n = n;
+    }
+    __syncthreads();
+    return s_n;
+}
+
 // b_i = (1/4) sum_j Gint_ij . m_j at the trial point of every active instance
 // (one thread per row and instance, instances fastest): computed once per
 // evaluation and read by both potential-solve stages (forward and adjoint
 // right-hand sides, the adjoint's surface hand-off), by the same arithmetic
-// (rhs_b) the solves used inline before.
-template <typename T, bool GEN>
+// (rhs_b) the solves used inline before.  VEC = 4 (batches of a multiple of 4 in
+// FP32, where the trial point has one copy): four instances a thread, so that the
+// row's entries are read once and the trial point in 16-byte vectors.
+template <typename T, bool GEN, int VEC>
 __global__ void k_rhs(MeshView M, BatchView<T> V) {
+    __shared__ int s_act[256 / VEC];
     const int B = V.B;
-    const size_t total = (size_t)M.N * B;
+    const unsigned G = active_list<VEC>(V.st, B, s_act);
+    const unsigned total = (unsigned)M.N * G;   // < 2^32: 96 bytes of the state each
     const typename GenTab<T>::V4* __restrict__ gA = GEN ? GenTab<T>::A(M) : nullptr;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        const int b = (int)(t % B);
-        const int row = (int)(t / B);
-        const InstState& s = V.st[b];
-        if (s.phase == PH_DONE) continue;
-        V.bvec[t] = rhs_b<T, GEN>(M.col, M.pkA, gA, M.rowptr[row], M.rowptr[row + 1], trial_m(V, s.cur, M.N), B, b);
+    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+        const int row = (int)(t / G), act = s_act[t - (unsigned)row * G], b = act >> 1;
+        if constexpr (VEC == 4) {
+            double f[4];   // of finished instances too: nothing reads theirs
+            rhs_b4<T, GEN>(M.col, M.pkA, gA, M.rowptr[row], M.rowptr[row + 1], trial_m(V, 0, M.N), B, b, f);
+            double2* o = reinterpret_cast<double2*>(V.bvec + (size_t)row * B + b);
+            o[0] = make_double2(f[0], f[1]);
+            o[1] = make_double2(f[2], f[3]);
+        } else {
+            V.bvec[(size_t)row * B + b] =
+                rhs_b<T, GEN>(M.col, M.pkA, gA, M.rowptr[row], M.rowptr[row + 1], trial_m(V, act & 1, M.N), B, b);
+        }
     }
 }
 
 template <typename T>
 void rhs_eval(const Launch& L, const MeshView& M, const BatchView<T>& V) {
-    const size_t total = (size_t)M.N * V.B;
-    size_t blocks = (total + 255) / 256;
-    if (blocks > (size_t)8 * L.num_sms) blocks = (size_t)8 * L.num_sms;
-    if (M.gen) k_rhs<T, true><<<(unsigned)blocks, 256, 0, L.stream>>>(M, V);
-    else k_rhs<T, false><<<(unsigned)blocks, 256, 0, L.stream>>>(M, V);
+    const bool v4 = sizeof(T) == 4 && V.B % 4 == 0;
+    const size_t total = (size_t)M.N * (v4 ? V.B / 4 : V.B);
+    size_t blocks = (total + 127) / 128;
+    if (blocks > (size_t)16 * L.num_sms) blocks = (size_t)16 * L.num_sms;
+    if (M.gen) {
+        if (v4) k_rhs<T, true, 4><<<(unsigned)blocks, 128, 0, L.stream>>>(M, V);
+        else k_rhs<T, true, 1><<<(unsigned)blocks, 128, 0, L.stream>>>(M, V);
+    } else {
+        if (v4) k_rhs<T, false, 4><<<(unsigned)blocks, 128, 0, L.stream>>>(M, V);
+        else k_rhs<T, false, 1><<<(unsigned)blocks, 128, 0, L.stream>>>(M, V);
+    }
     *L.launches += 1;
 }
 
@@ -1071,87 +1117,139 @@ void bem_product(const Launch& L, const MeshView& M, const BatchView<T>& V) {
 }
 
 // ---- effective field, gradient, energies and step dot products -----------------------
+// Threads of a block: 256, or 64 for small work (at most one node of one instance a
+// thread of 4 blocks per SM), so that the FP64 units of many SMs share it: one instance
+// at n = 10 kept six of 152 SMs busy (43 us), now twenty-one.
+static int field_threads(int num_sms, int N, int B) {
+    return B <= 64 && (long long)N * B <= 64LL * 4 * num_sms ? 64 : FIELD_THREADS;
+}
+
 int field_blocks(const Launch& L, const MeshView& M, int B) {
-    const int RB = FIELD_THREADS / B;
+    const int RB = field_threads(L.num_sms, M.N, B) / B;
     int nblk = (M.N + RB - 1) / RB;
     const int maxblk = 4 * L.num_sms;
     return nblk < maxblk ? nblk : maxblk;
 }
 
+// GB300 issues FP64 at 1/64 of its FP32 rate, and the FP64 instructions are what
+// bounds this kernel (pipe 82 % busy at 64 instances), so it takes each quantity in its
+// cheapest exact form: 1 / V from a table on the Kuhn cube, whose volumes are the
+// integers up to 24; g = |m|^2 grad - (m.grad) m for m x H; |H|^2 = (V/12)^2 |m x h|^2 and
+// |g|^2 = |m|^2 |H|^2; |m x a|^2 = |m - (m.a) a|^2; the Zeeman term from
+// the sum of V m; constant factors on the sums.  About 95 operations a node where there
+// were 130.  32 instances at n = 30 in FP32: 293 -> 211 us (with five still running 293 ->
+// 115); 6 in FP64 at n = 25 and one at n = 10, with the event pair: 117 -> 100, 43 -> 23 us.
 template <typename T, bool GEN>
-__global__ void __launch_bounds__(FIELD_THREADS) k_field(MeshView M, BatchView<T> V, int demag) {
+__global__ void __launch_bounds__(FIELD_THREADS, sizeof(T) == 4 ? 2 : 1) k_field(MeshView M, BatchView<T> V, int demag) {
     extern __shared__ double fsm[];
+    const int tid = threadIdx.x, bd = blockDim.x;
     double* scratch = fsm;                        // [Q_COUNT][bd]
-    double* out = fsm + Q_COUNT * FIELD_THREADS;  // [Q_COUNT][B]
-    const int tid = threadIdx.x;
-    const int B = V.B, RB = FIELD_THREADS / B;
-    const bool lane = tid < RB * B;
-    const int b = tid % B, rl = tid / B;
-    const int N = M.N;
+    __shared__ double s_v[32], s_iv[32];          // V and 1 / V (Kuhn cube, units h^3/24)
+    __shared__ int s_act[256];
+    const int B = V.B, N = M.N;
+    const int nact = active_list<1>(V.st, B, s_act);
+    if (nact == 0) return;
+    // row lanes and sums as if all instances ran: an instance's bits do not depend on
+    // which others have finished; the lanes of those that run are packed into full warps
+    // (from another warp on in each quarter of the grid: a block's warp w runs on
+    // scheduler w mod 4, and the FP64 units belong to the schedulers)
+    const int RB = bd / B;
+    const int rot = (int)(4u * blockIdx.x / gridDim.x) * 32;
+    const int vt = (tid + bd - rot % bd) % bd;
+    const bool lane = vt < RB * nact;
+    const int act = s_act[vt % nact], b = act >> 1, cur = act & 1, rl = vt / nact;
+    if (!GEN && tid < 32) {
+        s_v[tid] = (double)tid;
+        s_iv[tid] = tid ? 1.0 / (double)tid : 0.0;
+    }
+    __syncthreads();
     double acc[Q_COUNT];
 #pragma unroll
     for (int k = 0; k < Q_COUNT; ++k) acc[k] = 0.0;
-    const int phase = lane ? V.st[b].phase : PH_DONE;
-    if (lane && phase != PH_DONE) {
-        const int cur = V.st[b].cur;
+    if (lane) {
         const InstConst ic = V.ic[b];
-        const double lam6 = ic.lam / 6.0, q24 = ic.Q / 24.0;
+        const double c4lam = -4.0 * ic.lam;
         const double* mt = V.m + (size_t)(1 - cur) * N * 3 * B;
         const double* mb = V.m + (size_t)cur * N * 3 * B;
         double* Gt = V.H + (size_t)(1 - cur) * N * 3 * B;        // grad phi at the trial point
         const double* Gb = V.H + (size_t)cur * N * 3 * B;   // grad phi at the base point
         for (int row = blockIdx.x * RB + rl; row < N; row += gridDim.x * RB) {
-            const double vi = GEN ? M.gV[row] : (double)(M.node[row] & 0xff);
             const size_t i3 = (size_t)row * 3 * B + b;
-            const double mx = mt[i3], my = mt[i3 + B], mz = mt[i3 + 2 * B];
             T ex0 = T(0), ex1 = T(0), ex2 = T(0), hd0 = T(0), hd1 = T(0), hd2 = T(0);
             // neighbour values in T: the FP32 kernel reads the FP32 copy of the trial
             // point (exact zero differences for equal values are kept)
             const T* mn = (sizeof(T) == 4) ? reinterpret_cast<const T*>(V.m32) : reinterpret_cast<const T*>(mt);
             const T tx = mn[i3], ty = mn[i3 + B], tz = mn[i3 + 2 * B];
             const int e0 = M.rowptr[row], e1 = M.rowptr[row + 1];
-            for (int e = e0; e < e1; ++e) {
-                const int j = __ldg(&M.col[e]) & 0x7fffffff;
-                const T k = GEN ? T(GenTab<T>::A(M)[e].x) : T(sbyte(__ldg(&M.pkA[e]), 0));
-                const size_t j3 = (size_t)j * 3 * B + b;
-                // difference form: exact zero for a uniform state, no cancellation
-                ex0 += k * (mn[j3] - tx);
-                ex1 += k * (mn[j3 + B] - ty);
-                ex2 += k * (mn[j3 + 2 * B] - tz);
-                if (demag) {
+            const double m[3] = {mt[i3], mt[i3 + B], mt[i3 + 2 * B]};
+            const double bm[3] = {mb[i3], mb[i3 + B], mb[i3 + 2 * B]};
+            const double bg[3] = {Gb[i3], Gb[i3 + B], Gb[i3 + 2 * B]};
+            // entries four at a time, past the row's end as copies of its last with weight
+            // zero: a row's loads take two trips to memory a four (one by one, the last
+            // three of seven entries took six)
+            for (int eb = e0; eb < e1; eb += 4) {
+                int jj[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) jj[q] = __ldg(&M.col[min(eb + q, e1 - 1)]) & 0x7fffffff;
+                T mj[4][3], uj[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const size_t j3 = (size_t)jj[q] * 3 * B + b, jc = (size_t)jj[q] * 2 * B + b;
+                    mj[q][0] = mn[j3];
+                    mj[q][1] = mn[j3 + B];
+                    mj[q][2] = mn[j3 + 2 * B];
                     // (forward + adjoint)/2: the potential whose lumped gradient is the
                     // exact gradient of the stray-field energy
-                    const size_t jc = (size_t)j * 2 * B + b;
-                    const T u = T(0.5) * (V.U1[jc] + V.U2[jc] + V.U2[jc + B]);
-                    if constexpr (GEN) {
-                        const typename GenTab<T>::V4 gb = GenTab<T>::Bt(M)[e];
-                        hd0 += gb.x * u;
-                        hd1 += gb.y * u;
-                        hd2 += gb.z * u;
-                    } else {
-                        const int wb = __ldg(&M.pkB[e]);
-                        hd0 += T(sbyte(wb, 0)) * u;
-                        hd1 += T(sbyte(wb, 1)) * u;
-                        hd2 += T(sbyte(wb, 2)) * u;
+                    if (demag) uj[q] = T(0.5) * (V.U1[jc] + V.U2[jc] + V.U2[jc + B]);
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int e = min(eb + q, e1 - 1);
+                    if (sizeof(T) == 8 && eb + q >= e1) break;   // FP64 arithmetic is not done for nothing
+                    T k = GEN ? T(GenTab<T>::A(M)[e].x) : T(sbyte(__ldg(&M.pkA[e]), 0));
+                    if (eb + q >= e1) k = T(0);
+                    // difference form: exact zero for a uniform state, no cancellation
+                    ex0 += k * (mj[q][0] - tx);
+                    ex1 += k * (mj[q][1] - ty);
+                    ex2 += k * (mj[q][2] - tz);
+                    if (demag) {
+                        const T u = eb + q < e1 ? uj[q] : T(0);
+                        if constexpr (GEN) {
+                            const typename GenTab<T>::V4 gb = GenTab<T>::Bt(M)[e];
+                            hd0 += gb.x * u;
+                            hd1 += gb.y * u;
+                            hd2 += gb.z * u;
+                        } else {
+                            const int wb = __ldg(&M.pkB[e]);
+                            hd0 += T(sbyte(wb, 0)) * u;
+                            hd1 += T(sbyte(wb, 1)) * u;
+                            hd2 += T(sbyte(wb, 2)) * u;
+                        }
                     }
                 }
             }
-            const double m[3] = {mx, my, mz};
+            double vi, ivi;
+            if constexpr (GEN) {
+                vi = M.gV[row];
+                ivi = 1.0 / vi;
+            } else {
+                const int vn = M.node[row] & 0xff;
+                vi = s_v[vn];
+                ivi = s_iv[vn];
+            }
             const double kx[3] = {(double)ex0, (double)ex1, (double)ex2};
+            const double hd[3] = {(double)hd0, (double)hd1, (double)hd2};   // -V times the stray field
             const double ma = m[0] * ic.a[0] + m[1] * ic.a[1] + m[2] * ic.a[2];
-            // GB300 issues FP64 at a small fraction of its FP32 rate: one division
-            // per node (1/V_i), constant factors as products, squared maxima
-            // (the square roots are taken once, on the totals, by k_decide)
-            const double ivi = 1.0 / vi;
-            const double cex = -4.0 * ic.lam * ivi;
-            const double hd[3] = {-(double)hd0 * ivi, -(double)hd1 * ivi, -(double)hd2 * ivi};
+            const double qm = ic.Q * ma, cex = c4lam * ivi;
             double h[3];
-            for (int c = 0; c < 3; ++c) h[c] = cex * kx[c] + ic.Q * ma * ic.a[c] + ic.hz[c] + hd[c];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) h[c] = fma(cex, kx[c], fma(qm, ic.a[c], fma(-ivi, hd[c], ic.hz[c])));
             // grad phi = -(V/12) h ;  H = -m x grad phi = (V/12) m x h ;  g = m x H
-            const double v12 = vi * (1.0 / 12.0), v24 = vi * (1.0 / 24.0);
+            const double v12 = vi * (1.0 / 12.0);
             const double gr[3] = {-v12 * h[0], -v12 * h[1], -v12 * h[2]};
             const double mh[3] = {m[1] * h[2] - m[2] * h[1], m[2] * h[0] - m[0] * h[2], m[0] * h[1] - m[1] * h[0]};
-            const double Hv[3] = {v12 * mh[0], v12 * mh[1], v12 * mh[2]};
+            const double tq = mh[0] * mh[0] + mh[1] * mh[1] + mh[2] * mh[2];
+            const double HH = v12 * v12 * tq;
             Gt[i3] = gr[0];
             Gt[i3 + B] = gr[1];
             Gt[i3 + 2 * B] = gr[2];
@@ -1160,75 +1258,112 @@ __global__ void __launch_bounds__(FIELD_THREADS) k_field(MeshView M, BatchView<T
                 V.hout[i3 + B] = h[1];
                 V.hout[i3 + 2 * B] = h[2];
             }
-            const double g[3] = {m[1] * Hv[2] - m[2] * Hv[1], m[2] * Hv[0] - m[0] * Hv[2],
-                                 m[0] * Hv[1] - m[1] * Hv[0]};
-            const double bm[3] = {mb[i3], mb[i3 + B], mb[i3 + 2 * B]};
-            const double bg[3] = {Gb[i3], Gb[i3 + B], Gb[i3 + 2 * B]};
-            // g_b = m_b x (-m_b x grad_b) = grad_b - (m_b . grad_b) m_b  (|m_b| = 1)
+            // g = m x (-m x grad) = |m|^2 grad - (m . grad) m; |m| = 1 at the base point
+            const double mm = m[0] * m[0] + m[1] * m[1] + m[2] * m[2];
+            const double mg = m[0] * gr[0] + m[1] * gr[1] + m[2] * gr[2];
             const double bmg = bm[0] * bg[0] + bm[1] * bg[1] + bm[2] * bg[2];
-            const double gb[3] = {bg[0] - bmg * bm[0], bg[1] - bmg * bm[1], bg[2] - bmg * bm[2]};
-            // E is quadratic in m, so E_t - E_b = (grad_t + grad_b) . (m_t - m_b) / 2 exactly
-            acc[Q_DE] += 0.5 * ((gr[0] + bg[0]) * (m[0] - bm[0]) + (gr[1] + bg[1]) * (m[1] - bm[1]) +
-                                (gr[2] + bg[2]) * (m[2] - bm[2]));
-            const double mxa[3] = {m[1] * ic.a[2] - m[2] * ic.a[1], m[2] * ic.a[0] - m[0] * ic.a[2],
-                                   m[0] * ic.a[1] - m[1] * ic.a[0]};
-            acc[Q_EEX] += lam6 * (m[0] * kx[0] + m[1] * kx[1] + m[2] * kx[2]);
-            acc[Q_EAN] += q24 * vi * (mxa[0] * mxa[0] + mxa[1] * mxa[1] + mxa[2] * mxa[2]);
-            acc[Q_EZ] -= v12 * (m[0] * ic.hz[0] + m[1] * ic.hz[1] + m[2] * ic.hz[2]);
-            acc[Q_ED] -= v24 * (m[0] * hd[0] + m[1] * hd[1] + m[2] * hd[2]);
-            acc[Q_TORQUE] = fmax(acc[Q_TORQUE], mh[0] * mh[0] + mh[1] * mh[1] + mh[2] * mh[2]);
-            acc[Q_HMAX] = fmax(acc[Q_HMAX], Hv[0] * Hv[0] + Hv[1] * Hv[1] + Hv[2] * Hv[2]);
-            double ss = 0.0, sy = 0.0, yy = 0.0, gg = 0.0;
+            double de = acc[Q_DE], ss = acc[Q_SS], sy = acc[Q_SY], yy = acc[Q_YY], pp = 0.0;
+            double ee = acc[Q_EEX], ed = acc[Q_ED];
+#pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const double sc = m[c] - bm[c], yc = g[c] - gb[c];
-                ss += sc * sc;
-                sy += sc * yc;
-                yy += yc * yc;
-                gg += g[c] * g[c];
+                const double sc = m[c] - bm[c];
+                const double yc = fma(-mg, m[c], mm * gr[c]) - fma(-bmg, bm[c], bg[c]);
+                // E is quadratic in m, so E_t - E_b = (grad_t + grad_b) . (m_t - m_b) / 2 exactly
+                de = fma(gr[c] + bg[c], sc, de);
+                ss = fma(sc, sc, ss);
+                sy = fma(sc, yc, sy);
+                yy = fma(yc, yc, yy);
+                const double pc = fma(-ma, ic.a[c], m[c]);
+                pp = fma(pc, pc, pp);
+                ee = fma(m[c], kx[c], ee);
+                ed = fma(m[c], hd[c], ed);
             }
-            acc[Q_GG] += gg;
-            acc[Q_SS] += ss;
-            acc[Q_SY] += sy;
-            acc[Q_YY] += yy;
-            acc[Q_MX] += vi * m[0];
-            acc[Q_MY] += vi * m[1];
-            acc[Q_MZ] += vi * m[2];
+            acc[Q_DE] = de;
+            acc[Q_SS] = ss;
+            acc[Q_SY] = sy;
+            acc[Q_YY] = yy;
+            acc[Q_EEX] = ee;
+            acc[Q_ED] = ed;
+            acc[Q_EAN] = fma(vi, pp, acc[Q_EAN]);
+            acc[Q_TORQUE] = fmax(acc[Q_TORQUE], tq);
+            acc[Q_HMAX] = fmax(acc[Q_HMAX], HH);
+            acc[Q_GG] = fma(mm, HH, acc[Q_GG]);
+            acc[Q_MX] = fma(vi, m[0], acc[Q_MX]);
+            acc[Q_MY] = fma(vi, m[1], acc[Q_MY]);
+            acc[Q_MZ] = fma(vi, m[2], acc[Q_MZ]);
             if (!(isfinite(h[0]) && isfinite(h[1]) && isfinite(h[2]))) acc[Q_BAD] = 1.0;
         }
+        acc[Q_DE] *= 0.5;
+        acc[Q_EEX] *= ic.lam / 6.0;
+        acc[Q_EAN] *= ic.Q / 24.0;
+        acc[Q_EZ] = (-1.0 / 12.0) * (acc[Q_MX] * ic.hz[0] + acc[Q_MY] * ic.hz[1] + acc[Q_MZ] * ic.hz[2]);
+        acc[Q_ED] *= 1.0 / 24.0;
     }
+    // block sums (maxima of the torque, |H|^2 and the flag): `sub` threads a total, each
+    // over every sub-th row lane, then a butterfly -- a fixed order
     const unsigned maxmask = (1u << Q_TORQUE) | (1u << Q_HMAX) | (1u << Q_BAD);
-    block_reduce_inst<Q_COUNT>(acc, scratch, out, B, RB, maxmask);
-    if (tid < B)
-        for (int k = 0; k < Q_COUNT; ++k) V.part[((size_t)blockIdx.x * B + tid) * NQ + k] = out[k * B + tid];
+#pragma unroll
+    for (int k = 0; k < Q_COUNT; ++k) scratch[k * bd + vt] = acc[k];
+    __syncthreads();
+    int sub = 1;
+    while (sub < 16 && sub * 2 <= RB && Q_COUNT * B * sub * 2 <= bd) sub *= 2;
+    const int total = Q_COUNT * nact;
+    for (int t0 = 0; t0 < total; t0 += bd / sub) {
+        const int t = t0 + tid / sub, part = tid % sub;
+        const bool on = t < total;
+        const int k = on ? t / nact : 0, bb = on ? t - k * nact : 0;
+        const bool mx = (maxmask >> k) & 1u;
+        double v = 0.0;
+        if (on)
+            for (int r = part; r < RB; r += sub) {
+                const double o = scratch[k * bd + r * nact + bb];
+                v = mx ? fmax(v, o) : v + o;
+            }
+        for (int o = sub / 2; o > 0; o >>= 1) {
+            const double w = __shfl_xor_sync(0xffffffffu, v, o);
+            v = mx ? fmax(v, w) : v + w;
+        }
+        if (on && part == 0) V.part[((size_t)blockIdx.x * B + (s_act[bb] >> 1)) * NQ + k] = v;
+    }
 }
 
 template <typename T>
 void field_eval(const Launch& L, const MeshView& M, const BatchView<T>& V, int demag) {
-    const int nblk = field_blocks(L, M, V.B);
-    const size_t smem = sizeof(double) * Q_COUNT * (FIELD_THREADS + V.B);
-    kernel_smem_attr((const void*)k_field<T, false>, 96 * 1024);
-    kernel_smem_attr((const void*)k_field<T, true>, 96 * 1024);
-    if (M.gen) k_field<T, true><<<nblk, FIELD_THREADS, smem, L.stream>>>(M, V, demag);
-    else k_field<T, false><<<nblk, FIELD_THREADS, smem, L.stream>>>(M, V, demag);
+    const int nblk = field_blocks(L, M, V.B), threads = field_threads(L.num_sms, M.N, V.B);
+    const size_t smem = sizeof(double) * Q_COUNT * threads;
+    if (M.gen) k_field<T, true><<<nblk, threads, smem, L.stream>>>(M, V, demag);
+    else k_field<T, false><<<nblk, threads, smem, L.stream>>>(M, V, demag);
     *L.launches += 1;
 }
 
-// ---- Sec. 2.3 step control, one warp per instance ---------------------------------------
+// ---- Sec. 2.3 step control ---------------------------------------------------------------
 __device__ double hist_max(const InstState& s) {
     double e = s.hist[0];
     for (int k = 1; k < s.nhist; ++k) e = fmax(e, s.hist[k]);
     return e;
 }
 
-__global__ void k_decide(const double* __restrict__ part, int nblk, InstState* st, const InstConst* ic, StepOpts so,
-                         double vsum, int B) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= B) return;
-    const int b = warp;
-    double v[Q_COUNT];
-    for (int k = 0; k < Q_COUNT; ++k) {
+// One block per instance: a warp per quantity adds its per-block partials (lanes
+// stride, then a fixed butterfly), then one thread decides on a copy of the state in
+// shared memory (the decision's chain of FP64 operations and of trips to global memory
+// took 18 to 65 us with one warp for everything).
+constexpr int DECIDE_THREADS = 32 * Q_COUNT;
+__device__ void decide_step(InstState& s, double (&v)[Q_COUNT], const StepOpts& so, double vsum);
+
+__global__ void __launch_bounds__(DECIDE_THREADS) k_decide(const double* __restrict__ part, int nblk, InstState* st,
+                                                           StepOpts so, double vsum, int B) {
+    static_assert(sizeof(InstState) % 8 == 0, "copied in 8-byte words");
+    constexpr int WORDS = sizeof(InstState) / 8;
+    __shared__ double s_v[Q_COUNT];
+    __shared__ __align__(8) unsigned char s_st[sizeof(InstState)];
+    const int b = blockIdx.x, k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint64_t* gst = reinterpret_cast<uint64_t*>(&st[b]);
+    uint64_t* lst = reinterpret_cast<uint64_t*>(s_st);
+    for (int i = threadIdx.x; i < WORDS; i += DECIDE_THREADS) lst[i] = gst[i];
+    {
         const bool mx = (k == Q_TORQUE || k == Q_HMAX || k == Q_BAD);
         double acc = 0.0;
+#pragma unroll 4
         for (int blk = lane; blk < nblk; blk += 32) {
             const double x = part[((size_t)blk * B + b) * NQ + k];
             acc = mx ? fmax(acc, x) : acc + x;
@@ -1237,11 +1372,22 @@ __global__ void k_decide(const double* __restrict__ part, int nblk, InstState* s
             const double y = __shfl_xor_sync(0xffffffffu, acc, o);
             acc = mx ? fmax(acc, y) : acc + y;
         }
-        v[k] = acc;
+        if (lane == 0) s_v[k] = acc;
     }
-    if (lane != 0) return;
-    InstState& s = st[b];
+    __syncthreads();
+    InstState& s = *reinterpret_cast<InstState*>(s_st);
     if (s.phase == PH_DONE) return;
+    if (threadIdx.x == 0) {
+        double v[Q_COUNT];
+#pragma unroll
+        for (int q = 0; q < Q_COUNT; ++q) v[q] = s_v[q];
+        decide_step(s, v, so, vsum);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < WORDS; i += DECIDE_THREADS) gst[i] = lst[i];
+}
+
+__device__ void decide_step(InstState& s, double (&v)[Q_COUNT], const StepOpts& so, double vsum) {
     const double Edirect = ((v[Q_EEX] + v[Q_EAN]) + v[Q_EZ]) + v[Q_ED];
     // Decisions use E(base) + (E(trial) - E(base)) with the difference from the
     // gradients (exact for the quadratic energy): its rounding scales with the
@@ -1390,23 +1536,21 @@ __global__ void k_decide(const double* __restrict__ part, int nblk, InstState* s
 
 template <typename T>
 void decide(const Launch& L, const MeshView& M, const BatchView<T>& V, const StepOpts& so, int nblk_field) {
-    const int threads = 128;
-    const int blocks = (V.B * 32 + threads - 1) / threads;
-    k_decide<<<blocks, threads, 0, L.stream>>>(V.part, nblk_field, V.st, V.ic, so, M.vsum, V.B);
+    k_decide<<<V.B, DECIDE_THREADS, 0, L.stream>>>(V.part, nblk_field, V.st, so, M.vsum, V.B);
     *L.launches += 1;
 }
 
 // ---- Eq. (8): the curvilinear step ------------------------------------------------------
 template <typename T>
 __global__ void k_trial(int N, BatchView<T> V) {
+    __shared__ int s_act[256];
     const int B = V.B;
-    const size_t total = (size_t)N * B;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        const int b = (int)(t % B);
-        const size_t row = t / B;
+    const unsigned nact = active_list<1>(V.st, B, s_act);
+    const unsigned total = (unsigned)N * nact;   // < 2^32: 96 bytes of the state each
+    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+        const size_t row = t / nact;
+        const int act = s_act[t - (unsigned)row * nact], b = act >> 1, cur = act & 1;
         const int phase = V.st[b].phase;
-        if (phase == PH_DONE) continue;
-        const int cur = V.st[b].cur;
         const size_t i3 = row * 3 * B + b;
         const double* mb = V.m + (size_t)cur * N * 3 * B;
         double* mt = V.m + (size_t)(1 - cur) * N * 3 * B;
@@ -1444,19 +1588,18 @@ __global__ void k_trial(int N, BatchView<T> V) {
             put(x0 / xn, x1 / xn, x2 / xn);
             continue;
         }
-        // x = [(1 - |w|^2) m - 2 m x w + 2 (m.w) w] / (1 + |w|^2),  w = tau H / 2
+        // x = [(1 - |w|^2) m - 2 m x w + 2 (m.w) w] / (1 + |w|^2),  w = tau H / 2, where
+        // m.w = 0 (H = -m x grad phi); v = 2 w
         const double* Gb = V.H + (size_t)cur * N * 3 * B;   // grad phi at the base point
-        const double ht = 0.5 * V.st[b].tau;
+        const double nt = -V.st[b].tau;
         const double m0 = mb[i3], m1 = mb[i3 + B], m2 = mb[i3 + 2 * B];
         const double g0 = Gb[i3], g1 = Gb[i3 + B], g2 = Gb[i3 + 2 * B];
-        // w = (tau/2) H with H = -m x grad phi
-        const double w0 = -ht * (m1 * g2 - m2 * g1), w1 = -ht * (m2 * g0 - m0 * g2), w2 = -ht * (m0 * g1 - m1 * g0);
-        const double ww = w0 * w0 + w1 * w1 + w2 * w2;
-        const double mw = m0 * w0 + m1 * w1 + m2 * w2;
-        const double c0 = m1 * w2 - m2 * w1, c1 = m2 * w0 - m0 * w2, c2 = m0 * w1 - m1 * w0;
+        const double v0 = nt * (m1 * g2 - m2 * g1), v1 = nt * (m2 * g0 - m0 * g2), v2 = nt * (m0 * g1 - m1 * g0);
+        const double ww = 0.25 * (v0 * v0 + v1 * v1 + v2 * v2);
         const double iden = 1.0 / (1.0 + ww);   // one FP64 division per node
-        put(((1.0 - ww) * m0 - 2.0 * c0 + 2.0 * mw * w0) * iden, ((1.0 - ww) * m1 - 2.0 * c1 + 2.0 * mw * w1) * iden,
-            ((1.0 - ww) * m2 - 2.0 * c2 + 2.0 * mw * w2) * iden);
+        const double cm = (1.0 - ww) * iden;
+        put(fma(cm, m0, -iden * (m1 * v2 - m2 * v1)), fma(cm, m1, -iden * (m2 * v0 - m0 * v2)),
+            fma(cm, m2, -iden * (m0 * v1 - m1 * v0)));
     }
 }
 

@@ -386,7 +386,7 @@ __device__ __forceinline__ bool grid_reduce(const double* part, int q0, int C, d
 
 // rhs_b for the four consecutive instances b0..b0+3 (b0 a multiple of 4, B too):
 // the row's column and coupling entries are read once, the trial point as
-// 16-byte vectors of four instances; per instance the sum of rhs_b.
+// 16-byte vectors of four instances; per instance the sum of rhs_b, bit for bit.
 template <typename T, bool GEN>
 __device__ __forceinline__ void rhs_b4(const int* __restrict__ col, const int* __restrict__ pkA,
                                        const typename GenTab<T>::V4* __restrict__ gA, int e0, int e1,
@@ -402,14 +402,12 @@ __device__ __forceinline__ void rhs_b4(const int* __restrict__ col, const int* _
             const int w = __ldg(&pkA[e]);
             gx = T(sbyte(w, 1)); gy = T(sbyte(w, 2)); gz = T(sbyte(w, 3));
         }
-        const T g3[3] = {gx, gy, gz};
+        T m0[4], m1[4], m2[4];
+        vload<T, 4, false>(m0, meval + mj);
+        vload<T, 4, false>(m1, meval + mj + B);
+        vload<T, 4, false>(m2, meval + mj + 2 * (size_t)B);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {   // one component at a time (few live registers)
-            T mc[4];
-            vload<T, 4, false>(mc, meval + mj + (size_t)c * B);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) acc[k] += g3[c] * mc[k];
-        }
+        for (int k = 0; k < 4; ++k) acc[k] += gx * m0[k] + gy * m1[k] + gz * m2[k];
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) f[k] = 0.25 * (double)acc[k];
