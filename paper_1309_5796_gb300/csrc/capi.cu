@@ -297,10 +297,9 @@ VecLayout vec_layout(const Mesh& M, int B, int tsize) {
     L.q = take(tsize * N * C);
     L.ub_in = take(tsize * nb * C);
     L.ub_out = take(tsize * nb * C);
-    // 32 x nb partial sums of the transposed single-instance product; FP64
-    // batches also the K-split partials of the batched product (S x nb x 2B)
-    const size_t df = (tsize == 8 && B > 1) ? (size_t)bem_df_splits((int)nb, B, M.num_sms) * nb * C : 0;
-    L.bem_part = take(8 * (32 * nb > df ? 32 * nb : df));
+    // partial sums of the boundary products: gemv_parts() vectors of one instance, the
+    // K-split partials of a batch (S x nb x 2B)
+    L.bem_part = take(8 * (B == 1 ? (size_t)gemv_parts() * nb : (size_t)bem_df_splits((int)nb, B, M.num_sms) * nb * C));
     L.m32 = tsize == 4 ? take(4 * N * 3 * B) : 0;
     L.bvec = take(8 * N * B);
     // transformed planes of the fast solves of large cubes (FP64 batches: plain and
@@ -337,6 +336,7 @@ BatchView<T> batch_view(const lbm_ctx* ctx, const Mesh& M, const Inst& I, bool w
     v.ub_in = (T*)(base + L.ub_in);
     v.ub_out = (T*)(base + L.ub_out);
     v.bem_part = (T*)(base + L.bem_part);
+    v.bem_parts = gemv_parts();
     v.m32 = sizeof(T) == 4 ? (float*)(base + L.m32) : nullptr;
     v.bvec = (double*)(base + L.bvec);
     v.fs = L.fs_bytes ? (void*)(base + L.fs) : nullptr;

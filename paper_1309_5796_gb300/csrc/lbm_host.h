@@ -243,7 +243,8 @@ struct BatchView {
     T* r; T* z; T* p; T* q;    // [N][2B] PCG work vectors
     T* ub_in;    // [nb][2B] BEM input:  u1 on the surface | t = b_S - K_SI w
     T* ub_out;   // [nb][2B] BEM output: B u1_S | B^T t
-    T* bem_part; // column-split partial sums of the transposed product (scratch)
+    T* bem_part; // partial sums of the boundary products (scratch)
+    int bem_parts = 32;        // one instance: vectors of nb doubles in bem_part
     double* part;              // partial sums, >= maxblocks * B * NQ
     InstState* st;             // [B]
     const InstConst* ic;       // [B]
@@ -342,6 +343,7 @@ int field_blocks(const Launch& L, const MeshView& M, int B);
 // FP64-accurate batched BEM product on the FP32 units: K-split count and the
 // doubles of its partial-sum scratch (S * nb * 2B)
 int bem_df_splits(int nb, int B, int num_sms);
+int gemv_parts();
 // B_lo = fp32(B64 - B32) (nb x nb)
 void launch_bem_lo(const double* B64, const float* B32, float* B32lo, size_t n, cudaStream_t st);
 size_t pcg_part_elems(int num_sms, int B);

@@ -688,6 +688,12 @@ template <> struct DotAcc<double> {
     double s = 0.0;
     __device__ __forceinline__ void add(double a, double x) { s = fma(a, x, s); }
     __device__ __forceinline__ double value() const { return s; }
+    __device__ __forceinline__ void merge(const DotAcc& o) { s += o.s; }
+    __device__ __forceinline__ DotAcc from(int lanemask) const {
+        DotAcc o;
+        o.s = __shfl_xor_sync(0xffffffffu, s, lanemask);
+        return o;
+    }
 };
 template <> struct DotAcc<float> {
     float s = 0.f, c = 0.f;
@@ -698,77 +704,220 @@ template <> struct DotAcc<float> {
         s = t;
     }
     __device__ __forceinline__ double value() const { return (double)s - (double)c; }
+    // the sum of two, its rounding kept in c (TwoSum)
+    __device__ __forceinline__ void merge(const DotAcc& o) {
+        const float t = __fadd_rn(s, o.s), b = __fsub_rn(t, s);
+        const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(o.s, b));
+        c = __fsub_rn(__fadd_rn(c, o.c), err);
+        s = t;
+    }
+    __device__ __forceinline__ DotAcc from(int lanemask) const {
+        DotAcc o;
+        o.s = __shfl_xor_sync(0xffffffffu, s, lanemask);
+        o.c = __shfl_xor_sync(0xffffffffu, c, lanemask);
+        return o;
+    }
 };
 
-// y[row*inc] = sum_j A[row][j] x[j*inc]; one warp per row
-template <typename TA, typename T>
-__global__ void k_gemv(const TA* __restrict__ A, const T* __restrict__ x, T* __restrict__ y, int nb, int inc) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int row = warp; row < nb; row += nw) {
-        const TA* a = A + (size_t)row * nb;
-        DotAcc<T> acc;
-        for (int j = lane; j < nb; j += 32) acc.add(T(a[j]), x[(size_t)j * inc]);
-        double v = acc.value();
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) y[(size_t)row * inc] = T(v);
+// ---- both products of one instance ------------------------------------------------------
+// y0 = B x0 and y1 = B^T x1 (columns 0 and 1 of the surface arrays) in one pass over B.
+// The pass reads nb^2 words, and those reads bound it: two passes (a warp per row, then
+// columns over row chunks) took twice the memory's time.  A block takes a panel of rows
+// and a chunk of columns.  A thread owns the chunk's columns tid, tid + 256, ... (their
+// x0 and running sums in shared memory, private to the thread) and, for R rows at a
+// time, the rows' sums over its columns in registers (FP32: two neighbouring columns a
+// step where rows are 8-byte aligned); the next R loads are in flight while R products
+// are taken.  The R sums of a warp take R merges by shuffles for R rows
+// by a chunk, so a chunk is as wide as the grid's need for blocks allows.  Sums are
+// DotAcc's (compensated in FP32, FP64 in FP64) to a warp and FP64 across warps, panels and
+// chunks, all in a fixed order.
+// One instance, before -> after: FP32 at n = 80 1.91 -> 1.10 ms (5.9 GB), n = 40 141 -> 97 us,
+// n = 20 27 -> 20 us; FP64 at n = 10 21 -> 14 us, at n = 17 31 us both (FP64 units).
+constexpr int GV_THREADS = 256, GV_MAX_COLS = 4096;
+constexpr int GV_ROWS = 8;
+template <typename T> constexpr int GV_BLOCKS = sizeof(T) == 8 ? 2 : 3;   // per SM
+
+// a step's columns of a thread: their x0, and their sums
+template <typename T, int VEC> struct alignas(sizeof(T) * VEC) GvWords { T w[VEC]; };
+template <typename T, int VEC> struct alignas(sizeof(DotAcc<T>) * VEC) GvCols { DotAcc<T> s[VEC]; };
+template <typename T, int VEC> constexpr size_t gv_step_bytes() {
+    return GV_THREADS * (sizeof(GvCols<T, VEC>) + sizeof(GvWords<T, VEC>));
+}
+static_assert(gv_step_bytes<float, 1>() == 256 * 12 && gv_step_bytes<float, 2>() == 256 * 24 &&
+              gv_step_bytes<double, 1>() == 256 * 16, "no padding: the shared memory is sized by them");
+
+struct GemvSplit {
+    int kc, cc, rows, p;   // 256-column steps of a chunk, chunks, rows of a panel, panels
+};
+
+// cc + p partial vectors of nb doubles fit `cap`; blocks for two or one full waves where
+// the matrix has them (for which chunks get narrower), as many as it has otherwise.
+static GemvSplit gemv_split(int nb, int vec, int resident, int cap) {
+    const int step = GV_THREADS * vec, maxp = (nb + GV_ROWS - 1) / GV_ROWS, maxc = (nb + step - 1) / step;
+    int cc = (nb + GV_MAX_COLS - 1) / GV_MAX_COLS;
+    while (cc < maxc && cc < cap / 2 && cc * std::min(cap - cc, maxp) < resident) ++cc;
+    GemvSplit s;
+    s.kc = (nb + cc * step - 1) / (cc * step);
+    s.cc = (nb + s.kc * step - 1) / (s.kc * step);
+    const int most = std::max(1, std::min(cap - s.cc, maxp));
+    int p = 2 * resident / s.cc;
+    if (p > most) p = std::max(1, std::min(most, resident / s.cc));
+    s.rows = ((nb + p - 1) / p + GV_ROWS - 1) / GV_ROWS * GV_ROWS;
+    s.p = (nb + s.rows - 1) / s.rows;
+    return s;
+}
+
+// Partial vectors of the one-instance product: 160 let chunks be 4096 columns wide where
+// the matrix is larger than L2 (49 MB for the 38,402 surface nodes of 80 cells a side).
+int gemv_parts() { return 160; }
+
+template <typename T, int VEC>
+__global__ void __launch_bounds__(GV_THREADS, GV_BLOCKS<T>) k_gemv_both(const T* __restrict__ A, const T* __restrict__ x,
+                                                                        double* __restrict__ rowpart,
+                                                                        double* __restrict__ colpart, int nb, int kc,
+                                                                        int rows_per_panel) {
+    constexpr int R = GV_ROWS, STEP = GV_THREADS * VEC;
+    using Words = GvWords<T, VEC>;
+    using Cols = GvCols<T, VEC>;
+    extern __shared__ __align__(16) unsigned char gv_sm[];
+    __shared__ double s_row[GV_THREADS / 32][R];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int c0 = blockIdx.x * kc * STEP + tid * VEC;   // nb is a multiple of VEC
+    const int r0 = blockIdx.y * rows_per_panel, r1 = min(nb, r0 + rows_per_panel);
+    Cols* const col = reinterpret_cast<Cols*>(gv_sm) + tid;                                   // [kc][256]
+    Words* const x0 = reinterpret_cast<Words*>(gv_sm + sizeof(Cols) * kc * GV_THREADS) + tid;   // [kc][256]
+    const int steps = min(kc, (nb - c0 + STEP - 1) / STEP);   // of this thread (< 1: none)
+    for (int k = 0; k < steps; ++k) {
+        Cols c;
+        Words w;
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) {
+            c.s[v] = DotAcc<T>();
+            w.w[v] = x[2 * (size_t)(c0 + k * STEP + v)];
+        }
+        col[k * GV_THREADS] = c;
+        x0[k * GV_THREADS] = w;
+    }
+    for (int rg = r0; rg < r1; rg += R) {
+        DotAcc<T> row[R];
+        T x1[R];
+        const T* a = A + (size_t)rg * nb + c0;
+        const int last = r1 - 1 - rg;   // rows past the panel: the last one again, weight zero
+#pragma unroll
+        for (int r = 0; r < R; ++r) x1[r] = r <= last ? x[2 * (size_t)(rg + r) + 1] : T(0);
+        auto pass = [&](auto full) {
+            Words m[R], nx[R];
+            if (steps > 0) {
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    nx[r] = *reinterpret_cast<const Words*>(a + (size_t)(decltype(full)::value ? r : min(r, last)) * nb);
+            }
+            for (int k = 0; k < steps; ++k) {
+                if (k + 1 < steps) a += STEP;   // (past the last step: its words again)
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    m[r] = nx[r];
+                    nx[r] = *reinterpret_cast<const Words*>(a + (size_t)(decltype(full)::value ? r : min(r, last)) * nb);
+                }
+                Cols c = col[k * GV_THREADS];
+                const Words xv = x0[k * GV_THREADS];
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) {
+                        row[r].add(m[r].w[v], xv.w[v]);
+                        c.s[v].add(m[r].w[v], x1[r]);
+                    }
+                col[k * GV_THREADS] = c;
+            }
+        };
+        if (last >= R - 1) pass(std::true_type());
+        else pass(std::false_type());
+        // R sums over the 32 lanes: halves of the rows change sides at every step, so that
+        // lane l has row l mod R, of R lanes; then of all four groups of R lanes
+#pragma unroll
+        for (int h = R / 2; h > 0; h >>= 1) {
+            const bool up = lane & h;
+#pragma unroll
+            for (int r = 0; r < h; ++r) {
+                const DotAcc<T> send = up ? row[r] : row[r + h], got = send.from(h);
+                if (up) row[r] = row[r + h];
+                row[r].merge(got);
+            }
+        }
+#pragma unroll
+        for (int o = R; o < 32; o <<= 1) row[0].merge(row[0].from(o));
+        if (lane < R) s_row[warp][lane] = row[0].value();
+        __syncthreads();
+        if (tid < R && rg + tid < r1) {
+            double t = 0.0;
+#pragma unroll
+            for (int w = 0; w < GV_THREADS / 32; ++w) t += s_row[w][tid];
+            rowpart[(size_t)blockIdx.x * nb + rg + tid] = t;
+        }
+        __syncthreads();
+    }
+    for (int k = 0; k < steps; ++k)
+#pragma unroll
+        for (int v = 0; v < VEC; ++v)
+            colpart[(size_t)blockIdx.y * nb + c0 + k * STEP + v] = col[k * GV_THREADS].s[v].value();
+}
+
+// y[2 j] = sum of the cc row partials, y[2 j + 1] of the p column partials: 32 positions
+// by 8 lanes a block (blockIdx.y: which of the two)
+template <typename T>
+__global__ void __launch_bounds__(256) k_gemv_sum(const double* __restrict__ rowpart, int cc,
+                                                  const double* __restrict__ colpart, int p, int nb, T* __restrict__ y) {
+    __shared__ double s[8][32];
+    const int jx = threadIdx.x & 31, l = threadIdx.x >> 5, j = blockIdx.x * 32 + jx;
+    const double* part = blockIdx.y ? colpart : rowpart;
+    const int n = blockIdx.y ? p : cc;
+    double acc = 0.0;
+    if (j < nb) {
+#pragma unroll 4
+        for (int q = l; q < n; q += 8) acc += part[(size_t)q * nb + j];
+    }
+    s[l][jx] = acc;
+    __syncthreads();
+    if (l == 0 && j < nb) {
+#pragma unroll
+        for (int q = 1; q < 8; ++q) acc += s[q][jx];
+        y[2 * (size_t)j + blockIdx.y] = T(acc);
     }
 }
 
-// part[s][j] = sum_{i in chunk s} A[i][j] x[i*inc]: column-parallel, coalesced rows
-template <typename TA, typename T>
-__global__ void k_gemv_t_part(const TA* __restrict__ A, const T* __restrict__ x, double* __restrict__ part, int nb,
-                              int inc, int rows_per_chunk) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i0 = blockIdx.y * rows_per_chunk, i1 = min(nb, i0 + rows_per_chunk);
-    if (j >= nb) return;
-    DotAcc<T> acc;
-#pragma unroll 4
-    for (int i = i0; i < i1; ++i) acc.add(T(A[(size_t)i * nb + j]), x[(size_t)i * inc]);
-    part[(size_t)blockIdx.y * nb + j] = acc.value();
-}
-
-template <typename T>
-__global__ void k_sum_parts(const double* __restrict__ part, int S, int nb, T* __restrict__ y, int inc) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= nb) return;
-    double acc = 0.0;
-    for (int s = 0; s < S; ++s) acc += part[(size_t)s * nb + j];
-    y[(size_t)j * inc] = T(acc);
-}
-
-// Y[:, 0:ncols] = op(A) X[:, 0:ncols] with row strides ldx, ldy; 64x64 tiles,
-// 256 threads, 4x4 outputs each.  TRANS: op(A) = A^T.  Arithmetic in the
-// matrix type TA (vectors of type T are converted on load and store).
-template <typename TA, typename T, bool TRANS>
-__global__ void __launch_bounds__(256) k_gemm(const TA* __restrict__ A, const T* __restrict__ X, int ldx,
-                                              T* __restrict__ Y, int ldy, int nb, int ncols) {
+// ---- batched products -----------------------------------------------------------------
+// Y = op(A) X in FP64 arithmetic (batches whose mesh has no low words of B: their
+// allocation failed), 64x64 tiles, 256 threads, 4x4 outputs each.
+template <bool TRANS>
+__global__ void __launch_bounds__(256) k_gemm(const double* __restrict__ A, const double* __restrict__ X,
+                                              int ldx, double* __restrict__ Y, int ldy, int nb, int ncols) {
     constexpr int BM = 64, BN = 64, BK = 16;
-    __shared__ TA As[BK][BM + 4];
-    __shared__ TA Xs[BK][BN + 4];
+    __shared__ double As[BK][BM + 4];
+    __shared__ double Xs[BK][BN + 4];
     const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
     const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-    TA acc[4][4];
+    double acc[4][4];
     for (int i = 0; i < 4; ++i)
-        for (int j = 0; j < 4; ++j) acc[i][j] = TA(0);
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
     for (int k0 = 0; k0 < nb; k0 += BK) {
         for (int l = tid; l < BM * BK; l += 256) {
             int mm, kk;
             if (TRANS) { kk = l / BM; mm = l % BM; } else { mm = l / BK; kk = l % BK; }
             const int gm = m0 + mm, gk = k0 + kk;
-            TA v = TA(0);
+            double v = 0.0;
             if (gm < nb && gk < nb) v = TRANS ? A[(size_t)gk * nb + gm] : A[(size_t)gm * nb + gk];
             As[kk][mm] = v;
         }
         for (int l = tid; l < BK * BN; l += 256) {
             const int kk = l / BN, nn = l % BN;
             const int gk = k0 + kk, gn = n0 + nn;
-            Xs[kk][nn] = (gk < nb && gn < ncols) ? TA(X[(size_t)gk * ldx + gn]) : TA(0);
+            Xs[kk][nn] = (gk < nb && gn < ncols) ? X[(size_t)gk * ldx + gn] : 0.0;
         }
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
-            TA a[4], xv[4];
+            double a[4], xv[4];
             for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
             for (int j = 0; j < 4; ++j) xv[j] = Xs[kk][tx * 4 + j];
             for (int i = 0; i < 4; ++i)
@@ -779,23 +928,43 @@ __global__ void __launch_bounds__(256) k_gemm(const TA* __restrict__ A, const T*
     for (int i = 0; i < 4; ++i)
         for (int j = 0; j < 4; ++j) {
             const int gm = m0 + ty * 4 + i, gn = n0 + tx * 4 + j;
-            if (gm < nb && gn < ncols) Y[(size_t)gm * ldy + gn] = T(acc[i][j]);
+            if (gm < nb && gn < ncols) Y[(size_t)gm * ldy + gn] = acc[i][j];
         }
 }
 
-// ---- FP64-accurate batched BEM products on the FP32 units ------------------------------
-// Y = op(B) X for the FP64 vectors of FP64 batches (the FP64 phase of mixed
-// runs included), with B = B_hi + B_lo (B_hi the FP32 copy of B, B_lo the FP32
-// rounding of B - B_hi: together B to about 2^-48 relative) and x = x_hi + x_lo
-// the same way.  Per term a_hi x_hi is exact as p + e (e = fma(a_hi, x_hi, -p));
-// p is added to the high word of a double-FP32 accumulator with Knuth's TwoSum,
-// whose rounding error is exact; that error, e and the cross terms a_hi x_lo +
-// a_lo x_hi go into the low word (the a_lo x_lo term is 2^-48 of the term); the
-// two words are combined in FP64.  (Kahan compensation in FP32 is not enough:
-// it keeps each term to about FP32 precision.)  GB300 issues FP32 arithmetic
-// at many times its FP64 rate, so twelve FP32 instructions per term beat one
-// FP64 fused multiply-add.  The sum over K is split across blocks (blockIdx.z); the
-// partials part[z][row][c] (FP64) are added in a fixed order by k_sum_splits.
+// FP64 batches (the FP64 phase of mixed runs included) on the FP32 units, to better than
+// FP64 needs: B = B_hi + B_lo (B_hi the FP32 copy of B, B_lo the FP32 rounding of
+// B - B_hi: together B to about 2^-48 relative) and x = x_hi + x_lo the same way.  GB300
+// issues FP32 arithmetic at 64 times its FP64 rate, and those instructions bound the
+// product.  Over 8 terms the accumulator t starts at c = 2 sum |a_hi| |x_hi|, so that
+// t stays within [c/2, 3c/2] and t' = fma(a_hi, x_hi, t) has t' - t exact (Sterbenz)
+// and the rounding error e = fma(a_hi, x_hi, -(t' - t)); e and the cross terms
+// a_hi x_lo + a_lo x_hi go into a low word (the a_lo x_lo term is 2^-48 of the term).
+// Then t - c, exact again, is added to the high word of the result by Knuth's TwoSum and
+// the rest to its low word; the two are combined in FP64.  Eight instructions a term;
+// TwoSum for every term took twelve.  (Kahan compensation in FP32 is not enough: it
+// keeps each term to about FP32 precision.)  The diagonal (up to 0.9; the other entries
+// are a few hundredths at most) would give c, and with it the rounding of e, its size: it
+// is left out and added in FP64 with the splits.  FP32 batches (DF = false): FMA over
+// 8 terms, TwoSum for these.
+// A block of 256 threads takes 128 rows by up to 32 instances over a K range, both
+// products in one launch; columns are the instances that still run, and a block of at
+// most 8 or 16 of them takes a narrower tile (the tile of 64 columns of before multiplied
+// zeros: 90 % of it for six instances).  Each thread has 4, 2 or 1 rows by 4 instances;
+// the next tile is copied to shared memory behind the arithmetic (cp.async).  K is split so that the grid fills the chip;
+// the partials part[z][row][c] (FP64) are added in a fixed order by k_sum_splits.
+// FP64, 6 instances at n = 25 / 32 / 64 at n = 30, before -> after: 0.95 -> 0.15, 1.96 -> 0.75,
+// 1.97 -> 1.50 ms; FP32, 16 at n = 20 / 32 at n = 30: 0.64 -> 0.05, 2.4 -> 0.23 ms.  Errors
+// against extended precision, FP64: 1e-15 of the result where TwoSum had up to 6e-14.
+constexpr int DF_BM = 128, DF_BN = 32, DF_BK = 16, DF_G = 8, DF_THREADS = 256;
+
+struct __align__(16) DfSmem {
+    float ah[2][DF_BK][DF_BM + 4], al[2][DF_BK][DF_BM + 4];   // a tile and the next
+    float xh[2][DF_BK][DF_BN + 4], xl[2][DF_BK][DF_BN + 4];
+    float c[16][DF_THREADS];   // each thread its own
+    int list[256];
+};
+
 __global__ void k_bem_lo(const double* __restrict__ B64, const float* __restrict__ B32, float* __restrict__ lo,
                          size_t n) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
@@ -806,95 +975,193 @@ void launch_bem_lo(const double* B64, const float* B32, float* B32lo, size_t n, 
     k_bem_lo<<<1024, 256, 0, st>>>(B64, B32, B32lo, n);
 }
 
-template <bool TRANS>
-__global__ void __launch_bounds__(256) k_gemm_df(const float* __restrict__ Ahi, const float* __restrict__ Alo,
-                                                 const double* __restrict__ X, int ldx, double* __restrict__ part,
-                                                 int ldp, int nb, int ncols, int kchunk) {
-    constexpr int BM = 64, BN = 64, BK = 16;
-    __shared__ float Ah[BK][BM + 4], Al[BK][BM + 4], Xh[BK][BN + 4], Xl[BK][BN + 4];
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-    const int kbeg = blockIdx.z * kchunk, kend = min(nb, kbeg + kchunk);
-    float sh[4][4], sl[4][4];   // high and low words of the accumulators
+// four bytes to shared memory behind the arithmetic; zero if !on
+__device__ __forceinline__ void async4(float* dst, const float* src, bool on) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(on ? 4 : 0)
+                 : "memory");
+}
+
+template <typename T, bool TRANS, int BN>
+__device__ __forceinline__ void gemm_tile(const float* __restrict__ Ahi, const float* __restrict__ Alo,
+                                          const T* __restrict__ X, double* __restrict__ part, int C, int nb, int m0,
+                                          int kbeg, int kend, const int* list, int ncol, DfSmem& S) {
+    constexpr bool DF = sizeof(T) == 8;
+    constexpr int TX = BN / 4, TM = DF_BM * TX / DF_THREADS;   // threads across, rows of a thread
+    constexpr int NA = DF_BM * DF_BK / DF_THREADS, NX = (BN * DF_BK + DF_THREADS - 1) / DF_THREADS;
+    const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+    T fx[NX];
+    auto fetch = [&](int k0, int buf) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < NA; ++i) {
+            const int l = tid + i * DF_THREADS;
+            const int mm = TRANS ? l % DF_BM : l / DF_BK, kk = TRANS ? l / DF_BM : l % DF_BK;
+            const int gm = m0 + mm, gk = k0 + kk;
+            const bool on = gm < nb && gk < kend && gm != gk;   // the diagonal: k_sum_splits
+            const size_t at = !on ? 0 : TRANS ? (size_t)gk * nb + gm : (size_t)gm * nb + gk;
+            async4(&S.ah[buf][kk][mm], Ahi + at, on);
+            if (DF) async4(&S.al[buf][kk][mm], Alo + at, on);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+#pragma unroll
+        for (int i = 0; i < NX; ++i) {
+            const int l = tid + i * DF_THREADS, kk = l / BN, nn = l % BN;
+            fx[i] = (l < BN * DF_BK && k0 + kk < kend && nn < ncol) ? X[(size_t)(k0 + kk) * C + (list[nn] >> 1)] : T(0);
+        }
+    };
+    float sh[TM][4], sl[TM][4];   // high and low words of the results
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) sh[i][j] = sl[i][j] = 0.f;
-    for (int k0 = kbeg; k0 < kend; k0 += BK) {
-        for (int l = tid; l < BM * BK; l += 256) {
-            int mm, kk;
-            if (TRANS) { kk = l / BM; mm = l % BM; } else { mm = l / BK; kk = l % BK; }
-            const int gm = m0 + mm, gk = k0 + kk;
-            float h = 0.f, w = 0.f;
-            if (gm < nb && gk < kend) {
-                const size_t idx = TRANS ? (size_t)gk * nb + gm : (size_t)gm * nb + gk;
-                h = Ahi[idx];
-                w = Alo[idx];
+    fetch(kbeg, 0);
+    for (int k0 = kbeg, buf = 0; k0 < kend; k0 += DF_BK, buf ^= 1) {
+#pragma unroll
+        for (int i = 0; i < NX; ++i) {
+            const int l = tid + i * DF_THREADS, kk = l / BN, nn = l % BN;
+            if (l < BN * DF_BK) {
+                const float h = (float)fx[i];
+                S.xh[buf][kk][nn] = h;
+                if (DF) S.xl[buf][kk][nn] = (float)((double)fx[i] - (double)h);
             }
-            Ah[kk][mm] = h;
-            Al[kk][mm] = w;
         }
-        for (int l = tid; l < BK * BN; l += 256) {
-            const int kk = l / BN, nn = l % BN;
-            const int gk = k0 + kk, gn = n0 + nn;
-            const double v = (gk < kend && gn < ncols) ? X[(size_t)gk * ldx + gn] : 0.0;
-            const float h = (float)v;
-            Xh[kk][nn] = h;
-            Xl[kk][nn] = (float)(v - (double)h);
-        }
-        __syncthreads();
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();   // this tile is there; the other buffers' readers have passed it
+        if (k0 + DF_BK < kend) fetch(k0 + DF_BK, buf ^ 1);
+#pragma unroll 1
+        for (int kg = 0; kg < DF_BK; kg += DF_G) {
+            float t[TM][4], w[TM][4];
 #pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            float ah[4], al[4], xh[4], xl[4];
+            for (int i = 0; i < TM; ++i)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                ah[i] = Ah[kk][ty * 4 + i];
-                al[i] = Al[kk][ty * 4 + i];
-                xh[i] = Xh[kk][tx * 4 + i];
-                xl[i] = Xl[kk][tx * 4 + i];
+                for (int j = 0; j < 4; ++j) t[i][j] = w[i][j] = 0.f;
+            if (DF) {
+#pragma unroll
+                for (int kk = 0; kk < DF_G; ++kk) {
+                    float ah[TM];
+#pragma unroll
+                    for (int i = 0; i < TM; ++i) ah[i] = fabsf(S.ah[buf][kg + kk][ty * TM + i]);
+                    const float4 q = *reinterpret_cast<const float4*>(&S.xh[buf][kg + kk][tx * 4]);
+                    const float xh[4] = {fabsf(q.x), fabsf(q.y), fabsf(q.z), fabsf(q.w)};
+#pragma unroll
+                    for (int i = 0; i < TM; ++i)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) t[i][j] = __fmaf_rn(ah[i], xh[j], t[i][j]);
+                }
+#pragma unroll
+                for (int i = 0; i < TM; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        t[i][j] = __fmul_rn(2.0002f, t[i][j]);
+                        S.c[i * 4 + j][tid] = t[i][j];
+                    }
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int kk = 0; kk < DF_G; ++kk) {
+                float ah[TM], al[TM], xl[4];
+#pragma unroll
+                for (int i = 0; i < TM; ++i) {
+                    ah[i] = S.ah[buf][kg + kk][ty * TM + i];
+                    al[i] = DF ? S.al[buf][kg + kk][ty * TM + i] : 0.f;
+                }
+                const float4 q = *reinterpret_cast<const float4*>(&S.xh[buf][kg + kk][tx * 4]);
+                const float xh[4] = {q.x, q.y, q.z, q.w};
+                if (DF) {
+                    const float4 u = *reinterpret_cast<const float4*>(&S.xl[buf][kg + kk][tx * 4]);
+                    xl[0] = u.x; xl[1] = u.y; xl[2] = u.z; xl[3] = u.w;
+                }
+#pragma unroll
+                for (int i = 0; i < TM; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float tn = __fmaf_rn(ah[i], xh[j], t[i][j]);
+                        if (DF) {
+                            float e = __fmaf_rn(ah[i], xh[j], -__fsub_rn(tn, t[i][j]));
+                            e = __fmaf_rn(ah[i], xl[j], e);
+                            e = __fmaf_rn(al[i], xh[j], e);
+                            w[i][j] = __fadd_rn(w[i][j], e);
+                        }
+                        t[i][j] = tn;
+                    }
+            }
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const float p = __fmul_rn(ah[i], xh[j]);
-                    float e = __fmaf_rn(ah[i], xh[j], -p);   // exact: a_hi x_hi = p + e
-                    e = __fmaf_rn(ah[i], xl[j], e);
-                    e = __fmaf_rn(al[i], xh[j], e);
-                    // TwoSum: t + err = sh + p exactly
-                    const float t = __fadd_rn(sh[i][j], p);
-                    const float bp = __fsub_rn(t, sh[i][j]);
-                    const float ap = __fsub_rn(t, bp);
-                    const float err = __fadd_rn(__fsub_rn(sh[i][j], ap), __fsub_rn(p, bp));
-                    sh[i][j] = t;
-                    sl[i][j] = __fadd_rn(sl[i][j], __fadd_rn(err, e));
+                    const float p = DF ? __fsub_rn(t[i][j], S.c[i * 4 + j][tid]) : t[i][j];
+                    // TwoSum: s + err = sh + p exactly
+                    const float s = __fadd_rn(sh[i][j], p);
+                    const float bp = __fsub_rn(s, sh[i][j]);
+                    const float err = __fadd_rn(__fsub_rn(sh[i][j], __fsub_rn(s, bp)), __fsub_rn(p, bp));
+                    sh[i][j] = s;
+                    sl[i][j] = __fadd_rn(sl[i][j], DF ? __fadd_rn(err, w[i][j]) : err);
                 }
         }
-        __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int gm = m0 + ty * 4 + i, gn = n0 + tx * 4 + j;
-            if (gm < nb && gn < ncols)
-                part[((size_t)blockIdx.z * nb + gm) * ldp + gn] = (double)sh[i][j] + (double)sl[i][j];
+            const int gm = m0 + ty * TM + i, gn = tx * 4 + j;
+            if (gm < nb && gn < ncol)
+                part[(size_t)gm * C + (list[gn] >> 1)] = (double)sh[i][j] + (double)sl[i][j];
         }
 }
 
-// y[row][c] = sum over the S splits of part[s][row][c], in split order (C = 2B columns)
-__global__ void k_sum_splits(const double* __restrict__ part, int S, int nb, int C, double* __restrict__ y) {
+// blockIdx: x the row tile (those of B, then those of B^T), y 32 of the running
+// instances, z the K range.  st null: all B instances run.
+template <typename T>
+__global__ void __launch_bounds__(DF_THREADS, 2) k_gemm_split(const float* __restrict__ Ahi, const float* __restrict__ Alo,
+                                                              const T* __restrict__ X, double* __restrict__ part, int nb,
+                                                              int B, int kchunk, const InstState* st) {
+    extern __shared__ __align__(16) unsigned char df_sm[];
+    DfSmem& S = *reinterpret_cast<DfSmem*>(df_sm);
+    int nact = B;
+    if (st) {
+        nact = active_list<1>(st, B, S.list);
+    } else {
+        for (int b = threadIdx.x; b < B; b += DF_THREADS) S.list[b] = b * 2;
+        __syncthreads();
+    }
+    const int n0 = blockIdx.y * DF_BN, ncol = min(DF_BN, nact - n0);
+    if (ncol <= 0) return;
+    const int mt = gridDim.x / 2, C = 2 * B;
+    const bool trans = (int)blockIdx.x >= mt;
+    const int m0 = ((int)blockIdx.x - (trans ? mt : 0)) * DF_BM;
+    const int kbeg = blockIdx.z * kchunk, kend = min(nb, kbeg + kchunk);
+    const T* Xc = X + (trans ? B : 0);
+    double* P = part + (size_t)blockIdx.z * nb * C + (trans ? B : 0);
+    const int* list = S.list + n0;
+    if (trans) {
+        if (ncol <= 8) gemm_tile<T, true, 8>(Ahi, Alo, Xc, P, C, nb, m0, kbeg, kend, list, ncol, S);
+        else if (ncol <= 16) gemm_tile<T, true, 16>(Ahi, Alo, Xc, P, C, nb, m0, kbeg, kend, list, ncol, S);
+        else gemm_tile<T, true, 32>(Ahi, Alo, Xc, P, C, nb, m0, kbeg, kend, list, ncol, S);
+    } else {
+        if (ncol <= 8) gemm_tile<T, false, 8>(Ahi, Alo, Xc, P, C, nb, m0, kbeg, kend, list, ncol, S);
+        else if (ncol <= 16) gemm_tile<T, false, 16>(Ahi, Alo, Xc, P, C, nb, m0, kbeg, kend, list, ncol, S);
+        else gemm_tile<T, false, 32>(Ahi, Alo, Xc, P, C, nb, m0, kbeg, kend, list, ncol, S);
+    }
+}
+
+// y[row][c] = diagonal entry times x[row][c] plus the sum over the S splits of
+// part[s][row][c], in split order (C = 2B columns, those of the running instances)
+template <typename T>
+__global__ void k_sum_splits(const double* __restrict__ part, int S, int nb, int C, const T* __restrict__ A,
+                             const T* __restrict__ x, T* __restrict__ y, const InstState* st) {
     const size_t total = (size_t)nb * C;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        double acc = 0.0;
+        const int c = (int)(i % C), B = C / 2;
+        if (st && st[c < B ? c : c - B].phase == PH_DONE) continue;
+        double acc = (double)A[(i / C) * ((size_t)nb + 1)] * (double)x[i];
+#pragma unroll 4
         for (int z = 0; z < S; ++z) acc += part[(size_t)z * total + i];
-        y[i] = acc;
+        y[i] = T(acc);
     }
 }
 
 // K splits so that the two products fill about four waves of two blocks per SM
 int bem_df_splits(int nb, int B, int num_sms) {
-    const int tiles = ((nb + 63) / 64) * ((B + 63) / 64) * 2;
+    const int tiles = ((nb + DF_BM - 1) / DF_BM) * ((B + DF_BN - 1) / DF_BN) * 2;
     int S = (8 * num_sms + tiles - 1) / tiles;
     if (S > 16) S = 16;
     if (S < 1) S = 1;
@@ -905,112 +1172,45 @@ template <typename T> __host__ __device__ inline const T* bem_ptr(const MeshView
 template <> __host__ __device__ inline const double* bem_ptr<double>(const MeshView& M) { return M.B64; }
 template <> __host__ __device__ inline const float* bem_ptr<float>(const MeshView& M) { return M.B32; }
 
-// Row chunks of the column-parallel transposed product: enough blocks for about
-// eight per SM, so that the column loads of many warps are in flight (at most
-// 32 chunks: the partial sums are 32 x nb).
-int bem_chunks(int nb, int num_sms) {
-    const int colblocks = (nb + 255) / 256;
-    int S = (8 * num_sms + colblocks - 1) / colblocks;
-    if (S > 32) S = 32;
-    if (S < 1) S = 1;
-    return S;
-}
-
-// ---- autotuner: row chunks of the transposed single-instance product ------------------
-// At the first product of a (nb, matrix type, vector type, SM count) the
-// column-parallel kernel is timed with 4, 8, 16 and 32 row chunks (CUDA events
-// on the launching stream; it reads the live input and writes only the
-// partial-sum scratch); the fastest is kept for the process.
-static std::mutex g_chunks_mu;
-static std::map<std::tuple<int, int, int, int>, int> g_chunks;
-
-template <typename F>
-static int tuned_chunks(const Launch& L, int nb, int key_a, int key_b, F&& launch_with) {
-    const auto key = std::make_tuple(nb, key_a, key_b, L.num_sms);
-    // without tuning (a call that must not wait) the default shape, whatever an
-    // earlier call tuned: its summation order then does not depend on history
-    if (!L.tune) return bem_chunks(nb, L.num_sms);
-    {
-        std::lock_guard<std::mutex> lk(g_chunks_mu);
-        auto it = g_chunks.find(key);
-        if (it != g_chunks.end()) return it->second;
-    }
-    int best = bem_chunks(nb, L.num_sms);
-    float best_ms = -1.f;
-    cudaEvent_t e0, e1;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    for (int S : {4, 8, 16, 32}) {
-        float t[3];
-        for (int rep = 0; rep < 3; ++rep) {
-            cudaEventRecord(e0, L.stream);
-            launch_with(S);
-            cudaEventRecord(e1, L.stream);
-            cudaEventSynchronize(e1);
-            cudaEventElapsedTime(&t[rep], e0, e1);
-            *L.launches += 1;
-        }
-        const float med = std::max(std::min(t[0], t[1]), std::min(std::max(t[0], t[1]), t[2]));
-        if (best_ms < 0.f || med < best_ms) {
-            best = S;
-            best_ms = med;
-        }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    std::lock_guard<std::mutex> lk(g_chunks_mu);
-    g_chunks[key] = best;
-    return best;
-}
-
-int gemv_chunks_chosen(int nb, int key_a, int key_b, int num_sms) {
-    std::lock_guard<std::mutex> lk(g_chunks_mu);
-    auto it = g_chunks.find(std::make_tuple(nb, key_a, key_b, num_sms));
-    return it == g_chunks.end() ? 0 : it->second;
-}
-
-template <typename TA, typename T>
-static void bem_launch(const Launch& L, const TA* Bm, const MeshView& M, const BatchView<T>& V) {
+template <typename T>
+static void bem_launch(const Launch& L, const T* Bm, const MeshView& M, const BatchView<T>& V) {
     const int B = V.B, C = 2 * B, nb = M.nb;
+    double* part = reinterpret_cast<double*>(V.bem_part);
     if (B == 1) {
-        int blocks = (nb * 32 + 255) / 256;
-        if (blocks > 8 * L.num_sms) blocks = 8 * L.num_sms;
-        k_gemv<TA, T><<<blocks, 256, 0, L.stream>>>(Bm, V.ub_in, V.ub_out, nb, C);
-        const int S = tuned_chunks(L, nb, (int)sizeof(TA), (int)sizeof(T), [&](int s) {
-            k_gemv_t_part<TA, T><<<dim3((nb + 255) / 256, s), 256, 0, L.stream>>>(Bm, V.ub_in + 1,
-                                                                                 (double*)V.bem_part, nb, C,
-                                                                                 (nb + s - 1) / s);
-        });
-        const int rpc = (nb + S - 1) / S;
-        k_gemv_t_part<TA, T><<<dim3((nb + 255) / 256, S), 256, 0, L.stream>>>(Bm, V.ub_in + 1, (double*)V.bem_part,
-                                                                             nb, C, rpc);
-        k_sum_parts<T><<<(nb + 255) / 256, 256, 0, L.stream>>>((const double*)V.bem_part, S, nb, V.ub_out + 1, C);
-        *L.launches += 3;
-    } else if constexpr (std::is_same<TA, double>::value && std::is_same<T, double>::value) {
-        if (M.B32lo) {
-            // FP64 batches: the FP64-accurate product on the FP32 units
-            const int S = bem_df_splits(nb, B, L.num_sms);
-            const int kchunk = (((nb + S - 1) / S) + 15) / 16 * 16;
-            dim3 grid((nb + 63) / 64, (B + 63) / 64, S);
-            double* part = reinterpret_cast<double*>(V.bem_part);
-            k_gemm_df<false><<<grid, 256, 0, L.stream>>>(M.B32, M.B32lo, V.ub_in, C, part, C, nb, B, kchunk);
-            k_gemm_df<true><<<grid, 256, 0, L.stream>>>(M.B32, M.B32lo, V.ub_in + B, C, part + B, C, nb, B, kchunk);
-            size_t blocks = ((size_t)nb * C + 255) / 256;
-            if (blocks > (size_t)8 * L.num_sms) blocks = (size_t)8 * L.num_sms;
-            k_sum_splits<<<(unsigned)blocks, 256, 0, L.stream>>>(part, S, nb, C, V.ub_out);
-            *L.launches += 3;
-        } else {
-            dim3 grid((nb + 63) / 64, (B + 63) / 64);
-            k_gemm<TA, T, false><<<grid, 256, 0, L.stream>>>(Bm, V.ub_in, C, V.ub_out, C, nb, B);
-            k_gemm<TA, T, true><<<grid, 256, 0, L.stream>>>(Bm, V.ub_in + B, C, V.ub_out + B, C, nb, B);
-            *L.launches += 2;
-        }
-    } else {
-        dim3 grid((nb + 63) / 64, (B + 63) / 64);
-        k_gemm<TA, T, false><<<grid, 256, 0, L.stream>>>(Bm, V.ub_in, C, V.ub_out, C, nb, B);
-        k_gemm<TA, T, true><<<grid, 256, 0, L.stream>>>(Bm, V.ub_in + B, C, V.ub_out + B, C, nb, B);
+        const bool pairs = sizeof(T) == 4 && nb % 2 == 0;
+        const GemvSplit g = gemv_split(nb, pairs ? 2 : 1, GV_BLOCKS<T> * L.num_sms, V.bem_parts);
+        double* colpart = part + (size_t)g.cc * nb;
+        auto run = [&](auto fn, size_t step_bytes) {
+            const size_t smem = g.kc * step_bytes;
+            kernel_smem_attr((const void*)fn, 64 * 1024);
+            fn<<<dim3(g.cc, g.p), GV_THREADS, smem, L.stream>>>(Bm, V.ub_in, part, colpart, nb, g.kc, g.rows);
+        };
+        constexpr int W = sizeof(T) == 4 ? 2 : 1;
+        if (pairs) run(k_gemv_both<T, W>, gv_step_bytes<T, W>());
+        else run(k_gemv_both<T, 1>, gv_step_bytes<T, 1>());
+        k_gemv_sum<T><<<dim3((nb + 31) / 32, 2), 256, 0, L.stream>>>(part, g.cc, colpart, g.p, nb, V.ub_out);
         *L.launches += 2;
+        return;
     }
+    if constexpr (sizeof(T) == 8) {
+        if (!M.B32lo) {
+            dim3 grid((nb + 63) / 64, (B + 63) / 64);
+            k_gemm<false><<<grid, 256, 0, L.stream>>>(Bm, V.ub_in, C, V.ub_out, C, nb, B);
+            k_gemm<true><<<grid, 256, 0, L.stream>>>(Bm, V.ub_in + B, C, V.ub_out + B, C, nb, B);
+            *L.launches += 2;
+            return;
+        }
+    }
+    const int S = bem_df_splits(nb, B, L.num_sms);
+    const int kchunk = (((nb + S - 1) / S) + DF_BK - 1) / DF_BK * DF_BK;
+    const int splits = (nb + kchunk - 1) / kchunk;
+    const dim3 grid(2 * ((nb + DF_BM - 1) / DF_BM), (B + DF_BN - 1) / DF_BN, splits);
+    kernel_smem_attr((const void*)k_gemm_split<T>, (int)sizeof(DfSmem));
+    k_gemm_split<T><<<grid, DF_THREADS, sizeof(DfSmem), L.stream>>>(M.B32, M.B32lo, V.ub_in, part, nb, B, kchunk, V.st);
+    size_t blocks = ((size_t)nb * C + 255) / 256;
+    if (blocks > (size_t)8 * L.num_sms) blocks = (size_t)8 * L.num_sms;
+    k_sum_splits<T><<<(unsigned)blocks, 256, 0, L.stream>>>(part, splits, nb, C, Bm, V.ub_in, V.ub_out, V.st);
+    *L.launches += 2;
 }
 
 // ---- BEM products with the hierarchical (H-matrix) form of B -------------------------
@@ -1112,8 +1312,7 @@ void bem_product(const Launch& L, const MeshView& M, const BatchView<T>& V) {
         hm_product<T>(L, *M.hm, V.ub_in, V.ub_out, V.B);
         return;
     }
-    if constexpr (sizeof(T) == 4) bem_launch<float, T>(L, M.B32, M, V);
-    else bem_launch<double, T>(L, M.B64, M, V);
+    bem_launch<T>(L, bem_ptr<T>(M), M, V);
 }
 
 // ---- effective field, gradient, energies and step dot products -----------------------
