@@ -1335,8 +1335,9 @@ int field_blocks(const Launch& L, const MeshView& M, int B) {
 // cheapest exact form: 1 / V from a table on the Kuhn cube, whose volumes are the
 // integers up to 24; g = |m|^2 grad - (m.grad) m for m x H; |H|^2 = (V/12)^2 |m x h|^2 and
 // |g|^2 = |m|^2 |H|^2; |m x a|^2 = |m - (m.a) a|^2; the Zeeman term from
-// the sum of V m; constant factors on the sums.  About 95 operations a node where there
-// were 130.  32 instances at n = 30 in FP32: 293 -> 211 us (with five still running 293 ->
+// the sum of V m; constant factors on the sums; and at a first point, which has no
+// step behind it, nothing of the step's products.  About 95 operations a node (60 at a
+// first point) where there were 130.  32 instances at n = 30 in FP32: 293 -> 211 us (with five still running 293 ->
 // 115); 6 in FP64 at n = 25 and one at n = 10, with the event pair: 117 -> 100, 43 -> 23 us.
 template <typename T, bool GEN>
 __global__ void __launch_bounds__(FIELD_THREADS, sizeof(T) == 4 ? 2 : 1) k_field(MeshView M, BatchView<T> V, int demag) {
@@ -1367,6 +1368,7 @@ __global__ void __launch_bounds__(FIELD_THREADS, sizeof(T) == 4 ? 2 : 1) k_field
     for (int k = 0; k < Q_COUNT; ++k) acc[k] = 0.0;
     if (lane) {
         const InstConst ic = V.ic[b];
+        const bool init = V.st[b].phase == PH_INIT;   // the first point: no step behind it
         const double c4lam = -4.0 * ic.lam;
         const double* mt = V.m + (size_t)(1 - cur) * N * 3 * B;
         const double* mb = V.m + (size_t)cur * N * 3 * B;
@@ -1381,8 +1383,14 @@ __global__ void __launch_bounds__(FIELD_THREADS, sizeof(T) == 4 ? 2 : 1) k_field
             const T tx = mn[i3], ty = mn[i3 + B], tz = mn[i3 + 2 * B];
             const int e0 = M.rowptr[row], e1 = M.rowptr[row + 1];
             const double m[3] = {mt[i3], mt[i3 + B], mt[i3 + 2 * B]};
-            const double bm[3] = {mb[i3], mb[i3 + B], mb[i3 + 2 * B]};
-            const double bg[3] = {Gb[i3], Gb[i3 + B], Gb[i3 + 2 * B]};
+            double bm[3], bg[3];
+            if (!init) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    bm[c] = mb[i3 + (size_t)c * B];
+                    bg[c] = Gb[i3 + (size_t)c * B];
+                }
+            }
             // entries four at a time, past the row's end as copies of its last with weight
             // zero: a row's loads take two trips to memory a four (one by one, the last
             // three of seven entries took six)
@@ -1457,30 +1465,35 @@ __global__ void __launch_bounds__(FIELD_THREADS, sizeof(T) == 4 ? 2 : 1) k_field
                 V.hout[i3 + B] = h[1];
                 V.hout[i3 + 2 * B] = h[2];
             }
-            // g = m x (-m x grad) = |m|^2 grad - (m . grad) m; |m| = 1 at the base point
             const double mm = m[0] * m[0] + m[1] * m[1] + m[2] * m[2];
-            const double mg = m[0] * gr[0] + m[1] * gr[1] + m[2] * gr[2];
-            const double bmg = bm[0] * bg[0] + bm[1] * bg[1] + bm[2] * bg[2];
-            double de = acc[Q_DE], ss = acc[Q_SS], sy = acc[Q_SY], yy = acc[Q_YY], pp = 0.0;
-            double ee = acc[Q_EEX], ed = acc[Q_ED];
+            if (!init) {
+                // g = m x (-m x grad) = |m|^2 grad - (m . grad) m; |m| = 1 at the base point
+                const double mg = m[0] * gr[0] + m[1] * gr[1] + m[2] * gr[2];
+                const double bmg = bm[0] * bg[0] + bm[1] * bg[1] + bm[2] * bg[2];
+                double de = acc[Q_DE], ss = acc[Q_SS], sy = acc[Q_SY], yy = acc[Q_YY];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const double sc = m[c] - bm[c];
+                    const double yc = fma(-mg, m[c], mm * gr[c]) - fma(-bmg, bm[c], bg[c]);
+                    // E is quadratic in m, so E_t - E_b = (grad_t + grad_b) . (m_t - m_b) / 2 exactly
+                    de = fma(gr[c] + bg[c], sc, de);
+                    ss = fma(sc, sc, ss);
+                    sy = fma(sc, yc, sy);
+                    yy = fma(yc, yc, yy);
+                }
+                acc[Q_DE] = de;
+                acc[Q_SS] = ss;
+                acc[Q_SY] = sy;
+                acc[Q_YY] = yy;
+            }
+            double pp = 0.0, ee = acc[Q_EEX], ed = acc[Q_ED];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const double sc = m[c] - bm[c];
-                const double yc = fma(-mg, m[c], mm * gr[c]) - fma(-bmg, bm[c], bg[c]);
-                // E is quadratic in m, so E_t - E_b = (grad_t + grad_b) . (m_t - m_b) / 2 exactly
-                de = fma(gr[c] + bg[c], sc, de);
-                ss = fma(sc, sc, ss);
-                sy = fma(sc, yc, sy);
-                yy = fma(yc, yc, yy);
                 const double pc = fma(-ma, ic.a[c], m[c]);
                 pp = fma(pc, pc, pp);
                 ee = fma(m[c], kx[c], ee);
                 ed = fma(m[c], hd[c], ed);
             }
-            acc[Q_DE] = de;
-            acc[Q_SS] = ss;
-            acc[Q_SY] = sy;
-            acc[Q_YY] = yy;
             acc[Q_EEX] = ee;
             acc[Q_ED] = ed;
             acc[Q_EAN] = fma(vi, pp, acc[Q_EAN]);
