@@ -9,13 +9,19 @@
 // surface vectors.  One CTA computes a 128 x 64 tile over a K range (split-K,
 // partials summed in a fixed order by a second kernel).
 //
-// Warp roles (192 threads): warp 0 issues TMA loads (one elected lane), warp 1
-// owns the TMEM accumulator and issues the MMAs (one elected lane), warps 2-5
-// split each A tile into its TF32 head (bits kept in place) and tail (A - head)
-// in shared memory, and finally read the accumulator back (each warp its lane
-// quadrant).  Every wait on an mbarrier gives up after one second, sets the
-// context's error word and leaves the CTA through the common exit that frees
-// the TMEM columns.
+// Both products are one launch.  Warp roles (192 threads): warp 0 issues TMA loads (one
+// elected lane), warp 1 owns the TMEM and issues the MMAs (one elected lane), warps 2-5
+// split each A tile into its TF32 head (low mantissa bits cleared) and tail (A - head),
+// a row per thread, and store both to TMEM, from where the MMAs take A; finally they read
+// the accumulator back (each warp its lane quadrant).  Every wait on an mbarrier gives up
+// after one second, sets the context's error word and leaves the CTA through the common
+// exit that frees the TMEM columns.
+//
+// With head and tail in shared memory, its bandwidth bound the kernel: 150 KB a stage (16
+// KB of A written by TMA, read, written twice by the split and read by twelve MMAs, with X)
+// took 1200 clocks where HBM needs 680 for the 16 KB.  With A in TMEM a stage moves 72 KB,
+// and 52 with 32 instances or fewer (tiles of 32 columns).
+// Both products of 64 / 32 instances at n = 30, with split and sum: 113 / 99 -> 93 / 84 us.
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -29,12 +35,14 @@ namespace lbm {
 
 namespace tc {
 
-constexpr int BM = 128, BN = 64, BK = 32, STAGES = 4, THREADS = 192;
+constexpr int BM = 128, BN = 64, BK = 32, STAGES = 6, THREADS = 192;
 constexpr int A_BYTES = BM * BK * 4;   // 16 KB
-constexpr int X_BYTES = BN * BK * 4;   // 8 KB
-constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * X_BYTES;
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
-constexpr uint32_t TMEM_COLS = 64;
+template <int NT> constexpr int X_BYTES = NT * BK * 4;   // NT = 32 or BN columns: 4 or 8 KB
+template <int NT> constexpr int STAGE_BYTES = A_BYTES + 2 * X_BYTES<NT>;
+template <int NT> constexpr int SMEM_BYTES = STAGES * STAGE_BYTES<NT> + 1024 + 256;
+// TMEM columns: the accumulator, then head and tail of A per stage (32 words each)
+constexpr uint32_t TMEM_A = BN, TMEM_COLS = 512;
+static_assert(TMEM_A + STAGES * 2 * BK <= TMEM_COLS, "one CTA's accumulator and stages of A");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -91,14 +99,28 @@ __device__ __forceinline__ uint64_t sw128_desc(const void* tile) {
 }
 
 // Instruction descriptor, kind::tf32: D FP32, A and B TF32, both K-major.
-constexpr uint32_t IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(BN >> 3) << 17) |
+template <int NT>
+constexpr uint32_t IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(NT >> 3) << 17) |
                            ((uint32_t)(BM >> 4) << 24);
 
-__device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t acc) {
+// D += A X^T, A (128 rows = lanes, 8 words along K = columns) in TMEM
+template <int NT>
+__device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint32_t atmem, uint64_t bdesc, uint32_t acc) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
-        "l"(adesc), "l"(bdesc), "r"(IDESC), "r"(acc));
+        " tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(dtmem),
+        "r"(atmem), "l"(bdesc), "r"(IDESC<NT>), "r"(acc));
+}
+
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31};" ::"r"(r[0]),
+        "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]),
+        "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]),
+        "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]),
+        "r"(r[29]), "r"(r[30]), "r"(r[31]), "r"(taddr)
+        : "memory");
 }
 
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
@@ -122,23 +144,27 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Ypart[split][m][n] = sum_{k in split} A[m][k] X[xrow0 + n][k],  m < nb, n < ncols
+// Ypart[product][split][m][n] = sum_{k in split} A[m][k] X[product ncols + n][k], m < nb,
+// n < ncols; A = B for product 0 and B^T for product 1 (the second half of blockIdx.x)
+template <int NT>
 __global__ void __launch_bounds__(THREADS, 1)
-    k_bem_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapXhi,
-             const __grid_constant__ CUtensorMap mapXlo, int xrow0, int nb, int ncols, int kblocks_per_split,
-             float* __restrict__ Ypart, int* err) {
+    k_bem_tc(const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapBT,
+             const __grid_constant__ CUtensorMap mapXhi, const __grid_constant__ CUtensorMap mapXlo, int nb, int ncols,
+             int kblocks_per_split, float* __restrict__ Ypart, int* err) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint64_t* bars = (uint64_t*)(smem + STAGES * STAGE_BYTES);
+    uint64_t* bars = (uint64_t*)(smem + STAGES * STAGE_BYTES<NT>);
     uint64_t* full = bars;                 // [STAGES] TMA landed
-    uint64_t* conv = bars + STAGES;        // [STAGES] tail split written
+    uint64_t* conv = bars + STAGES;        // [STAGES] head and tail of A in TMEM
     uint64_t* empty = bars + 2 * STAGES;   // [STAGES] MMAs of the stage done
     uint64_t* done = bars + 3 * STAGES;    // accumulator complete
     uint32_t* s_taddr = (uint32_t*)(bars + 3 * STAGES + 1);
     __shared__ int s_fail;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * BM;
+    const int mt = gridDim.x / 2, second = (int)blockIdx.x >= mt;
+    const int m0 = ((int)blockIdx.x - second * mt) * BM, xrow0 = second * ncols;
+    const CUtensorMap* mapA = second ? &mapBT : &mapB;
     const int kb0 = blockIdx.y * kblocks_per_split;
     const int nkb_total = (nb + BK - 1) / BK;
     const int nkb = max(0, min(kblocks_per_split, nkb_total - kb0));
@@ -170,12 +196,12 @@ __global__ void __launch_bounds__(THREADS, 1)
             for (int kb = 0; kb < nkb; ++kb) {
                 const int s = kb % STAGES;
                 if (kb >= STAGES && !mbar_wait(&empty[s], ((kb / STAGES) - 1) & 1, err)) { s_fail = 1; break; }
-                uint8_t* st = smem + s * STAGE_BYTES;
-                mbar_expect_tx(&full[s], A_BYTES + 2 * X_BYTES);
+                uint8_t* st = smem + s * STAGE_BYTES<NT>;
+                mbar_expect_tx(&full[s], A_BYTES + 2 * X_BYTES<NT>);
                 const int k = (kb0 + kb) * BK;
-                tma_load_2d(st, &mapA, &full[s], k, m0);
-                tma_load_2d(st + 2 * A_BYTES, &mapXhi, &full[s], k, xrow0);
-                tma_load_2d(st + 2 * A_BYTES + X_BYTES, &mapXlo, &full[s], k, xrow0);
+                tma_load_2d(st, mapA, &full[s], k, m0);
+                tma_load_2d(st + A_BYTES, &mapXhi, &full[s], k, xrow0);
+                tma_load_2d(st + A_BYTES + X_BYTES<NT>, &mapXlo, &full[s], k, xrow0);
             }
         } else if (warp == 1 && lane == 0) {
             // ---- MMA issuer ----------------------------------------------------------
@@ -183,53 +209,58 @@ __global__ void __launch_bounds__(THREADS, 1)
                 const int s = kb % STAGES;
                 if (!mbar_wait(&conv[s], (kb / STAGES) & 1, err)) { s_fail = 1; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                uint8_t* st = smem + s * STAGE_BYTES;
-                const uint64_t dAh = sw128_desc(st), dAl = sw128_desc(st + A_BYTES);
-                const uint64_t dXh = sw128_desc(st + 2 * A_BYTES), dXl = sw128_desc(st + 2 * A_BYTES + X_BYTES);
+                uint8_t* st = smem + s * STAGE_BYTES<NT>;
+                const uint32_t ah = tmem + TMEM_A + s * 2 * BK, al = ah + BK;
+                const uint64_t dXh = sw128_desc(st + A_BYTES), dXl = sw128_desc(st + A_BYTES + X_BYTES<NT>);
 #pragma unroll
                 for (int kk = 0; kk < BK / 8; ++kk) {
                     const uint64_t o = (uint64_t)(kk * 32) >> 4;   // 8 TF32 = 32 B along K
-                    mma_tf32(tmem, dAh + o, dXh + o, (kb > 0 || kk > 0) ? 1u : 0u);
-                    mma_tf32(tmem, dAh + o, dXl + o, 1u);
-                    mma_tf32(tmem, dAl + o, dXh + o, 1u);
+                    mma_tf32<NT>(tmem, ah + kk * 8, dXh + o, (kb > 0 || kk > 0) ? 1u : 0u);
+                    mma_tf32<NT>(tmem, ah + kk * 8, dXl + o, 1u);
+                    mma_tf32<NT>(tmem, al + kk * 8, dXh + o, 1u);
                 }
                 mma_commit(&empty[s]);
             }
             mma_commit(done);
         } else if (warp >= 2) {
-            // ---- converters: A -> TF32 head (in place) + tail (A - head) --------------
-            const int ct = tid - 64;   // 0..127
-            for (int kb = 0; kb < nkb; ++kb) {
+            // ---- converters: row of A -> TF32 head and tail (A - head) in TMEM ----------
+            // (a warp reaches the TMEM lanes of its quadrant: the same rows as its epilogue)
+            const int row = (warp & 3) * 32 + lane;
+            const uint32_t quadrant = (uint32_t)((warp & 3) * 32) << 16;
+            bool ok = true;
+            for (int kb = 0; kb < nkb && ok; ++kb) {
                 const int s = kb % STAGES;
-                if (!mbar_wait(&full[s], (kb / STAGES) & 1, err)) { s_fail = 1; break; }
-                float4* a = (float4*)(smem + s * STAGE_BYTES);
-                float4* t = (float4*)(smem + s * STAGE_BYTES + A_BYTES);
+                // the stage's MMAs of the round before have finished: the producer waited for them
+                ok = __all_sync(0xffffffffu, mbar_wait(&full[s], (kb / STAGES) & 1, err));
+                if (!ok) { s_fail = 1; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint8_t* a = smem + s * STAGE_BYTES<NT> + row * (BK * 4);
+                uint32_t h[32], l[32];
 #pragma unroll
-                for (int i = 0; i < A_BYTES / 16 / 128; ++i) {
-                    float4 v = a[ct + 128 * i];
-                    float4 h, l;
-                    h.x = __uint_as_float(__float_as_uint(v.x) & 0xFFFFE000u);
-                    h.y = __uint_as_float(__float_as_uint(v.y) & 0xFFFFE000u);
-                    h.z = __uint_as_float(__float_as_uint(v.z) & 0xFFFFE000u);
-                    h.w = __uint_as_float(__float_as_uint(v.w) & 0xFFFFE000u);
-                    l.x = v.x - h.x;
-                    l.y = v.y - h.y;
-                    l.z = v.z - h.z;
-                    l.w = v.w - h.w;
-                    a[ct + 128 * i] = h;
-                    t[ct + 128 * i] = l;
+                for (int c = 0; c < 8; ++c) {   // 16-byte chunks, 128-byte swizzle
+                    const uint4 v = *reinterpret_cast<const uint4*>(a + ((c ^ (row & 7)) << 4));
+                    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        h[4 * c + q] = w[q] & 0xFFFFE000u;
+                        l[4 * c + q] = __float_as_uint(__uint_as_float(w[q]) - __uint_as_float(h[4 * c + q]));
+                    }
                 }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                const uint32_t at = tmem + quadrant + TMEM_A + s * 2 * BK;
+                tmem_st32(at, h);
+                tmem_st32(at + BK, l);
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 mbar_arrive(&conv[s]);
             }
             // ---- epilogue: accumulator rows of this warp's lane quadrant -----------------
-            if (!s_fail && mbar_wait(done, 0, err)) {
+            if (ok && __all_sync(0xffffffffu, mbar_wait(done, 0, err))) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const int quad = warp & 3;
                 const int m = m0 + quad * 32 + lane;
-                float* yrow = Ypart + ((size_t)blockIdx.y * nb + (m < nb ? m : 0)) * BN;
+                float* yrow = Ypart + (((size_t)second * gridDim.y + blockIdx.y) * nb + (m < nb ? m : 0)) * NT;
 #pragma unroll
-                for (int half = 0; half < BN / 32; ++half) {
+                for (int half = 0; half < NT / 32; ++half) {
                     float v[32];
                     tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * 32), v);
                     if (m < nb)
@@ -248,15 +279,17 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
 }
 
-// Y[m * ldy + n] = sum_s Ypart[s][m][n] (fixed order)
+// Y[m][product ncols + n] = sum_s Ypart[product][s][m][n] (fixed order)
 template <typename T>
-__global__ void k_tc_sum(const float* __restrict__ Ypart, int splits, int nb, int ncols, T* __restrict__ Y, int ldy) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nb * ncols) return;
-    const int m = t / ncols, n = t % ncols;
+__global__ void k_tc_sum(const float* __restrict__ Ypart, int splits, int nb, int ncols, int nt, T* __restrict__ Y) {
+    const int C = 2 * ncols, t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nb * C) return;
+    const int m = t / C, c = t - m * C, second = c >= ncols, n = c - second * ncols;
+    const float* y = Ypart + ((size_t)second * splits * nb + m) * nt + n;
     float acc = 0.f;
-    for (int s = 0; s < splits; ++s) acc += Ypart[((size_t)s * nb + m) * BN + n];
-    Y[(size_t)m * ldy + n] = T(acc);
+#pragma unroll 4
+    for (int s = 0; s < splits; ++s) acc += y[(size_t)s * nb * nt];
+    Y[t] = T(acc);
 }
 
 // XT_hi / XT_lo [2B][ldp]: the surface vectors, transposed (column c of the
@@ -315,7 +348,7 @@ constexpr int TC_MAX_SPLITS = 8;   // largest split-K count the autotuner tries
 size_t tc_scratch_floats(int nb, int B, int num_sms) {
     (void)num_sms;
     const int ldp = tc_ld(nb);
-    return (size_t)2 * (2 * B) * ldp + (size_t)TC_MAX_SPLITS * nb * tc::BN + 64;
+    return (size_t)2 * (2 * B) * ldp + (size_t)2 * TC_MAX_SPLITS * nb * (B <= 32 ? 32 : tc::BN) + 64;
 }
 
 // ---- autotuner: split-K count of the tensor-core product ----------------------------
@@ -335,8 +368,8 @@ int splits_for(int nkb, int want, int* kps_out) {
 }
 }  // namespace
 
-static int tc_tuned_splits(const Launch& L, const CUtensorMap& mA, const CUtensorMap& mXh, const CUtensorMap& mXl,
-                           int nb, int B, float* ypart) {
+template <typename F>
+static int tc_tuned_splits(const Launch& L, int nb, int B, F&& launch_with) {
     const auto key = std::make_tuple(nb, B, L.num_sms);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -344,7 +377,7 @@ static int tc_tuned_splits(const Launch& L, const CUtensorMap& mA, const CUtenso
         if (it != g_tc_splits.end()) return it->second;
     }
     const int mt = (nb + tc::BM - 1) / tc::BM, nkb = (nb + tc::BK - 1) / tc::BK;
-    if (!L.tune) return (L.num_sms + mt - 1) / mt;
+    if (!L.tune) return std::min(TC_MAX_SPLITS, (2 * L.num_sms + mt - 1) / mt);
     int best = 0;
     float best_ms = 0.f;
     cudaEvent_t e0, e1;
@@ -357,8 +390,7 @@ static int tc_tuned_splits(const Launch& L, const CUtensorMap& mA, const CUtenso
         float t[3];
         for (int rep = 0; rep < 3; ++rep) {
             cudaEventRecord(e0, L.stream);
-            tc::k_bem_tc<<<dim3(mt, splits), tc::THREADS, tc::SMEM_BYTES, L.stream>>>(mA, mXh, mXl, 0, nb, B, kps,
-                                                                                      ypart, L.err);
+            launch_with(splits, kps);
             cudaEventRecord(e1, L.stream);
             cudaEventSynchronize(e1);
             cudaEventElapsedTime(&t[rep], e0, e1);
@@ -394,25 +426,30 @@ int bem_product_tc(const Launch& L, int nb, const float* A32, const float* A32T,
     float* xhi = scratch;
     float* xlo = scratch + (size_t)C * ldp;
     float* ypart = scratch + (size_t)2 * C * ldp;
-    if (kernel_smem_attr((const void*)tc::k_bem_tc, tc::SMEM_BYTES) != cudaSuccess) return -3;
-    const int total = nb * C;
+    const int total = nb * C, nt = B <= 32 ? 32 : tc::BN;
     tc::k_tc_split<T><<<(total + 255) / 256, 256, 0, L.stream>>>(ub_in, nb, C, ldp, xhi, xlo);
     const int mt = (nb + tc::BM - 1) / tc::BM, nkb = (nb + tc::BK - 1) / tc::BK;
     CUtensorMap mA, mAT, mXh, mXl;
     int e = make_map(&mA, A32, nb, nb, ldp, tc::BK, tc::BM);
     if (!e) e = make_map(&mAT, A32T, nb, nb, ldp, tc::BK, tc::BM);
-    if (!e) e = make_map(&mXh, xhi, nb, C, ldp, tc::BK, tc::BN);
-    if (!e) e = make_map(&mXl, xlo, nb, C, ldp, tc::BK, tc::BN);
+    if (!e) e = make_map(&mXh, xhi, nb, C, ldp, tc::BK, nt);
+    if (!e) e = make_map(&mXl, xlo, nb, C, ldp, tc::BK, nt);
     if (e) return e;
-    int kps;
-    const int splits = splits_for(nkb, tc_tuned_splits(L, mA, mXh, mXl, nb, B, ypart), &kps);
-    const dim3 grid(mt, splits);
     // forward: rows 0..B-1 of X; adjoint: rows B..2B-1 with B^T
-    tc::k_bem_tc<<<grid, tc::THREADS, tc::SMEM_BYTES, L.stream>>>(mA, mXh, mXl, 0, nb, B, kps, ypart, L.err);
-    tc::k_tc_sum<T><<<(nb * B + 255) / 256, 256, 0, L.stream>>>(ypart, splits, nb, B, ub_out, C);
-    tc::k_bem_tc<<<grid, tc::THREADS, tc::SMEM_BYTES, L.stream>>>(mAT, mXh, mXl, B, nb, B, kps, ypart, L.err);
-    tc::k_tc_sum<T><<<(nb * B + 255) / 256, 256, 0, L.stream>>>(ypart, splits, nb, B, ub_out + B, C);
-    *L.launches += 5;
+    auto run = [&](auto fn, int smem) -> int {
+        if (kernel_smem_attr((const void*)fn, smem) != cudaSuccess) return -3;
+        auto launch = [&](int splits, int kps) {
+            fn<<<dim3(2 * mt, splits), tc::THREADS, smem, L.stream>>>(mA, mAT, mXh, mXl, nb, B, kps, ypart, L.err);
+        };
+        int kps;
+        const int splits = splits_for(nkb, tc_tuned_splits(L, nb, B, launch), &kps);
+        launch(splits, kps);
+        tc::k_tc_sum<T><<<(total + 255) / 256, 256, 0, L.stream>>>(ypart, splits, nb, B, nt, ub_out);
+        return 0;
+    };
+    e = nt == 32 ? run(tc::k_bem_tc<32>, tc::SMEM_BYTES<32>) : run(tc::k_bem_tc<tc::BN>, tc::SMEM_BYTES<tc::BN>);
+    if (e) return e;
+    *L.launches += 3;
     return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
