@@ -310,9 +310,9 @@ VecLayout vec_layout(const Mesh& M, int B, int tsize) {
         if (tsize == 8) L.fs_bytes = std::max(L.fs_bytes, C * 8 * fast_scratch_words(M.n, 8));
     }
     L.fs = take(L.fs_bytes);
-    // space-transformation boundary: the FP64 grid potential and seven CG vectors, FP32
-    // ones in the room of five FP64 ones in FP32 batches
-    L.shx = M.shell ? take(8 * (tsize == 8 ? 8 : 6) * (size_t)M.shell->Ng * B) : 0;
+    // space-transformation boundary: the FP64 grid potential and six CG vectors, FP32
+    // ones in the room of three FP64 ones in FP32 batches
+    L.shx = M.shell ? take(8 * (tsize == 8 ? 7 : 4) * (size_t)M.shell->Ng * B) : 0;
     L.total = o;
     return L;
 }

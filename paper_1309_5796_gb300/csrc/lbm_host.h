@@ -252,7 +252,7 @@ struct BatchView {
     float* m32 = nullptr;      // FP32 batches: [N][3][B] FP32 copy of the trial point (else null)
     double* bvec = nullptr;    // [N][B] divergence right-hand side b = G m at the trial point (rhs_eval)
     void* fs = nullptr;        // transformed planes of the fast solves of large cubes (fast_scratch_words)
-    double* shx = nullptr;     // [Ng][B] FP64 grid potential, then seven CG work vectors (space-transformation boundary)
+    double* shx = nullptr;     // [Ng][B] FP64 grid potential, then six CG work vectors (space-transformation boundary)
 };
 
 struct Launch {

@@ -34,7 +34,7 @@ struct ShellArgs {
     const InstState* st;
     const double* bvec;           // [N][B] divergence right-hand side of the magnet
     double* x;                    // [Ng][B] FP64 grid potential
-    W *r, *z, *z2, *dd, *p, *q, *d;   // [Ng][B] work vectors (d: this solve's correction of x)
+    W *r, *z, *z2, *p, *q, *d;   // [Ng][B] work vectors (d: this solve's correction of x)
     double tol2;
     int max_iter;
     unsigned* bar;
@@ -126,8 +126,8 @@ __device__ __forceinline__ void kuhn_apply(const C (&c)[16], const V* v, ptrdiff
     }
 }
 
-constexpr int SH_DEG = 8;             // products of a CG iteration
-constexpr double SH_RATIO = 60.0;     // of the polynomial's interval
+constexpr int SH_DEG = 16;            // products of a CG iteration
+constexpr double SH_RATIO = 400.0;    // of the polynomial's interval
 
 // Threads hold VEC consecutive instances of one row: thread tid works on
 // instances c0 = (tid % G) VEC .. c0 + VEC - 1 (G = B / VEC) of row lane tid / G.
@@ -141,15 +141,17 @@ constexpr double SH_RATIO = 60.0;     // of the polynomial's interval
 //     MP_INNER (or met the tolerance), x += d; the solve ends on the FP64
 //     residual test (restarted CG, as the magnet's mixed-iteration solves).
 // Per CG iteration:
-//   B: alpha = rho / p.q, d += alpha p, r -= alpha q, z = dd = D^-1 r / theta, r.r
-//   C: SH_DEG - 1 steps dd = c1 dd + c2 D^-1 (r - K z), z' = z + dd; r.z with the last
+//   B: alpha = rho / p.q, d += alpha p, r -= alpha q, z = D^-1 r / theta, r.r
+//   C: SH_DEG - 1 steps z'' = z' + c1 (z' - z) + c2 D^-1 (r - K z'), z'' in z's place (no
+//      vector for the steps themselves); r.z with the last
 //   A: w = K z, p = z + beta p, q = w + beta q (= K p), p.q
-// The polynomial is Chebyshev's on [b / 60, b], b a bound of the eigenvalues of
-// D^-1 K: on the 54^3-cell grid 51 iterations of eight products where Jacobi-CG
-// takes 358 of one, and a product with its step moves 5 vector words and one
-// barrier where a CG iteration moves 12 and four.  (Multigrid and fast
-// diagonalisation stall on the shell's growing tangential stiffness.)
-// Measured on that grid: 32 instances 14.9 ms a solve, before 24.1; one 3.0, before 5.7.
+// The polynomial is Chebyshev's on [b / 400, b], b a bound of the eigenvalues of
+// D^-1 K: on the 54^3-cell grid 29 iterations of 16 products where Jacobi-CG takes 358 of
+// one, and a product with its step moves 4 vector words and one barrier where a CG
+// iteration moves 12 and four.  (Degree 8 on [b / 60, b]: 61 iterations, 25 % more time;
+// 20 on [b / 800, b] gives 3 % more on that grid and takes 14 % longer on small FP64 ones.
+// Multigrid and fast diagonalisation stall on the shell's growing tangential stiffness.)
+// Measured on that grid: 32 instances 10.5 ms a solve, one 2.5; at first 24.1 and 5.7.
 // Every block has one run of consecutive rows, so that the L1 serves a product's
 // neighbours along x and y and about three of its fifteen reads go to L2 (with
 // rows dealt round all blocks and loads past the L1, all fifteen did).
@@ -209,7 +211,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
     W* z = A.z;
     W* zo = A.z2;   // the steps alternate between the two
     for (int cycle = 0;; ++cycle) {
-        // residual of the current x: r = f - K x, z = dd = D^-1 r / theta, zero outer faces
+        // residual of the current x: r = f - K x, z = D^-1 r / theta, zero outer faces
         {
             R0 v[2][VEC];   // r.r, f.f
 #pragma unroll
@@ -222,7 +224,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
                     stv<VEC>(A.r + i, zero);
                     stv<VEC>(z + i, zero);
                     stv<VEC>(zo + i, zero);
-                    stv<VEC>(A.dd + i, zero);
                     stv<VEC>(A.p + i, zero);
                     stv<VEC>(A.q + i, zero);
                     stv<VEC>(A.d + i, zero);
@@ -260,7 +261,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
                 }
                 stv<VEC>(A.r + i, rw);
                 stv<VEC>(z + i, zw);
-                stv<VEC>(A.dd + i, zw);
             }
             if (!publish(v)) return;
         }
@@ -300,8 +300,15 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
                     CoefLoad<W>::row(coefW + (size_t)row * 16, c);
                     W w[VEC], rv[VEC], tv[VEC], zv[VEC];
                     ldv<VEC, false>(rv, A.r + i);
-                    ldv<VEC, false>(tv, A.dd + i);
                     ldv<VEC, false>(zv, z + i);
+                    if (st > 1) {   // the last step, from the z before, whose place the next takes
+                        ldv<VEC, false>(tv, zo + i);
+#pragma unroll
+                        for (int k = 0; k < VEC; ++k) tv[k] = zv[k] - tv[k];
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < VEC; ++k) tv[k] = zv[k];
+                    }
                     kuhn_apply<VEC>(c, z + i, sx, sy, sz, kind == 2, w);
                     const W di = c2 * c[15];
 #pragma unroll
@@ -310,7 +317,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
                         zv[k] += tv[k];
                         if (run[k]) v1[0][k] += rv[k] * zv[k];
                     }
-                    stv<VEC>(A.dd + i, tv);
                     stv<VEC>(zo + i, zv);
                 }
                 W* t = z;
@@ -393,7 +399,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
                 stv<VEC>(A.d + i, xa);
                 stv<VEC>(A.r + i, ra);
                 stv<VEC>(zo + i, pa);
-                stv<VEC>(A.dd + i, pa);
             }
             W* t = z;
             z = zo;
@@ -461,14 +466,13 @@ int launch_shell(const Launch& L, const ShellDev& S, const double* bvec, double*
     a.st = st;
     a.bvec = bvec;
     a.x = shx;
-    W* w = reinterpret_cast<W*>(shx + Gv);   // seven work vectors after x
+    W* w = reinterpret_cast<W*>(shx + Gv);   // six work vectors after x
     a.r = w;
     a.z = w + Gv;
     a.p = w + 2 * Gv;
     a.q = w + 3 * Gv;
     a.d = w + 4 * Gv;
     a.z2 = w + 5 * Gv;
-    a.dd = w + 6 * Gv;
     a.tol2 = tol * tol;
     a.max_iter = max_iter;
     a.bar = L.bar;
