@@ -12,17 +12,17 @@
 //   B  alpha = rho / p.q, d += alpha p, r -= alpha q, z = dd = D^-1 r / theta, sums r.r, r
 //   C  DEG - 1 steps dd = c1 dd + c2 D^-1 (r - K z), z += dd; sum r.z with the last
 //   A  p = z + beta p, q = K z + beta q (= K p), sum p.q
-// The polynomial is Chebyshev's on [b / 60, b], b a bound of the eigenvalues of
-// D^-1 K (Gershgorin, at most 4 for linear tetrahedra): eight products then do the
-// work of six CG iterations (187 -> 30 x 8 on a ball of 19 683 nodes) with one plain
-// cluster barrier each in place of two reductions.
+// The polynomial is Chebyshev's on [b / ratio, b], b a bound of the eigenvalues of
+// D^-1 K (Gershgorin, at most 4 for linear tetrahedra), its degree by size (cc_degree):
+// on a ball of 19 683 nodes 15 iterations of 16 products do the work of 187 CG
+// iterations, with one plain cluster barrier a product in place of two reductions.
 // A sum goes from the warps (W) to a total per CTA that is pushed to every CTA's
 // shared memory before the barrier, and is added there over the CTAs (FP64) in a
 // fixed order.  The launch shape depends on the sizes and the batch only, so a
 // solve gives the same bits every time.
 //
-// Measured (both stages of both chains): one instance on 19 683 nodes in FP32 1.8 ms,
-// 7.2 with the grid-wide kernel; 16 on 3 375 nodes in FP64 4.2 ms, before 8.5.
+// Measured (both stages of both chains): one instance on 19 683 nodes in FP32 1.7 ms,
+// 7.2 with the grid-wide kernel; 16 on 3 375 nodes in FP64 4.0 ms, before 8.5.
 // What bounds it: latency, in FP64 also the FP64 units.  A cluster barrier costs 400 to 650 clocks, a reduction
 // with its barrier about 1700, a product of 15 entries a row about 2000 at two rows
 // a thread (distributed shared memory serves 19 bytes a clock to an SM).
@@ -42,9 +42,17 @@ namespace {
 constexpr size_t CC_SMEM_MAX = 225 * 1024;
 constexpr int CC_MAX_CL = 16;
 constexpr int CC_NQ = 4;            // most quantities of one reduction
-constexpr int CC_DEG = 8;           // products of an iteration
-constexpr double CC_RATIO = 60.0;   // of the polynomial's interval
-constexpr int CC_VECS = 7;          // z, z', dd, r, p, q, d
+constexpr int CC_VECS = 7;          // z, z', dd, r, p, q, d (dd from z and z' instead: 2 to 4 % slower)
+
+// Products of an iteration and the ratio of the polynomial's interval.  A higher degree
+// saves reductions, but the last iteration's surplus weighs more where few are needed:
+// both stages of one instance in FP32 on 19 683 nodes 1.83 ms at degree 8 on [b / 60, b],
+// 1.71 at 16 on [b / 240, b]; 16 in FP64 on 3 375 nodes 4.18 at 4 on [b / 60, b], 4.02 at
+// 6 on [b / 120, b], 4.54 at 8 on [b / 240, b]; one in FP64 on 729 nodes 1.04, 1.14, 1.44.
+void cc_degree(int rows, int& deg, double& ratio) {
+    deg = rows >= 8192 ? 16 : rows >= 3000 ? 6 : 4;
+    ratio = rows >= 8192 ? 240.0 : rows >= 3000 ? 120.0 : 60.0;
+}
 
 extern __shared__ __align__(16) unsigned char cc_sm[];
 
@@ -106,7 +114,8 @@ struct CcGeo {
     int rows, rpc, cl;                 // rows of a system, rows per CTA, CTAs per cluster
     int nvec;                          // vectors in shared memory: z, z', then dd, r, p, q, d
     int deg;                           // products of an iteration
-    float b;                           // bound of the eigenvalues of D^-1 K
+    double ratio;                      // the polynomial's interval: [b / ratio, b]
+    double th, de;                     // its centre and half-width
     int ent;                           // general meshes: most entries of a CTA when they are in shared memory, else 0
     unsigned mul, shift;               // j / rpc = umulhi(j, mul) >> shift
     unsigned o_dinv, o_ent, o_ptr, o_scr, o_slot, o_col, smem;
@@ -374,7 +383,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
                 // the same totals in every CTA of the cluster: every CTA leaves together
                 if (__syncthreads_and(tid < VEC ? s_flag[tid] : 1)) break;
                 // ---- C: z = p(D^-1 K) D^-1 r -----------------------------------------
-                const W hi_b = W(g.b), th = W(0.5 * (1.0 + 1.0 / CC_RATIO)) * hi_b, de = W(0.5 * (1.0 - 1.0 / CC_RATIO)) * hi_b;
+                const W th = W(g.th), de = W(g.de);
                 W ab[VEC], v1[1][VEC];
                 if (it == 0) {   // later iterations: done with the update of r
 #pragma unroll
@@ -700,7 +709,7 @@ void cc_try(const Launch& L, int rows, int cols, const int* emax, CcChoice& best
         const int most = sizeof(W) == 8 ? 512 : 1024, per = (g.rpc + most - 1) / most;
         const int threads = std::min(most, std::max(128, ((g.rpc + per - 1) / per + 31) & ~31));
         if (g.nvec < 3) continue;   // dd has no global room
-        g.deg = rows >= 4096 ? CC_DEG : CC_DEG / 2;
+        cc_degree(rows, g.deg, g.ratio);
         int r = cc_resident<T, W, VEC>(g, threads);
         if (L.max_blocks > 0) r = std::min(r, std::max(1, L.max_blocks / g.cl));
         if (r < 1) continue;
@@ -763,7 +772,9 @@ cudaError_t cc_fem(const Launch& L, const MeshView& M, const BatchView<T>& V, co
     CcArgs<T, W> a = {};
     a.P = P;
     a.g = c.g;
-    a.g.b = M.jac_bound;
+    // b: a bound of the eigenvalues of D^-1 K
+    a.g.th = 0.5 * (1.0 + 1.0 / c.g.ratio) * M.jac_bound;
+    a.g.de = 0.5 * (1.0 - 1.0 / c.g.ratio) * M.jac_bound;
     // z, z' and dd are in shared memory (cc_try); r, p, q, d have the batch's work vectors
     a.v[1] = reinterpret_cast<W*>(V.r);
     a.v[2] = reinterpret_cast<W*>(V.p);
