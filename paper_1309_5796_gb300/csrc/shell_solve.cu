@@ -35,6 +35,8 @@ struct ShellArgs {
     const double* bvec;           // [N][B] divergence right-hand side of the magnet
     double* x;                    // [Ng][B] FP64 grid potential
     W *r, *z, *z2, *p, *q, *d;   // [Ng][B] work vectors (d: this solve's correction of x)
+    double th, de;                // centre and half-width of the polynomial's interval
+    int deal;                     // rows dealt round all blocks instead of a run for each
     double tol2;
     int max_iter;
     unsigned* bar;
@@ -128,6 +130,8 @@ __device__ __forceinline__ void kuhn_apply(const C (&c)[16], const V* v, ptrdiff
 
 constexpr int SH_DEG = 16;            // products of a CG iteration
 constexpr double SH_RATIO = 400.0;    // of the polynomial's interval
+// rows and instances from which on FP64 batches deal their rows round all blocks
+constexpr double SH_DEAL = 1.2e6;
 
 // Threads hold VEC consecutive instances of one row: thread tid works on
 // instances c0 = (tid % G) VEC .. c0 + VEC - 1 (G = B / VEC) of row lane tid / G.
@@ -194,10 +198,15 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
     const W* coefW;
     if constexpr (std::is_same<W, double>::value) coefW = A.S.coef64;
     else coefW = A.S.coef32;
-    const int rpb = (Ng + (int)gridDim.x - 1) / (int)gridDim.x;
-    const int rlo = (int)blockIdx.x * rpb, rhi = lane ? min(Ng, rlo + rpb) : 0;   // idle lanes have no rows
+    // a run of consecutive rows for each block (the header says why), or, where the FP64
+    // units bind, rows dealt round all blocks, so that each has its share of the 7- and of
+    // the 15-point rows (29 instances on 54 872 nodes 39.0 -> 34.5 ms a solve, 32 on 91 125
+    // 77 -> 70; 8 on 24 389 nodes, below the line, would go from 5.6 to 7.1)
+    const int rpb = (Ng + (int)gridDim.x - 1) / (int)gridDim.x, rstep = A.deal ? (int)gridDim.x * RB : RB;
+    const int rlo = (int)blockIdx.x * (A.deal ? RB : rpb);
+    const int rhi = !lane ? 0 : A.deal ? Ng : min(Ng, rlo + rpb);   // idle lanes have no rows
     const int row0 = rlo + rl;
-    const W bnd = W(A.S.jac_bound), th = W(0.5 * (1.0 + 1.0 / SH_RATIO)) * bnd, de = W(0.5 * (1.0 - 1.0 / SH_RATIO)) * bnd;
+    const W th = W(A.th), de = W(A.de);
     unsigned epoch = 0;
     // totals of v over the grid into out (NQ quantities of B instances)
     auto publish = [&](auto& v) -> bool {
@@ -217,7 +226,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
 #pragma unroll
             for (int k = 0; k < VEC; ++k) v[0][k] = v[1][k] = R0(0);
             const W zero[VEC] = {};
-            for (int row = row0; row < rhi; row += RB) {
+            for (int row = row0; row < rhi; row += rstep) {
                 const size_t i = (size_t)row * B + c0;
                 const int kind = __ldg(&A.S.kind[row]);
                 if (kind == 0) {   // outer face: u = 0
@@ -286,13 +295,15 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
 #pragma unroll
             for (int k = 0; k < VEC; ++k) run[k] = act[k] && !s_flag[c0 + k];
             // ---- C: outer-face rows (kind 0) keep zero ----
-            W v1[1][VEC], rho_c = de / th;
+            W v1[1][VEC];
+            W rho_c = de / th;
             for (int st = 1; st < SH_DEG; ++st) {
+                const bool last = st + 1 == SH_DEG;
                 const W rn = W(1) / (W(2) * th / de - rho_c), c1 = rn * rho_c, c2 = W(2) * rn / de;
                 rho_c = rn;
 #pragma unroll
                 for (int k = 0; k < VEC; ++k) v1[0][k] = W(0);
-                for (int row = row0; row < rhi; row += RB) {
+                for (int row = row0; row < rhi; row += rstep) {
                     const int kind = __ldg(&A.S.kind[row]);
                     if (kind == 0) continue;
                     const size_t i = (size_t)row * B + c0;
@@ -315,14 +326,14 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
                     for (int k = 0; k < VEC; ++k) {
                         tv[k] = c1 * tv[k] + di * (rv[k] - w[k]);
                         zv[k] += tv[k];
-                        if (run[k]) v1[0][k] += rv[k] * zv[k];
+                        if (last && run[k]) v1[0][k] += rv[k] * zv[k];
                     }
                     stv<VEC>(zo + i, zv);
                 }
                 W* t = z;
                 z = zo;
                 zo = t;
-                if (st + 1 < SH_DEG && !grid_sync(A.bar, gridDim.x, epoch, A.err)) return;
+                if (!last && !grid_sync(A.bar, gridDim.x, epoch, A.err)) return;
             }
             if (!publish(v1)) return;   // r.z
             if (tid < B) {
@@ -339,7 +350,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
                 ab[k] = s_abw[c0 < B ? c0 + k : 0];
                 v1[0][k] = W(0);
             }
-            for (int row = row0; row < rhi; row += RB) {
+            for (int row = row0; row < rhi; row += rstep) {
                 const int kind = __ldg(&A.S.kind[row]);
                 if (kind == 0) continue;
                 const size_t i = (size_t)row * B + c0;
@@ -378,7 +389,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
                 ab[k] = s_abw[c0 < B ? c0 + k : 0];
                 v1[0][k] = W(0);
             }
-            for (int row = row0; row < rhi; row += RB) {
+            for (int row = row0; row < rhi; row += rstep) {
                 const size_t i = (size_t)row * B + c0;
                 const W dt = __ldg(coefW + (size_t)row * 16 + 15) / th;
                 W xa[VEC], pa[VEC], ra[VEC], qa[VEC];
@@ -407,7 +418,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
         }
         // fold the cycle's correction into x before anything reads x
         if (it > 0)
-            for (int row = row0; row < rhi; row += RB) {
+            for (int row = row0; row < rhi; row += rstep) {
                 const size_t i = (size_t)row * B + c0;
                 double xv[VEC];
                 W dv[VEC];
@@ -473,6 +484,9 @@ int launch_shell(const Launch& L, const ShellDev& S, const double* bvec, double*
     a.q = w + 3 * Gv;
     a.d = w + 4 * Gv;
     a.z2 = w + 5 * Gv;
+    a.th = 0.5 * (1.0 + 1.0 / SH_RATIO) * S.jac_bound;
+    a.de = 0.5 * (1.0 - 1.0 / SH_RATIO) * S.jac_bound;
+    a.deal = sizeof(W) == 8 && (double)S.Ng * B >= SH_DEAL;
     a.tol2 = tol * tol;
     a.max_iter = max_iter;
     a.bar = L.bar;
