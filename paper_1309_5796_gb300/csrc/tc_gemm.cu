@@ -377,13 +377,16 @@ static int tc_tuned_splits(const Launch& L, int nb, int B, F&& launch_with) {
         if (it != g_tc_splits.end()) return it->second;
     }
     const int mt = (nb + tc::BM - 1) / tc::BM, nkb = (nb + tc::BK - 1) / tc::BK;
-    if (!L.tune) return std::min(TC_MAX_SPLITS, (2 * L.num_sms + mt - 1) / mt);
+    // at least as many as fill the chip with one product: the tensor cores' FP32 sums lose
+    // accuracy with their length (twice the error at twice the K range)
+    const int least = std::min(std::min(TC_MAX_SPLITS, nkb), (L.num_sms + mt - 1) / mt);
+    if (!L.tune) return least;
     int best = 0;
     float best_ms = 0.f;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    for (int want = 1; want <= TC_MAX_SPLITS; ++want) {
+    for (int want = least; want <= TC_MAX_SPLITS; ++want) {
         int kps;
         const int splits = splits_for(nkb, want, &kps);
         if (splits != want) continue;
@@ -404,7 +407,7 @@ static int tc_tuned_splits(const Launch& L, int nb, int B, F&& launch_with) {
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (best == 0) best = 1;
+    if (best == 0) best = least;
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_tc_splits[key] = best;
     return best;
