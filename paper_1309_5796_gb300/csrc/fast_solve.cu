@@ -42,8 +42,9 @@
 //
 // A result does not depend on how many systems share a cluster, how many CTAs
 // it has or how many threads they run: every sum is taken per chunk of 32
-// quadruples of mirrored nodes of one plane, then over the chunks of a plane,
-// then over the planes, each in a fixed order.
+// quadruples of mirrored nodes of one plane (small cubes in FP64: of 8, a lane
+// per node), then over
+// the chunks of a plane, then over the planes, each in a fixed order.
 #include <math.h>
 #include <stdint.h>
 
@@ -60,6 +61,7 @@ namespace {
 constexpr size_t FS_SMEM_MAX = 226 * 1024;   // dynamic; the rest of the 227 KB is static
 constexpr int FS_MAX_N1 = 97;       // largest cube: 96 cells
 constexpr int FS_NQ = 5;            // most quantities of one reduction
+constexpr int FS_NODE_H = 9;        // FP64: largest half side with a lane per node (n <= 17)
 constexpr int FS_MAX_CL = 16;
 constexpr int FS_SPLIT = 8;         // parts of a row of H
 
@@ -151,7 +153,7 @@ struct FsGeo {
     // pair (k, n-k) stands at k, the odd one at n-k, so folding is in place
     int n, s2, h, ho, hp, hop, ldx, ss;
     int cl, ppc;                          // CTAs per cluster, planes per CTA
-    int nch;                              // chunks of 32 quadruples of a plane
+    int nch;                              // chunks of a plane's sums: 32 quadruples, small cubes in FP64 8
     int zc, pr;                           // positions per CTA in P2, and per round of them
     int spl;                              // TS = false: planes per round of P1 and P3
     int matw;                             // words of one kind's transform matrices
@@ -350,7 +352,7 @@ __device__ __forceinline__ void edge_node(int e, int n, int& i, int& j, int& k) 
 // values frozen.
 template <typename T, typename W, int VEC, bool TS>
 __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(const __grid_constant__ FsArgs<T, W> A) {
-    constexpr bool MP = sizeof(T) != sizeof(W);
+    constexpr bool MP = sizeof(T) != sizeof(W), ND = sizeof(W) == 8;
     const FsGeo& g = A.g;
     W* buf = reinterpret_cast<W*>(fs_sm);                       // TS: own planes [ppc][VEC][ss]; else a round of planes
     W* zb = reinterpret_cast<W*>(fs_sm + g.o_z);                // P2: [s2][VEC * pr] (TS = false: in buf's room)
@@ -496,10 +498,11 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
             int at[4];     // in a sheet
         };
         auto quads = [&](int pa, int pb, auto&& f) {
-            const bool wide = nw >= g.nch;
-            const int ps = wide ? nw / g.nch : 1, pf = wide ? warp / g.nch : 0, cf = wide ? warp - pf * g.nch : warp;
+            const int nc = (h * h + 31) / 32;
+            const bool wide = nw >= nc;
+            const int ps = wide ? nw / nc : 1, pf = wide ? warp / nc : 0, cf = wide ? warp - pf * nc : warp;
             if (pf >= ps) return;
-            for (int ch = cf; ch < g.nch; ch += wide ? g.nch : nw) {
+            for (int ch = cf; ch < nc; ch += wide ? nc : nw) {
                 Quad q;
                 const int e = ch * 32 + lane;
                 q.y = e / h;
@@ -551,6 +554,55 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                 f(u, z0, a);
             }
         };
+        // Small cubes in FP64: the same with a lane per node, a warp per chunk of 8
+        // quadruples.  A warp's FP64 instruction takes its scheduler 64 clocks, and a plane of
+        // 11 x 11 nodes is one warp of quadruples: four nodes one after the other on one of an
+        // SM's four schedulers.  One instance at n = 10: 57 -> 51 us a stage; at n = 25, whose
+        // planes are six warps of quadruples, the lanes' index work costs 3 %.
+        bool nodewise = false;
+        if constexpr (ND) nodewise = h <= FS_NODE_H;
+        struct Node {
+            int y, x;      // of the quadruple
+            bool mx, my, on;
+            int row, at;
+        };
+        auto each = [&](int pa, int pb, auto&& f) {
+            const int nc = g.nch;
+            const bool wide = nw >= nc;
+            const int ps = wide ? nw / nc : 1, pf = wide ? warp / nc : 0, cf = wide ? warp - pf * nc : warp;
+            if (pf >= ps) return;
+            for (int ch = cf; ch < nc; ch += wide ? nc : nw) {
+                Node q;
+                const int e = ch * 8 + (lane >> 2);
+                q.y = e / h;
+                q.x = e - q.y * h;
+                q.mx = lane & 1;
+                q.my = lane & 2;
+                q.on = q.y < h && (!q.mx || q.x < ho) && (!q.my || q.y < ho);
+                if (!q.on) q.y = q.x = 0, q.mx = q.my = false;
+                const int xm = q.mx ? n - q.x : q.x, ym = q.my ? n - q.y : q.y;
+                q.row = ym * s2 + xm;
+                q.at = ym * ldx + xm + (q.mx ? gap : 0);
+                for (int pl = pa + pf; pl < pb; pl += ps) f(pl, ch, q);
+            }
+        };
+        // (K v) at a node: the arithmetic of stencil, the weights (1, 2, 3 or 6) by selection
+        auto stencil1 = [&](const Node& q, int kk, const W* s, const W* sm, const W* sp, W& z0) -> W {
+            const bool ex = q.x == 0, ey = q.y == 0, ek = kk == 0 || kk == n, lo_end = kk == 0;
+            const W vx = ey && ek ? (lo_end != q.my ? W(2) : W(1)) : ey || ek ? W(3) : W(6);
+            const W vy = ex && ek ? (lo_end != q.mx ? W(2) : W(1)) : ex || ek ? W(3) : W(6);
+            const W vz = ex && ey ? (q.mx == q.my ? W(2) : W(1)) : ex || ey ? W(3) : W(6);
+            const int xo = ex ? 0 : -1, xi = q.x + 1 < h ? 1 : 1 + gap, xim = n - q.x - 1 >= h ? -1 : -1 - gap;
+            const int yo = ey ? 0 : -ldx;
+            const W* z = s + q.at;
+            z0 = z[0];
+            W a = vx * (z0 - z[q.mx ? -xo : xo]);
+            a = fma_(vx, z0 - z[q.mx ? xim : xi], a);
+            a = fma_(vy, z0 - z[q.my ? -yo : yo], a);
+            a = fma_(vy, z0 - z[q.my ? -ldx : ldx], a);
+            a = fma_(vz, z0 - sm[q.at], a);
+            return fma_(vz, z0 - sp[q.at], a);
+        };
         // the sheets of the planes below and above plane kk (its own where there is none)
         auto below = [&](int kk, int pl) -> const W* { return kk == 0 ? s_plane[0] : (TS && pl > 0 ? buf + (pl - 1) * VEC * ss : s_plane[kk - 1]); };
         auto above = [&](int kk, int pl) -> const W* { return kk == n ? s_plane[n] : (TS && pl + 1 < np ? buf + (pl + 1) * VEC * ss : s_plane[kk + 1]); };
@@ -600,7 +652,56 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
         for (int cycle = 0;; ++cycle) {
             // residual of the current x into r; sums r.r, r, f.f, f (f: the norm
             // reference, Dirichlet: f - K_IS x_S) and (MP, Neumann) V x for the gauge
-            quads(0, np, [&](int pl, int ch, const Quad& q) {
+            if constexpr (ND) if (nodewise) each(0, np, [&](int pl, int ch, const Node& q) {
+                const int kk = k0 + pl;
+                const bool surf = q.x == 0 || q.y == 0 || kk == 0 || kk == n, froz = !neu && surf;
+                W v[4][VEC];
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) v[0][k] = v[1][k] = v[2][k] = v[3][k] = W(0);
+                if (q.on) {
+                    const int l = pl * pn + q.row;
+                    double fb[VEC];
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k) fb[k] = 0.0;
+                    if (!froz && (neu || !mode)) {
+                        ldc<VEC, false>(fb, bv + (ptrdiff_t)l * B);
+                        if (mode && surf) {   // the BEM term of the adjoint Neumann system
+                            const int bp = (int)((unsigned)nodes[l] >> 16);
+#pragma unroll
+                            for (int k = 0; k < VEC; ++k) fb[k] += (double)P.V.ub_out[(size_t)(bp - 1) * C + c0 + k];
+                        }
+                    }
+                    const W *s = own(kk, pl), *sm = below(kk, pl), *sp = above(kk, pl);
+                    const bool nx = q.x == 1, nx2 = q.x + 1 == n, ny = q.y == 1, ny2 = q.y + 1 == n, nk = kk == 1, nk2 = kk + 1 == n;
+                    const bool ref_differs = !froz && !neu && mode && (nx || nx2 || ny || ny2 || nk || nk2);
+                    W rv[VEC];
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k, s += ss, sm += ss, sp += ss) {
+                        W kx = W(0), z0, ref = act[k] ? W(fb[k]) : W(0);
+                        rv[k] = ref;
+                        if (!froz) kx = stencil1(q, kk, s, sm, sp, z0), rv[k] -= kx;
+                        if (ref_differs) {   // neighbours on the surface
+                            const int xi = q.x + 1 < h ? 1 : 1 + gap, xim = n - q.x - 1 >= h ? -1 : -1 - gap;
+                            const W* z = s + q.at;
+                            W t = W(0);
+                            if (nx) t += z[q.mx ? 1 : -1];
+                            if (nx2) t += z[q.mx ? xim : xi];
+                            if (ny) t += z[q.my ? ldx : -ldx];
+                            if (ny2) t += z[q.my ? -ldx : ldx];
+                            if (nk) t += sm[q.at];
+                            if (nk2) t += sp[q.at];
+                            ref = fma_(W(6), t, ref);
+                        }
+                        v[0][k] = rv[k] * rv[k];
+                        v[1][k] = rv[k];
+                        v[2][k] = ref * ref;
+                        v[3][k] = ref;
+                    }
+                    stc<VEC>(r + (ptrdiff_t)l * VEC, rv);
+                }
+                put(v, 0, pl, ch);
+            });
+            if (!nodewise) quads(0, np, [&](int pl, int ch, const Quad& q) {
                 const int kk = k0 + pl;
                 const bool surf = q.x == 0 || q.y == 0 || kk == 0 || kk == n;
                 W v[4][VEC];
@@ -922,7 +1023,33 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                 W keep[VEC];   // 0: the system has converged and stays as it is
 #pragma unroll
                 for (int k = 0; k < VEC; ++k) keep[k] = s_flag[k] ? W(0) : W(1);
-                quads(0, np, [&](int pl, int ch, const Quad& q) {
+                if constexpr (ND) if (nodewise) each(0, np, [&](int pl, int ch, const Node& q) {
+                    W v[2][VEC];   // r.r, sum r
+                    const int kk = k0 + pl;
+                    const bool froz = !neu && (q.x == 0 || q.y == 0 || kk == 0 || kk == n);
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k) v[0][k] = v[1][k] = W(0);
+                    if (q.on) {
+                        W rv[VEC], dv[VEC];
+                        const ptrdiff_t o = (ptrdiff_t)(pl * pn + q.row) * VEC;
+                        ldc<VEC, false>(rv, r + o);
+                        ldc<VEC, false>(dv, d + o);
+                        const W *s = own(kk, pl), *sm = below(kk, pl), *sp = above(kk, pl);
+#pragma unroll
+                        for (int k = 0; k < VEC; ++k, s += ss, sm += ss, sp += ss) {
+                            W z0, a = stencil1(q, kk, s, sm, sp, z0);
+                            if (froz) a = W(0);
+                            rv[k] = fma_(-keep[k], a, rv[k] - mean[k]);
+                            dv[k] = fma_(keep[k], z0, dv[k]);
+                            v[0][k] = rv[k] * rv[k];
+                            v[1][k] = rv[k];
+                        }
+                        stc<VEC>(r + o, rv);
+                        stc<VEC>(d + o, dv);
+                    }
+                    put(v, 0, pl, ch);
+                });
+                if (!nodewise) quads(0, np, [&](int pl, int ch, const Quad& q) {
                     W v[2][VEC];   // r.r, sum r
 #pragma unroll
                     for (int k = 0; k < VEC; ++k) v[0][k] = v[1][k] = W(0);
@@ -1029,7 +1156,18 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
         for (int k = 0; k < VEC; ++k) mean[k] = 0.0;
         if (neu) {
             if (!ended) {   // MP: the residual pass that ended the solve has summed V x
-                quads(0, np, [&](int pl, int ch, const Quad& q) {
+                if constexpr (ND) if (nodewise) each(0, np, [&](int pl, int ch, const Node& q) {
+                    W v[1][VEC], xv[VEC];
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k) xv[k] = W(0);
+                    const int l = pl * pn + q.row;
+                    if (q.on) ldc<VEC, false>(xv, d + (ptrdiff_t)l * VEC);
+                    const W vi = W(nodes[l] & 0xff);
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k) v[0][k] = vi * xv[k];
+                    put(v, 4, pl, ch);
+                });
+                if (!nodewise) quads(0, np, [&](int pl, int ch, const Quad& q) {
                     T v[1][VEC];
 #pragma unroll
                     for (int k = 0; k < VEC; ++k) v[0][k] = T(0);
@@ -1148,7 +1286,6 @@ FsGeo base_geo(int n) {
     g.hop = (g.ho + 3) & ~3;
     g.ldx = g.hp + g.hop;
     g.ss = g.s2 * g.ldx;
-    g.nch = (g.h * g.h + 31) / 32;
     g.matw = 2 * (g.hp * g.hp + g.hop * g.hop);
     g.ne = 12 * n - 4;
     return g;
@@ -1161,6 +1298,7 @@ bool fit_geo(FsGeo& g, int vec, int ppc, size_t word, int threads, bool ts) {
     g.cl = (g.s2 + ppc - 1) / ppc;
     if (g.cl > FS_MAX_CL) return false;
     g.er = (g.ne + g.cl - 1) / g.cl;
+    g.nch = word == 8 && g.h <= FS_NODE_H ? (g.h * g.h + 7) / 8 : (g.h * g.h + 31) / 32;
     auto up = [](size_t b) { return (b + 15) & ~(size_t)15; };
     const size_t mat = up(g.matw * word), part = up(sizeof(double) * (size_t)ppc * g.nch * FS_NQ * vec);
     const size_t slot = up(sizeof(double) * 2 * (size_t)ppc * FS_NQ * vec);
