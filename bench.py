@@ -344,7 +344,7 @@ def run_reference(args, ws, rank):
 # kernels, from one ncu capture each of the batched workload (profiles/), used to
 # report the roofline's measured traffic per launch: (bytes/ms) x average launch ms.
 PROFILED_DRAM_BYTES_PER_MS = {
-    "fp32": (1109.2e6 / 6.216, "profiles/k_pcg_cluster_fp32_batched64_n30.md"),
+    "fp32": (73.2e6 / 0.3332, "profiles/k_fast_solve_fp32_batched64_n30.md"),
 }
 
 
@@ -362,14 +362,19 @@ def pinned_copy(a: np.ndarray):
         return np.array(a, dtype=np.float64, order="C"), None, "pageable"
 
 
-def pcg_bytes_per_row(kind):
-    """Algorithmic bytes of one PCG iteration per row and system: z gather, p rw,
-    q rw (phase A); x rw, r rw, p and q read, z write (phase B) = 12 vector
-    words.  FP32 solves: 12 x 4 B; plain FP64: 12 x 8 B; FP64 solves iterated in
-    FP32: 12 x 4 B (the FP32 correction takes x's place; it is folded into the
-    FP64 x once per restart cycle, not counted).  The int8 stiffness tables are
-    shared by all systems and not counted."""
-    return {"fp32": 48, "fp64": 96, "fp64_fp32iter": 48}[kind]
+def pcg_bytes_per_row(kind, pcg_kernel=0):
+    """Algorithmic bytes of one step of a potential solve per row and system.  Kuhn
+    cubes by fast diagonalisation (pcg_kernel 0): a step's vectors and transforms
+    stay on the chip; a solve reads and writes x and reads the FP64 right-hand
+    side (FP32: 2 x 4 + 8 B, FP64 x: 2 x 8 + 8 B), and the two systems of a stage
+    take three steps together (a pair and one): 2/3 of that a step.
+    Conjugate-gradient kernels (pcg_kernel 1, 2), an iteration: z gather, p rw, q
+    rw (phase A); x rw, r rw, p and q read, z write (phase B) = 12 vector words of
+    4 B (FP32, and FP64 solves iterated in FP32, whose FP32 correction takes x's
+    place) or 8 B (plain FP64)."""
+    if pcg_kernel:
+        return {"fp32": 48, "fp64": 96, "fp64_fp32iter": 48}[kind]
+    return {"fp32": 32 / 3, "fp64": 16, "fp64_fp32iter": 16}[kind]
 
 
 # Algorithmic bytes of one unit of each kernel kind on a single instance (B = 1),
@@ -381,11 +386,10 @@ def pcg_bytes_per_row(kind):
 #     the node word (4 B), the trial point (24 B FP64 + 12 B FP32 copy in the
 #     FP32 phase, or 24 B), the base point and its gradient (48 B), three
 #     potential columns (12 or 24 B), the new gradient (24 B);
-#   potential solves, per row and sweep of the two systems (forward, adjoint):
-#     12 FP32 words per system (z, p, q; x or d, r, p, q, z) and the row's
-#     stiffness entries, pointer and node word (36 B);
-#   BEM products, per evaluation: the forward and the transposed product each
-#     read the matrix once (4 or 8 B per entry; with B_H its stored values).
+#   potential solves, per row and stage: the two systems' x read and written and
+#     the right-hand side (2 x 16 B in the FP32 phase, 2 x 24 B with FP64 x);
+#   BEM products, per evaluation: the two products read the dense matrix once
+#     (4 or 8 B per entry), with B_H each its own packed form (stored values).
 def large_leg(local, n, hm_eps, max_iter=100000, warmup=1):
     """One instance on an n^3-cell cube (random start, -3 T, mixed precision):
     time to solution and per-kernel achieved bandwidth against the measured HBM
@@ -443,15 +447,14 @@ def large_leg(local, n, hm_eps, max_iter=100000, warmup=1):
         ctx.profile_enable(False)
         inst.destroy()
         n32, n64 = prof["pcg1_fp32"]["launches"], prof["pcg1_fp64"]["launches"]
-        sweeps = sum(prof["cg_sweeps"])
         kern = {
             "trial_update": (prof["trial_update"], (n32 * 84 + n64 * 72) * N),
             "field": (prof["field"], (n32 + n64) * (12 * nnz + 124 * N)),
             "potential_solves": ({"ms": sum(prof[k]["ms"] for k in ("pcg1_fp32", "pcg2_fp32", "pcg1_fp64", "pcg2_fp64")),
                                   "launches": sum(prof[k]["launches"] for k in ("pcg1_fp32", "pcg2_fp32", "pcg1_fp64",
                                                                                 "pcg2_fp64"))},
-                                 sweeps * N * (2 * 48 + 36)),
-            "bem_products": (prof["bem_product"], (n32 * 2 * 4 + n64 * 2 * 8) * stored),
+                                 (n32 * 32 + n64 * 48) * 2 * N),
+            "bem_products": (prof["bem_product"], (n32 * 4 + n64 * 8) * (2 if eps > 0 else 1) * stored),
         }
         per = {}
         for k, (p, by) in kern.items():
@@ -472,8 +475,8 @@ def large_leg(local, n, hm_eps, max_iter=100000, warmup=1):
 
 
 # DRAM bytes per ms of k_shell_pcg kernel time from the ncu capture in
-# profiles/k_shell_pcg_fp32_batched64_n30_shell4x8.md (185.02 GB in 37.659 ms)
-PROFILED_SHELL_DRAM_BYTES_PER_MS = 185.02e9 / 37.659
+# profiles/k_shell_pcg_fp32_batched64_n30_shell4x8.md (59.21 GB in 22.007 ms)
+PROFILED_SHELL_DRAM_BYTES_PER_MS = 59.21e9 / 22.007
 
 
 def shell_leg(ctx, local, insts, a=4, s=8, precision="mixed"):
@@ -528,9 +531,12 @@ def shell_leg(ctx, local, insts, a=4, s=8, precision="mixed"):
     ctx.mesh_destroy(mesh)
     sw = prof["cg_sweeps"]
     word = 4 if (precision == "mixed" or opts.cg_mixed_iter) else 8
-    rec = 68 if word == 4 else 136
+    rec = 64 if word == 4 else 128
     solve_ms = prof["pcg1_fp32"]["ms"] + prof["pcg1_fp64"]["ms"]
-    by = (sw[0] + sw[2]) * rows * (12 * word * B + rec)
+    # an iteration of degree 16: 3 words a row in the first Chebyshev step, 4 in each
+    # of the 14 others, 12 in the two CG passes; the stencil record 17 times
+    words, recs = 3 + 14 * 4 + 12, 17
+    by = (sw[0] + sw[2]) * rows * (words * word * B + recs * rec)
     gbs = by / (solve_ms / 1e3) / 1e9 if solve_ms > 0 else None
     nlaunch = prof["pcg1_fp32"]["launches"] + prof["pcg1_fp64"]["launches"]
     avg_ms = solve_ms / max(1, nlaunch)
@@ -547,7 +553,7 @@ def shell_leg(ctx, local, insts, a=4, s=8, precision="mixed"):
                             "bytes": int(by), "GB_s": round(gbs, 1) if gbs else None,
                             "frac": round(gbs / hbm_peak, 4) if gbs else None,
                             "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)",
-                            "algorithmic_bytes_per_sweep": rows * (12 * word * B + rec),
+                            "algorithmic_bytes_per_sweep": rows * (words * word * B + recs * rec),
                             "avg_launch_ms": round(avg_ms, 3),
                             "bytes_per_launch": by / max(1, nlaunch),
                             "traffic": PROFILED_SHELL_DRAM_BYTES_PER_MS * avg_ms if word == 4 else None,
@@ -639,10 +645,8 @@ def run_ours(args, ws, rank, local):
 
     if rank != 0:
         return
-    # roofline of the dominant kernel: the potential solves (k_pcg).  Algorithmic
-    # bytes per system-iteration and row: z gather, p rw, q rw (phase A), x rw,
-    # r rw, p, q read, z write (phase B) = 12 vector words; the int8 matrix and
-    # the row tables are shared by all 2B systems and not counted.
+    # roofline of the dominant kernel: the potential solves.  The tables are shared
+    # by all 2B systems and not counted.
     peaks = {}
     try:
         peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
@@ -656,18 +660,19 @@ def run_ours(args, ws, rank, local):
     for name, idx, kind in (("fp32", 0, "fp32"), ("fp64", 1, fp64_kind)):
         ms = kinds[f"pcg1_{name}"]["ms"] + kinds[f"pcg2_{name}"]["ms"]
         nl = kinds[f"pcg1_{name}"]["launches"] + kinds[f"pcg2_{name}"]["launches"]
-        by = prof["cg_iters"][idx] * pcg_bytes_per_row(kind) * N
+        by = prof["cg_iters"][idx] * pcg_bytes_per_row(kind, args.pcg_kernel) * N
         pcg[name] = dict(ms=ms, launches=nl, bytes=by, kind=kind)
     dom = max(pcg, key=lambda k: pcg[k]["ms"])
     d = pcg[dom]
     achieved = d["bytes"] / (d["ms"] / 1e3) / 1e9 if d["ms"] > 0 else 0.0
     avg_ms = d["ms"] / max(d["launches"], 1)
     traffic, traffic_src = None, None
-    if d["kind"] in PROFILED_DRAM_BYTES_PER_MS and args.workload == "batched":
+    if d["kind"] in PROFILED_DRAM_BYTES_PER_MS and args.workload == "batched" and not args.pcg_kernel:
         rate, traffic_src = PROFILED_DRAM_BYTES_PER_MS[d["kind"]]
         traffic = rate * avg_ms
-    roofline = {"bound": "hbm", "kernel": f"k_pcg_cluster ({d['kind']} potential solves, forward + adjoint)",
-                "bytes_per_row_system_iteration": pcg_bytes_per_row(d["kind"]),
+    roofline = {"bound": "hbm", "kernel": f"{'k_pcg_cluster' if args.pcg_kernel else 'k_fast_solve'} ({d['kind']} potential "
+                                          "solves, forward + adjoint)",
+                "bytes_per_row_system_iteration": pcg_bytes_per_row(d["kind"], args.pcg_kernel),
                 "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                 "frac": achieved / hbm_peak, "traffic": traffic,
                 "traffic_source": (f"ncu dram__bytes_read.sum + dram__bytes_write.sum per ms of kernel time "
@@ -853,14 +858,14 @@ def run_large(args, ws, rank, local):
     except Exception:
         pass
     hbm_peak = float(peaks.get("hbm_gbs", 6800.0))
-    # one evaluation = one forward and one transposed product: the FP32 matrix in
-    # the FP32 phase, the FP64 matrix in FP64 runs and in the FP64 phase of mixed
+    # one evaluation = one forward and one transposed product in one pass over the
+    # FP32 matrix in the FP32 phase, the FP64 matrix in FP64 runs and in the FP64 phase of mixed
     # runs (one BEM scope per evaluation: as many as first-stage solves)
     word = 8 if prec == lbm.LBM_FP64 else 4
     bem = prof["bem_product"]
     n32, n64 = prof["pcg1_fp32"]["launches"], prof["pcg1_fp64"]["launches"]
-    bem_bytes = (n32 * 2 * 4 + n64 * 2 * 8) * nb * nb if n32 + n64 == bem["launches"] else \
-        bem["launches"] * 2 * word * nb * nb
+    bem_bytes = (n32 * 4 + n64 * 8) * nb * nb if n32 + n64 == bem["launches"] else \
+        bem["launches"] * word * nb * nb
     achieved = bem_bytes / (bem["ms"] / 1e3) / 1e9 if bem["ms"] > 0 else 0.0
     kinds = {k: v for k, v in prof.items() if k not in ("cg_iters", "cg_sweeps")}
     line = {"metric": "solves/s, one instance on a large cube", "value": 1e3 / statistics.mean(ms),
@@ -874,7 +879,7 @@ def run_large(args, ws, rank, local):
             "mesh_setup_s": setup_s, "status": res["status"], "iterations": res["iterations"],
             "evaluations": res["evaluations"], "torque": res["torque"], "energy_J": res["energy"][4],
             "gpu_launches": launches, "clocks": clocks,
-            "roofline": {"bound": "hbm", "kernel": "BEM products (forward row GEMV + transposed column GEMV)",
+            "roofline": {"bound": "hbm", "kernel": "k_gemv_both (forward and transposed BEM product)",
                          "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
                          "traffic": None, "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)",
                          "bytes_per_launch": bem_bytes / max(bem["launches"], 1),
