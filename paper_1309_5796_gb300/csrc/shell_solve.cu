@@ -130,8 +130,9 @@ __device__ __forceinline__ void kuhn_apply(const C (&c)[16], const V* v, ptrdiff
 
 constexpr int SH_DEG = 16;            // products of a CG iteration
 constexpr double SH_RATIO = 400.0;    // of the polynomial's interval
-// rows and instances from which on FP64 batches deal their rows round all blocks
-constexpr double SH_DEAL = 1.2e6;
+// rows times instances from which on FP64 batches deal their rows round all blocks: odd
+// batches, one instance a thread, and even ones, two
+constexpr double SH_DEAL1 = 3e5, SH_DEAL2 = 8e5;
 
 // Threads hold VEC consecutive instances of one row: thread tid works on
 // instances c0 = (tid % G) VEC .. c0 + VEC - 1 (G = B / VEC) of row lane tid / G.
@@ -200,8 +201,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
     else coefW = A.S.coef32;
     // a run of consecutive rows for each block (the header says why), or, where the FP64
     // units bind, rows dealt round all blocks, so that each has its share of the 7- and of
-    // the 15-point rows (29 instances on 54 872 nodes 39.0 -> 34.5 ms a solve, 32 on 91 125
-    // 77 -> 70; 8 on 24 389 nodes, below the line, would go from 5.6 to 7.1)
+    // the 15-point rows (ms a solve, runs -> dealt: 29 instances on 54 872 nodes 39.0 -> 34.3,
+    // 25 on 35 937 19.6 -> 17.4, 9 on 35 937 8.9 -> 8.1, 16 on 50 653 19.0 -> 17.7; below
+    // the lines 24 on 29 791 14.0 -> 14.2, 16 on 24 389 8.4 -> 9.3)
     const int rpb = (Ng + (int)gridDim.x - 1) / (int)gridDim.x, rstep = A.deal ? (int)gridDim.x * RB : RB;
     const int rlo = (int)blockIdx.x * (A.deal ? RB : rpb);
     const int rhi = !lane ? 0 : A.deal ? Ng : min(Ng, rlo + rpb);   // idle lanes have no rows
@@ -486,7 +488,7 @@ int launch_shell(const Launch& L, const ShellDev& S, const double* bvec, double*
     a.z2 = w + 5 * Gv;
     a.th = 0.5 * (1.0 + 1.0 / SH_RATIO) * S.jac_bound;
     a.de = 0.5 * (1.0 - 1.0 / SH_RATIO) * S.jac_bound;
-    a.deal = sizeof(W) == 8 && (double)S.Ng * B >= SH_DEAL;
+    a.deal = sizeof(W) == 8 && (double)S.Ng * B >= (VEC == 1 && B > 1 ? SH_DEAL1 : SH_DEAL2);
     a.tol2 = tol * tol;
     a.max_iter = max_iter;
     a.bar = L.bar;
