@@ -101,15 +101,17 @@ __device__ __forceinline__ void stv(W* p, const W (&d)[VEC]) {
     }
 }
 
-// (K v)_row for VEC instances: v points at the row's first value; sx, sy, sz
+// (K v)_row for VEC instances (ADD: plus w): v points at the row's first value; sx, sy, sz
 // are the strides of one grid step along x, y, z in v.
-template <int VEC, typename R, typename C, typename V>
+template <int VEC, bool ADD = false, typename R, typename C, typename V>
 __device__ __forceinline__ void kuhn_apply(const C (&c)[16], const V* v, ptrdiff_t sx, ptrdiff_t sy, ptrdiff_t sz,
                                            bool full, R (&w)[VEC]) {
     const ptrdiff_t off[15] = {0, sx, -sx, sy, -sy, sz, -sz, sx + sy, -sx - sy, sx + sz, -sx - sz, sy + sz, -sy - sz,
                                sx + sy + sz, -sx - sy - sz};
+    if (!ADD) {
 #pragma unroll
-    for (int k = 0; k < VEC; ++k) w[k] = R(0);
+        for (int k = 0; k < VEC; ++k) w[k] = R(0);
+    }
 #pragma unroll
     for (int j = 0; j < 7; ++j) {
         V t[VEC];
@@ -156,7 +158,7 @@ constexpr double SH_DEAL1 = 3e5, SH_DEAL2 = 8e5;
 // iteration moves 12 and four.  (Degree 8 on [b / 60, b]: 61 iterations, 25 % more time;
 // 20 on [b / 800, b] gives 3 % more on that grid and takes 14 % longer on small FP64 ones.
 // Multigrid and fast diagonalisation stall on the shell's growing tangential stiffness.)
-// Measured on that grid: 32 instances 10.5 ms a solve, one 2.5; at first 24.1 and 5.7.
+// Measured on that grid: 32 instances 10.3 ms a solve, one 2.4; at first 24.1 and 5.7.
 // Every block has one run of consecutive rows, so that the L1 serves a product's
 // neighbours along x and y and about three of its fifteen reads go to L2 (with
 // rows dealt round all blocks and loads past the L1, all fifteen did).
@@ -201,7 +203,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
     else coefW = A.S.coef32;
     // a run of consecutive rows for each block (the header says why), or, where the FP64
     // units bind, rows dealt round all blocks, so that each has its share of the 7- and of
-    // the 15-point rows (ms a solve, runs -> dealt: 29 instances on 54 872 nodes 39.0 -> 34.3,
+    // the 15-point rows (ms a solve, runs -> dealt, with five FP64 operations
+    // a step besides the product, now three: 29 instances on 54 872 nodes 39.0 -> 34.3,
     // 25 on 35 937 19.6 -> 17.4, 9 on 35 937 8.9 -> 8.1, 16 on 50 653 19.0 -> 17.7; below
     // the lines 24 on 29 791 14.0 -> 14.2, 16 on 24 389 8.4 -> 9.3)
     const int rpb = (Ng + (int)gridDim.x - 1) / (int)gridDim.x, rstep = A.deal ? (int)gridDim.x * RB : RB;
@@ -301,7 +304,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
             W rho_c = de / th;
             for (int st = 1; st < SH_DEG; ++st) {
                 const bool last = st + 1 == SH_DEG;
-                const W rn = W(1) / (W(2) * th / de - rho_c), c1 = rn * rho_c, c2 = W(2) * rn / de;
+                const W rn = W(1) / (W(2) * th / de - rho_c), c1 = rn * rho_c, c2 = W(2) * rn / de, c3 = W(1) + c1;
                 rho_c = rn;
 #pragma unroll
                 for (int k = 0; k < VEC; ++k) v1[0][k] = W(0);
@@ -314,20 +317,18 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
                     W w[VEC], rv[VEC], tv[VEC], zv[VEC];
                     ldv<VEC, false>(rv, A.r + i);
                     ldv<VEC, false>(zv, z + i);
-                    if (st > 1) {   // the last step, from the z before, whose place the next takes
-                        ldv<VEC, false>(tv, zo + i);
+                    // z'' = (1 + c1) z' - c1 z - c2 D^-1 (K z' - r), in the place of z (none at first)
 #pragma unroll
-                        for (int k = 0; k < VEC; ++k) tv[k] = zv[k] - tv[k];
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < VEC; ++k) tv[k] = zv[k];
+                    for (int k = 0; k < VEC; ++k) {
+                        tv[k] = W(0);
+                        w[k] = -rv[k];
                     }
-                    kuhn_apply<VEC>(c, z + i, sx, sy, sz, kind == 2, w);
+                    if (st > 1) ldv<VEC, false>(tv, zo + i);
+                    kuhn_apply<VEC, true>(c, z + i, sx, sy, sz, kind == 2, w);
                     const W di = c2 * c[15];
 #pragma unroll
                     for (int k = 0; k < VEC; ++k) {
-                        tv[k] = c1 * tv[k] + di * (rv[k] - w[k]);
-                        zv[k] += tv[k];
+                        zv[k] = c3 * zv[k] - c1 * tv[k] - di * w[k];
                         if (last && run[k]) v1[0][k] += rv[k] * zv[k];
                     }
                     stv<VEC>(zo + i, zv);
