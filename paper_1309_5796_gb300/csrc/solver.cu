@@ -1334,7 +1334,7 @@ int field_blocks(const Launch& L, const MeshView& M, int B) {
 // bounds this kernel (pipe 82 % busy at 64 instances), so it takes each quantity in its
 // cheapest exact form: 1 / V from a table on the Kuhn cube, whose volumes are the
 // integers up to 24; g = |m|^2 grad - (m.grad) m for m x H; |H|^2 = (V/12)^2 |m x h|^2 and
-// |g|^2 = |m|^2 |H|^2; |m x a|^2 = |m - (m.a) a|^2; the Zeeman term from
+// |g|^2 = |m|^2 |H|^2; |m x a|^2 = |a|^2 |m - (m.a) a|^2 (|a| 1 or 0); the Zeeman term from
 // the sum of V m; constant factors on the sums; and at a first point, which has no
 // step behind it, nothing of the step's products.  About 95 operations a node (60 at a
 // first point) where there were 130.  32 instances at n = 30 in FP32: 293 -> 211 us (with five still running 293 ->
@@ -1507,7 +1507,8 @@ __global__ void __launch_bounds__(FIELD_THREADS, sizeof(T) == 4 ? 2 : 1) k_field
         }
         acc[Q_DE] *= 0.5;
         acc[Q_EEX] *= ic.lam / 6.0;
-        acc[Q_EAN] *= ic.Q / 24.0;
+        // |m x a|^2 = |a|^2 |m - (m.a) a|^2 for a unit axis and for none (a = 0: no anisotropy)
+        acc[Q_EAN] *= ic.Q / 24.0 * (ic.a[0] * ic.a[0] + ic.a[1] * ic.a[1] + ic.a[2] * ic.a[2]);
         acc[Q_EZ] = (-1.0 / 12.0) * (acc[Q_MX] * ic.hz[0] + acc[Q_MY] * ic.hz[1] + acc[Q_MZ] * ic.hz[2]);
         acc[Q_ED] *= 1.0 / 24.0;
     }

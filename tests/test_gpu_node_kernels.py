@@ -69,3 +69,34 @@ def test_bits_do_not_depend_on_who_has_finished(ctx):
     assert min(r["evaluations"] for r in res2) < res2[k]["evaluations"]
     assert res2[k]["evaluations"] == res[k]["evaluations"]
     assert np.array_equal(again[k], relaxed[k])
+
+
+@pytest.mark.parametrize("prec", [lbm.LBM_FP64, lbm.LBM_MIXED])
+def test_no_easy_axis_no_anisotropy(ctx, prec):
+    """A material without an easy axis (0, 0, 0) has no anisotropy energy and no anisotropy
+    field, whatever its K1, beside an instance with an axis (whose energy is the sum of
+    K1 V |m x a|^2: every term of it is positive here)."""
+    n, B = 5, 2
+    mesh, N = ctx.mesh_cube(2e-9, n), (n + 1) ** 3
+    m = np.stack([m_perturbed(N, 31 + b, 0.3, (0.4, 0.1, 1.0)) for b in range(B)])
+    out = {}
+    for k1 in (K1_JM3, 0.0):
+        inst = ctx.instance_create(mesh, B, prec)
+        inst.set_material(JS_T, A_JM, k1, [[0.0, 0.0, 0.0], [0.0, 0.0, 1.0]])
+        inst.set_field(np.array([0.1, 0.0, -0.7]))
+        inst.set_m(m)
+        out[k1] = inst.evaluate(lbm.default_opts(prec))
+        inst.destroy()
+    (res, h, _), (plain, h0, _) = out[K1_JM3], out[0.0]
+    assert res[0]["energy"] == plain[0]["energy"] and np.array_equal(h[0], h0[0])
+    assert res[0]["energy"][1] == 0.0 < res[1]["energy"][1]
+    if prec == lbm.LBM_FP64:   # the entry point that allocates nothing
+        torch = pytest.importorskip("torch")
+        d_m = torch.from_numpy(m[0]).to("cuda")
+        d_e = torch.zeros(5, dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        ctx.evaluate_noalloc(mesh, JS_T, A_JM, K1_JM3, [0.0, 0.0, 0.0], np.array([0.1, 0.0, -0.7]), d_m.data_ptr(),
+                             d_energy=d_e.data_ptr())
+        torch.cuda.synchronize()
+        assert float(d_e[1]) == 0.0 and float(d_e[0]) > 0.0
+    ctx.mesh_destroy(mesh)
