@@ -862,7 +862,10 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                         s_it[tid] += 1;
                     }
                     // every solve takes a step (Neumann: a pair): it costs little, and the
-                    // error is then rounding's, not the tolerance's; a pair is completed
+                    // error is then rounding's, not the tolerance's; a pair is completed.
+                    // A system that has met the test waits for the others of its cluster: the
+                    // second step of a pair belongs to the first one, which it has not taken.
+                    const bool stays = !first && s_flag[tid];
                     const bool must = (first && cycle == 0) || (neu && (it & 1));
                     int conv;
                     if constexpr (MP) {
@@ -870,9 +873,9 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                             s_done[tid] = !a || (!must && !(rr > s_tol[tid])) || s_it[tid] >= P.max_iter;
                             s_tin[tid] = fmax(s_tol[tid], MP_INNER * MP_INNER * rr);
                         }
-                        conv = s_done[tid] || (!must && !(rr > s_tin[tid])) || s_it[tid] >= P.max_iter;
+                        conv = stays || s_done[tid] || (!must && !(rr > s_tin[tid])) || s_it[tid] >= P.max_iter;
                     } else {
-                        conv = !a || (!must && !(rr > s_tol[tid])) || it >= P.max_iter;
+                        conv = stays || !a || (!must && !(rr > s_tol[tid])) || it >= P.max_iter;
                     }
                     s_flag[tid] = conv;
                     s_mean[tid] = neu ? sr / (double)N : 0.0;

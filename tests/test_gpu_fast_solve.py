@@ -84,3 +84,28 @@ def test_bits_do_not_depend_on_the_batch(ctx, n, prec):
         assert np.array_equal(u[B][0], u[1][0])
     assert np.array_equal(u[12][:3], u[3])
     ctx.mesh_destroy(mesh)
+
+
+@pytest.mark.parametrize("n,B", [(8, 192), (14, 192), (20, 128)])
+def test_a_converged_system_waits(ctx, n, B):
+    """Tolerances near and below FP32's rounding, where the systems that share a cluster
+    (two do at these sizes) need different numbers of pairs of steps: one that has
+    converged takes no further step, so every instance's first-stage potential has the
+    bits it has alone."""
+    mesh = ctx.mesh_cube(2e-9, n)
+    m = _m(n, B, 11)
+    rng = np.random.default_rng(5)
+    m[1::4] = rng.standard_normal(m[1::4].shape)   # rough right-hand sides beside smooth ones
+    m[2::4, :, :2] *= 0.02
+    m /= np.linalg.norm(m, axis=-1, keepdims=True)
+    mixed = 0
+    for tol in (1e-7, 7e-8, 5e-8, 4e-8, 3e-8, 2e-8, 1e-8, 1e-13):
+        counts = set()
+        u = _run(ctx, mesh, n, B, 1, m, cg_tol=tol)[2]
+        for b in (*range(12), B // 2, B - 1):
+            res, _, one = _run(ctx, mesh, n, 1, 1, m[b:b + 1], cg_tol=tol)
+            counts.add(res[0]["cg_iters1"])
+            assert np.array_equal(u[b, 0], one[0, 0]), (tol, b)
+        mixed += len(counts) > 1
+    assert mixed   # some instances did take more steps than others
+    ctx.mesh_destroy(mesh)
