@@ -605,17 +605,12 @@ int run_chunk(lbm_ctx* ctx, const Launch& L, const Mesh& M, Inst* I, const Batch
     ChunkGraph& g = I->graph;
     std::vector<char> key(sizeof(lbm_solve_opts) + 10 * sizeof(int64_t));
     {
-        // the launch shape of the cluster potential solves (it follows the active
-        // instances; querying it here also caches its occupancy before a capture)
-        int64_t shape = 0;   // the other solves' shapes do not follow the active instances
-        if (!(M.shell && o.demag)) {
-            shape = fast_shape(L, M.view(), I->B, sizeof(T) == 8, o.cg_mixed_iter != 0);
-            if (!shape && (!M.gen || o.pcg_kernel != 0))
-                shape = pcg_cluster_shape(L, M.view(), I->B, sizeof(T) == 8, o.cg_mixed_iter != 0);
-        }
+        // the kernel of the potential solves and, where it follows the active instances,
+        // its launch shape (asking here also caches the occupancies before a capture)
+        const int64_t route = M.shell && o.demag ? 0 : pcg_route(L, M.view(), I->B, sizeof(T) == 8, o.cg_mixed_iter != 0);
         const int64_t k[10] = {chunk, (int64_t)sizeof(T), I->B, (int64_t)(intptr_t)M.hm, (int64_t)(intptr_t)M.B32lo,
                                (int64_t)(intptr_t)M.tcA, ctx->prof ? 1 : 0, (int64_t)(intptr_t)V.m,
-                               (int64_t)(intptr_t)M.shell, shape};
+                               (int64_t)(intptr_t)M.shell, route};
         memcpy(key.data(), &o, sizeof(lbm_solve_opts));
         memcpy(key.data() + sizeof(lbm_solve_opts), k, sizeof k);
     }

@@ -785,6 +785,12 @@ cudaError_t cc_fem(const Launch& L, const MeshView& M, const BatchView<T>& V, co
 
 }  // namespace
 
+bool cluster_cg_takes(const Launch& L, const MeshView& M, int B, bool fp64, bool mixed_iter) {
+    if (!M.gen || L.pcg_kernel != 0 || L.wait_test) return false;
+    if (!fp64) return cc_choose<float, float>(L, M.N, 2 * B, M.emax).vec != 0;
+    return (mixed_iter ? cc_choose<double, float>(L, M.N, 2 * B, M.emax) : cc_choose<double, double>(L, M.N, 2 * B, M.emax)).vec != 0;
+}
+
 // General meshes: 1 when launched (*err its status), 0 when the cluster shapes do
 // not take it (z of a system exceeds a cluster's shared memory).
 template <typename T>

@@ -1460,7 +1460,8 @@ FsChoice choose(const Launch& L, const MeshView& M, int B) {
     if constexpr (sizeof(T) == 4) try_shapes<T, W, 4, true>(L, M.n, B, groups[2], c, cost);
     if constexpr (sizeof(T) == sizeof(W)) try_shapes<T, W, 2, true>(L, M.n, B, groups[1], c, cost);
     try_shapes<T, W, 1, true>(L, M.n, B, groups[0], c, cost);
-    if (!c.vec) try_shapes<T, W, 1, false>(L, M.n, B, groups[0], c, cost);
+    // (where batches have room for the planes in global memory)
+    if (!c.vec && fast_scratch_words(M.n, sizeof(W))) try_shapes<T, W, 1, false>(L, M.n, B, groups[0], c, cost);
     std::lock_guard<std::mutex> lk(mu);
     if (known.size() >= 4096) known.clear();
     known.emplace(key, c);
@@ -1521,6 +1522,7 @@ cudaError_t solve_as(const Launch& L, const MeshView& M, const BatchView<T>& V, 
 template <typename T, typename W>
 int64_t shape_as(const Launch& L, const MeshView& M, int B) {
     const FsChoice c = choose<T, W>(L, M, B);
+    if (!c.vec) return 0;
     return ((((int64_t)c.vec * 32 + c.g.cl) * 2 + c.ts) * 1024 + c.clusters) * 2048 + c.threads;
 }
 

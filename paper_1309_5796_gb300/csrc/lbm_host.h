@@ -276,7 +276,14 @@ struct Launch {
 int pcg_cluster_shape(const Launch& L, const MeshView& M, int B, bool fp64, bool mixed_iter);
 // The same for the fast-diagonalisation solves (0: they do not take this launch).
 int64_t fast_shape(const Launch& L, const MeshView& M, int B, bool fp64, bool mixed_iter);
-// CG preconditioned by fast diagonalisation on Kuhn cubes (fast_solve.cu): 1 when
+// Whether the polynomially preconditioned cluster CG takes this launch (its shape
+// follows the sizes and the batch only).
+bool cluster_cg_takes(const Launch& L, const MeshView& M, int B, bool fp64, bool mixed_iter);
+// The kernel that pcg_solve takes (low two bits, PcgRoute) and its shape where that
+// follows the active instances: what a captured chunk depends on besides the options.
+enum PcgRoute { ROUTE_GRID = 0, ROUTE_FAST = 1, ROUTE_CLUSTER_CG = 2, ROUTE_PCG_CLUSTER = 3 };
+int64_t pcg_route(const Launch& L, const MeshView& M, int B, bool fp64, bool mixed_iter);
+// Fast diagonalisation with iterative refinement on Kuhn cubes (fast_solve.cu): 1 when
 // launched (*err its status), 0 when it does not qualify.
 template <typename T>
 int fast_solve(const Launch& L, const MeshView& M, const BatchView<T>& V, int mode, double tol, int max_iter,

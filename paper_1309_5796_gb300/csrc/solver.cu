@@ -641,18 +641,29 @@ static cudaError_t dispatch_pcg(const Launch& L, const MeshView& M, PcgArgs<T>& 
     return vec4 ? launch_pcg<T, false, V4, GEN, MP>(L, M, a, C) : launch_pcg<T, false, 2, GEN, MP>(L, M, a, C);
 }
 
+// Kuhn cubes: fast diagonalisation; uploaded meshes: the polynomially preconditioned
+// cluster CG where it takes them; then, and where the caller asks for one of the
+// diagonally preconditioned kernels, these.
+int64_t pcg_route(const Launch& L, const MeshView& M, int B, bool fp64, bool mixed_iter) {
+    if (const int64_t s = fast_shape(L, M, B, fp64, mixed_iter)) return s << 2 | ROUTE_FAST;
+    if (cluster_cg_takes(L, M, B, fp64, mixed_iter)) return ROUTE_CLUSTER_CG;
+    if (const int64_t s = pcg_cluster_shape(L, M, B, fp64, mixed_iter)) return s << 2 | ROUTE_PCG_CLUSTER;
+    return ROUTE_GRID;
+}
+
 // mixed_iter (FP64 only): iterate in FP32 with FP64 residual replacement.
 template <typename T>
 int pcg_solve(const Launch& L, const MeshView& M, const BatchView<T>& V, int mode, double tol, int max_iter,
               bool mixed_iter) {
-    // Kuhn cubes, unless the caller asks for one of the diagonally preconditioned kernels
-    cudaError_t fe;
-    if (fast_solve<T>(L, M, V, mode, tol, max_iter, mixed_iter, &fe)) return fe == cudaSuccess ? 0 : (int)fe;
-    if (cluster_cg_fem<T>(L, M, V, mode, tol, max_iter, mixed_iter, &fe)) return fe == cudaSuccess ? 0 : (int)fe;
-    if (L.pcg_kernel != 1) {
-        cudaError_t ce;
-        if (pcg_solve_cluster<T>(L, M, V, mode, tol, max_iter, mixed_iter, &ce)) return ce == cudaSuccess ? 0 : (int)ce;
+    cudaError_t ce = cudaSuccess;
+    int taken = 1;   // 0: the kernel of this route does not take the launch after all
+    switch (pcg_route(L, M, V.B, sizeof(T) == 8, mixed_iter) & 3) {
+        case ROUTE_FAST: taken = fast_solve<T>(L, M, V, mode, tol, max_iter, mixed_iter, &ce); break;
+        case ROUTE_CLUSTER_CG: taken = cluster_cg_fem<T>(L, M, V, mode, tol, max_iter, mixed_iter, &ce); break;
+        case ROUTE_PCG_CLUSTER: taken = pcg_solve_cluster<T>(L, M, V, mode, tol, max_iter, mixed_iter, &ce); break;
+        default: taken = 0;
     }
+    if (taken) return (int)ce;
     const int C = 2 * V.B;
     PcgArgs<T> a{M, V, mode, tol * tol, max_iter, L.bar, L.err, L.sweeps, L.fin};
     // one CTA is fastest for small FP32 work (no grid barriers); FP64 arithmetic
