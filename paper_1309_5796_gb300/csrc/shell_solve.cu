@@ -281,7 +281,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
         if (tid < B) {
             const double rr = out[tid];
             if (cycle == 0) s_tol[tid] = A.tol2 * out[B + tid];
-            s_done[tid] = !s_act[tid] || rr <= s_tol[tid] || s_it[tid] >= A.max_iter;
+            // (a residual that is no number ends the solve: no step mends it)
+            s_done[tid] = !s_act[tid] || !(rr > s_tol[tid]) || s_it[tid] >= A.max_iter;
             s_tin[tid] = RES64 ? fmax(s_tol[tid], MP_INNER * MP_INNER * rr) : s_tol[tid];
             s_rhop[tid] = 1.0;
         }
@@ -293,7 +294,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
                     s_rhop[tid] = s_rho[tid];
                     if (!s_flag[tid]) s_it[tid] += 1;
                 }
-                s_flag[tid] = s_done[tid] || out[tid] <= s_tin[tid] || s_it[tid] >= A.max_iter;
+                s_flag[tid] = s_done[tid] || !(out[tid] > s_tin[tid]) || s_it[tid] >= A.max_iter;
             }
             if (__syncthreads_and(tid < B ? s_flag[tid] : 1)) break;
             bool run[VEC];

@@ -90,3 +90,33 @@ def test_nonfinite_magnetisation(ctx, prec):
     assert all(x["status"] == lbm.LBM_OK for x in r)
     inst.destroy()
     ctx.mesh_destroy(mesh)
+
+
+@pytest.mark.parametrize("prec", [lbm.LBM_FP64, lbm.LBM_MIXED])
+def test_nonfinite_magnetisation_with_the_transformed_grid(ctx, prec):
+    """The solve of a non-finite instance ends at once with the space-transformation
+    boundary too (it does not iterate to cg_max_iter), and its neighbours' results stay."""
+    n, B = 4, 3
+    N = (n + 1) ** 3
+    m0 = np.stack([m_random_sphere(N, 80 + b) for b in range(B)])
+    mesh = ctx.mesh_cube(2e-9, n)
+    ctx.mesh_shell(mesh, 2, 3)
+
+    def run(m):
+        inst = ctx.instance_create(mesh, len(m), prec)
+        inst.set_material(JS_T, A_JM, K1_JM3, [0.0, 0.0, 1.0])
+        inst.set_field(np.array([0.0, 0.0, -1.0]))
+        inst.set_m(m)
+        out = inst.evaluate(lbm.default_opts(prec))
+        inst.destroy()
+        return out
+
+    good, h0, _ = run(m0)
+    m0[1, 7] = [np.nan, 0.0, 1.0]
+    res, h, _ = run(m0)
+    ctx.mesh_destroy(mesh)
+    assert res[1]["status"] == lbm.LBM_E_NAN
+    for b in (0, 2):
+        assert res[b]["status"] == lbm.LBM_OK and res[b]["cg_iters1"] == good[b]["cg_iters1"]
+        assert np.array_equal(h[b], h0[b])
+    assert res[1]["cg_iters1"] <= max(res[0]["cg_iters1"], res[2]["cg_iters1"])
