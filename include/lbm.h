@@ -469,7 +469,9 @@ typedef struct {
 typedef struct {
     int32_t slots;           /* batch width of each group (default 16) */
     int32_t chunk;           /* iterations issued per group between polls (default 8) */
-    int32_t max_pcg_blocks;  /* cooperative grid cap per group (default 0: a quarter of the SMs) */
+    int32_t max_pcg_blocks;  /* cap on the blocks of a group's potential solves at a time (default
+                                0: a quarter of the SMs); the space-transformation solve takes
+                                one block per SM whatever it says */
     double  mem_reserve;     /* fraction of device memory kept free (default 0.05) */
     lbm_solve_opts opt;      /* solve options of every request */
     int32_t shell_a;         /* > 0: every group's cube gets the space-transformation */

@@ -710,8 +710,7 @@ void cc_try(const Launch& L, int rows, int cols, const int* emax, CcChoice& best
         const int threads = std::min(most, std::max(128, ((g.rpc + per - 1) / per + 31) & ~31));
         if (g.nvec < 3) continue;   // dd has no global room
         cc_degree(rows, g.deg, g.ratio);
-        int r = cc_resident<T, W, VEC>(g, threads);
-        if (L.max_blocks > 0) r = std::min(r, std::max(1, L.max_blocks / g.cl));
+        const int r = cc_resident<T, W, VEC>(g, threads);
         if (r < 1) continue;
         const int waves = (cols / VEC + r - 1) / r;
         // an iteration's time in rows of a thread block: the rows' vectors (twice as
@@ -786,7 +785,8 @@ cudaError_t cc_fem(const Launch& L, const MeshView& M, const BatchView<T>& V, co
 }  // namespace
 
 bool cluster_cg_takes(const Launch& L, const MeshView& M, int B, bool fp64, bool mixed_iter) {
-    if (!M.gen || L.pcg_kernel != 0 || L.wait_test) return false;
+    // (a cap on the blocks, L.max_blocks, comes with served cubes only; the other kernels keep to it)
+    if (!M.gen || L.pcg_kernel != 0 || L.wait_test || L.max_blocks > 0) return false;
     if (!fp64) return cc_choose<float, float>(L, M.N, 2 * B, M.emax).vec != 0;
     return (mixed_iter ? cc_choose<double, float>(L, M.N, 2 * B, M.emax) : cc_choose<double, double>(L, M.N, 2 * B, M.emax)).vec != 0;
 }
@@ -797,7 +797,7 @@ template <typename T>
 int cluster_cg_fem(const Launch& L, const MeshView& M, const BatchView<T>& V, int mode, double tol, int max_iter,
                    bool mixed_iter, cudaError_t* err) {
     *err = cudaSuccess;
-    if (!M.gen || L.pcg_kernel != 0 || L.wait_test) return 0;
+    if (!M.gen || L.pcg_kernel != 0 || L.wait_test || L.max_blocks > 0) return 0;
     PcgArgs<T> P{M, V, mode, tol * tol, max_iter, L.bar, L.err, L.sweeps, L.fin};
     bool ok = false;
     if constexpr (sizeof(T) == 4) *err = cc_fem<T, float>(L, M, V, P, &ok);

@@ -170,6 +170,7 @@ struct FsArgs {
     const W* inv;      // [2 kinds][s2 modes][ss] 1 / 6(l_a + l_b + l_c) (0: no such mode, or the constant)
     const W* edge;     // [ne][ne] H (symmetric)
     W* gt;             // TS = false: [group][s2][VEC][ss]
+    int first, clusters;   // this launch's first cluster, and those of all launches of the solve
 };
 
 // Register tile of the transforms: rows x columns per thread.  FP32: 4 x 4, so
@@ -380,7 +381,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
 
     // the cluster's group of VEC systems: the k-th one with an active instance
     if (warp == 0) {
-        const int ng = C / VEC, want = (int)cl_index();
+        const int ng = C / VEC, want = A.first + (int)cl_index();
         int found = -1, cnt = 0;
         for (int base = 0; base < ng; base += 32) {
             bool a = false;
@@ -396,7 +397,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
         }
         if (lane == 0) {
             s_grp = found;
-            if (rank == 0 && want == 0 && cnt > (int)(gridDim.x / g.cl)) atomicOr(A.P.err, DEV_ERR_SHAPE);
+            if (rank == 0 && want == 0 && cnt > A.clusters) atomicOr(A.P.err, DEV_ERR_SHAPE);
         }
     }
     __syncthreads();
@@ -1250,12 +1251,12 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                       (unsigned long long)s_it[tid]);
         for (int k = 0; k < VEC; ++k) itmax = max(itmax, s_it[k]);
     }
-    // sweep counter: the largest step count of the launch (the last cluster to
+    // sweep counter: the largest step count of the solve (its last cluster to
     // finish adds it and clears the two counter words)
     if (rank == 0 && tid == 0) {
         atomicMax(&A.P.bar[2], (unsigned)itmax);
         __threadfence();
-        if (atomicAdd(&A.P.bar[3], 1u) == gridDim.x / g.cl - 1) {
+        if (atomicAdd(&A.P.bar[3], 1u) == (unsigned)A.clusters - 1u) {
             __threadfence();
             const unsigned km = atomicExch(&A.P.bar[2], 0u);
             atomicExch(&A.P.bar[3], 0u);
@@ -1380,6 +1381,7 @@ int resident(const FsGeo& g, int threads) {
 struct FsChoice {
     FsGeo g;
     int vec = 0, threads = 0, clusters = 0;
+    int per = 0;   // clusters of one launch (all of them without a cap on the blocks)
     bool ts = true;
 };
 
@@ -1395,7 +1397,7 @@ void try_shapes(const Launch& L, int n, int B, int groups, FsChoice& best, doubl
             FsGeo g = base_geo(n);
             if (!fit_geo(g, VEC, ppc, sizeof(W), threads, TS)) continue;
             int r = resident<T, W, VEC, TS>(g, threads);
-            if (L.max_blocks > 0) r = std::min(r, std::max(1, L.max_blocks / cl));
+            if (L.max_blocks > 0) r = std::min(r, L.max_blocks / cl);
             if (r < 1) continue;
             const int waves = (groups + r - 1) / r;
             // CTAs that share an SM share its issue slots; a CTA's own rows take their
@@ -1415,13 +1417,19 @@ void try_shapes(const Launch& L, int n, int B, int groups, FsChoice& best, doubl
                 best.threads = threads;
                 best.ts = TS;
                 best.clusters = waves > 1 ? 2 * B / VEC : std::min(r, 2 * B / VEC);
+                best.per = best.clusters;
+                if (L.max_blocks > 0) {   // waves as launches one after the other, none for idle groups only
+                    best.clusters = std::min(waves * r, 2 * B / VEC);
+                    best.per = r;
+                }
             }
         }
     }
 }
 
 // The launch for a batch: VEC systems per cluster, planes per CTA, threads.  Clusters
-// are independent, so more of them than can be resident at once run in waves.  The
+// are independent, so more of them than can be resident at once run in waves; a cap on
+// the blocks (L.max_blocks: size groups that share the chip) makes the waves launches.  The
 // constants are fitted to some 400 measured shapes of 25 sizes and batches (n = 10 to
 // 80, 1 to 64 instances), on which the rule's shape is within 5 % of the fastest (1 % on
 // average): 64 instances at n = 30 run one system on two CTAs of 16 planes and 512
@@ -1469,9 +1477,8 @@ FsChoice choose(const Launch& L, const MeshView& M, int B) {
 }
 
 template <typename T, typename W, int VEC, bool TS>
-cudaError_t launch_fast(const Launch& L, const FsArgs<T, W>& a, const FsChoice& c) {
+cudaError_t launch_fast(const Launch& L, FsArgs<T, W>& a, const FsChoice& c) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(c.clusters * c.g.cl));
     cfg.blockDim = dim3((unsigned)c.threads);
     cfg.dynamicSmemBytes = c.g.smem;
     cfg.stream = L.stream;
@@ -1482,7 +1489,14 @@ cudaError_t launch_fast(const Launch& L, const FsArgs<T, W>& a, const FsChoice& 
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_fast_solve<T, W, VEC, TS>, a);
+    cudaError_t e = cudaSuccess;
+    a.clusters = c.clusters;
+    for (a.first = 0; a.first < c.clusters && e == cudaSuccess; a.first += c.per) {
+        cfg.gridDim = dim3((unsigned)(std::min(c.per, c.clusters - a.first) * c.g.cl));
+        e = cudaLaunchKernelEx(&cfg, k_fast_solve<T, W, VEC, TS>, a);
+        *L.launches += 1;
+    }
+    return e;
 }
 
 template <typename T, typename W>
@@ -1548,9 +1562,7 @@ int fast_solve(const Launch& L, const MeshView& M, const BatchView<T>& V, int mo
     if constexpr (sizeof(T) == 4) *err = solve_as<T, float>(L, M, V, P, &ok);
     else if (mixed_iter) *err = solve_as<T, float>(L, M, V, P, &ok);
     else *err = solve_as<T, double>(L, M, V, P, &ok);
-    if (!ok && *err == cudaSuccess) return 0;
-    *L.launches += 1;
-    return 1;
+    return ok || *err != cudaSuccess;
 }
 
 template int fast_solve<float>(const Launch&, const MeshView&, const BatchView<float>&, int, double, int, bool, cudaError_t*);

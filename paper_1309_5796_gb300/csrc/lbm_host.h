@@ -263,7 +263,7 @@ struct Launch {
     int64_t* launches; // host counter of kernel launches
     unsigned long long* sweeps;  // device counters [4]: batched PCG iterations per stage and precision
     double* fin;                 // device scratch for grid reductions (>= 4 * 512 doubles)
-    int max_blocks;              // cap on the cooperative PCG grid (0: one block per SM)
+    int max_blocks;              // cap on the blocks of a potential solve's launch (0: one block per SM)
     bool tune = true;            // launch-shape autotuning allowed (it waits on events)
     bool wait_test = false;      // solves must take a kernel with a grid barrier (lbm_set_wait_limit's test hook)
     int pcg_kernel = 0;          // 0 choose, 1 grid-wide kernel, 2 prefer clusters (lbm_solve_opts)

@@ -105,3 +105,25 @@ def test_size_groups_overlap_on_the_device(ctx):
             if tr[i, 0] != tr[j, 0] and max(tr[i, 1], tr[j, 1]) < min(tr[i, 2], tr[j, 2]):
                 overlaps += 1
     assert overlaps > 0
+
+
+def test_the_block_cap_holds_for_cubes(ctx):
+    """max_pcg_blocks caps the blocks of a group's potential solves: with one block a solve
+    takes a launch for each of the batch's systems, with the device's it takes one; the
+    results have the same bits."""
+    req = _req(6, 17, -5.0, 3.0)
+    N = (req["n"] + 1) ** 3
+    out = []
+    for cap in (1, 100000):
+        ctx.serve_start(slots=4, chunk=4, max_pcg_blocks=cap)
+        try:
+            k0 = ctx.launch_count()
+            r, m = ctx.wait(ctx.submit(**req), N, timeout_s=300)
+        finally:
+            ctx.serve_stop()   # the loop has ended: its counter is still
+        out.append((r, m, ctx.launch_count() - k0))
+    (ra, ma, la), (rb, mb, lb) = out
+    assert ra["status"] == rb["status"] == lbm.LBM_OK
+    assert ra["energy"] == rb["energy"] and np.array_equal(ma, mb)
+    # an evaluation is at most 7 launches with one a solve; its two solves have two systems to serve
+    assert la >= lb + 2 * ra["evaluations"]
