@@ -417,26 +417,45 @@ void free_mesh(Mesh* m) {
     delete m;
 }
 
+// Byte offsets of the fast-diagonalisation tables of a Kuhn cube inside one allocation.
+struct FastLayout {
+    size_t i64, m32, i32, row, col, e64, e32, total;
+};
+FastLayout fast_layout(int n) {
+    FastTables t;
+    fast_sizes(n, t);
+    const size_t nm = 2 * (size_t)t.words, ni = 2 * t.inv, ne = 12 * (size_t)n - 4;
+    FastLayout L;
+    size_t o = align256(8 * nm);
+    auto take = [&o](size_t bytes) { const size_t at = o; o += align256(bytes); return at; };
+    L.i64 = take(8 * ni);
+    L.m32 = take(4 * nm);
+    L.i32 = take(4 * ni);
+    L.row = take(8 * 2 * ((size_t)n + 1));
+    L.col = take(8 * 2 * (size_t)t.ldx);
+    L.e64 = take(8 * ne * ne);
+    L.e32 = take(4 * ne * ne);
+    L.total = o;
+    return L;
+}
+
 // The fast-diagonalisation tables of a Kuhn cube (fast_solve.cu).
 int fast_upload(lbm_ctx* ctx, Mesh* M) {
     FastTables t;
     fast_tables(M->n, t);
-    const size_t nm = t.mat.size(), ni = 2 * t.inv, nr = t.lam_row.size(), nc = t.lam_col.size();
+    const size_t nm = t.mat.size(), nr = t.lam_row.size(), nc = t.lam_col.size();
     const size_t ne = 12 * (size_t)M->n - 4, ne2 = ne * ne;
-    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    const size_t o_i64 = up(8 * nm), o_m32 = o_i64 + up(8 * ni), o_i32 = o_m32 + up(4 * nm), o_r = o_i32 + up(4 * ni),
-                 o_c = o_r + up(8 * nr), o_e64 = o_c + up(8 * nc), o_e32 = o_e64 + up(8 * ne2),
-                 total = o_e32 + up(4 * ne2);
-    CK(cudaMalloc(&M->fast_mem, total));
+    const FastLayout L = fast_layout(M->n);
+    CK(cudaMalloc(&M->fast_mem, L.total));
     char* base = (char*)M->fast_mem;
     const std::vector<float> m32(t.mat.begin(), t.mat.end());
     cudaStream_t st = ctx->stream;
     CK(cudaMemcpyAsync(base, t.mat.data(), 8 * nm, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(base + o_m32, m32.data(), 4 * nm, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(base + o_r, t.lam_row.data(), 8 * nr, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(base + o_c, t.lam_col.data(), 8 * nc, cudaMemcpyHostToDevice, st));
-    launch_fast_inv(M->n, (const double*)(base + o_r), (const double*)(base + o_c), (double*)(base + o_i64),
-                    (float*)(base + o_i32), st);
+    CK(cudaMemcpyAsync(base + L.m32, m32.data(), 4 * nm, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(base + L.row, t.lam_row.data(), 8 * nr, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(base + L.col, t.lam_col.data(), 8 * nc, cudaMemcpyHostToDevice, st));
+    launch_fast_inv(M->n, (const double*)(base + L.row), (const double*)(base + L.col), (double*)(base + L.i64),
+                    (float*)(base + L.i32), st);
     ctx->launches += 2;
     {   // the correction of the cube's edges
         std::vector<double> A, X(ne2), H;
@@ -444,27 +463,27 @@ int fast_upload(lbm_ctx* ctx, Mesh* M) {
         double* w = nullptr;   // A, T1, T2; X in H's place
         CK(cudaMalloc(&w, 3 * 8 * ne2));
         cudaError_t e = cudaMemcpyAsync(w, A.data(), 8 * ne2, cudaMemcpyHostToDevice, st);
-        launch_inverse_newton((int)ne, w, (double*)(base + o_e64), w + ne2, w + 2 * ne2, st);
+        launch_inverse_newton((int)ne, w, (double*)(base + L.e64), w + ne2, w + 2 * ne2, st);
         ctx->launches += 9;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(X.data(), base + o_e64, 8 * ne2, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(X.data(), base + L.e64, 8 * ne2, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         cudaFree(w);
         CK(e);
         fast_edge_matrix(M->n, X, H);
         const std::vector<float> h32(H.begin(), H.end());
-        CK(cudaMemcpyAsync(base + o_e64, H.data(), 8 * ne2, cudaMemcpyHostToDevice, st));
-        CK(cudaMemcpyAsync(base + o_e32, h32.data(), 4 * ne2, cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(base + L.e64, H.data(), 8 * ne2, cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(base + L.e32, h32.data(), 4 * ne2, cudaMemcpyHostToDevice, st));
         CK(cudaStreamSynchronize(st));
     }
     CK(cudaGetLastError());
     M->fast = new FastDev();
     M->fast->mat64 = (const double*)base;
-    M->fast->inv64 = (const double*)(base + o_i64);
-    M->fast->mat32 = (const float*)(base + o_m32);
-    M->fast->inv32 = (const float*)(base + o_i32);
-    M->fast->edge64 = (const double*)(base + o_e64);
-    M->fast->edge32 = (const float*)(base + o_e32);
-    M->bytes += total;
+    M->fast->inv64 = (const double*)(base + L.i64);
+    M->fast->mat32 = (const float*)(base + L.m32);
+    M->fast->inv32 = (const float*)(base + L.i32);
+    M->fast->edge64 = (const double*)(base + L.e64);
+    M->fast->edge32 = (const float*)(base + L.e32);
+    M->bytes += L.total;
     return LBM_OK;
 }
 
@@ -2395,17 +2414,32 @@ void group_free(lbm_ctx* ctx, Group* G) {
     delete G;
 }
 
-size_t group_estimate(int n, int slots, int shell_a, int shell_s) {
-    const size_t N = (size_t)(n + 1) * (n + 1) * (n + 1);
-    const size_t nb = N - (size_t)(n > 1 ? (n - 1) * (n - 1) * (n - 1) : 0);
-    size_t mesh = 12 * nb * nb + 100 * N;
-    size_t per_slot = 8 * (2 * N * 3 * 2 + 3 * N) * 2 + (4 + 8) * (12 * N + 4 * nb) + 40 * N;
-    if (shell_a > 0) {   // the grid's stencil records and, per slot, its FP64 vectors in both batches
-        const size_t g1 = (size_t)n + 2 * ((size_t)shell_a + shell_s) + 1, Ng = g1 * g1 * g1;
-        mesh += (16 * 12 + 9) * Ng;
-        per_slot += (6 + 8) * 8 * Ng;
+// Device memory that a size group takes: the mesh with both copies of B, its low words
+// and its tables, the grid's records, and the two batches, with what assembling B takes
+// while they are not there yet; 64 MB for graphs, kernels and rounding up.
+size_t group_estimate(const lbm_ctx* ctx, int n, int slots, int shell_a, int shell_s) {
+    Mesh M;
+    FastDev fast;
+    ShellDev shell;
+    M.n = n;
+    M.N = (n + 1) * (n + 1) * (n + 1);
+    M.nb = M.N - (n > 1 ? (n - 1) * (n - 1) * (n - 1) : 0);
+    M.num_sms = ctx->num_sms;
+    M.fast = &fast;
+    const size_t N = M.N, nb = M.nb;
+    size_t mesh = (slots > 1 ? 16 : 12) * nb * nb + 230 * N + fast_layout(n).total;
+    if (shell_a > 0) {
+        const size_t g1 = (size_t)n + 2 * ((size_t)shell_a + shell_s) + 1;
+        shell.Ng = (int)(g1 * g1 * g1);
+        M.shell = &shell;
+        mesh += (16 * 12 + 9) * (size_t)shell.Ng;
     }
-    return mesh + per_slot * slots + ((size_t)64 << 20);
+    const size_t assembly = 8 * 3 * 12 * (size_t)n * n * std::min((size_t)2 * ctx->num_sms, nb);
+    size_t batches = 0;
+    for (int tsize : {4, 8})
+        batches += vec_bytes(M, slots, tsize) + 8 * part_elems(ctx, slots) + 40 * N * slots +
+                   (sizeof(InstState) + sizeof(InstConst)) * slots;
+    return mesh + std::max(assembly, batches + 24 * N) + ((size_t)64 << 20);
 }
 
 // Create (or reuse) the group of cube size n, evicting idle groups when the
@@ -2414,7 +2448,7 @@ Group* group_get(Server& S, int n, double cell) {
     auto it = S.groups.find(n);
     if (it != S.groups.end()) return it->second;
     lbm_ctx* ctx = S.ctx;
-    const size_t need = group_estimate(n, S.opt.slots, S.opt.shell_a, S.opt.shell_s);
+    const size_t need = group_estimate(ctx, n, S.opt.slots, S.opt.shell_a, S.opt.shell_s);
     for (;;) {
         size_t fr = 0, tot = 0;
         cudaMemGetInfo(&fr, &tot);

@@ -1578,11 +1578,16 @@ size_t fast_scratch_words(int n, size_t word) {
     return (size_t)(n + 1) * base_geo(n).ss;
 }
 
-void fast_tables(int n, FastTables& t) {
+void fast_sizes(int n, FastTables& t) {
     const FsGeo g = base_geo(n);
     t.words = g.matw;
     t.inv = (size_t)g.s2 * g.ss;
     t.ldx = g.ldx;
+}
+
+void fast_tables(int n, FastTables& t) {
+    const FsGeo g = base_geo(n);
+    fast_sizes(n, t);
     t.mat.assign((size_t)2 * g.matw, 0.0);
     t.lam_row.assign((size_t)2 * g.s2, -1.0);
     t.lam_col.assign((size_t)2 * g.ldx, -1.0);

@@ -186,6 +186,7 @@ struct FastTables {
     size_t inv = 0;                    // words of one kind's 1 / eigenvalues
     std::vector<double> mat, lam_row, lam_col;   // [2 kinds]
 };
+void fast_sizes(int n, FastTables& t);   // words, ldx and inv alone
 void fast_tables(int n, FastTables& t);
 // Correction of the edge nodes: A = 1 + R E, and H = E - E X with X = A^-1 (host,
 // ne x ne row-major, ne = 12 n - 4); launch_inverse_newton: X = A^-1 on the device for

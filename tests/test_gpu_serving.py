@@ -127,3 +127,41 @@ def test_the_block_cap_holds_for_cubes(ctx):
     assert ra["energy"] == rb["energy"] and np.array_equal(ma, mb)
     # an evaluation is at most 7 launches with one a solve; its two solves have two systems to serve
     assert la >= lb + 2 * ra["evaluations"]
+
+
+def test_a_group_is_admitted_with_the_memory_it_takes(ctx):
+    """The memory a size group is said to need covers what it takes: with 8 MB less than
+    that free (the rest reserved) a request waits, with it and some more it runs."""
+    import time
+
+    import torch
+    req = _req(30, 12, -4.0, 3.0)
+    torch.cuda.mem_get_info()
+
+    def free():
+        return torch.cuda.mem_get_info()
+
+    def serve(reserve):
+        ctx.serve_start(slots=64, chunk=8, mem_reserve=reserve)
+        try:
+            t = ctx.submit(**req)
+            time.sleep(1.0)
+            st = ctx.serve_stats()
+            if not st["active_slots"] and not st["completed"]:
+                return st, None
+            used = f0 - free()[0]
+            ctx.wait(t, None, timeout_s=300)
+            return st, used
+        finally:
+            ctx.serve_stop()
+
+    f0, tot = free()
+    serve(0.0)                       # modules, kernels and pools of a first run
+    f0 = free()[0]
+    st, used = serve(0.0)
+    assert used > 0 and st["stalls"] == 0
+    f0 = free()[0]
+    st, none = serve((f0 - used + (8 << 20)) / tot)
+    assert none is None and st["stalls"] > 0
+    st, again = serve((f0 - used - (256 << 20)) / tot)
+    assert again is not None and st["stalls"] == 0
