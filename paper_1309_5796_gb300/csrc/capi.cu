@@ -297,9 +297,6 @@ VecLayout vec_layout(const Mesh& M, int B, int tsize) {
     L.q = take(tsize * N * C);
     L.ub_in = take(tsize * nb * C);
     L.ub_out = take(tsize * nb * C);
-    // partial sums of the boundary products: gemv_parts() vectors of one instance, the
-    // K-split partials of a batch (S x nb x 2B)
-    L.bem_part = take(8 * (B == 1 ? (size_t)gemv_parts() * nb : (size_t)bem_df_splits((int)nb, B, M.num_sms) * nb * C));
     L.m32 = tsize == 4 ? take(4 * N * 3 * B) : 0;
     L.bvec = take(8 * N * B);
     // transformed planes of the fast solves of large cubes (FP64 batches: plain and
@@ -313,9 +310,16 @@ VecLayout vec_layout(const Mesh& M, int B, int tsize) {
     // space-transformation boundary: the FP64 grid potential and six CG vectors, FP32
     // ones in the room of three FP64 ones in FP32 batches
     L.shx = M.shell ? take(8 * (tsize == 8 ? 7 : 4) * (size_t)M.shell->Ng * B) : 0;
+    // last, as not every batch has them (vec_bytes): partial sums of the boundary products,
+    // gemv_parts() vectors of one instance, the K-split partials of a batch (S x nb x 2B)
+    L.bem_part = take(8 * (B == 1 ? (size_t)gemv_parts() * nb : (size_t)bem_df_splits((int)nb, B, M.num_sms) * nb * C));
     L.total = o;
     return L;
 }
+
+// Whether a batch takes boundary products that sum partials: not with the space
+// transformation (no boundary matrix), nor on the tensor cores (their own scratch).
+bool bem_sums(const Mesh& M, bool use_tc) { return !M.shell && !use_tc; }
 
 template <typename T>
 BatchView<T> batch_view(const lbm_ctx* ctx, const Mesh& M, const Inst& I, bool with_hout) {
@@ -335,7 +339,7 @@ BatchView<T> batch_view(const lbm_ctx* ctx, const Mesh& M, const Inst& I, bool w
     v.q = (T*)(base + L.q);
     v.ub_in = (T*)(base + L.ub_in);
     v.ub_out = (T*)(base + L.ub_out);
-    v.bem_part = (T*)(base + L.bem_part);
+    v.bem_part = bem_sums(M, I.use_tc) ? (T*)(base + L.bem_part) : nullptr;
     v.bem_parts = gemv_parts();
     v.m32 = sizeof(T) == 4 ? (float*)(base + L.m32) : nullptr;
     v.bvec = (double*)(base + L.bvec);
@@ -347,7 +351,10 @@ BatchView<T> batch_view(const lbm_ctx* ctx, const Mesh& M, const Inst& I, bool w
     return v;
 }
 
-size_t vec_bytes(const Mesh& M, int B, int tsize) { return vec_layout(M, B, tsize).total; }
+size_t vec_bytes(const Mesh& M, int B, int tsize, bool use_tc = false) {
+    const VecLayout L = vec_layout(M, B, tsize);
+    return bem_sums(M, use_tc) ? L.total : L.bem_part;
+}
 
 // A new magnetisation starts its potential solves from zero (not from the
 // previous solve's potentials), so that a solve depends only on its inputs.
@@ -1688,7 +1695,8 @@ int lbm_instance_create(lbm_ctx* ctx, lbm_mesh mesh, int32_t batch, int32_t prec
     I->B = batch;
     I->precision = precision;
     I->tsize = precision == LBM_FP64 ? 8 : 4;
-    const size_t vb = vec_bytes(*M, batch, precision == LBM_FP64 ? 8 : 4), pe = part_elems(ctx, batch);
+    const bool use_tc = precision == LBM_MIXED_TC && batch >= 2 && batch <= 64;
+    const size_t vb = vec_bytes(*M, batch, I->tsize, use_tc), pe = part_elems(ctx, batch);
     const size_t N = M->N;
 #define CKI(call)                                                                                   \
     do {                                                                                            \
@@ -1709,7 +1717,7 @@ int lbm_instance_create(lbm_ctx* ctx, lbm_mesh mesh, int32_t batch, int32_t prec
     CKI(cudaMemsetAsync(I->st, 0, sizeof(InstState) * batch, ctx->stream));
 #undef CKI
     I->bytes = vb + pe * 8 + (sizeof(InstState) + sizeof(InstConst)) * batch + 40 * batch * N;
-    if (precision == LBM_MIXED_TC && batch >= 2 && batch <= 64) {
+    if (use_tc) {
         // tensor-core BEM products: padded B / B^T per mesh, split/partial scratch per instance
         const size_t pad = sizeof(float) * (size_t)M->nb * tc_ld(M->nb);
         if (!M->tcA) {

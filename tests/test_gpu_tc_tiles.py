@@ -30,3 +30,22 @@ def test_tiles(n, B):
     assert np.abs(ht - ha).max() <= 2e-5 * np.abs(ha).max()
     for x, y in zip(ra, rt):
         assert abs(x["energy"][4] - y["energy"][4]) <= 2e-5 * (abs(x["energy"][4]) + 1e-20)
+
+
+def test_no_room_for_sums_that_no_product_takes():
+    """A batch whose boundary products run on the tensor cores holds their scratch and not
+    the partial sums of the other batched product as well (8 splits x nb x 2B doubles here,
+    44 MB; two words of each vector and 8 splits x nb x B x 2 FP32 sums, 28 MB)."""
+    from paper_1309_5796_gb300 import build
+    build.build()
+    torch = pytest.importorskip("torch")
+    with lbm.Context(0) as ctx:
+        mesh = ctx.mesh_cube(2e-9, 30)
+        used = {}
+        for prec in (lbm.LBM_MIXED_TC, lbm.LBM_MIXED, lbm.LBM_MIXED_TC):   # the first brings the mesh's padded copies
+            f0 = torch.cuda.mem_get_info()[0]
+            inst = ctx.instance_create(mesh, 64, prec)
+            used[prec] = f0 - torch.cuda.mem_get_info()[0]
+            inst.destroy()
+        ctx.mesh_destroy(mesh)
+    assert 0 < used[lbm.LBM_MIXED_TC] <= used[lbm.LBM_MIXED] - (10 << 20)
