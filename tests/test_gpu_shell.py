@@ -283,3 +283,34 @@ def test_shell_serving(ctx):
         scale = max(abs(ref.E), p.Kd * (r["n"] * p.cell) ** 3)
         assert res["status"] == lbm.LBM_OK, r
         assert abs(res["energy"][4] - ref.E) / scale < 1e-6, (r["n"], res["energy"][4], ref.E)
+
+
+# plain FP64 batches on either side of the sizes from which rows are dealt round the blocks
+# (17^3 nodes times 61 and 63, 162 and 164; the first pair one instance a thread, the second
+# two), FP64 iterated in FP32 and FP32 of every width, on a grid with a short last block
+@pytest.mark.parametrize("B,prec,mixed", [
+    (61, lbm.LBM_FP64, 0), (63, lbm.LBM_FP64, 0), (162, lbm.LBM_FP64, 0), (164, lbm.LBM_FP64, 0),
+    (163, lbm.LBM_FP64, 1), (162, lbm.LBM_FP64, 1), (1, lbm.LBM_MIXED, 0), (63, lbm.LBM_MIXED, 0),
+    (162, lbm.LBM_MIXED, 0), (164, lbm.LBM_MIXED, 0)])
+def test_shell_batches_against_the_oracle(ctx, B, prec, mixed):
+    """Fields of a few instances of wide batches, the oracle's to 1e-10 (FP64 to a 1e-13
+    residual), 1e-7 (iterated in FP32 to 1e-10) and 2e-5 (FP32), as the bars above."""
+    n, a, s = 6, 1, 4
+    N = (n + 1) ** 3
+    axis = tilted_axis(5.0, 0.7)
+    m0 = np.stack([m_random_sphere(N, 500 + b) for b in range(B)])
+    mesh, info = _shell_mesh(ctx, n, a, s)
+    assert info["grid_nodes"] == 17 ** 3
+    inst = ctx.instance_create(mesh, B, prec)
+    inst.set_material(JS_T, A_JM, K1_JM3, axis)
+    inst.set_field(np.array([0.1, 0.2, -1.0]))
+    inst.set_m(m0)
+    opts = lbm.default_opts(prec, cg_mixed_iter=1, cg_tol=1e-10) if mixed else lbm.default_opts(prec)
+    _, h, _ = inst.evaluate(opts, want_u=False)
+    inst.destroy()
+    ctx.mesh_destroy(mesh)
+    rtol = 2e-5 if prec else (1e-7 if mixed else 1e-10)
+    p = ShellProblem(n, JS_T, A_JM, K1_JM3, axis, a, s)
+    for b in sorted({0, 1 % B, B // 2, B - 1}):
+        ev = p.evaluate(m0[b], np.array([0.1, 0.2, -1.0]))
+        assert np.abs(h[b] - ev.h).max() <= rtol * np.abs(ev.h).max(), b
