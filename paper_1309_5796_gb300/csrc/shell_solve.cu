@@ -36,6 +36,7 @@ struct ShellArgs {
     double* x;                    // [Ng][B] FP64 grid potential
     W *r, *z, *z2, *p, *q, *d;   // [Ng][B] work vectors (d: this solve's correction of x)
     double th, de;                // centre and half-width of the polynomial's interval
+    int deg;                      // products of a CG iteration
     int deal;                     // rows dealt round all blocks instead of a run for each
     double tol2;
     int max_iter;
@@ -130,8 +131,36 @@ __device__ __forceinline__ void kuhn_apply(const C (&c)[16], const V* v, ptrdiff
     }
 }
 
-constexpr int SH_DEG = 16;            // products of a CG iteration
-constexpr double SH_RATIO = 400.0;    // of the polynomial's interval
+// Products of a CG iteration and the ratio of the polynomial's interval.  A higher degree
+// saves reductions and their barriers; but an iteration is a whole number of polynomials,
+// and a small grid needs few: 11^3 nodes 97 plain CG iterations in FP64, twenty of degree
+// 16.  ms an evaluation at degree, ratio (first plain CG, last what every grid had):
+//   6^3, 64 instances in FP64    0.95 | 3, 8: 0.84   4, 15: 0.91   8, 60: 1.28
+//   7^3, 64 in FP64              1.13 | 3, 8: 1.06   4, 15: 1.04   6, 30: 1.13   8, 60: 1.35
+//   9^3, 64 in FP64                   | 4, 15: 1.40   6, 30: 1.38   8, 60: 1.51   16, 400: 3.06
+//   11^3, 256 in FP64            3.71 | 6, 30: 3.06   8, 60: 3.31   12, 220: 4.60   16, 400: 6.05
+//   11^3, 64 in FP32             1.03 | 6, 30: 0.72   8, 60: 0.72   12, 220: 0.82   16, 400: 1.03
+//   17^3, 64 in FP64                  | 8, 60: 4.21   8, 100: 4.08   12, 220: 4.49   16, 400: 5.24
+//   21^3, 128 in FP64            13.3 | 8, 100: 11.7   12, 220: 11.7   16, 400: 13.4
+//   27^3, 16 in FP32                  | 8, 100: 1.62   12, 220: 1.48   16, 400: 1.39
+//   39^3, 32 in FP64                  | 8, 100: 39.1   12, 220: 38.0   16, 400: 37.1
+// The lines lie between these sizes.
+void sh_degree(int rows, int& deg, double& ratio) {
+    struct Step {
+        int rows, deg;
+        double ratio;
+    };
+    static constexpr Step steps[] = {{280, 3, 8.0},     {600, 4, 15.0},     {1000, 6, 30.0},
+                                     {2500, 8, 60.0},   {6500, 8, 100.0},   {14000, 12, 220.0}};
+    deg = 16;
+    ratio = 400.0;
+    for (const Step& t : steps)
+        if (rows <= t.rows) {
+            deg = t.deg;
+            ratio = t.ratio;
+            return;
+        }
+}
 // rows times instances from which on FP64 batches deal their rows round all blocks: odd
 // batches, one instance a thread, and even ones, two
 constexpr double SH_DEAL1 = 3e5, SH_DEAL2 = 8e5;
@@ -149,15 +178,15 @@ constexpr double SH_DEAL1 = 3e5, SH_DEAL2 = 8e5;
 //     residual test (restarted CG, as the magnet's mixed-iteration solves).
 // Per CG iteration:
 //   B: alpha = rho / p.q, d += alpha p, r -= alpha q, z = D^-1 r / theta, r.r
-//   C: SH_DEG - 1 steps z'' = z' + c1 (z' - z) + c2 D^-1 (r - K z'), z'' in z's place (no
+//   C: deg - 1 steps z'' = z' + c1 (z' - z) + c2 D^-1 (r - K z'), z'' in z's place (no
 //      vector for the steps themselves); r.z with the last
 //   A: w = K z, p = z + beta p, q = w + beta q (= K p), p.q
-// The polynomial is Chebyshev's on [b / 400, b], b a bound of the eigenvalues of
-// D^-1 K: on the 54^3-cell grid 29 iterations of 16 products where Jacobi-CG takes 358 of
-// one, and a product with its step moves 4 vector words and one barrier where a CG
-// iteration moves 12 and four.  (Degree 8 on [b / 60, b]: 61 iterations, 25 % more time;
-// 20 on [b / 800, b] gives 3 % more on that grid and takes 14 % longer on small FP64 ones.
-// Multigrid and fast diagonalisation stall on the shell's growing tangential stiffness.)
+// The polynomial is Chebyshev's on [b / ratio, b], b a bound of the eigenvalues of
+// D^-1 K, its degree by size (sh_degree): on the 54^3-cell grid 29 iterations of 16
+// products where Jacobi-CG takes 358 of one, and a product with its step moves 4 vector
+// words and one barrier where a CG iteration moves 12 and four.  (20 on [b / 800, b] gives
+// 3 % more on that grid.  Multigrid and fast diagonalisation stall on the shell's growing
+// tangential stiffness.)
 // Measured on that grid: 32 instances 10.3 ms a solve, one 2.4; at first 24.1 and 5.7.
 // Every block has one run of consecutive rows, so that the L1 serves a product's
 // neighbours along x and y and about three of its fifteen reads go to L2 (with
@@ -303,8 +332,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
             // ---- C: outer-face rows (kind 0) keep zero ----
             W v1[1][VEC];
             W rho_c = de / th;
-            for (int st = 1; st < SH_DEG; ++st) {
-                const bool last = st + 1 == SH_DEG;
+            for (int st = 1; st < A.deg; ++st) {
+                const bool last = st + 1 == A.deg;
                 const W rn = W(1) / (W(2) * th / de - rho_c), c1 = rn * rho_c, c2 = W(2) * rn / de, c3 = W(1) + c1;
                 rho_c = rn;
 #pragma unroll
@@ -488,8 +517,10 @@ int launch_shell(const Launch& L, const ShellDev& S, const double* bvec, double*
     a.q = w + 3 * Gv;
     a.d = w + 4 * Gv;
     a.z2 = w + 5 * Gv;
-    a.th = 0.5 * (1.0 + 1.0 / SH_RATIO) * S.jac_bound;
-    a.de = 0.5 * (1.0 - 1.0 / SH_RATIO) * S.jac_bound;
+    double ratio;
+    sh_degree(S.Ng, a.deg, ratio);
+    a.th = 0.5 * (1.0 + 1.0 / ratio) * S.jac_bound;
+    a.de = 0.5 * (1.0 - 1.0 / ratio) * S.jac_bound;
     a.deal = sizeof(W) == 8 && (double)S.Ng * B >= (VEC == 1 && B > 1 ? SH_DEAL1 : SH_DEAL2);
     a.tol2 = tol * tol;
     a.max_iter = max_iter;

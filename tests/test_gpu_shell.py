@@ -314,3 +314,22 @@ def test_shell_batches_against_the_oracle(ctx, B, prec, mixed):
     for b in sorted({0, 1 % B, B // 2, B - 1}):
         ev = p.evaluate(m0[b], np.array([0.1, 0.2, -1.0]))
         assert np.abs(h[b] - ev.h).max() <= rtol * np.abs(ev.h).max(), b
+
+
+# grids of 6^3 to 25^3 nodes: sizes on either side of those at which the polynomial changes
+@pytest.mark.parametrize("prec,rtol", [(lbm.LBM_FP64, 1e-10), (lbm.LBM_MIXED, 2e-5)])
+@pytest.mark.parametrize("n,a,s", [
+    (1, 1, 1), (2, 1, 1), (2, 1, 2), (3, 1, 2), (2, 1, 4), (3, 1, 4), (5, 2, 4), (6, 2, 4), (9, 2, 5), (8, 3, 5)])
+def test_shell_polynomial_degrees(ctx, n, a, s, prec, rtol):
+    axis, field = tilted_axis(5.0, 0.7), np.array([0.1, 0.2, -1.0])
+    m0 = m_random_sphere((n + 1) ** 3, 700 + n)
+    mesh, _ = _shell_mesh(ctx, n, a, s)
+    inst = ctx.instance_create(mesh, 1, prec)
+    inst.set_material(JS_T, A_JM, K1_JM3, axis)
+    inst.set_field(field)
+    inst.set_m(m0)
+    _, h, _ = inst.evaluate(lbm.default_opts(prec), want_u=False)
+    inst.destroy()
+    ctx.mesh_destroy(mesh)
+    ev = ShellProblem(n, JS_T, A_JM, K1_JM3, axis, a, s).evaluate(m0, field)
+    assert np.abs(h[0] - ev.h).max() <= rtol * np.abs(ev.h).max()
