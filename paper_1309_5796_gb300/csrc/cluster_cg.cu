@@ -40,6 +40,15 @@ namespace lbm {
 namespace {
 
 constexpr size_t CC_SMEM_MAX = 225 * 1024;
+// A CTA whose matrix entries are in global memory: the products read them a row a thread,
+// so a line has to stay in the L1 (what the shared memory leaves of 256 KB) until its next
+// entries are used.  Less shared memory, and vectors that go to global memory instead, are
+// faster then (ms an evaluation with all of it -> with this much): FP32, 4 / 8 instances on
+// 59 319 nodes 23.1 -> 11.5 / 32.6 -> 15.7, one on 117 649 64 -> 25, 5 iterated in FP32 on
+// 74 088 128 -> 43.  In FP64, where the units bind too, 4 on 46 656 39.4 -> 35.4 and one on
+// 59 319 41.8 -> 36.7 at 200 KB; less than that takes vectors of small shapes (12 on 24 389
+// 30 -> 43 ms at 130 KB).
+template <typename W> constexpr size_t CC_SMEM_BARE = (sizeof(W) == 8 ? 200 : 130) * 1024;
 constexpr int CC_MAX_CL = 16;
 constexpr int CC_NQ = 4;            // most quantities of one reduction
 constexpr int CC_VECS = 7;          // z, z', dd, r, p, q, d (dd from z and z' instead: 2 to 4 % slower)
@@ -113,6 +122,7 @@ __device__ __forceinline__ void cc_put(X* p, const X (&d)[VEC]) {
 struct CcGeo {
     int rows, rpc, cl;                 // rows of a system, rows per CTA, CTAs per cluster
     int nvec;                          // vectors in shared memory: z, z', then dd, r, p, q, d
+    int fit;                           // as many as would fit it
     int deg;                           // products of an iteration
     double ratio;                      // the polynomial's interval: [b / ratio, b]
     double th, de;                     // its centre and half-width
@@ -623,14 +633,14 @@ struct CcChoice {
 };
 
 // Shared memory of a shape; false when not even z fits.
-bool cc_fit(CcGeo& g, int vec, size_t word, int entries) {
+bool cc_fit(CcGeo& g, int vec, size_t word, int entries, size_t bare) {
     auto up = [](size_t b) { return (b + 15) & ~(size_t)15; };
     const size_t scr = up(std::max(word * 32 * CC_NQ * vec, sizeof(double) * 32 * vec));
     const size_t slot = up(sizeof(double) * 2 * CC_NQ * vec * CC_MAX_CL);
     const size_t col = up(sizeof(double) * (CC_NQ + 6) * vec + sizeof(int) * 3 * vec + 4 * CC_MAX_CL);
     const size_t one = word * vec * (size_t)g.rpc, di = up(word * (size_t)g.rpc), fixed = scr + slot + col + di;
     if (up(2 * one) + fixed > CC_SMEM_MAX) return false;
-    g.nvec = (int)std::min<size_t>(CC_VECS, (CC_SMEM_MAX - fixed - 16) / one);
+    g.nvec = g.fit = (int)std::min<size_t>(CC_VECS, (CC_SMEM_MAX - fixed - 16) / one);
     size_t o = up(one * g.nvec);
     g.o_dinv = (unsigned)o;
     o += di;
@@ -644,6 +654,13 @@ bool cc_fit(CcGeo& g, int vec, size_t word, int entries) {
             g.o_ptr = (unsigned)o;
             o += pt;
         }
+    }
+    if (!g.ent) {
+        while (g.nvec > 3 && up(one * g.nvec) + fixed + 16 > bare) --g.nvec;
+        o = up(one * g.nvec);
+        g.o_dinv = (unsigned)o;
+        o += di;
+        g.o_ent = g.o_ptr = (unsigned)o;
     }
     g.o_scr = (unsigned)o;
     o += scr;
@@ -705,7 +722,7 @@ void cc_try(const Launch& L, int rows, int cols, const int* emax, CcChoice& best
         g.rpc = (rows + cl - 1) / cl;
         if (g.rpc < 32 && cl > 1) continue;
         g.cl = (rows + g.rpc - 1) / g.rpc;   // every CTA has rows
-        if (!cc_fit(g, VEC, sizeof(W), emax[cl])) continue;
+        if (!cc_fit(g, VEC, sizeof(W), emax[cl], CC_SMEM_BARE<W>)) continue;
         const int most = sizeof(W) == 8 ? 512 : 1024, per = (g.rpc + most - 1) / most;
         const int threads = std::min(most, std::max(128, ((g.rpc + per - 1) / per + 31) & ~31));
         if (g.nvec < 3) continue;   // dd has no global room
@@ -714,10 +731,10 @@ void cc_try(const Launch& L, int rows, int cols, const int* emax, CcChoice& best
         if (r < 1) continue;
         const int waves = (cols / VEC + r - 1) / r;
         // an iteration's time in rows of a thread block: the rows' vectors (twice as
-        // dear in global memory), their matrix entries, and barriers and latencies
-        // worth about 3000 rows
+        // dear in global memory, unless they went there for the L1's sake), their matrix
+        // entries, and barriers and latencies worth about 3000 rows
         const double mat = g.ent ? 2.0 : 6.0;
-        const double cost = waves * (g.rpc * (VEC * (1.0 + 0.25 * (CC_VECS - g.nvec)) * (sizeof(W) == 8 ? 24.0 : 1.0) + mat) + 3000.0);
+        const double cost = waves * (g.rpc * (VEC * (1.0 + 0.25 * (CC_VECS - g.fit)) * (sizeof(W) == 8 ? 24.0 : 1.0) + mat) + 3000.0);
         if (best.vec == 0 || cost < best_cost) {
             best_cost = cost;
             best.g = g;

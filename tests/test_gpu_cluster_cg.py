@@ -79,3 +79,13 @@ def test_transformed_grid(ctx, n, a, s, B, prec):
     ctx.mesh_shell(mesh, a, s)
     _compare(ctx, mesh, (n + 1) ** 3, B, prec)
     ctx.mesh_destroy(mesh)
+
+
+# entries in global memory, where some of the vectors follow them: one, two and four
+# systems a cluster, all seven vectors to three in shared memory
+@pytest.mark.parametrize("n,B,prec", [(30, 3, 0), (34, 5, 1), (34, 8, 1), (38, 4, 1), (38, 12, 1), (38, 5, 0)])
+def test_meshes_beyond_the_shared_memory(ctx, n, B, prec):
+    xyz, tets = ball_mesh(n)
+    mesh = ctx.mesh_upload(xyz, tets)
+    _compare(ctx, mesh, xyz.shape[0], B, prec)
+    ctx.mesh_destroy(mesh)
