@@ -629,7 +629,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
 
 struct CcChoice {
     CcGeo g;
-    int vec = 0, threads = 0;
+    int vec = 0, threads = 0, waves = 0;
 };
 
 // Shared memory of a shape; false when not even z fits.
@@ -740,8 +740,23 @@ void cc_try(const Launch& L, int rows, int cols, const int* emax, CcChoice& best
             best.g = g;
             best.vec = VEC;
             best.threads = threads;
+            best.waves = waves;
         }
     }
+}
+
+// Where the Jacobi-CG kernels, which spread a product over the whole chip, are faster: many
+// systems in plain FP64, whose clusters run in waves (the polynomial takes about a quarter
+// more products, and FP64 units are what bounds both), and the largest meshes (a system has
+// sixteen SMs and its entries come from global memory).  ms an evaluation here / there, plain
+// FP64: 64 instances on 3 375 nodes 17.4 / 12.6, 128 33.6 / 19.7, 96 on 1 331 8.6 / 7.5, 32 on
+// 15 625 49.8 / 44.5 (three to seven waves); one or two waves 1.0 to 2.3 times faster here
+// over 60 such shapes of 343 to 42 875 nodes; one on 74 088 46.7 / 37.5, on 59 319 36.7 / 34.5.
+// Iterated in FP32: one on 74 088 26.5 / 25.8, on 91 125 33.5 / 31.8, five 61 / 44; FP32: one on
+// 91 125 17.3 / 16.6, eight 54 / 41, four on 117 649 57 / 31, one on 166 375 45 / 23.
+bool cc_slower(int rows, int cols, int waves, bool fp32, bool fp64_vectors) {
+    if (fp64_vectors) return rows > 65000 || waves >= 5 || (waves >= 3 && (cols >= 80 || rows >= 14000));
+    return rows > (fp32 && cols < 16 ? 100000 : 80000);
 }
 
 template <typename T, typename W>
@@ -751,6 +766,7 @@ CcChoice cc_choose(const Launch& L, int rows, int cols, const int* emax) {
     if constexpr (sizeof(W) == 4) cc_try<T, W, 4>(L, rows, cols, emax, c, cost);
     cc_try<T, W, 2>(L, rows, cols, emax, c, cost);
     cc_try<T, W, 1>(L, rows, cols, emax, c, cost);
+    if (cc_slower(rows, cols, c.waves, sizeof(T) == 4, sizeof(W) == 8)) c.vec = 0;
     return c;
 }
 

@@ -89,3 +89,16 @@ def test_meshes_beyond_the_shared_memory(ctx, n, B, prec):
     mesh = ctx.mesh_upload(xyz, tets)
     _compare(ctx, mesh, xyz.shape[0], B, prec)
     ctx.mesh_destroy(mesh)
+
+
+@pytest.mark.parametrize("n,B,same", [(10, 128, True), (10, 24, False), (14, 80, True), (40, 1, True)])
+def test_plain_fp64_in_many_waves_goes_to_the_grid(ctx, n, B, same):
+    """Plain FP64 batches whose clusters would run in many waves, and the largest meshes,
+    take the grid-wide kernel (its bits); smaller ones do not."""
+    xyz, tets = ball_mesh(n)
+    mesh = ctx.mesh_upload(xyz, tets)
+    _, _, u = _run(ctx, mesh, xyz.shape[0], B, 0)
+    _, _, g = _run(ctx, mesh, xyz.shape[0], B, 0, pcg_kernel=1)
+    ctx.mesh_destroy(mesh)
+    assert np.array_equal(u, g) == same
+    assert max(_off(u, g)) <= 1e-9
