@@ -54,13 +54,19 @@ constexpr int CC_NQ = 4;            // most quantities of one reduction
 constexpr int CC_VECS = 7;          // z, z', dd, r, p, q, d (dd from z and z' instead: 2 to 4 % slower)
 
 // Products of an iteration and the ratio of the polynomial's interval.  A higher degree
-// saves reductions, but the last iteration's surplus weighs more where few are needed:
-// both stages of one instance in FP32 on 19 683 nodes 1.83 ms at degree 8 on [b / 60, b],
-// 1.71 at 16 on [b / 240, b]; 16 in FP64 on 3 375 nodes 4.18 at 4 on [b / 60, b], 4.02 at
-// 6 on [b / 120, b], 4.54 at 8 on [b / 240, b]; one in FP64 on 729 nodes 1.04, 1.14, 1.44.
+// saves reductions, but the last iteration's surplus weighs more where few are needed.
+// ms an evaluation at 4 on [b / 60, b], 6 on [b / 120, b], 8, 12 and 16 on [b / 240, b]:
+// FP64, one instance on 27 nodes 0.59, 0.73 (2 on [b / 15, b]: 0.38), on 729 1.12, 1.23, 1.48,
+// 1.42, 1.36, on 2 197 1.65, 1.61, 1.86, 1.78, 1.67, on 4 913 2.89, 2.64, 2.78, 2.67, 2.58, on
+// 9 261 4.76, 4.37, 4.35, 4.17, 4.21, on 19 683 11.3, 10.7, 10.3, 10.5, 10.6, 32 on 3 375 9.2,
+// 9.8, 12.0, 11.4, 11.5; FP32, one on 1 331 0.50, 0.45, 0.48, 0.47, 0.43, on 4 913 0.83, 0.74,
+// 0.73, 0.70, 0.69, on 9 261 1.27, 1.15, 1.07, 1.05, 1.08, on 19 683 2.19, 2.03, 1.94, 1.94,
+// 1.92, 32 on 2 197 1.15, 1.13, 1.21, 1.19, 1.22; FP64 iterated in FP32 as FP32.  Within 8 %
+// of the best of these in FP64, within 12 % for one FP32 instance between the lines (up to
+// 20 % on 1 331 to 2 197 nodes) and 3 % for thirty-two.
 void cc_degree(int rows, int& deg, double& ratio) {
-    deg = rows >= 8192 ? 16 : rows >= 3000 ? 6 : 4;
-    ratio = rows >= 8192 ? 240.0 : rows >= 3000 ? 120.0 : 60.0;
+    deg = rows >= 8192 ? 16 : rows >= 3000 ? 6 : rows >= 90 ? 4 : 2;
+    ratio = rows >= 8192 ? 240.0 : rows >= 3000 ? 120.0 : rows >= 90 ? 60.0 : 15.0;
 }
 
 extern __shared__ __align__(16) unsigned char cc_sm[];
