@@ -125,6 +125,58 @@ __device__ __forceinline__ void st4(double* p, const double (&v)[4]) {
 __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
 
+// Sums that have to be better than FP32's: FP64 where the values are, or, of FP32 values,
+// pairs of FP32 words with every rounding kept (Knuth's TwoSum, the product's error by
+// FMA), 48 bits at a sixth of the time of GB300's FP64 units.
+struct Pair {
+    float s = 0.f, e = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+        e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
+        s = t;
+    }
+    __device__ __forceinline__ void fma(float a, float b) {
+        const float p = __fmul_rn(a, b);
+        add(p);
+        e = __fadd_rn(e, __fmaf_rn(a, b, -p));
+    }
+};
+struct Sum64 {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double x) { s += x; }
+    __device__ __forceinline__ void fma(double a, double b) { s = __fma_rn(a, b, s); }
+};
+template <typename T> struct SumOf { using type = Sum64; };
+template <> struct SumOf<float> { using type = Pair; };
+__device__ __forceinline__ float shfl_x(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ double shfl_x(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ Pair shfl_x(Pair v, int o) {
+    v.s = shfl_x(v.s, o);
+    v.e = shfl_x(v.e, o);
+    return v;
+}
+__device__ __forceinline__ Sum64 shfl_x(Sum64 v, int o) {
+    v.s = shfl_x(v.s, o);
+    return v;
+}
+__device__ __forceinline__ float plus(float a, float b) { return a + b; }
+__device__ __forceinline__ double plus(double a, double b) { return a + b; }
+__device__ __forceinline__ Sum64 plus(Sum64 a, Sum64 b) {
+    a.s += b.s;
+    return a;
+}
+__device__ __forceinline__ Pair plus(Pair a, Pair b) {   // the same bits either way round
+    const float e = __fadd_rn(a.e, b.e);
+    a.e = 0.f;
+    a.add(b.s);
+    a.e = __fadd_rn(a.e, e);
+    return a;
+}
+__device__ __forceinline__ double total(float v) { return (double)v; }
+__device__ __forceinline__ double total(double v) { return v; }
+__device__ __forceinline__ double total(Sum64 v) { return v.s; }
+__device__ __forceinline__ double total(Pair v) { return (double)v.s + (double)v.e; }
+
 // VEC consecutive columns of one row; CG: through L2 (values other CTAs write)
 template <int VEC, bool CG, typename X>
 __device__ __forceinline__ void ldc(X (&d)[VEC], const X* p) {
@@ -341,8 +393,9 @@ __device__ __forceinline__ void edge_node(int e, int n, int& i, int& j, int& k) 
 }
 
 // T: type of the potential x and of the residual f - K x; W: type of the
-// refinement (transforms, r, the sum of the steps) and of the dot products inside
-// a chunk (sums over chunks, planes and CTAs in FP64).  T = W: d starts as x and
+// refinement (transforms, r, the sum of the steps) and of a step's dot products inside
+// a chunk (sums over chunks, planes and CTAs in FP64; those of the first residual, of its
+// reference and of the gauge in FP64 or pairs (SumOf) from the node on).  T = W: d starts as x and
 // collects the steps; the first residual's stencil runs on a copy of x in the
 // planes' place, so x is read once and written once (a system's values lie 2B words
 // apart in it).  T = double, W = float (solves iterated in FP32): cycles of the FP64
@@ -354,6 +407,7 @@ __device__ __forceinline__ void edge_node(int e, int n, int& i, int& j, int& k) 
 template <typename T, typename W, int VEC, bool TS>
 __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(const __grid_constant__ FsArgs<T, W> A) {
     constexpr bool MP = sizeof(T) != sizeof(W), ND = sizeof(W) == 8;
+    using Acc = typename SumOf<T>::type;
     const FsGeo& g = A.g;
     W* buf = reinterpret_cast<W*>(fs_sm);                       // TS: own planes [ppc][VEC][ss]; else a round of planes
     W* zb = reinterpret_cast<W*>(fs_sm + g.o_z);                // P2: [s2][VEC * pr] (TS = false: in buf's room)
@@ -476,17 +530,34 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
             par ^= 1;
             __syncthreads();
         };
-        // chunk sums of the quantities a0, a0 + 1, ... in v into part (whole warp)
+        // chunk sums of the quantities a0, a0 + 1, ... in v into part (whole warp): halves of
+        // the values change sides at every step while there are several, so that each step
+        // adds half as many; the sum of a value is the same butterfly's in any case
         auto put = [&](auto& v, int a0, int pl, int ch) {
-            constexpr int NQ = sizeof(v) / sizeof(v[0]);
+            constexpr int NV = sizeof(v) / sizeof(v[0][0]);
+            using X = typename std::remove_reference<decltype(v[0][0])>::type;
+            X f[NV];
 #pragma unroll
-            for (int a = 0; a < NQ; ++a)
+            for (int i = 0; i < NV; ++i) f[i] = v[i / VEC][i % VEC];
+            int at = 0;
 #pragma unroll
-                for (int k = 0; k < VEC; ++k) {
+            for (int o = 16, n2 = NV; o > 0; o >>= 1) {
+                if (n2 % 2 == 0) {
+                    n2 >>= 1;
+                    const bool up = lane & o;
+                    if (up) at += n2;
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) v[a][k] += __shfl_xor_sync(0xffffffffu, v[a][k], o);
-                    if (lane == 0) part[((pl * g.nch + ch) * FS_NQ + a0 + a) * VEC + k] = (double)v[a][k];
+                    for (int i = 0; i < n2; ++i) {
+                        const X send = up ? f[i] : f[i + n2], keep = up ? f[i + n2] : f[i];
+                        f[i] = plus(keep, shfl_x(send, o));
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < n2; ++i) f[i] = plus(f[i], shfl_x(f[i], o));
                 }
+            }
+            static_assert((NV & (NV - 1)) == 0 && NV <= 16, "one value a lane is left");
+            if ((lane & (32 / NV - 1)) == 0) part[((pl * g.nch + ch) * FS_NQ + a0) * VEC + at] = total(f[0]);
         };
         // f(pl, ch, q) for every chunk ch of the CTA's planes [pa, pb), a warp per chunk, a
         // lane per quadruple of mirrored nodes: u = 0 (y, x), 1 (y, n-x), 2 (n-y, x),
@@ -705,79 +776,75 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
             if (!nodewise) quads(0, np, [&](int pl, int ch, const Quad& q) {
                 const int kk = k0 + pl;
                 const bool surf = q.x == 0 || q.y == 0 || kk == 0 || kk == n;
-                W v[4][VEC];
+                Acc v[4][VEC];
                 double vx[1][VEC];
 #pragma unroll
-                for (int k = 0; k < VEC; ++k) {
-                    v[0][k] = v[1][k] = v[2][k] = v[3][k] = W(0);
-                    vx[0][k] = 0.0;
-                }
+                for (int k = 0; k < VEC; ++k) vx[0][k] = 0.0;
                 const bool froz = !neu && surf;
-                // the right-hand side at node u (none in the stage-2 forward system)
-                auto rhs = [&](int u, T (&f)[VEC]) {
+                // node: r = f - kx stored; sums of r.r and of the square of the reference f - ks (f:
+                // none in the stage-2 forward system), of Neumann systems also of r and f
+                auto node = [&](int l, const T (&kx)[VEC], const T (&ks)[VEC], bool differs) {
+                    double f[VEC];
+                    const bool rhs = !froz && (neu || !mode);
 #pragma unroll
-                    for (int k = 0; k < VEC; ++k) f[k] = T(0);
-                    if (froz || (mode && !neu)) return;
-                    double fb[VEC];
-                    ldc<VEC, false>(fb, bv + (ptrdiff_t)(pl * pn + q.row[u]) * B);
-                    if (mode && surf) {   // the BEM term of the adjoint Neumann system
-                        const int bp = (int)((unsigned)nodes[pl * pn + q.row[u]] >> 16);
+                    for (int k = 0; k < VEC; ++k) f[k] = 0.0;
+                    if (rhs) {
+                        ldc<VEC, false>(f, bv + (ptrdiff_t)l * B);
+                        if (mode && surf) {   // the BEM term of the adjoint Neumann system
+                            const int bp = (int)((unsigned)nodes[l] >> 16);
 #pragma unroll
-                        for (int k = 0; k < VEC; ++k) fb[k] += (double)P.V.ub_out[(size_t)(bp - 1) * C + c0 + k];
+                            for (int k = 0; k < VEC; ++k) f[k] += (double)P.V.ub_out[(size_t)(bp - 1) * C + c0 + k];
+                        }
                     }
-#pragma unroll
-                    for (int k = 0; k < VEC; ++k) f[k] = act[k] ? T(fb[k]) : T(0);
-                };
-                auto done = [&](int u, const T (&f)[VEC], const T (&kx)[VEC], const T (&ks)[VEC]) {
                     W rv[VEC];
 #pragma unroll
                     for (int k = 0; k < VEC; ++k) {
-                        rv[k] = W(f[k] - kx[k]);
-                        const W ref = W(f[k] - ks[k]);
-                        v[0][k] = fma_(rv[k], rv[k], v[0][k]);
-                        v[1][k] += rv[k];
-                        v[2][k] = fma_(ref, ref, v[2][k]);
-                        v[3][k] += ref;
+                        const T ft = act[k] ? T(f[k]) : T(0), rt = ft - kx[k];
+                        rv[k] = W(rt);
+                        if (froz) continue;
+                        v[0][k].fma(rt, rt);
+                        if (neu) v[1][k].add(rt);
+                        if (!rhs && !differs) continue;
+                        const T ref = ft - ks[k];
+                        v[2][k].fma(ref, ref);
+                        if (neu) v[3][k].add(ref);
                     }
-                    stc<VEC>(r + (ptrdiff_t)(pl * pn + q.row[u]) * VEC, rv);
+                    stc<VEC>(r + (ptrdiff_t)l * VEC, rv);
                 };
                 if constexpr (!MP) {
-                    T kx[4][VEC], ks[4][VEC];
+                    T kx[4][VEC];
 #pragma unroll
                     for (int u = 0; u < 4; ++u)
 #pragma unroll
-                        for (int k = 0; k < VEC; ++k) kx[u][k] = ks[u][k] = T(0);
-                    if (!froz) {
-                        const W *s = own(kk, pl), *sm = below(kk, pl), *sp = above(kk, pl);
+                        for (int k = 0; k < VEC; ++k) kx[u][k] = T(0);
+                    const W *s = own(kk, pl), *sm = below(kk, pl), *sp = above(kk, pl);
+                    if (!froz)
 #pragma unroll
-                        for (int k = 0; k < VEC; ++k) {
+                        for (int k = 0; k < VEC; ++k)
                             stencil(q, kk, s + k * ss, sm + k * ss, sp + k * ss, [&](int u, W, W a) { kx[u][k] = a; });
-                            if (!neu && mode) {   // neighbours on the surface
-                                const bool nx = q.x == 1, nx2 = q.x + 1 == n, ny = q.y == 1, ny2 = q.y + 1 == n;
-                                if (!(nx || nx2 || ny || ny2 || kk == 1 || kk + 1 == n)) continue;
-                                const int xi = q.x + 1 < h ? 1 : 1 + gap, xim = n - q.x - 1 >= h ? -1 : -1 - gap;
-#pragma unroll
-                                for (int u = 0; u < 4; ++u) {
-                                    if (!q.has[u]) continue;
-                                    const W* z = s + k * ss + q.at[u];
-                                    W t = W(0);
-                                    if (nx) t += z[(u & 1) ? 1 : -1];
-                                    if (nx2) t += z[(u & 1) ? xim : xi];
-                                    if (ny) t += z[(u & 2) ? ldx : -ldx];
-                                    if (ny2) t += z[(u & 2) ? -ldx : ldx];
-                                    if (kk == 1) t += sm[k * ss + q.at[u]];
-                                    if (kk + 1 == n) t += sp[k * ss + q.at[u]];
-                                    ks[u][k] = W(-6) * t;
-                                }
-                            }
-                        }
-                    }
+                    // neighbours on the surface (K_IS x_S of the stage-2 forward system)
+                    const bool nx = q.x == 1, nx2 = q.x + 1 == n, ny = q.y == 1, ny2 = q.y + 1 == n;
+                    const bool differs = !froz && !neu && mode && (nx || nx2 || ny || ny2 || kk == 1 || kk + 1 == n);
+                    const int xi = q.x + 1 < h ? 1 : 1 + gap, xim = n - q.x - 1 >= h ? -1 : -1 - gap;
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         if (!q.has[u]) continue;
-                        T f[VEC];
-                        rhs(u, f);
-                        done(u, f, kx[u], ks[u]);
+                        T ks[VEC];
+#pragma unroll
+                        for (int k = 0; k < VEC; ++k) {
+                            ks[k] = T(0);
+                            if (!differs) continue;
+                            const W* z = s + k * ss + q.at[u];
+                            double t = 0.0;
+                            if (nx) t += (double)z[(u & 1) ? 1 : -1];
+                            if (nx2) t += (double)z[(u & 1) ? xim : xi];
+                            if (ny) t += (double)z[(u & 2) ? ldx : -ldx];
+                            if (ny2) t += (double)z[(u & 2) ? -ldx : ldx];
+                            if (kk == 1) t += (double)sm[k * ss + q.at[u]];
+                            if (kk + 1 == n) t += (double)sp[k * ss + q.at[u]];
+                            ks[k] = T(-6.0 * t);
+                        }
+                        node(pl * pn + q.row[u], kx[u], ks, differs);
                     }
                 } else {
                     const int co[3] = {q.x, q.y, kk};
@@ -787,9 +854,10 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                         const bool mx = u & 1, my = u & 2;
                         if (!(mx ? (my ? q.has[3] : q.has[1]) : (my ? q.has[2] : q.has[0]))) continue;
                         const int j = my ? n - q.y : q.y, i = mx ? n - q.x : q.x, l = pl * pn + j * s2 + i;
-                        T kx[VEC], ks[VEC], f[VEC];
+                        T kx[VEC], ks[VEC];
+                        bool differs = false;
 #pragma unroll
-                        for (int k = 0; k < VEC; ++k) kx[k] = ks[k] = f[k] = T(0);
+                        for (int k = 0; k < VEC; ++k) kx[k] = ks[k] = T(0);
                         if (!froz) {
                             const T* xp = x + (ptrdiff_t)l * C;
                             T xi[VEC];
@@ -809,38 +877,19 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                                     const T w = T(wt[a]);
 #pragma unroll
                                     for (int k = 0; k < VEC; ++k) kx[k] = fma_(w, xi[k] - xj[k], kx[k]);
-                                    if (!neu && mode && (ca == 0 || ca == n))   // the neighbour lies on the surface
+                                    if (!neu && mode && (ca == 0 || ca == n)) {   // the neighbour lies on the surface
+                                        differs = true;
 #pragma unroll
                                         for (int k = 0; k < VEC; ++k) ks[k] -= T(6) * xj[k];
+                                    }
                                 }
                             if (neu) {
                                 const double vi = (double)(nodes[l] & 0xff);
 #pragma unroll
                                 for (int k = 0; k < VEC; ++k) vx[0][k] = fma_(vi, (double)xi[k], vx[0][k]);
                             }
-                            if (neu || !mode) {
-                                double fb[VEC];
-                                ldc<VEC, false>(fb, bv + (ptrdiff_t)l * B);
-                                if (mode && surf) {   // the BEM term of the adjoint Neumann system
-                                    const int bp = (int)((unsigned)nodes[l] >> 16);
-#pragma unroll
-                                    for (int k = 0; k < VEC; ++k) fb[k] += (double)P.V.ub_out[(size_t)(bp - 1) * C + c0 + k];
-                                }
-#pragma unroll
-                                for (int k = 0; k < VEC; ++k) f[k] = act[k] ? T(fb[k]) : T(0);
-                            }
                         }
-                        W rv[VEC];
-#pragma unroll
-                        for (int k = 0; k < VEC; ++k) {
-                            rv[k] = W(f[k] - kx[k]);
-                            const W ref = W(f[k] - ks[k]);
-                            v[0][k] = fma_(rv[k], rv[k], v[0][k]);
-                            v[1][k] += rv[k];
-                            v[2][k] = fma_(ref, ref, v[2][k]);
-                            v[3][k] += ref;
-                        }
-                        stc<VEC>(r + (ptrdiff_t)l * VEC, rv);
+                        node(l, kx, ks, differs);
                     }
                 }
                 put(v, 0, pl, ch);
@@ -1172,9 +1221,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                     put(v, 4, pl, ch);
                 });
                 if (!nodewise) quads(0, np, [&](int pl, int ch, const Quad& q) {
-                    T v[1][VEC];
-#pragma unroll
-                    for (int k = 0; k < VEC; ++k) v[0][k] = T(0);
+                    Acc v[1][VEC];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         if (!q.has[u]) continue;
@@ -1187,7 +1234,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                             ldc<VEC, false>(xv, d + (ptrdiff_t)l * VEC);
                         }
 #pragma unroll
-                        for (int k = 0; k < VEC; ++k) v[0][k] = fma_(vi, xv[k], v[0][k]);
+                        for (int k = 0; k < VEC; ++k) v[0][k].fma(vi, xv[k]);
                     }
                     put(v, 4, pl, ch);
                 });
