@@ -145,7 +145,8 @@ struct CcArgs {
 };
 
 // T: type of the potential x and of the residual f - K x; W: type of the CG
-// vectors and of the sums inside a CTA.  T = W: CG to the tolerance.  T = double,
+// vectors and of an iteration's sums inside a CTA (the residual's, its reference's and
+// the gauge's are FP64).  T = W: CG to the tolerance.  T = double,
 // W = float: cycles of the FP64 residual and FP32 CG until it has reduced that
 // residual by MP_INNER; the solve ends on the FP64 residual test.
 template <typename T, typename W, int VEC>
@@ -219,21 +220,25 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
             for (int i = tid; i <= cnt; i += nt) eptr[i] = P.M.kptr[lo + i] - e0;
         }
         int par = 0;
-        // Totals over the cluster of NQ quantities of VEC columns into out[q * VEC + k].
-        auto reduce = [&](auto& v) {
+        // Totals over the cluster of NQ quantities of VEC columns into out[(q0 + q) * VEC + k];
+        // of W, or of FP64 (two W words of scr hold one: at most CC_NQ / 2 quantities).
+        auto reduce = [&](auto& v, int q0) {
             constexpr int NQ = sizeof(v) / sizeof(v[0]), NV = NQ * VEC;
+            using X = typename std::remove_reference<decltype(v[0][0])>::type;
+            static_assert(NQ * sizeof(X) <= CC_NQ * sizeof(W), "scr holds them");
+            X* const sc = reinterpret_cast<X*>(scr);   // [32 warps][NV]
 #pragma unroll
             for (int a = 0; a < NQ; ++a)
 #pragma unroll
                 for (int k = 0; k < VEC; ++k) {
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) v[a][k] += __shfl_xor_sync(0xffffffffu, v[a][k], o);
-                    if (lane == 0) scr[warp * (CC_NQ * VEC) + a * VEC + k] = v[a][k];
+                    if (lane == 0) sc[warp * NV + a * VEC + k] = v[a][k];
                 }
             __syncthreads();
             const uint32_t sl = cc_addr(slots + par * CC_NQ * VEC * CC_MAX_CL);
             for (int w = warp; w < NV; w += nw) {
-                W t = lane < nw ? scr[lane * (CC_NQ * VEC) + w] : W(0);
+                X t = lane < nw ? sc[lane * NV + w] : X(0);
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
                 if (lane < g.cl) cc_st(cc_peer(sl + (uint32_t)(w * CC_MAX_CL + (int)rank) * 8u, (unsigned)lane), (double)t);
@@ -243,7 +248,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
                 double t = lane < g.cl ? slots[(par * CC_NQ * VEC + w) * CC_MAX_CL + lane] : 0.0;
 #pragma unroll
                 for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-                if (lane == 0) out[w] = t;
+                if (lane == 0) out[q0 * VEC + w] = t;
             }
             par ^= 1;   // rewritten only after a further barrier, when every CTA has read it
             __syncthreads();
@@ -308,12 +313,12 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
             }
         cc_sync();
         for (int cycle = 0;; ++cycle) {
-            {   // residual of the current x into r; sums r.r, r, f.f, f (f: the norm reference)
-                W v[4][VEC];
+            {   // residual of the current x into r; FP64 sums r.r, r and f.f, f (f: the norm reference)
+                double v[2][VEC], vf[2][VEC];
 #pragma unroll
-                for (int a = 0; a < 4; ++a)
+                for (int a = 0; a < 2; ++a)
 #pragma unroll
-                    for (int k = 0; k < VEC; ++k) v[a][k] = W(0);
+                    for (int k = 0; k < VEC; ++k) v[a][k] = vf[a][k] = 0.0;
                 for (int l = tid; l < cnt; l += nt) {
                     const int row = lo + l;
                     W rv[VEC];
@@ -323,10 +328,14 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
                         for (int k = 0; k < VEC; ++k) rv[k] = W(0);
                     } else {
                         const T* kvT = GenTab<T>::k(P.M);
-                        T xi[VEC], kx[VEC], f[VEC], ks[VEC];
+                        T xi[VEC], kx[VEC];
+                        double f[VEC], ks[VEC];
                         cc_get<VEC, true>(xi, x + (size_t)row * C + c0);
 #pragma unroll
-                        for (int k = 0; k < VEC; ++k) kx[k] = f[k] = ks[k] = T(0);
+                        for (int k = 0; k < VEC; ++k) {
+                            kx[k] = T(0);
+                            f[k] = ks[k] = 0.0;
+                        }
                         const int e0 = P.M.kptr[row], e1 = P.M.kptr[row + 1];
 #pragma unroll 4
                         for (int e = e0; e < e1; ++e) {
@@ -338,32 +347,32 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
 #pragma unroll
                             for (int k = 0; k < VEC; ++k) {
                                 kx[k] = cc_fma(kv, xj[k] - xi[k], kx[k]);
-                                if (s) ks[k] = cc_fma(kv, xj[k], ks[k]);   // K_IS x_S
+                                if (s) ks[k] = fma((double)kv, (double)xj[k], ks[k]);   // K_IS x_S
                             }
                         }
                         if (!(mode == 1 && !neu)) {
-                            double fb[VEC];
-                            cc_get<VEC, false>(fb, P.V.bvec + (size_t)row * B + b0);
+                            cc_get<VEC, false>(f, P.V.bvec + (size_t)row * B + b0);
 #pragma unroll
                             for (int k = 0; k < VEC; ++k) {
-                                if (!act[k]) fb[k] = 0.0;
-                                if (mode == 1 && bp) fb[k] += (double)P.V.ub_out[(size_t)(bp - 1) * C + c0 + k];
-                                f[k] = T(fb[k]);
+                                if (!act[k]) f[k] = 0.0;
+                                if (mode == 1 && bp) f[k] += (double)P.V.ub_out[(size_t)(bp - 1) * C + c0 + k];
                             }
                         }
 #pragma unroll
                         for (int k = 0; k < VEC; ++k) {
-                            rv[k] = W(f[k] - kx[k]);
-                            const W ref = W(f[k] - ks[k]);
-                            v[0][k] = cc_fma(rv[k], rv[k], v[0][k]);
-                            v[1][k] += rv[k];
-                            v[2][k] = cc_fma(ref, ref, v[2][k]);
-                            v[3][k] += ref;
+                            const T rt = T(f[k]) - kx[k];
+                            rv[k] = W(rt);
+                            const double rd = (double)rt, ref = f[k] - ks[k];
+                            v[0][k] = fma(rd, rd, v[0][k]);
+                            v[1][k] += rd;
+                            vf[0][k] = fma(ref, ref, vf[0][k]);
+                            vf[1][k] += ref;
                         }
                     }
                     cc_put<VEC>(r + (size_t)l * VEC, rv);
                 }
-                reduce(v);
+                reduce(v, 0);
+                reduce(vf, 2);
                 if (tid < VEC) {
                     const double sf = out[3 * VEC + tid], ff = out[2 * VEC + tid];
                     if (cycle == 0) s_tol[tid] = P.tol2 * (neu ? fmax(ff - sf * sf / (double)R, 0.0) : ff);
@@ -445,7 +454,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
                     if (!last) cc_sync();
                     cur ^= 1;
                 }
-                reduce(v1);   // r.z
+                reduce(v1, 0);   // r.z
                 if (tid < VEC) {
                     const double rho = out[tid];
                     s_ab[tid] = (it == 0 || s_flag[tid]) ? W(0) : W(rho) / W(s_rhop[tid]);
@@ -479,7 +488,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
                     cc_put<VEC>(p + (size_t)l * VEC, pv);
                     cc_put<VEC>(q + (size_t)l * VEC, qv);
                 }
-                reduce(v1);   // p.q
+                reduce(v1, 0);   // p.q
                 if (tid < VEC) s_ab[tid] = s_flag[tid] ? W(0) : W(s_rho[tid]) / W(out[tid]);
                 __syncthreads();
                 // ---- B, and the first step of the next polynomial -------------------------
@@ -514,7 +523,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
                     cc_put<VEC>(dd + (size_t)l * VEC, zv);
                 }
                 cur ^= 1;
-                reduce(u);
+                reduce(u, 0);
             }
             // fold the cycle's correction into x before anything reads x
             for (int l = tid; it > 0 && l < cnt; l += nt) {
@@ -550,32 +559,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
 #pragma unroll
                 for (int k = 0; k < VEC; ++k) pv[0][k] = fma(vi, (double)xv[k], pv[0][k]);
             }
-            // FP64 sums of the CTA through the warps' room (two W words hold one)
-            {
-                double* scd = reinterpret_cast<double*>(scr);
-#pragma unroll
-                for (int k = 0; k < VEC; ++k) {
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) pv[0][k] += __shfl_xor_sync(0xffffffffu, pv[0][k], o);
-                    if (lane == 0) scd[warp * VEC + k] = pv[0][k];
-                }
-                __syncthreads();
-                const uint32_t sl = cc_addr(slots + par * CC_NQ * VEC * CC_MAX_CL);
-                for (int w = warp; w < VEC; w += nw) {
-                    double t = lane < nw ? scd[lane * VEC + w] : 0.0;
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-                    if (lane < g.cl) cc_st(cc_peer(sl + (uint32_t)(w * CC_MAX_CL + (int)rank) * 8u, (unsigned)lane), t);
-                }
-                cc_sync();
-                for (int w = warp; w < VEC; w += nw) {
-                    double t = lane < g.cl ? slots[(par * CC_NQ * VEC + w) * CC_MAX_CL + lane] : 0.0;
-#pragma unroll
-                    for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-                    if (lane == 0) out[w] = t;
-                }
-                __syncthreads();
-            }
+            reduce(pv, 0);
             T mean[VEC];
 #pragma unroll
             for (int k = 0; k < VEC; ++k) mean[k] = T(out[k] / P.M.vsum);
