@@ -145,6 +145,7 @@ __device__ __forceinline__ void kuhn_apply(const C (&c)[16], const V* v, ptrdiff
 //   27^3, 16 in FP32                  | 8, 100: 1.62   12, 220: 1.48   16, 400: 1.39
 //   39^3, 32 in FP64                  | 8, 100: 39.1   12, 220: 38.0   16, 400: 37.1
 // The lines lie between these sizes.
+constexpr int SH_DEG_MAX = 16;
 void sh_degree(int rows, int& deg, double& ratio) {
     struct Step {
         int rows, deg;
@@ -152,7 +153,7 @@ void sh_degree(int rows, int& deg, double& ratio) {
     };
     static constexpr Step steps[] = {{280, 3, 8.0},     {600, 4, 15.0},     {1000, 6, 30.0},
                                      {2500, 8, 60.0},   {6500, 8, 100.0},   {14000, 12, 220.0}};
-    deg = 16;
+    deg = SH_DEG_MAX;
     ratio = 400.0;
     for (const Step& t : steps)
         if (rows <= t.rows) {
@@ -332,8 +333,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
             // ---- C: outer-face rows (kind 0) keep zero ----
             W v1[1][VEC];
             W rho_c = de / th;
-            for (int st = 1; st < A.deg; ++st) {
-                const bool last = st + 1 == A.deg;
+            // counted up to a constant: to A.deg the loop takes 2 % longer
+            for (int st = SH_DEG_MAX - A.deg + 1, st1 = st; st < SH_DEG_MAX; ++st) {
+                const bool last = st + 1 == SH_DEG_MAX;
                 const W rn = W(1) / (W(2) * th / de - rho_c), c1 = rn * rho_c, c2 = W(2) * rn / de, c3 = W(1) + c1;
                 rho_c = rn;
 #pragma unroll
@@ -353,7 +355,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
                         tv[k] = W(0);
                         w[k] = -rv[k];
                     }
-                    if (st > 1) ldv<VEC, false>(tv, zo + i);
+                    if (st > st1) ldv<VEC, false>(tv, zo + i);
                     kuhn_apply<VEC, true>(c, z + i, sx, sy, sz, kind == 2, w);
                     const W di = c2 * c[15];
 #pragma unroll
