@@ -159,7 +159,6 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint64_t* empty = bars + 2 * STAGES;   // [STAGES] MMAs of the stage done
     uint64_t* done = bars + 3 * STAGES;    // accumulator complete
     uint32_t* s_taddr = (uint32_t*)(bars + 3 * STAGES + 1);
-    __shared__ int s_fail;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int mt = gridDim.x / 2, second = (int)blockIdx.x >= mt;
@@ -170,7 +169,6 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int nkb = max(0, min(kblocks_per_split, nkb_total - kb0));
 
     if (tid == 0) {
-        s_fail = 0;
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&conv[s], 128);
@@ -195,7 +193,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             // ---- producer: TMA loads of A, X_hi, X_lo per stage -----------------
             for (int kb = 0; kb < nkb; ++kb) {
                 const int s = kb % STAGES;
-                if (kb >= STAGES && !mbar_wait(&empty[s], ((kb / STAGES) - 1) & 1, err)) { s_fail = 1; break; }
+                if (kb >= STAGES && !mbar_wait(&empty[s], ((kb / STAGES) - 1) & 1, err)) break;
                 uint8_t* st = smem + s * STAGE_BYTES<NT>;
                 mbar_expect_tx(&full[s], A_BYTES + 2 * X_BYTES<NT>);
                 const int k = (kb0 + kb) * BK;
@@ -207,7 +205,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             // ---- MMA issuer ----------------------------------------------------------
             for (int kb = 0; kb < nkb; ++kb) {
                 const int s = kb % STAGES;
-                if (!mbar_wait(&conv[s], (kb / STAGES) & 1, err)) { s_fail = 1; break; }
+                if (!mbar_wait(&conv[s], (kb / STAGES) & 1, err)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 uint8_t* st = smem + s * STAGE_BYTES<NT>;
                 const uint32_t ah = tmem + TMEM_A + s * 2 * BK, al = ah + BK;
@@ -232,7 +230,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 const int s = kb % STAGES;
                 // the stage's MMAs of the round before have finished: the producer waited for them
                 ok = __all_sync(0xffffffffu, mbar_wait(&full[s], (kb / STAGES) & 1, err));
-                if (!ok) { s_fail = 1; break; }
+                if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint8_t* a = smem + s * STAGE_BYTES<NT> + row * (BK * 4);
                 uint32_t h[32], l[32];
