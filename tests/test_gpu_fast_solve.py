@@ -109,3 +109,17 @@ def test_a_converged_system_waits(ctx, n, B):
         mixed += len(counts) > 1
     assert mixed   # some instances did take more steps than others
     ctx.mesh_destroy(mesh)
+
+
+@pytest.mark.parametrize("n,prec,opts,tol", [
+    (82, 0, dict(cg_mixed_iter=1, cg_tol=1e-10), 1e-6), (96, 1, dict(), 2e-5)])
+def test_the_largest_cubes(ctx, n, prec, opts, tol):
+    """FP64 solves iterated in FP32 with their planes in global memory, and the largest
+    cube there is."""
+    mesh = ctx.mesh_cube(2e-9, n)
+    m = _m(n, 1, 5)
+    _, h, u = _run(ctx, mesh, n, 1, prec, m, **opts)
+    _, hr, ur = _run(ctx, mesh, n, 1, prec, m, pcg_kernel=1, **opts)
+    ctx.mesh_destroy(mesh)
+    assert np.linalg.norm(u - ur) <= tol * np.linalg.norm(ur)
+    assert np.linalg.norm(h - hr) <= tol * np.linalg.norm(hr)
