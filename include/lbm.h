@@ -73,7 +73,14 @@ typedef struct {
                                (the paper's grad h^T grad h test, Sec. 3.1) */
     int32_t max_iter;       /* accepted steps per minimisation */
     double  cg_tol;         /* relative residual |r|/|b| of both potential solves */
-    int32_t cg_max_iter;    /* iteration cap of each potential solve */
+    int32_t cg_max_iter;    /* iteration cap of each potential solve, in the iterations of
+                               the solve it takes (pcg_kernel): refinement steps of the
+                               fast diagonalisation (Neumann solves take them in pairs: a
+                               cap of 1 ends one halfway), or CG iterations, of one matrix
+                               product in the Jacobi-preconditioned kernels, of 2 to 16
+                               in the polynomially preconditioned one of uploaded meshes
+                               and of 3 to 16 on the grid of lbm_mesh_shell.  The counters
+                               of lbm_result and lbm_profile_stats count the same */
     double  c1;             /* Armijo constant of the line search */
     int32_t max_backtracks; /* step halvings before LBM_E_LINESEARCH */
     int32_t memory;         /* nonmonotone memory (20 in Sec. 2.3) */
@@ -112,18 +119,23 @@ typedef struct {
                                FP32 phase of a mixed run then hands the instance to the
                                FP64 phase (which ignores it).  0 = never.  Default 200
                                for the mixed precisions, 0 for LBM_FP64 */
-    int32_t pcg_kernel;     /* potential-solve kernel: 0 (default) chooses; 1 Jacobi-
-                               preconditioned CG, grid-wide kernel (one CTA for small
-                               work, else a cooperative grid); 2 the same iteration
-                               with one thread-block cluster per group of systems
-                               (taken when the batch has a multiple of 4, at least 16
-                               instances, FP32 work vectors and z of a cluster's
+    int32_t pcg_kernel;     /* potential-solve kernel of the FEM/BEM chain: 0 (default)
+                               chooses; 1 Jacobi-preconditioned CG, grid-wide kernel (one
+                               CTA for small work, else a cooperative grid); 2 the same
+                               iteration with one thread-block cluster per group of
+                               systems (taken when the batch has a multiple of 4, at
+                               least 16 instances, FP32 work vectors and z of a cluster's
                                systems fits its shared memory; otherwise as 1).
                                0 on a Kuhn cube: fast diagonalisation with iterative
-                               refinement to the same residual tests (each iteration
-                               of the counters is one refinement step, at least one a
-                               solve); on a general mesh 2 where it qualifies, else 1.
-                               Results agree to the solves' tolerance */
+                               refinement to the same residual tests (at least one step a
+                               solve).  0 on an uploaded mesh: CG with a Chebyshev
+                               polynomial as preconditioner, one cluster per group of
+                               systems, to the same tests; on meshes of more than 65 000
+                               nodes (80 000 to 100 000 with FP32 work vectors) and for
+                               plain FP64 batches too wide for the chip's clusters 2 where
+                               it qualifies, else 1.  Results agree to the solves'
+                               tolerance.  The solve of lbm_mesh_shell has one kernel,
+                               whatever this says */
     int32_t use_graphs;     /* 1 (default): each chunk of check_every iterations is
                                captured once as a CUDA graph (per batch, options and
                                mesh operators) and replayed; the first chunk of a solve
@@ -156,7 +168,7 @@ typedef struct {
     int32_t iterations;     /* accepted steps */
     int32_t evaluations;    /* energy-gradient evaluations (incl. the initial one) */
     int32_t line_searches;  /* times the line search was entered */
-    int64_t cg_iters1;      /* total iterations of the Neumann (u1) solves */
+    int64_t cg_iters1;      /* total iterations (cg_max_iter) of the Neumann (u1) solves */
     int64_t cg_iters2;      /* total iterations of the Dirichlet (u2) solves */
     double  energy[5];      /* exchange, anisotropy, Zeeman, stray field, total (J) */
     double  torque;         /* max_i |m_i x h_i| / Js at the final state */
@@ -383,8 +395,10 @@ int lbm_mesh_hmatrix(lbm_ctx* ctx, lbm_mesh mesh, double eps, double eta, int32_
  * potential vanishes on the outer face (the image of infinity).  From then on
  * every stray-field evaluation of the mesh's instances (minimise, evaluate,
  * serving; every precision) solves the one symmetric system K_grid u = b on
- * the grid (FP64 Jacobi-PCG on the device, cg_tol / cg_max_iter of the solve
- * options, warm-started from the instance's previous grid potential) instead
+ * the grid (CG with a Chebyshev polynomial of the Jacobi-scaled matrix as
+ * preconditioner, in FP32 for FP32 phases and cg_mixed_iter, else in FP64; cg_tol
+ * / cg_max_iter of the solve options, warm-started from the instance's previous
+ * grid potential) instead
  * of the two Poisson solves and the boundary product; its iterations count as
  * cg_iters1 and its time as the first potential solve.  The field at the
  * magnet's nodes is the exact gradient field of the discrete stray-field
