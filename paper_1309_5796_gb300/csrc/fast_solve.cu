@@ -125,7 +125,7 @@ __device__ __forceinline__ void st4(double* p, const double (&v)[4]) {
 __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// Sums that have to be better than FP32's: FP64 where the values are, or, of FP32 values,
+// Sums that have to be better than FP32's: FP64 of FP64 values, or, of FP32 ones,
 // pairs of FP32 words with every rounding kept (Knuth's TwoSum, the product's error by
 // FMA), 48 bits at a sixth of the time of GB300's FP64 units.
 struct Pair {
@@ -407,7 +407,6 @@ __device__ __forceinline__ void edge_node(int e, int n, int& i, int& j, int& k) 
 template <typename T, typename W, int VEC, bool TS>
 __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(const __grid_constant__ FsArgs<T, W> A) {
     constexpr bool MP = sizeof(T) != sizeof(W), ND = sizeof(W) == 8;
-    using Acc = typename SumOf<T>::type;
     const FsGeo& g = A.g;
     W* buf = reinterpret_cast<W*>(fs_sm);                       // TS: own planes [ppc][VEC][ss]; else a round of planes
     W* zb = reinterpret_cast<W*>(fs_sm + g.o_z);                // P2: [s2][VEC * pr] (TS = false: in buf's room)
@@ -776,7 +775,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
             if (!nodewise) quads(0, np, [&](int pl, int ch, const Quad& q) {
                 const int kk = k0 + pl;
                 const bool surf = q.x == 0 || q.y == 0 || kk == 0 || kk == n;
-                Acc v[4][VEC];
+                typename SumOf<W>::type v[4][VEC];
                 double vx[1][VEC];
 #pragma unroll
                 for (int k = 0; k < VEC; ++k) vx[0][k] = 0.0;
@@ -799,13 +798,13 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                     W rv[VEC];
 #pragma unroll
                     for (int k = 0; k < VEC; ++k) {
-                        const T ft = act[k] ? T(f[k]) : T(0), rt = ft - kx[k];
-                        rv[k] = W(rt);
+                        const T ft = act[k] ? T(f[k]) : T(0);
+                        rv[k] = W(ft - kx[k]);
                         if (froz) continue;
-                        v[0][k].fma(rt, rt);
-                        if (neu) v[1][k].add(rt);
+                        v[0][k].fma(rv[k], rv[k]);
+                        if (neu) v[1][k].add(rv[k]);
                         if (!rhs && !differs) continue;
-                        const T ref = ft - ks[k];
+                        const W ref = W(ft - ks[k]);
                         v[2][k].fma(ref, ref);
                         if (neu) v[3][k].add(ref);
                     }
@@ -1221,7 +1220,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                     put(v, 4, pl, ch);
                 });
                 if (!nodewise) quads(0, np, [&](int pl, int ch, const Quad& q) {
-                    Acc v[1][VEC];
+                    typename SumOf<T>::type v[1][VEC];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         if (!q.has[u]) continue;
