@@ -21,7 +21,7 @@
 // fixed order.  The launch shape depends on the sizes and the batch only, so a
 // solve gives the same bits every time.
 //
-// Measured (both stages of both chains): one instance on 19 683 nodes in FP32 1.7 ms,
+// Measured (both stages of both chains): one instance on 19 683 nodes in FP32 1.83 ms,
 // 7.2 with the grid-wide kernel; 16 on 3 375 nodes in FP64 4.0 ms, before 8.5.
 // What bounds it: latency, in FP64 also the FP64 units.  A cluster barrier costs 400 to 650 clocks, a reduction
 // with its barrier about 1700, a product of 15 entries a row about 2000 at two rows

@@ -26,7 +26,7 @@
 //
 // Measured on GB300 (two stages of both chains, FP64 n = 10 / FP32 n = 20, 80, one
 // instance / FP32 n = 30, 64 instances, before: diagonally preconditioned CG):
-// 0.13 / 0.13 / 1.5 / 0.72 ms, before 6.1 / 5.6 / 36 / 12 ms.
+// 0.11 / 0.14 / 1.57 / 0.77 ms, before 6.1 / 5.6 / 36 / 12 ms.
 //
 // One thread-block cluster solves VEC systems (columns of the [N][2B] layout)
 // of one kind; CTA r owns the z-planes [r ppc, (r+1) ppc).  Per step:
@@ -1479,7 +1479,7 @@ void try_shapes(const Launch& L, int n, int B, int groups, FsChoice& best, doubl
 // constants are fitted to some 400 measured shapes of 25 sizes and batches (n = 10 to
 // 80, 1 to 64 instances), on which the rule's shape is within 5 % of the fastest (1 % on
 // average): 64 instances at n = 30 run one system on two CTAs of 16 planes and 512
-// threads (0.36 ms a stage; 0.46 on sixteen CTAs of two planes, 0.80 on one CTA), one
+// threads (0.36 ms a stage in that measurement; 0.46 on sixteen CTAs of two planes, 0.80 on one CTA), one
 // instance at n = 20 on eleven CTAs of two planes (62 us; 120 on two CTAs).
 template <typename T, typename W>
 FsChoice choose(const Launch& L, const MeshView& M, int B) {

@@ -188,7 +188,8 @@ constexpr double SH_DEAL1 = 3e5, SH_DEAL2 = 8e5;
 // words and one barrier where a CG iteration moves 12 and four.  (20 on [b / 800, b] gives
 // 3 % more on that grid.  Multigrid and fast diagonalisation stall on the shell's growing
 // tangential stiffness.)
-// Measured on that grid: 32 instances 10.3 ms a solve, one 2.4; at first 24.1 and 5.7.
+// Measured on that grid: 0.36 ms an iteration of 32 instances, 0.083 of one; an evaluation of
+// smooth states (34 iterations) 12.5 and 2.9 ms, with Jacobi-CG 28.6 and 6.8.
 // Every block has one run of consecutive rows, so that the L1 serves a product's
 // neighbours along x and y and about three of its fifteen reads go to L2 (with
 // rows dealt round all blocks and loads past the L1, all fifteen did).
@@ -233,10 +234,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_shell_pcg(ShellArgs<W> A) {
     else coefW = A.S.coef32;
     // a run of consecutive rows for each block (the header says why), or, where the FP64
     // units bind, rows dealt round all blocks, so that each has its share of the 7- and of
-    // the 15-point rows (ms a solve, runs -> dealt, with five FP64 operations
-    // a step besides the product, now three: 29 instances on 54 872 nodes 39.0 -> 34.3,
-    // 25 on 35 937 19.6 -> 17.4, 9 on 35 937 8.9 -> 8.1, 16 on 50 653 19.0 -> 17.7; below
-    // the lines 24 on 29 791 14.0 -> 14.2, 16 on 24 389 8.4 -> 9.3)
+    // the 15-point rows (ms an evaluation, runs -> dealt.  Odd batches above the line: 13
+    // instances on 29 791 nodes 9.90 -> 9.12, 33 20.3 -> 18.2, 3 on 117 649 15.7 -> 15.9,
+    // 25 94.3 -> 84.1, 17 on 166 375 104 -> 90; below it 9 on 29 791 7.46 -> 7.67, 7 6.26 ->
+    // 6.55.  Even ones above: 32 on 29 791 17.3 -> 15.3, 8 on 117 649 30.2 -> 28.4, 32 104 ->
+    // 91.5, 16 on 166 375 86.4 -> 76.5; below 8 on 29 791 6.25 -> 7.01, 4 on 166 375 25.3 ->
+    // 26.8, 2 16.0 -> 18.5, though 16 on 29 791 10.5 -> 9.2, 4 on 117 649 17.5 -> 16.1)
     const int rpb = (Ng + (int)gridDim.x - 1) / (int)gridDim.x, rstep = A.deal ? (int)gridDim.x * RB : RB;
     const int rlo = (int)blockIdx.x * (A.deal ? RB : rpb);
     const int rhi = !lane ? 0 : A.deal ? Ng : min(Ng, rlo + rpb);   // idle lanes have no rows

@@ -741,7 +741,9 @@ template <> struct DotAcc<float> {
 // are taken.  The R sums of a warp take R merges by shuffles for R rows
 // by a chunk, so a chunk is as wide as the grid's need for blocks allows.  Sums are
 // DotAcc's (compensated in FP32, FP64 in FP64) to a warp and FP64 across warps, panels and
-// chunks, all in a fixed order.
+// chunks, all in a fixed order.  Against 64 bits FP32 results are off by 3.4e-8 to 4.6e-8 of
+// their norm for 8 to 11 618 surface nodes (with FP64 sums over the lanes 3.7e-8 to 6.4e-8:
+// the rounding of the result in both), FP64 ones by 1.5e-16 to 4.1e-16 (1.5e-16 to 3.9e-16).
 // One instance, before -> after: FP32 at n = 80 1.91 -> 1.10 ms (5.9 GB), n = 40 141 -> 97 us,
 // n = 20 27 -> 20 us; FP64 at n = 10 21 -> 14 us, at n = 17 31 us both (FP64 units).
 constexpr int GV_THREADS = 256, GV_MAX_COLS = 4096;
