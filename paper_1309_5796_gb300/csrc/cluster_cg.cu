@@ -739,14 +739,19 @@ void cc_try(const Launch& L, int rows, int cols, const int* emax, CcChoice& best
 // systems in plain FP64, whose clusters run in waves (the polynomial takes about a quarter
 // more products, and FP64 units are what bounds both), and the largest meshes (a system has
 // sixteen SMs and its entries come from global memory).  ms an evaluation here / there, plain
-// FP64: 64 instances on 3 375 nodes 17.4 / 12.6, 128 33.6 / 19.7, 96 on 1 331 8.6 / 7.5, 32 on
-// 15 625 49.8 / 44.5 (three to seven waves); one or two waves 1.0 to 2.3 times faster here
-// over 60 such shapes of 343 to 42 875 nodes; one on 74 088 46.7 / 37.5, on 59 319 36.7 / 34.5.
-// Iterated in FP32: one on 74 088 26.5 / 25.8, on 91 125 33.5 / 31.8, five 61 / 44; FP32: one on
-// 91 125 17.3 / 16.6, eight 54 / 41, four on 117 649 57 / 31, one on 166 375 45 / 23.
-bool cc_slower(int rows, int cols, int waves, bool fp32, bool fp64_vectors) {
-    if (fp64_vectors) return rows > 65000 || waves >= 5 || (waves >= 3 && (cols >= 80 || rows >= 14000));
-    return rows > (fp32 && cols < 16 ? 100000 : 80000);
+// FP64, systems a cluster by waves: 2 by 5, 64 instances on 3 375 nodes 17.4 / 12.6; 2 by 3,
+// 96 on 1 331 8.6 / 7.5, 40 on 12 167 44.0 / 38.0, 20 on 29 791 71 / 62, but 20 on 12 167 23.7 /
+// 27.3, 40 on 4 913 14.6 / 15.6; 2 by 4, 48 on 3 375 13.9 / 13.3 (as its instances finish, a
+// minimisation is faster here); 1 by 3, 9 on 19 683 25.5 / 28.4, on 29 791 39.6 / 39.5, 8 on
+// 46 656 62 / 55, on 50 653 70 / 64; 1 by 4, 25 on 9 261 20.3 / 24.4, 24 on 24 389 59.9 / 57.3; one or two waves 1.0 to
+// 2.3 times faster here over 60 such shapes of 343 to 42 875 nodes; one on 74 088 46.7 / 37.5, on
+// 59 319 36.7 / 34.5.  Iterated in FP32: one on 74 088 26.5 / 25.8, on 91 125 33.5 / 31.8, five
+// 61 / 44; FP32: one on 91 125 17.3 / 16.6, eight 54 / 41, four on 117 649 57 / 31, one on
+// 166 375 45 / 23.
+bool cc_slower(int rows, int cols, int vec, int waves, bool fp32, bool fp64_vectors) {
+    if (!fp64_vectors) return rows > (fp32 && cols < 16 ? 100000 : 80000);
+    const bool wide = cols >= 100 || rows >= 14000 || (cols >= 80 && rows >= 10000);
+    return rows > 65000 || waves >= 5 || (wide && waves >= (vec == 2 ? 3 : 4)) || (rows >= 45000 && waves >= 3);
 }
 
 template <typename T, typename W>
@@ -756,7 +761,7 @@ CcChoice cc_choose(const Launch& L, int rows, int cols, const int* emax) {
     if constexpr (sizeof(W) == 4) cc_try<T, W, 4>(L, rows, cols, emax, c, cost);
     cc_try<T, W, 2>(L, rows, cols, emax, c, cost);
     cc_try<T, W, 1>(L, rows, cols, emax, c, cost);
-    if (cc_slower(rows, cols, c.waves, sizeof(T) == 4, sizeof(W) == 8)) c.vec = 0;
+    if (cc_slower(rows, cols, c.vec, c.waves, sizeof(T) == 4, sizeof(W) == 8)) c.vec = 0;
     return c;
 }
 
