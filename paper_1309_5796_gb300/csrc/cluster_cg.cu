@@ -23,9 +23,9 @@
 //
 // Measured (both stages of both chains): one instance on 19 683 nodes in FP32 1.83 ms,
 // 7.2 with the grid-wide kernel; 16 on 3 375 nodes in FP64 4.0 ms, before 8.5.
-// What bounds it: latency, in FP64 also the FP64 units.  A cluster barrier costs 400 to 650 clocks, a reduction
-// with its barrier about 1700, a product of 15 entries a row about 2000 at two rows
-// a thread (distributed shared memory serves 19 bytes a clock to an SM).
+// What bounds it: latency, in FP64 also the FP64 units.  A cluster barrier costs 400 to 650
+// clocks, a reduction with its barrier about 1700, a product of 15 entries a row about 2000
+// at two rows a thread (distributed shared memory serves 19 bytes a clock to an SM).
 #include <math.h>
 #include <stdint.h>
 
@@ -703,7 +703,7 @@ int cc_resident(const CcGeo& g, int threads) {
 // rows: of a system; cols: systems; emax[cl]: most matrix entries of a CTA when the
 // rows are dealt to cl CTAs
 template <typename T, typename W, int VEC>
-void cc_try(const Launch& L, int rows, int cols, const int* emax, CcChoice& best, double& best_cost) {
+void cc_try(int rows, int cols, const int* emax, CcChoice& best, double& best_cost) {
     if ((cols / 2) % VEC) return;
     for (int cl = CC_MAX_CL; cl >= 1; cl = cl > 8 ? cl - 2 : cl / 2) {
         CcGeo g = {};
@@ -743,11 +743,11 @@ void cc_try(const Launch& L, int rows, int cols, const int* emax, CcChoice& best
 // 96 on 1 331 8.6 / 7.5, 40 on 12 167 44.0 / 38.0, 20 on 29 791 71 / 62, but 20 on 12 167 23.7 /
 // 27.3, 40 on 4 913 14.6 / 15.6; 2 by 4, 48 on 3 375 13.9 / 13.3 (as its instances finish, a
 // minimisation is faster here); 1 by 3, 9 on 19 683 25.5 / 28.4, on 29 791 39.6 / 39.5, 8 on
-// 46 656 62 / 55, on 50 653 70 / 64; 1 by 4, 25 on 9 261 20.3 / 24.4, 24 on 24 389 59.9 / 57.3; one or two waves 1.0 to
-// 2.3 times faster here over 60 such shapes of 343 to 42 875 nodes; one on 74 088 46.7 / 37.5, on
-// 59 319 36.7 / 34.5.  Iterated in FP32: one on 74 088 26.5 / 25.8, on 91 125 33.5 / 31.8, five
-// 61 / 44; FP32: one on 91 125 17.3 / 16.6, eight 54 / 41, four on 117 649 57 / 31, one on
-// 166 375 45 / 23.
+// 46 656 62 / 55, on 50 653 70 / 64; 1 by 4, 25 on 9 261 20.3 / 24.4, 24 on 24 389 59.9 /
+// 57.3; one or two waves 1.0 to 2.3 times faster here over 60 such shapes of 343 to 42 875
+// nodes; one on 74 088 46.7 / 37.5, on 59 319 36.7 / 34.5.  Iterated in FP32: one on 74 088 26.5
+// / 25.8, on 91 125 33.5 / 31.8, five 61 / 44; FP32: one on 91 125 17.3 / 16.6, eight 54 / 41,
+// four on 117 649 57 / 31, one on 166 375 45 / 23.
 bool cc_slower(int rows, int cols, int vec, int waves, bool fp32, bool fp64_vectors) {
     if (!fp64_vectors) return rows > (fp32 && cols < 16 ? 100000 : 80000);
     const bool wide = cols >= 100 || rows >= 14000 || (cols >= 80 && rows >= 10000);
@@ -755,12 +755,12 @@ bool cc_slower(int rows, int cols, int vec, int waves, bool fp32, bool fp64_vect
 }
 
 template <typename T, typename W>
-CcChoice cc_choose(const Launch& L, int rows, int cols, const int* emax) {
+CcChoice cc_choose(int rows, int cols, const int* emax) {
     CcChoice c;
     double cost = 0.0;
-    if constexpr (sizeof(W) == 4) cc_try<T, W, 4>(L, rows, cols, emax, c, cost);
-    cc_try<T, W, 2>(L, rows, cols, emax, c, cost);
-    cc_try<T, W, 1>(L, rows, cols, emax, c, cost);
+    if constexpr (sizeof(W) == 4) cc_try<T, W, 4>(rows, cols, emax, c, cost);
+    cc_try<T, W, 2>(rows, cols, emax, c, cost);
+    cc_try<T, W, 1>(rows, cols, emax, c, cost);
     if (cc_slower(rows, cols, c.vec, c.waves, sizeof(T) == 4, sizeof(W) == 8)) c.vec = 0;
     return c;
 }
@@ -793,7 +793,7 @@ cudaError_t cc_launch_vec(const Launch& L, const CcArgs<T, W>& a, const CcChoice
 template <typename T, typename W>
 cudaError_t cc_fem(const Launch& L, const MeshView& M, const BatchView<T>& V, const PcgArgs<T>& P, bool* ok) {
     const int cols = 2 * V.B;
-    const CcChoice c = cc_choose<T, W>(L, M.N, cols, M.emax);
+    const CcChoice c = cc_choose<T, W>(M.N, cols, M.emax);
     *ok = c.vec != 0;
     if (!c.vec) return cudaSuccess;
     CcArgs<T, W> a = {};
@@ -815,8 +815,8 @@ cudaError_t cc_fem(const Launch& L, const MeshView& M, const BatchView<T>& V, co
 bool cluster_cg_takes(const Launch& L, const MeshView& M, int B, bool fp64, bool mixed_iter) {
     // (a cap on the blocks, L.max_blocks, comes with served cubes only; the other kernels keep to it)
     if (!M.gen || L.pcg_kernel != 0 || L.wait_test || L.max_blocks > 0) return false;
-    if (!fp64) return cc_choose<float, float>(L, M.N, 2 * B, M.emax).vec != 0;
-    return (mixed_iter ? cc_choose<double, float>(L, M.N, 2 * B, M.emax) : cc_choose<double, double>(L, M.N, 2 * B, M.emax)).vec != 0;
+    if (!fp64) return cc_choose<float, float>(M.N, 2 * B, M.emax).vec != 0;
+    return (mixed_iter ? cc_choose<double, float>(M.N, 2 * B, M.emax) : cc_choose<double, double>(M.N, 2 * B, M.emax)).vec != 0;
 }
 
 // General meshes: 1 when launched (*err its status), 0 when the cluster shapes do

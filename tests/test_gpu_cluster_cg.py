@@ -1,8 +1,11 @@
-"""Jacobi-CG with a cluster per group of systems (csrc/cluster_cg.cu) against the
-grid-wide kernels (lbm_solve_opts.pcg_kernel = 1): uploaded meshes and the
-space-transformation boundary.
+"""Potential solves of uploaded meshes by CG with a Chebyshev polynomial as
+preconditioner, a cluster per group of systems (csrc/cluster_cg.cu), against the
+grid-wide Jacobi-CG (lbm_solve_opts.pcg_kernel = 1), and of the space-transformation
+boundary, whose one kernel (csrc/shell_solve.cu) the option does not reach: there FP32
+and FP64 iterated in FP32 are compared with plain FP64 (the oracle's comparison is in
+test_gpu_shell.py).
 
-Both run the same iteration to the same relative residual: 1e-13 (FP64), 1e-10
+All solve to the same relative residual: 1e-13 (FP64), 1e-10
 (FP64 iterated in FP32) or 1e-6 (FP32).  In FP64 the condition numbers (a few
 hundred for cells of one size, a few thousand for the grids) leave fields and
 potentials within 1e-9 and 1e-6.  An FP32 solve is taken against the FP64 one: no

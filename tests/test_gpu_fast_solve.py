@@ -1,6 +1,6 @@
 """Potential solves on Kuhn cubes by fast diagonalisation (csrc/fast_solve.cu)
 against the diagonally preconditioned CG of the grid-wide kernel
-(lbm_solve_opts.pcg_kernel = 1), which general meshes use.
+(lbm_solve_opts.pcg_kernel = 1).
 
 Both solve to a relative residual of 1e-13 (FP64), 1e-10 (FP64 iterated in
 FP32) or 1e-6 (FP32).  The smallest nonzero eigenvalue of the stiffness over its
