@@ -172,6 +172,8 @@ __device__ __forceinline__ Pair plus(Pair a, Pair b) {   // the same bits either
     a.e = __fadd_rn(a.e, e);
     return a;
 }
+__device__ __forceinline__ float scaled(float a, Pair v) { return __fmaf_rn(a, v.s, __fmul_rn(a, v.e)); }
+__device__ __forceinline__ double scaled(double a, Sum64 v) { return a * v.s; }
 __device__ __forceinline__ double total(float v) { return (double)v; }
 __device__ __forceinline__ double total(double v) { return v; }
 __device__ __forceinline__ double total(Sum64 v) { return v.s; }
@@ -721,8 +723,8 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
         const int step = TS ? max(np, 1) : g.spl;
         bool ended = false;
         for (int cycle = 0;; ++cycle) {
-            // residual of the current x into r; sums r.r, r, f.f, f (f: the norm
-            // reference, Dirichlet: f - K_IS x_S) and (MP, Neumann) V x for the gauge
+            // residual of the current x into r; sums r.r, f.f (f: the norm reference,
+            // Dirichlet: f - K_IS x_S) and, Neumann, r, f and (MP) V x for the gauge
             if constexpr (ND) if (nodewise) each(0, np, [&](int pl, int ch, const Node& q) {
                 const int kk = k0 + pl;
                 const bool surf = q.x == 0 || q.y == 0 || kk == 0 || kk == n, froz = !neu && surf;
@@ -764,8 +766,8 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                             ref = fma_(W(6), t, ref);
                         }
                         v[0][k] = rv[k] * rv[k];
-                        v[1][k] = rv[k];
-                        v[2][k] = ref * ref;
+                        v[1][k] = ref * ref;
+                        v[2][k] = rv[k];
                         v[3][k] = ref;
                     }
                     stc<VEC>(r + (ptrdiff_t)l * VEC, rv);
@@ -802,10 +804,10 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                         rv[k] = W(ft - kx[k]);
                         if (froz) continue;
                         v[0][k].fma(rv[k], rv[k]);
-                        if (neu) v[1][k].add(rv[k]);
+                        if (neu) v[2][k].add(rv[k]);
                         if (!rhs && !differs) continue;
                         const W ref = W(ft - ks[k]);
-                        v[2][k].fma(ref, ref);
+                        v[1][k].fma(ref, ref);
                         if (neu) v[3][k].add(ref);
                     }
                     stc<VEC>(r + (ptrdiff_t)l * VEC, rv);
@@ -834,14 +836,14 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                             ks[k] = T(0);
                             if (!differs) continue;
                             const W* z = s + k * ss + q.at[u];
-                            double t = 0.0;
-                            if (nx) t += (double)z[(u & 1) ? 1 : -1];
-                            if (nx2) t += (double)z[(u & 1) ? xim : xi];
-                            if (ny) t += (double)z[(u & 2) ? ldx : -ldx];
-                            if (ny2) t += (double)z[(u & 2) ? -ldx : ldx];
-                            if (kk == 1) t += (double)sm[k * ss + q.at[u]];
-                            if (kk + 1 == n) t += (double)sp[k * ss + q.at[u]];
-                            ks[k] = T(-6.0 * t);
+                            typename SumOf<W>::type t;
+                            if (nx) t.add(z[(u & 1) ? 1 : -1]);
+                            if (nx2) t.add(z[(u & 1) ? xim : xi]);
+                            if (ny) t.add(z[(u & 2) ? ldx : -ldx]);
+                            if (ny2) t.add(z[(u & 2) ? -ldx : ldx]);
+                            if (kk == 1) t.add(sm[k * ss + q.at[u]]);
+                            if (kk + 1 == n) t.add(sp[k * ss + q.at[u]]);
+                            ks[k] = scaled(W(-6), t);
                         }
                         node(pl * pn + q.row[u], kx[u], ks, differs);
                     }
@@ -891,22 +893,25 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_fast_solve(c
                         node(l, kx, ks, differs);
                     }
                 }
-                put(v, 0, pl, ch);
-                if constexpr (MP)
-                    if (neu) put(vx, 4, pl, ch);
+                if (neu) {
+                    put(v, 0, pl, ch);
+                    if constexpr (MP) put(vx, 4, pl, ch);
+                } else {
+                    put(reinterpret_cast<typename SumOf<W>::type(&)[2][VEC]>(v), 0, pl, ch);
+                }
             });
-            reduce(MP && neu ? 5 : 4);
+            reduce(!neu ? 2 : MP ? 5 : 4);
             int it = 0;
             for (;; ++it) {
                 const bool first = it == 0;
                 if (tid < VEC) {
                     // Neumann: residual (and first of all the reference) without their means
-                    const double sr = out[VEC + tid];
+                    const double sr = neu ? out[(first ? 2 : 1) * VEC + tid] : 0.0;
                     const double rr = neu ? fmax(out[tid] - sr * sr / (double)N, 0.0) : out[tid];
                     const bool a = P.V.st[b0 + tid].phase != PH_DONE;
                     if (first) {
-                        const double sf = out[3 * VEC + tid];
-                        s_tol[tid] = P.tol2 * (neu ? fmax(out[2 * VEC + tid] - sf * sf / (double)N, 0.0) : out[2 * VEC + tid]);
+                        const double ff = out[VEC + tid], sf = neu ? out[3 * VEC + tid] : 0.0;
+                        s_tol[tid] = P.tol2 * (neu ? fmax(ff - sf * sf / (double)N, 0.0) : ff);
                     } else if (!s_flag[tid]) {
                         s_it[tid] += 1;
                     }
