@@ -145,8 +145,8 @@ struct CcArgs {
 };
 
 // T: type of the potential x and of the residual f - K x; W: type of the CG
-// vectors and of an iteration's sums inside a CTA (the residual's, its reference's and
-// the gauge's are FP64).  T = W: CG to the tolerance.  T = double,
+// vectors and of an iteration's sums inside a CTA (the residual's and its reference's are
+// SumOf's, the gauge's FP64).  T = W: CG to the tolerance.  T = double,
 // W = float: cycles of the FP64 residual and FP32 CG until it has reduced that
 // residual by MP_INNER; the solve ends on the FP64 residual test.
 template <typename T, typename W, int VEC>
@@ -221,7 +221,8 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
         }
         int par = 0;
         // Totals over the cluster of NQ quantities of VEC columns into out[(q0 + q) * VEC + k];
-        // of W, or of FP64 (two W words of scr hold one: at most CC_NQ / 2 quantities).
+        // of W, or of what keeps more (SumOf, FP64; two FP32 words of scr hold one: at most
+        // CC_NQ / 2 quantities then).
         auto reduce = [&](auto& v, int q0) {
             constexpr int NQ = sizeof(v) / sizeof(v[0]), NV = NQ * VEC;
             using X = typename std::remove_reference<decltype(v[0][0])>::type;
@@ -232,16 +233,17 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
 #pragma unroll
                 for (int k = 0; k < VEC; ++k) {
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) v[a][k] += __shfl_xor_sync(0xffffffffu, v[a][k], o);
+                    for (int o = 16; o > 0; o >>= 1) v[a][k] = plus(v[a][k], shfl_x(v[a][k], o));
                     if (lane == 0) sc[warp * NV + a * VEC + k] = v[a][k];
                 }
             __syncthreads();
             const uint32_t sl = cc_addr(slots + par * CC_NQ * VEC * CC_MAX_CL);
             for (int w = warp; w < NV; w += nw) {
-                X t = lane < nw ? sc[lane * NV + w] : X(0);
+                X t{};
+                if (lane < nw) t = sc[lane * NV + w];
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-                if (lane < g.cl) cc_st(cc_peer(sl + (uint32_t)(w * CC_MAX_CL + (int)rank) * 8u, (unsigned)lane), (double)t);
+                for (int o = 16; o > 0; o >>= 1) t = plus(t, shfl_x(t, o));
+                if (lane < g.cl) cc_st(cc_peer(sl + (uint32_t)(w * CC_MAX_CL + (int)rank) * 8u, (unsigned)lane), total(t));
             }
             cc_sync();
             for (int w = warp; w < NV; w += nw) {
@@ -313,12 +315,8 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
             }
         cc_sync();
         for (int cycle = 0;; ++cycle) {
-            {   // residual of the current x into r; FP64 sums r.r, r and f.f, f (f: the norm reference)
-                double v[2][VEC], vf[2][VEC];
-#pragma unroll
-                for (int a = 0; a < 2; ++a)
-#pragma unroll
-                    for (int k = 0; k < VEC; ++k) v[a][k] = vf[a][k] = 0.0;
+            {   // residual of the current x into r; sums r.r, r and f.f, f (f: the norm reference)
+                typename SumOf<W>::type v[2][VEC], vf[2][VEC];
                 for (int l = tid; l < cnt; l += nt) {
                     const int row = lo + l;
                     W rv[VEC];
@@ -329,15 +327,18 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
                     } else {
                         const T* kvT = GenTab<T>::k(P.M);
                         T xi[VEC], kx[VEC];
-                        double f[VEC], ks[VEC];
+                        double f[VEC];
+                        typename SumOf<T>::type ks[VEC];
                         cc_get<VEC, true>(xi, x + (size_t)row * C + c0);
 #pragma unroll
                         for (int k = 0; k < VEC; ++k) {
                             kx[k] = T(0);
-                            f[k] = ks[k] = 0.0;
+                            f[k] = 0.0;
                         }
                         const int e0 = P.M.kptr[row], e1 = P.M.kptr[row + 1];
-#pragma unroll 4
+                        // entries in flight; with four, wider FP32 vectors spill in every product
+                        constexpr int RU = sizeof(W) == 8 || (VEC == 1 && !MP) ? 4 : 2;
+#pragma unroll RU
                         for (int e = e0; e < e1; ++e) {
                             const int j = (int)((unsigned)__ldg(&P.M.kent[e]) >> 8);
                             const T kv = __ldg(&kvT[e]);
@@ -347,7 +348,7 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
 #pragma unroll
                             for (int k = 0; k < VEC; ++k) {
                                 kx[k] = cc_fma(kv, xj[k] - xi[k], kx[k]);
-                                if (s) ks[k] = fma((double)kv, (double)xj[k], ks[k]);   // K_IS x_S
+                                if (s) ks[k].fma(kv, xj[k]);   // K_IS x_S
                             }
                         }
                         if (!(mode == 1 && !neu)) {
@@ -360,13 +361,12 @@ __global__ void __launch_bounds__(sizeof(W) == 8 ? 512 : 1024, 1) k_cluster_cg(c
                         }
 #pragma unroll
                         for (int k = 0; k < VEC; ++k) {
-                            const T rt = T(f[k]) - kx[k];
-                            rv[k] = W(rt);
-                            const double rd = (double)rt, ref = f[k] - ks[k];
-                            v[0][k] = fma(rd, rd, v[0][k]);
-                            v[1][k] += rd;
-                            vf[0][k] = fma(ref, ref, vf[0][k]);
-                            vf[1][k] += ref;
+                            rv[k] = W(T(f[k]) - kx[k]);
+                            const W ref = W(T(f[k]) - scaled(T(1), ks[k]));
+                            v[0][k].fma(rv[k], rv[k]);
+                            v[1][k].add(rv[k]);
+                            vf[0][k].fma(ref, ref);
+                            vf[1][k].add(ref);
                         }
                     }
                     cc_put<VEC>(r + (size_t)l * VEC, rv);

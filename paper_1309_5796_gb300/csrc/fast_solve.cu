@@ -125,60 +125,6 @@ __device__ __forceinline__ void st4(double* p, const double (&v)[4]) {
 __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// Sums that have to be better than FP32's: FP64 of FP64 values, or, of FP32 ones,
-// pairs of FP32 words with every rounding kept (Knuth's TwoSum, the product's error by
-// FMA), 48 bits at a sixth of the time of GB300's FP64 units.
-struct Pair {
-    float s = 0.f, e = 0.f;
-    __device__ __forceinline__ void add(float x) {
-        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
-        e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
-        s = t;
-    }
-    __device__ __forceinline__ void fma(float a, float b) {
-        const float p = __fmul_rn(a, b);
-        add(p);
-        e = __fadd_rn(e, __fmaf_rn(a, b, -p));
-    }
-};
-struct Sum64 {
-    double s = 0.0;
-    __device__ __forceinline__ void add(double x) { s += x; }
-    __device__ __forceinline__ void fma(double a, double b) { s = __fma_rn(a, b, s); }
-};
-template <typename T> struct SumOf { using type = Sum64; };
-template <> struct SumOf<float> { using type = Pair; };
-__device__ __forceinline__ float shfl_x(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
-__device__ __forceinline__ double shfl_x(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
-__device__ __forceinline__ Pair shfl_x(Pair v, int o) {
-    v.s = shfl_x(v.s, o);
-    v.e = shfl_x(v.e, o);
-    return v;
-}
-__device__ __forceinline__ Sum64 shfl_x(Sum64 v, int o) {
-    v.s = shfl_x(v.s, o);
-    return v;
-}
-__device__ __forceinline__ float plus(float a, float b) { return a + b; }
-__device__ __forceinline__ double plus(double a, double b) { return a + b; }
-__device__ __forceinline__ Sum64 plus(Sum64 a, Sum64 b) {
-    a.s += b.s;
-    return a;
-}
-__device__ __forceinline__ Pair plus(Pair a, Pair b) {   // the same bits either way round
-    const float e = __fadd_rn(a.e, b.e);
-    a.e = 0.f;
-    a.add(b.s);
-    a.e = __fadd_rn(a.e, e);
-    return a;
-}
-__device__ __forceinline__ float scaled(float a, Pair v) { return __fmaf_rn(a, v.s, __fmul_rn(a, v.e)); }
-__device__ __forceinline__ double scaled(double a, Sum64 v) { return a * v.s; }
-__device__ __forceinline__ double total(float v) { return (double)v; }
-__device__ __forceinline__ double total(double v) { return v; }
-__device__ __forceinline__ double total(Sum64 v) { return v.s; }
-__device__ __forceinline__ double total(Pair v) { return (double)v.s + (double)v.e; }
-
 // VEC consecutive columns of one row; CG: through L2 (values other CTAs write)
 template <int VEC, bool CG, typename X>
 __device__ __forceinline__ void ldc(X (&d)[VEC], const X* p) {
