@@ -130,9 +130,9 @@ typedef struct {
                                refinement to the same residual tests (at least one step a
                                solve).  0 on an uploaded mesh: CG with a Chebyshev
                                polynomial as preconditioner, one cluster per group of
-                               systems, to the same tests; on meshes of more than 65 000
-                               nodes (80 000 to 100 000 with FP32 work vectors) and for
-                               plain FP64 batches too wide for the chip's clusters 2 where
+                               systems, to the same tests; for plain FP64 batches too
+                               wide for the chip's clusters, and in FP64 on meshes of
+                               more than 65 000 nodes (80 000 with cg_mixed_iter), 2 where
                                it qualifies, else 1.  Results agree to the solves'
                                tolerance.  The solve of lbm_mesh_shell has one kernel,
                                whatever this says */

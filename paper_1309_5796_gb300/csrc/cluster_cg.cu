@@ -746,10 +746,13 @@ void cc_try(int rows, int cols, const int* emax, CcChoice& best, double& best_co
 // 46 656 62 / 55, on 50 653 70 / 64; 1 by 4, 25 on 9 261 20.3 / 24.4, 24 on 24 389 59.9 /
 // 57.3; one or two waves 1.0 to 2.3 times faster here over 60 such shapes of 343 to 42 875
 // nodes; one on 74 088 46.7 / 37.5, on 59 319 36.7 / 34.5.  Iterated in FP32: one on 74 088 26.5
-// / 25.8, on 91 125 33.5 / 31.8, five 61 / 44; FP32: one on 91 125 17.3 / 16.6, eight 54 / 41,
-// four on 117 649 57 / 31, one on 166 375 45 / 23.
+// / 25.8, on 91 125 33.5 / 31.8, five 61 / 44, one on 166 375 99 / 44.  FP32 solves stay here at
+// any size: there Jacobi-CG of one reduction a product does not always come to its tolerance
+// (fields off by 1.4e-6 here and up to 2e-5 there for one instance on 117 649 nodes, 1e-2 for
+// five, after 5000 iterations; on 166 375 45 ms here, 23 there, both within 2e-6).
 bool cc_slower(int rows, int cols, int vec, int waves, bool fp32, bool fp64_vectors) {
-    if (!fp64_vectors) return rows > (fp32 && cols < 16 ? 100000 : 80000);
+    if (fp32) return false;
+    if (!fp64_vectors) return rows > 80000;
     const bool wide = cols >= 100 || rows >= 14000 || (cols >= 80 && rows >= 10000);
     return rows > 65000 || waves >= 5 || (wide && waves >= (vec == 2 ? 3 : 4)) || (rows >= 45000 && waves >= 3);
 }
